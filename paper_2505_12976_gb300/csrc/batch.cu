@@ -310,14 +310,14 @@ __device__ void closure(E* __restrict__ W, int32_t mp, BatchSmem& sm) {
     __syncthreads();
     for (int32_t t = g; t < 2 * (nb - 1); t += kGroups) {  // row, then column panel tiles
       if (t < nb - 1)
-        Ops::update(W, mp, r, t + (t >= r), r, ts, lt, bar);
+        tiles::tile_update(W, mp, r, t + (t >= r), r, ts, lt, bar);
       else
-        Ops::update(W, mp, (t - (nb - 1)) + ((t - (nb - 1)) >= r), r, r, ts, lt, bar);
+        tiles::tile_update(W, mp, (t - (nb - 1)) + ((t - (nb - 1)) >= r), r, r, ts, lt, bar);
     }
     __syncthreads();
     for (int32_t t = g; t < (nb - 1) * (nb - 1); t += kGroups) {
       int32_t i = t / (nb - 1), j = t % (nb - 1);
-      Ops::update(W, mp, i + (i >= r), j + (j >= r), r, ts, lt, bar);
+      tiles::tile_update(W, mp, i + (i >= r), j + (j >= r), r, ts, lt, bar);
     }
     __syncthreads();
   }

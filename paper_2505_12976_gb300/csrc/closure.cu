@@ -6,9 +6,13 @@
 // else 0. They are packed into a zero-padded square workspace W (int16 when
 // every count fits in 15 bits, else int32) whose rows and columns follow a
 // relabeling of the candidates: candidates with at least one outgoing edge
-// first, then those without (ids kept in order inside each group). The
-// closure commutes with relabeling, and rows without edges stay zero, so
-// their tiles are never touched.
+// first, strongest first (most outgoing edges, or most ballots), then those
+// without edges in id order. The closure commutes with relabeling, and rows
+// without edges stay zero, so their tiles are never touched. The order
+// among the warm candidates puts like widths into the same 64 x 64 tiles: a
+// majority graph is close to an order, so below the diagonal most tiles are
+// zero, and above it a tile's smallest entry soon reaches what a further
+// pivot block could offer, which lets most tile updates be skipped (below).
 //
 // Only the candidates with edges (the "warm" ones, nw of them) need work:
 // rows of cold candidates are zero in W and in p. W holds the warm rows only
@@ -36,16 +40,26 @@
 //   3. updates every other tile: X(i, j) = max(X, W(i, r) (x) W(r, j)),
 // where (x) is the (max, min) product. Widths only grow and every value
 // written is the width of a real path, so the order of the updates inside a
-// phase does not matter and the result is the exact closure. An update whose
-// operand tile is all zero cannot change anything and is skipped.
+// phase does not matter and the result is the exact closure. An update
+// cannot change anything when min(max A, max B) <= min X over the tiles'
+// entries, and is skipped; each tile's progress word carries its largest and
+// smallest entry for that test. Updates left by it, of nb^3 (counted on the
+// CPU, blocked Floyd-Warshall): 0.9% for Plackett-Luce Zipf(1.1) top-20 lists
+// at m = 8192, 3.7% at m = 2048, 4.6% for top-200 lists at m = 2048, 2.1% for
+// Mallows(0.98) full rankings and 92% for impartial culture at m = 1024. The
+// closure went from 390 to 10.8 ms at m = 16384 (int32, top-20, 0.7% of the
+// updates left) and from 309 to 13.0 ms at m = 18407 (int16, top-200, 4%); it
+// is now bound by the chain diagonal tile - panels - next diagonal tile of
+// its 256 to 288 rounds, about 40 us each. Where every update is needed
+// (uniform random d, m = 8192) the tests and bounds cost 5%.
 //
 // All rounds run in ONE persistent cooperative launch: the CTAs take work
 // items from a global queue in a fixed order in which the next round's
 // diagonal and panel items come right after the current round's tiles in
 // that row and column ("lookahead"), so they overlap the rest of the round.
-// Each tile carries a progress word (rounds applied, plus a nonzero bit); an
-// item waits (bounded, clock-limited spin) until the tiles it reads have
-// reached its round. Every wait is on an item earlier in the queue, which a
+// Each tile carries a progress word (rounds applied, bounds of its entries);
+// an item, up to 32 tiles of one tile row or column, waits (bounded,
+// clock-limited spin) until the tiles it reads have reached its round. Every wait is on an item earlier in the queue, which a
 // resident CTA already holds, so the schedule cannot deadlock.
 #include <cooperative_groups.h>
 
@@ -63,17 +77,33 @@ namespace {
 using tiles::kB;        // block / tile size
 using tiles::kThreads;  // threads per CTA
 using tiles::BlockBarrier;
+using tiles::Bounds;
 using tiles::Ops;
-using tiles::diag_closure;
 using tiles::diag_closure_local;
 
-constexpr uint32_t kNZ = 1u << 30;         // progress word: tile has a nonzero entry
-constexpr uint32_t kRoundMask = kNZ - 1u;  // progress word: rounds applied
+// Progress word of a tile: rounds applied (12 bits), then the largest entry
+// (rounded up) and the smallest (rounded down) as 26-bit values of
+// 2^shift each, shift chosen so that the bound on the counts fits.
+constexpr int kBoundBits = 26;
+constexpr uint32_t kBoundMax = (1u << kBoundBits) - 1u;
+
+__device__ __forceinline__ uint64_t make_word(uint32_t rounds, Bounds b, int shift) {
+  const uint32_t mx = min((uint32_t(max(b.mx, 0)) + ((1u << shift) - 1u)) >> shift, kBoundMax);
+  const uint32_t mn = min(uint32_t(max(b.mn, 0)) >> shift, kBoundMax);
+  return (uint64_t(rounds) << (2 * kBoundBits)) | (uint64_t(mx) << kBoundBits) | mn;
+}
+__device__ __forceinline__ uint32_t word_rounds(uint64_t w) { return uint32_t(w >> (2 * kBoundBits)); }
+__device__ __forceinline__ uint32_t word_max(uint64_t w) { return uint32_t(w >> kBoundBits) & kBoundMax; }
+__device__ __forceinline__ uint32_t word_min(uint64_t w) { return uint32_t(w) & kBoundMax; }
+__device__ __forceinline__ uint64_t word_at(uint64_t w, uint32_t rounds) {  // the same bounds, more rounds applied
+  return (w & ((uint64_t(1) << (2 * kBoundBits)) - 1u)) | (uint64_t(rounds) << (2 * kBoundBits));
+}
+
 constexpr long long kSpinLimitCycles = 4000000000LL;  // ~2 s at 2 GHz, unless the context sets another
 
 // ------------------------------------------------------------ relabel
 
-// rowflag[i] = 1 iff candidate i has an outgoing edge (some j with
+// rowflag[i] = the number of outgoing edges of candidate i (the j with
 // d[i][j] > d[j][i]); also reports SCHULZE_EDATA for an entry outside
 // [0, bound]. Each CTA takes 64 x 64 block pairs (A, B), A <= B: thread
 // (r, c) holds d[A+r][B+c..c+3] and d[B+r][A+c..c+3] in registers (16-byte
@@ -130,19 +160,19 @@ __global__ void __launch_bounds__(256) rowflag_kernel(const int32_t* __restrict_
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int r = rq + 16 * q;
-      bool e0 = false, e1 = false;
+      uint32_t e = 0;  // side 0 in the low half, side 1 in the high half
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int c = c4 + e;
-        e0 |= (A + r != B + c) && x1[q][e] > T[c][r];
-        if (A != B) e1 |= x2[q][e] > t1[c][r];
+      for (int x = 0; x < 4; ++x) {
+        const int c = c4 + x;  // (on the diagonal both sides are the same entry: not counted)
+        e += x1[q][x] > T[c][r] ? 1u : 0u;
+        if (A != B) e += x2[q][x] > t1[c][r] ? 0x10000u : 0u;
       }
       // padding entries are 0 on both sides, so they never count
-      const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, e0), b1 = __ballot_sync(0xFFFFFFFFu, e1);
+#pragma unroll
+      for (int o = 8; o; o >>= 1) e += __shfl_xor_sync(0xFFFFFFFFu, e, o);
       if ((lane & 15) == 0) {
-        const uint32_t sh = lane & 16;
-        if ((b0 >> sh) & 0xFFFFu) atomicOr(&rowflag[A + r], 1);
-        if ((b1 >> sh) & 0xFFFFu) atomicOr(&rowflag[B + r], 1);
+        if (e & 0xFFFFu) atomicAdd(&rowflag[A + r], int32_t(e & 0xFFFFu));
+        if (e >> 16) atomicAdd(&rowflag[B + r], int32_t(e >> 16));
       }
     }
     __syncthreads();
@@ -150,27 +180,56 @@ __global__ void __launch_bounds__(256) rowflag_kernel(const int32_t* __restrict_
   if (bad) set_status(status, SCHULZE_EDATA);
 }
 
-// Stable partition: perm[new] = old, candidates with edges first; inv[old] = new.
-// The flags come from rowflag_kernel; when the tally set *hint_valid it has
-// written the relabeling of its own flags already, and this launch returns.
+// perm[new] = old, inv[old] = new: candidates with edges first, strongest
+// first, then the others in id order. Strength is the number of outgoing
+// edges (rowflag_kernel), or, when the tally set *hint_valid, the number of
+// ballots that list the candidate (hint). It is sorted by counting over
+// kStrengths classes (equal sizes for edge counts, relative steps of 1/128
+// for ballots; any order inside a class): the closure needs like candidates
+// near each other, not an exact order. The tally has written a warm-first
+// relabeling already when its hint is valid; it is kept where the cluster
+// closure takes the whole warm square (warm_max), whose cost does not depend
+// on the order.
+constexpr int kStrengths = 4096;
+
+__device__ __forceinline__ int strength_class(uint32_t x, bool ballots, int32_t m) {
+  if (ballots) {  // x >= 1: exponent and the seven bits after the leading one
+    const int lz = __clz(x);
+    return kStrengths - 1 - ((31 - lz) * 128 + int((x << lz >> 24) & 127u));
+  }
+  return kStrengths - 1 - int(uint64_t(x) * kStrengths / uint64_t(m));  // x < m
+}
+
 __global__ void __launch_bounds__(1024) relabel_kernel(const int32_t* __restrict__ rowflag, int32_t m,
                                                        int32_t* __restrict__ perm, int32_t* __restrict__ inv,
                                                        int32_t* __restrict__ warm_out,
-                                                       const int32_t* __restrict__ hint_valid) {
+                                                       const int32_t* __restrict__ hint,
+                                                       const int32_t* __restrict__ hint_valid, int32_t warm_max) {
   pdl_enter_early();
   __shared__ uint32_t part[33];
+  __shared__ uint32_t cls[kStrengths];
   extern __shared__ uint32_t relabel_smem[];  // m words when m <= kScanSmem
-  if (hint_valid && *hint_valid) return;
+  const bool hv = hint_valid && *hint_valid;
+  if (hv && *warm_out <= warm_max) return;
+  const int32_t* strength = hv ? hint : rowflag;
   // rank[c] = 1 for warm c, scanned into the warm rank (in shared memory, or
   // in place in inv for long candidate lists)
   uint32_t* rank = m <= kScanSmem ? relabel_smem : reinterpret_cast<uint32_t*>(inv);
-  for (int32_t c = threadIdx.x; c < m; c += blockDim.x) rank[c] = rowflag[c] ? 1u : 0u;
+  for (int t = threadIdx.x; t < kStrengths; t += blockDim.x) cls[t] = 0u;
+  __syncthreads();
+  for (int32_t c = threadIdx.x; c < m; c += blockDim.x) {
+    const int32_t x = strength[c];
+    rank[c] = x ? 1u : 0u;
+    if (x) atomicAdd(&cls[strength_class(uint32_t(x), hv, m)], 1u);
+  }
   __syncthreads();
   const int32_t warm = int32_t(block_exclusive_scan(rank, m, part));
+  block_exclusive_scan(cls, kStrengths, part);
   if (threadIdx.x == 0) *warm_out = warm;
   for (int32_t c = threadIdx.x; c < m; c += blockDim.x) {
-    const int32_t before = int32_t(rank[c]);                 // warm candidates before c
-    const int32_t nw = rowflag[c] ? before : warm + (c - before);  // cold ones keep their order
+    const int32_t x = strength[c];
+    const int32_t nw = x ? int32_t(atomicAdd(&cls[strength_class(uint32_t(x), hv, m)], 1u))
+                         : warm + (c - int32_t(rank[c]));  // rank[c] warm candidates before c
     perm[nw] = c;
     inv[c] = nw;
   }
@@ -180,8 +239,10 @@ __global__ void __launch_bounds__(1024) relabel_kernel(const int32_t* __restrict
 // m x m, on the diagonal and where d does not beat its transpose; w is d, or
 // the margin d - d^T with `margin`). One CTA
 // pass per row a: with x = perm[a], the threads walk b, reading d[x][perm b]
-// (along row x) and d[perm b][x] (down column x); a warp that writes a
-// nonzero sets the nonzero bit of its 64 x 64 tile's progress word.
+// (along row x) and d[perm b][x] (down column x), and each warp adds its part
+// of the bounds of the 64 x 64 tile to tmax and tmin (tmin holds INT32_MAX -
+// min, so that both start at zero): the largest entry, and the smallest one
+// among the warm rows and the existing columns, off the diagonal.
 //
 // With the tally's flags (hint valid), a candidate y without edges is one no
 // ballot lists, so d[y][x] = 0 and that read is skipped.
@@ -190,7 +251,8 @@ __global__ void __launch_bounds__(1024) relabel_kernel(const int32_t* __restrict
 template <typename E>
 __global__ void __launch_bounds__(512) pack_kernel(const int32_t* __restrict__ d, int32_t m, int32_t mp,
                                                    const int32_t* __restrict__ perm, const int32_t* __restrict__ warm,
-                                                   E* __restrict__ W, uint32_t* __restrict__ prog, int32_t nb,
+                                                   E* __restrict__ W, int32_t* __restrict__ tmax,
+                                                   int32_t* __restrict__ tmin, int32_t nb,
                                                    const int32_t* __restrict__ hint,
                                                    const int32_t* __restrict__ hint_valid, int32_t* __restrict__ ucol,
                                                    int margin) {
@@ -223,7 +285,13 @@ __global__ void __launch_bounds__(512) pack_kernel(const int32_t* __restrict__ d
         const int32_t b = b0 + q * blockDim.x + threadIdx.x;
         const int32_t out = v[q] > u[q] ? (margin ? v[q] - u[q] : v[q]) : 0;
         if (b < bend) wrow[b] = E(out);
-        if (__any_sync(0xFFFFFFFFu, out != 0) && lane == 0) atomicOr(&prog[(a / kB) * nb + (b / kB)], kNZ);
+        const int32_t mx = __reduce_max_sync(0xFFFFFFFFu, out);
+        const int32_t mn = __reduce_min_sync(0xFFFFFFFFu, a < *warm && b < m && b != a ? out : INT32_MAX);
+        if (lane == 0 && b < bend) {
+          const int32_t t = (a / kB) * nb + b / kB;
+          if (mx > 0) atomicMax(&tmax[t], mx);
+          if (mn < INT32_MAX) atomicMax(&tmin[t], INT32_MAX - max(mn, 0));
+        }
       }
     }
   }
@@ -310,154 +378,158 @@ __global__ void __launch_bounds__(256) widen_kernel(const E* __restrict__ W, int
 
 // ----------------------------------------------------- work queue
 
-enum ItemKind : int32_t { kDiag = 0, kPanel = 1, kTile = 2 };
+enum ItemKind : int32_t { kDiag = 0, kPanel = 1, kTile = 2, kStop = 3 };
+
+// A work item: cnt tiles in round r, with the running index v0 + t * stride
+// for tile t. The index runs along tile row or column fix, or (kGrid) over
+// the n x n tiles of R(r) row by row; tile indices are counted without the
+// `skip` indices r, r + 1, ...
+enum ItemShape : int32_t { kRow = 0, kColumn = 1, kGrid = 2 };
 struct Item {
-  int32_t kind, r, i, j;
+  int32_t kind, r, shape, fix, v0, stride, cnt, skip, n;
+  __device__ __forceinline__ void tile(int32_t t, int32_t& i, int32_t& j) const {
+    int32_t x = v0 + t * stride, y = fix;
+    if (shape == kGrid) y = x / n, x -= y * n, y = y < r ? y : y + skip;
+    x = x < r ? x : x + skip;
+    i = shape == kColumn ? x : y, j = shape == kColumn ? y : x;
+  }
 };
 
 // The candidates with outgoing edges occupy the first nbr tile rows after
 // relabeling; the other rows of W are zero and stay zero, and a round over a
 // block of them cannot change anything (min(x, 0) = 0). So rounds run over
-// r < nbr and only tile rows i < nbr are updated. The queue is written for
-// nc >= nbr tile columns (nbr * nbr * nc items); the closure runs it on the
-// warm square (nc = nbr) and leaves the cold columns to cold_product_kernel.
+// r < nbr on the nbr x nbr tiles of the warm square; cold_product_kernel does
+// the cold columns.
 //
 // Queue order, stage by stage:
 //   stage 0:             D(0) P(0) L(0)
-//   stage s (1..nbr-1):  D(s) P(s) R(s-1) L(s)     (no L in the last one)
+//   stage s (1..nbr-2):  D(s) P(s) X(s-1) R(s-1) L(s)
+//   stage nbr-1:         D(s) P(s) R(s-1)
 //   stage nbr:           R(nbr-1)
-// D(r): diagonal tile; P(r): row panel (r, j != r) then column panel
-// (i < nbr, i != r); L(r): round-r tiles that are the next round's panels
-// (tile row r+1, then tile column r+1); R(r): the other round-r tiles.
+// D(r): diagonal tile; P(r): the panel tiles (r, r+1) and (r+1, r) the next
+// diagonal tile waits for, then the rest of row panel r and of column panel
+// r; L(r): round-r tiles that the next round's panels are made of, the next
+// diagonal tile (r+1, r+1) first, then tile row r+1, then tile column r+1;
+// X(r): the round-r tiles of tile row and column r+2, which L(r+1) is made
+// of, ahead of R(r): the other round-r tiles. P, L and X come in items of at
+// most gp tiles, R in items of at most gr: about two items per CTA and round,
+// or 16 where most tiles need their update (a round then ends with CTAs
+// waiting for its last items). One tile per item costs nothing at few tiles
+// and keeps the chain of the panels short; at many tiles the tests of 32
+// tiles, a lane each, cost one round trip to the progress words instead of 32
+// (a skipped tile by itself would take its CTA about a microsecond). The
+// tiles of an item are spread evenly over their range: those that need an
+// update lie next to each other (m = 16384 top-20: 480 of 65536 in a round),
+// and items of neighbours left some CTAs with most of them (the closure took
+// 28.5 ms, 10.8 ms spread).
 struct Shape {
-  int32_t nbr, nb;
-  int64_t P, L, Rmid, Rlast;
+  int32_t nbr, gp, gr;
+  int32_t sp, sp_last;  // items per panel side, r < nbr - 1 and r = nbr - 1 (no r + 1 to leave out)
+  int32_t xc;           // items of the column side of X (its row side has sp)
+  int32_t P, L;         // items of P(r), L(r), r < nbr - 1
+  int32_t X, R;         // items of X(r), R(r), r < nbr - 2
+  int32_t P_last, R_pen, R_last;  // P(nbr - 1), R(nbr - 2), R(nbr - 1)
 };
 
-__device__ __forceinline__ Shape make_shape(int32_t nbr, int32_t nb) {
+__device__ __forceinline__ Shape make_shape(int32_t nbr, int32_t grid, bool dense) {  // nbr >= 3
   Shape sh;
-  sh.nbr = nbr, sh.nb = nb;
-  sh.P = int64_t(nb - 1) + (nbr - 1);
-  sh.L = int64_t(nb - 1) + (nbr - 2);
-  sh.Rmid = int64_t(nbr - 2) * (nb - 2);
-  sh.Rlast = int64_t(nbr - 1) * (nb - 1);
+  sh.nbr = nbr;
+  sh.gr = min(32, max(1, nbr * nbr / ((dense ? 16 : 2) * grid)));
+  sh.gp = min(4, max(1, nbr / 64));
+  const int32_t q = nbr - 2;
+  sh.sp = (q + sh.gp - 1) / sh.gp, sh.sp_last = (q + sh.gp) / sh.gp;
+  sh.xc = (q - 1 + sh.gp - 1) / sh.gp;
+  sh.P = 2 + 2 * sh.sp, sh.L = 1 + 2 * sh.sp, sh.P_last = 2 * sh.sp_last;
+  sh.X = sh.sp + sh.xc, sh.R = ((q - 1) * (q - 1) + sh.gr - 1) / sh.gr;
+  sh.R_pen = (q * q + sh.gr - 1) / sh.gr, sh.R_last = ((q + 1) * (q + 1) + sh.gr - 1) / sh.gr;
   return sh;
 }
 
-__device__ __forceinline__ int64_t stage_size(int32_t s, const Shape& sh) {
-  int64_t z = 0;
-  if (s < sh.nbr) z += 1 + sh.P;
-  if (s >= 1) z += (s - 1 < sh.nbr - 1) ? sh.Rmid : sh.Rlast;
-  if (s < sh.nbr - 1) z += sh.L;
-  return z;
+__device__ __forceinline__ uint32_t queue_items(const Shape& sh) {
+  return uint32_t(sh.nbr) + uint32_t(sh.nbr - 1) * uint32_t(sh.P + sh.L) +
+         uint32_t(sh.nbr - 2) * uint32_t(sh.X + sh.R) + uint32_t(sh.P_last + sh.R_pen + sh.R_last);
 }
 
-__device__ Item decode_item(int64_t t, const Shape& sh) {
-  const int32_t nbr = sh.nbr, nb = sh.nb;
-  int32_t s;
-  const int64_t s0 = stage_size(0, sh);
-  if (t < s0) {
-    s = 0;
-  } else {
-    t -= s0;
-    const int64_t mid = int64_t(nbr) * nb;  // stages 1 .. nbr-2 all hold nbr * nb items
-    const int64_t nmid = nbr >= 2 ? nbr - 2 : 0;
-    if (t < nmid * mid) {
+// item t of the queue, t < queue_items(sh)
+__device__ Item decode_item(uint32_t t, const Shape& sh) {
+  const int32_t nbr = sh.nbr, q = nbr - 2;
+  const uint32_t first = 1 + sh.P + sh.L, mid = first + sh.X + sh.R;
+  int32_t s = 0;
+  if (t >= first) {
+    t -= first;
+    if (t < uint32_t(q) * mid) {
       s = 1 + int32_t(t / mid);
-      t -= int64_t(s - 1) * mid;
+      t -= uint32_t(s - 1) * mid;
     } else {
-      t -= nmid * mid;
-      s = 1 + int32_t(nmid);
-      const int64_t z = stage_size(s, sh);
-      if (t >= z) {
-        t -= z;
-        s += 1;
-      }
+      t -= uint32_t(q) * mid;
+      s = nbr - 1;
+      const uint32_t z = 1 + sh.P_last + sh.R_pen;
+      if (t >= z) t -= z, s = nbr;
     }
   }
-  Item it{kDiag, 0, 0, 0};
+  const bool last = s == nbr - 1;
+  auto one = [](int32_t kind, int32_t r, int32_t i, int32_t j) { return Item{kind, r, kRow, i, j, 0, 1, 0, 0}; };
+  // item a of the `items` that share the n tiles (or n x n) of a range
+  auto part = [](int32_t kind, int32_t r, int32_t shape, int32_t fix, int32_t a, int32_t items, int32_t n, int32_t skip) {
+    const int32_t range = shape == kGrid ? n * n : n;
+    return Item{kind, r, shape, fix, a, items, (range - a + items - 1) / items, skip, n};
+  };
   if (s < nbr) {
-    if (t == 0) {
-      it.kind = kDiag, it.r = s, it.i = s, it.j = s;
-      return it;
-    }
+    if (t == 0) return one(kDiag, s, s, s);
     t -= 1;
-    if (t < sh.P) {
-      it.kind = kPanel, it.r = s;
-      if (t < nb - 1) {
-        it.i = s, it.j = int32_t(t) + (t >= s);
-      } else {
-        const int32_t q = int32_t(t - (nb - 1));
-        it.i = q + (q >= s), it.j = s;
+    const uint32_t P = last ? sh.P_last : sh.P;
+    if (t < P) {
+      if (!last) {
+        if (t < 2) return t == 0 ? one(kPanel, s, s, s + 1) : one(kPanel, s, s + 1, s);
+        t -= 2;
       }
-      return it;
+      const int32_t sp = last ? sh.sp_last : sh.sp, a = int32_t(t);
+      return part(kPanel, s, a < sp ? kRow : kColumn, s, a < sp ? a : a - sp, sp, last ? q + 1 : q, last ? 1 : 2);
     }
-    t -= sh.P;
+    t -= P;
   }
   if (s >= 1) {
-    const int32_t r = s - 1;
-    it.kind = kTile, it.r = r;
-    if (r == nbr - 1) {
-      const int32_t wc = nb - 1;
-      if (t < sh.Rlast) {
-        const int32_t a = int32_t(t / wc), b = int32_t(t % wc);
-        it.i = a + (a >= r), it.j = b + (b >= r);
-        return it;
-      }
-      t -= sh.Rlast;
-    } else {
-      const int32_t wc = nb - 2;
-      if (t < sh.Rmid) {
-        const int32_t a = int32_t(t / wc), b = int32_t(t % wc);
-        it.i = a < r ? a : a + 2;
-        it.j = b < r ? b : b + 2;
-        return it;
-      }
-      t -= sh.Rmid;
+    const int32_t r = s - 1, skip = s == nbr ? 1 : last ? 2 : 3;
+    if (skip == 3) {
+      const int32_t a = int32_t(t);
+      if (a < sh.sp) return part(kTile, r, kRow, r + 2, a, sh.sp, q, 2);
+      if (a < sh.X) return part(kTile, r, kColumn, r + 2, a - sh.sp, sh.xc, q - 1, 3);
+      t -= sh.X;
     }
+    const int32_t R = skip == 1 ? sh.R_last : skip == 2 ? sh.R_pen : sh.R;
+    if (int32_t(t) < R) return part(kTile, r, kGrid, 0, int32_t(t), R, nbr - skip, skip);
+    t -= R;
   }
-  const int32_t r = s;  // L(s)
-  it.kind = kTile, it.r = r;
-  if (t < nb - 1) {
-    it.i = r + 1, it.j = int32_t(t) + (t >= r);
-  } else {
-    const int32_t q = int32_t(t - (nb - 1));
-    it.i = q < r ? q : q + 2, it.j = r + 1;
-  }
-  return it;
+  // L(s)
+  if (t == 0) return one(kTile, s, s + 1, s + 1);
+  const int32_t a = int32_t(t) - 1;
+  return part(kTile, s, a < sh.sp ? kRow : kColumn, s + 1, a < sh.sp ? a : a - sh.sp, sh.sp, q, 2);
 }
 
 struct Sync {
-  uint32_t* prog;                // [nb * nb] progress words
+  unsigned long long* prog;      // [nb * nb] progress words
+  const int32_t* tmax;           // [nb * nb] bounds of the packed tiles (pack_kernel)
+  const int32_t* tmin;
   uint32_t* head;                // queue head
   uint32_t* abort_flag;          // set when a wait times out
   int32_t* status;
   const int32_t* warm;           // candidates with outgoing edges
   unsigned long long* counters;  // [0] tile updates done, [1] diagonal closures done, [2] items
   long long spin_limit;          // clock cycles a wait may take before it gives up
+  int32_t shift;                 // progress word bounds are in units of 2^shift
 };
 
-// Thread 0 waits until prog[idx] has applied at least `need` rounds; returns
-// the word, or 0xFFFFFFFF after a timeout (which also raises the abort flag).
-__device__ uint32_t wait_round(const Sync& sy, int32_t idx, uint32_t need) {
-  const long long t0 = clock64();
-  for (;;) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(sy.prog + idx) : "memory");
-    if ((v & kRoundMask) >= need) return v;
-    if (*reinterpret_cast<volatile uint32_t*>(sy.abort_flag)) return 0xFFFFFFFFu;
-    if (clock64() - t0 > sy.spin_limit) {
-      set_status(sy.status, SCHULZE_ETIMEOUT);
-      atomicExch(sy.abort_flag, 1u);
-      return 0xFFFFFFFFu;
-    }
-    __nanosleep(64);
-  }
+// Progress words are read and written relaxed, with one fence between the
+// reads an item waits for and its work, and one between the work and its word
+// (an acquire per read would make the three reads of a test wait for one
+// another).
+__device__ __forceinline__ uint64_t load_word(const unsigned long long* p) {
+  uint64_t v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
 }
-
-__device__ __forceinline__ void publish(const Sync& sy, int32_t idx, uint32_t word) {
-  __threadfence();
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(sy.prog + idx), "r"(word) : "memory");
+__device__ __forceinline__ void store_word(unsigned long long* p, uint64_t v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 // Warm squares up to this size are closed by closure_cluster_kernel (the
@@ -466,148 +538,152 @@ __device__ __forceinline__ void publish(const Sync& sy, int32_t idx, uint32_t wo
 template <typename E>
 constexpr int32_t kClusterMaxWarm = sizeof(E) == 2 ? 256 : 192;
 
-// CTAs per SM: five for int32 lanes (at most 96 registers a thread; the
-// tile update needs 92), which measured fastest against four and six; seven
-// for packed int16 lanes (72 registers, as the unbounded build took)
-#define SCHULZE_PERSIST_BOUNDS __launch_bounds__(kThreads, sizeof(E) == 2 ? 7 : 5)
-// The next work item of a persistent CTA, as thread 0 prepares it while the
-// CTA computes the current one: the item, the progress words it waits for
-// (own tile: `need` rounds applied; panel: the closed diagonal; tile: both
-// panels) and their values as first loaded.
-struct Pending {
+// CTAs per SM: five for int32 lanes (at most 96 registers a thread), which
+// measured fastest against four and six; six for packed int16 lanes (80
+// registers; seven spill, uniform random d at m = 1000: 0.506 against 0.474
+// ms for the whole call, m = 8192: 29.15 against 29.41 ms)
+#define SCHULZE_PERSIST_BOUNDS __launch_bounds__(kThreads, sizeof(E) == 2 ? 6 : 5)
+
+// Warp 1 runs the schedule: it claims the CTA's next queue slot while the CTA
+// works on the current item, and between items its lane t waits for the
+// words tile t of the new item depends on (own tile: the rounds before;
+// panel: the closed diagonal; tile: both panels) and tests its bounds: a tile
+// that cannot change is passed on to the next round at once, the others are
+// computed one after another by the CTA and published by thread 0 as they are
+// done (the last one while warp 1 is at the next item already). The schedule
+// stays deadlock-free: every wait is on an item earlier in the queue, and a
+// CTA holds at most one claimed, unstarted item, later in the queue than its
+// current one, so the earliest unfinished item is always being worked on.
+struct Slot {  // an item and its tiles to compute
   Item it;
-  int32_t dep[3];
-  uint32_t need[3];
-  uint32_t val[3];
+  uint32_t mask;
 };
 
-__device__ __forceinline__ uint32_t load_acquire(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
+// warp 1: the item of queue slot t into *s (kStop at the end of the queue or
+// after a failed wait); out of line, as the tile update needs the registers
+__device__ __noinline__ void next_item(const Sync& sy, uint32_t t, int32_t nbr, int32_t nb, bool dense, Slot* s) {
+  const int lane = threadIdx.x & 31;
+  if (lane == 0) {
+    const Shape sh = make_shape(nbr, int32_t(gridDim.x), dense);
+    if (t >= queue_items(sh) || *reinterpret_cast<volatile uint32_t*>(sy.abort_flag)) s->it.kind = kStop;
+    else s->it = decode_item(t, sh);
+  }
+  __syncwarp();
+  const Item it = s->it;
+  const uint32_t r = uint32_t(it.r);
+  bool ok = true, need = false;
+  if (it.kind != kStop && lane < it.cnt) {
+    int32_t i, j;
+    it.tile(lane, i, j);
+    const int32_t own = i * nb + j;
+    const bool ta = it.kind != kDiag, tb = it.kind == kTile;
+    const int32_t da = it.kind == kTile ? i * nb + it.r : it.r * nb + it.r, db = it.r * nb + j;
+    uint64_t w0 = r ? load_word(sy.prog + own) : 0, w1 = ta ? load_word(sy.prog + da) : 0,
+             w2 = tb ? load_word(sy.prog + db) : 0;
+    const long long t0 = clock64();
+    for (;;) {
+      const bool m0 = word_rounds(w0) < r, m1 = ta && word_rounds(w1) <= r, m2 = tb && word_rounds(w2) <= r;
+      if (!(m0 || m1 || m2)) break;
+      if (*reinterpret_cast<volatile uint32_t*>(sy.abort_flag)) ok = false;
+      if (ok && clock64() - t0 > sy.spin_limit) {
+        set_status(sy.status, SCHULZE_ETIMEOUT);
+        atomicExch(sy.abort_flag, 1u);
+        ok = false;
+      }
+      if (!ok) break;
+      __nanosleep(32);
+      if (m0) w0 = load_word(sy.prog + own);
+      if (m1) w1 = load_word(sy.prog + da);
+      if (m2) w2 = load_word(sy.prog + db);
+    }
+    __threadfence();
+    if (r == 0) w0 = make_word(0, Bounds{sy.tmax[own], INT32_MAX - sy.tmin[own]}, sy.shift);
+    // what the update can offer at most, against the tile's smallest entry
+    const uint32_t offer = it.kind == kDiag    ? word_max(w0)
+                           : it.kind == kPanel ? min(word_max(w1), word_max(w0))
+                                               : min(word_max(w1), word_max(w2));
+    need = offer > (it.kind == kDiag ? 0u : word_min(w0));
+    if (ok && !need) store_word(sy.prog + own, word_at(w0, r + 1));
+  }
+  const uint32_t mask = __ballot_sync(0xFFFFFFFFu, need), fail = __ballot_sync(0xFFFFFFFFu, !ok);
+  if (lane == 0) {
+    s->mask = mask;
+    if (fail) s->it.kind = kStop;
+  }
 }
 
-template <typename E, int kMix>
-__global__ void SCHULZE_PERSIST_BOUNDS closure_persistent_kernel(E* __restrict__ W, int32_t ld, int32_t nb, Sync sy) {
+// Whether at least three quarters of the tile updates look needed: 128
+// triples of tiles, tested on the packed bounds (every CTA samples the same
+// ones).
+__device__ __forceinline__ bool sample_dense(const Sync& sy, int32_t nbr, int32_t nb) {
+  uint32_t h = (threadIdx.x + 1u) * 2654435761u;
+  auto draw = [&]() {
+    h ^= h >> 15, h *= 2246822519u, h ^= h >> 13;
+    return int32_t(h % uint32_t(nbr));
+  };
+  const int32_t i = draw(), k = draw(), j = draw();
+  const bool need = min(sy.tmax[i * nb + k], sy.tmax[k * nb + j]) > INT32_MAX - sy.tmin[i * nb + j];
+  return __syncthreads_count(need) >= kThreads * 3 / 4;
+}
+
+template <typename E>
+__global__ void SCHULZE_PERSIST_BOUNDS closure_persistent_kernel(E* W, int32_t ld, int32_t m, int32_t nb,
+                                                                 const __grid_constant__ Sync sy) {
   pdl_enter_early();
-  __shared__ __align__(16) typename Ops<E, kMix>::Smem sm;
+  __shared__ __align__(16) typename Ops<E>::Smem sm;
   __shared__ __align__(16) int32_t rowbuf[2][kB];
-  __shared__ int32_t s_item[2][4];  // kind, round, tile row, tile column (double-buffered)
-  __shared__ uint32_t s_flags[2];   // bit 0: skip the update; bit 1: tile already nonzero
-  __shared__ int32_t s_slow[2];     // the next item still has to wait (double-buffered)
-  constexpr uint32_t kFail = 0xFFFFFFFFu;
-  const int32_t nbr = (*sy.warm + kB - 1) / kB;
-  if (*sy.warm <= kClusterMaxWarm<E>) return;  // closure_cluster_kernel's case
-  const Shape sh = make_shape(nbr, nbr);  // the warm square; nb is the progress-word row stride
-  const int64_t total_items = int64_t(nbr) * nbr * nbr;
-  // Thread 0 runs the schedule. While the CTA computes item i it claims the
-  // next queue slot, decodes it and loads the progress words it depends on.
-  // After its own part of item i it looks at them again without waiting:
-  // when all are there, it writes the next item into the other half of the
-  // double buffer, which the barrier ending item i makes visible, so one
-  // barrier per item is left besides the operand barrier inside the update.
-  // When one is not there yet, nothing waits before item i is published (the
-  // missing tile may itself wait, through other CTAs, for item i): thread 0
-  // publishes, then waits (bounded) and hands the item over behind one more
-  // barrier. The schedule stays deadlock-free: a CTA holds at most one
-  // claimed, unstarted item, later in the queue than its current one, and
-  // only waits once its current item is published, so the earliest
-  // unfinished item is always being computed (its dependencies are earlier,
-  // hence finished) and completes.
-  __shared__ Pending nx;  // thread 0's alone (kept out of every thread's registers)
-  auto issue = [&](uint32_t t) {  // thread 0: claim decoded, dependencies' words loaded
-    nx.it = Item{-1, 0, 0, 0};
-    nx.dep[0] = nx.dep[1] = nx.dep[2] = -1;
-    if (int64_t(t) >= total_items || *reinterpret_cast<volatile uint32_t*>(sy.abort_flag)) return;
-    nx.it = decode_item(int64_t(t), sh);
-    const Item& it = nx.it;
-    const uint32_t r = uint32_t(it.r);
-    nx.dep[0] = it.i * nb + it.j, nx.need[0] = r;  // rounds 0 .. r-1 applied
-    if (it.kind == kPanel) {
-      nx.dep[1] = it.r * nb + it.r, nx.need[1] = r + 1;
-    } else if (it.kind == kTile) {
-      nx.dep[1] = it.i * nb + it.r, nx.need[1] = r + 1;
-      nx.dep[2] = it.r * nb + it.j, nx.need[2] = r + 1;
-    }
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-      if (nx.dep[q] >= 0) nx.val[q] = load_acquire(sy.prog + nx.dep[q]);
-  };
-  // thread 0, no waiting: every dependency of the next item there (those not
-  // seen yet are loaded once more)
-  auto ready = [&]() -> bool {
-    if (nx.it.kind < 0) return true;
-    bool all = true;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      if (nx.dep[q] < 0 || (nx.val[q] & kRoundMask) >= nx.need[q]) continue;
-      nx.val[q] = load_acquire(sy.prog + nx.dep[q]);
-      all = all && (nx.val[q] & kRoundMask) >= nx.need[q];
-    }
-    return all;
-  };
-  // thread 0: wait for what is still missing (bounded), decide the flags,
-  // write the next item into s_item[buf]
-  auto decide = [&](int buf) {
-    if (nx.it.kind >= 0) {
-      bool ok = true;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        if (nx.dep[q] < 0 || !ok || (nx.val[q] & kRoundMask) >= nx.need[q]) continue;
-        nx.val[q] = wait_round(sy, nx.dep[q], nx.need[q]);
-        ok = nx.val[q] != kFail;
+  // two slots: warp 1 writes the next one while the others read the current
+  __shared__ Slot s_slot[2];
+  __shared__ uint32_t s_done[3];  // tile updates, diagonal closures, items
+  __shared__ Bounds s_bd[2][kThreads / 32];
+  const int32_t nw = *sy.warm;
+  if (nw <= kClusterMaxWarm<E>) return;  // closure_cluster_kernel's case
+  const int32_t nbr = (nw + kB - 1) / kB;  // nb is the progress words' row stride
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const bool dense = sample_dense(sy, nbr, nb);
+  if (tid < 3) s_done[tid] = 0u;
+  uint32_t next = 0;  // warp 1, lane 0: the claimed queue slot
+  if (tid == 32) next = atomicAdd(sy.head, 1u);
+  for (int buf = 0, par = 0;; buf ^= 1) {
+    if (wid == 1) next_item(sy, next, nbr, nb, dense, &s_slot[buf]);
+    __syncthreads();
+    const Slot& sl = s_slot[buf];
+    const int32_t kind = sl.it.kind, r = sl.it.r;
+    if (kind == kStop) break;
+    if (tid == 32) next = atomicAdd(sy.head, 1u), ++s_done[2];  // in flight during this item
+    int32_t cur_a = -1, cur_b = -1;  // staged operand tiles: (cur_a, r) and (r, cur_b)
+    for (uint32_t mask = sl.mask; mask; mask &= mask - 1) {
+      int32_t i, j;
+      sl.it.tile(__ffs(int(mask)) - 1, i, j);
+      Bounds bd;
+      const int32_t vr = nw - i * kB, vc = m - j * kB;  // candidates with edges / candidates from the tile's corner on
+      E* Cg = W + int64_t(i) * kB * ld + int64_t(j) * kB;
+      if (kind == kDiag) {
+        diag_closure_local<E>(W, ld, r, vr, vc, rowbuf, tid, BlockBarrier{}, bd);
+      } else {
+        // the tiles of a panel side share an operand
+        if (cur_a != i) Ops<E>::load_a(W + int64_t(i) * kB * ld + int64_t(r) * kB, ld, sm, tid);
+        if (cur_b != j) Ops<E>::load_b(W + int64_t(r) * kB * ld + int64_t(j) * kB, ld, sm, tid);
+        cur_a = i, cur_b = j;
+          Ops<E>::template multiply<true>(Cg, ld, sm, tid, BlockBarrier{}, bd, i == j || vr < kB || vc < kB, i == j,
+                                          vr, vc);
       }
-      if (!ok) nx.it.kind = -1;
-    }
-    uint32_t flags = 0;
-    if (nx.it.kind >= 0) {
-      __threadfence();
-      const uint32_t own = nx.val[0];
-      if (nx.it.kind == kDiag) {
-        if (!(own & kNZ)) flags |= 1u;
-      } else if (nx.it.kind == kPanel) {
-        if (!(nx.val[1] & kNZ) || !(own & kNZ)) flags |= 1u;
-      } else if (!(nx.val[1] & kNZ) || !(nx.val[2] & kNZ)) {
-        flags |= 1u;
+      const int32_t mx = __reduce_max_sync(0xFFFFFFFFu, bd.mx), mn = __reduce_min_sync(0xFFFFFFFFu, bd.mn);
+      if (lane == 0) s_bd[par][wid] = Bounds{mx, mn};
+      __syncthreads();  // every store of the tile and its bounds done, operands free
+      if (tid == 0) {
+        Bounds b = s_bd[par][0];
+#pragma unroll
+        for (int w = 1; w < kThreads / 32; ++w) b.mx = max(b.mx, s_bd[par][w].mx), b.mn = min(b.mn, s_bd[par][w].mn);
+        __threadfence();
+        store_word(sy.prog + (i * nb + j), make_word(r + 1, b, sy.shift));
+        ++s_done[kind == kDiag ? 1 : 0];
       }
-      if (own & kNZ) flags |= 2u;
+      par ^= 1;
     }
-    s_item[buf][0] = nx.it.kind, s_item[buf][1] = nx.it.r, s_item[buf][2] = nx.it.i, s_item[buf][3] = nx.it.j;
-    s_flags[buf] = flags;
-  };
-  if (threadIdx.x == 0) {
-    issue(atomicAdd(sy.head, 1u));
-    decide(0);  // nothing computed yet: waiting here delays no one
   }
   __syncthreads();
-  for (int buf = 0;; buf ^= 1) {
-    const int32_t kind = s_item[buf][0], r = s_item[buf][1], i = s_item[buf][2], j = s_item[buf][3];
-    const uint32_t flags = s_flags[buf];
-    if (kind < 0) return;
-    if (threadIdx.x == 0) issue(atomicAdd(sy.head, 1u));  // loads in flight during this item
-    bool nz = (flags & 2u) != 0;
-    if (!(flags & 1u)) {
-      if (kind == kDiag)
-        nz = diag_closure_local<E>(W, ld, r, rowbuf, threadIdx.x, BlockBarrier{});
-      else
-        nz = Ops<E, kMix>::update_local(W, ld, i, j, r, sm, threadIdx.x, BlockBarrier{});
-    }
-    if (threadIdx.x == 0) {
-      const bool fast = ready();
-      if (fast) decide(buf ^ 1);
-      s_slow[buf] = fast ? 0 : 1;
-    }
-    nz = __syncthreads_or(nz) != 0;  // every store of the tile done; next item or s_slow[buf] visible
-    if (threadIdx.x == 0) {
-      publish(sy, i * nb + j, uint32_t(r + 1) | (nz ? kNZ : 0u));
-      if (!(flags & 1u)) atomicAdd(&sy.counters[kind == kDiag ? 1 : 0], 1ull);
-      atomicAdd(&sy.counters[2], 1ull);
-    }
-    if (s_slow[buf]) {  // the next item's tiles were not all there: wait now that this one is published
-      if (threadIdx.x == 0) decide(buf ^ 1);
-      __syncthreads();
-    }
-  }
+  if (tid < 3) atomicAdd(&sy.counters[tid], (unsigned long long)s_done[tid]);
 }
 
 // Warm squares of at most kClusterMaxWarm candidates: the closure by
@@ -624,8 +700,7 @@ __global__ void SCHULZE_PERSIST_BOUNDS closure_persistent_kernel(E* __restrict__
 // after the first sweep in which no CTA changed anything, when S (x) S <= S
 // held for the whole square, i.e. S is closed. Rows of cold candidates are
 // zero and stay zero; columns run over all of S. Each CTA then writes its
-// rows back into W and sets the nonzero bits of the 64 x 64 tiles of W for
-// cold_product_kernel.
+// rows back into W.
 constexpr int kClusterCtas = 8;
 constexpr int kClusterThreads = 512;
 constexpr int kMaxSweeps = 40;  // > ceil(log2 256) + 1: never reached
@@ -656,8 +731,8 @@ __device__ __forceinline__ bool differs(const uint4& a, const uint4& b) {
 
 template <typename E>
 __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterThreads, 1)
-    closure_cluster_kernel(E* __restrict__ W, int32_t ld, int32_t nb, const int32_t* __restrict__ warm,
-                           uint32_t* __restrict__ prog, unsigned long long* counters) {
+    closure_cluster_kernel(E* __restrict__ W, int32_t ld, const int32_t* __restrict__ warm,
+                           unsigned long long* counters) {
   pdl_enter();
   using AW = typename std::conditional<sizeof(E) == 2, uint32_t, int2>::type;  // a row's entries k, k + 1
   namespace cg = cooperative_groups;
@@ -667,7 +742,6 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
   extern __shared__ __align__(16) unsigned char cluster_smem[];
   uint4* S4 = reinterpret_cast<uint4*>(cluster_smem);
   const AW* A = reinterpret_cast<const AW*>(cluster_smem);  // row i, entries k, k + 1: A[i * n / 2 + k / 2]
-  __shared__ uint32_t tnz[4][4];                  // 64 x 64 tiles of W holding a nonzero
   __shared__ uint32_t flags[2][kClusterCtas];     // CTA o changed something in the sweep (two buffers)
   const int32_t n = (nw + kB - 1) / kB * kB;      // square side: whole 64-wide tiles
   constexpr int kPer16 = 16 / sizeof(E);          // entries per 16-byte piece
@@ -693,7 +767,6 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
       }
     }
   }
-  if (t < 16) tnz[t >> 2][t & 3] = 0u;
   if (t < 2 * kClusterCtas) flags[t / kClusterCtas][t % kClusterCtas] = 0u;
   cl.sync();  // every copy loaded, every flag clear, before any remote write
   const int32_t own = int32_t(q) < nw ? (nw - int32_t(q) + kClusterCtas - 1) / kClusterCtas : 0;
@@ -738,8 +811,8 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
     if (t < kClusterCtas) flags[sweeps & 1][t] = 0u;  // rewritten two sweeps on, after the next barrier
     if (!more) break;  // the same decision in every CTA
   }
-  // each CTA writes its rows back with a zero diagonal; nonzero bits per
-  // 64 x 64 tile of W. No CTA writes into another any more.
+  // each CTA writes its rows back with a zero diagonal. No CTA writes into
+  // another any more.
   for (int32_t it = t; it < own * Q; it += kClusterThreads) {
     const int32_t r = it / Q, c = it % Q;
     const int32_t i = int32_t(q) + kClusterCtas * r, j0 = c * kPer16;
@@ -754,10 +827,7 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
       v.w = w == 3 ? v.w & keep : v.w;
     }
     *reinterpret_cast<uint4*>(W + int64_t(i) * ld + j0) = v;
-    if (v.x | v.y | v.z | v.w) tnz[i / kB][j0 / kB] = 1u;
   }
-  __syncthreads();
-  if (t < 16 && tnz[t >> 2][t & 3]) atomicOr(&prog[(t >> 2) * nb + (t & 3)], kNZ);
   if (t == 0 && q == 0)  // entry updates, in 64 x 64 x 64 tile units
     atomicAdd(&counters[0], (unsigned long long)sweeps * uint64_t(nw) * uint64_t(nw) * uint64_t(n) / 262144ull);
 }
@@ -887,14 +957,15 @@ __global__ void __launch_bounds__(512, 1) cold_strip_kernel(E* __restrict__ W, i
 // value either one sees is the width of a real path and the closed square
 // composes with itself without growing (p(i,x) and p(x,y) give a walk no
 // wider than p(i,y)), so the result is the exact closure either way.
-template <typename E, int kMix>
+template <typename E>
 __global__ void __launch_bounds__(kThreads) cold_product_kernel(E* __restrict__ W, int32_t ld, int32_t nb,
                                                                  int32_t m, const int32_t* __restrict__ warm,
-                                                                 const uint32_t* __restrict__ prog,
+                                                                 const unsigned long long* __restrict__ prog,
+                                                                 const int32_t* __restrict__ tmax,
                                                                  unsigned long long* counters,
                                                                  const int32_t* __restrict__ hint_valid) {
   pdl_enter_early();
-  __shared__ __align__(16) typename Ops<E, kMix>::Smem sm;
+  __shared__ __align__(16) typename Ops<E>::Smem sm;
   if (*warm <= kClusterMaxWarm<E>) return;  // cold_strip_kernel's case
   if (hint_valid && *hint_valid && (*warm + kB - 1) / kB * kB < m) return;  // uniform cold columns
   const int32_t nbr = (*warm + kB - 1) / kB;
@@ -904,9 +975,8 @@ __global__ void __launch_bounds__(kThreads) cold_product_kernel(E* __restrict__ 
   for (int64_t t = blockIdx.x; t < items; t += gridDim.x) {
     const int32_t i = int32_t(t / nc), j = nbr + int32_t(t % nc);
     for (int32_t k = 0; k < nbr; ++k) {
-      const uint32_t a = prog[i * nb + k], b = prog[k * nb + j];
-      if ((a & kNZ) && (b & kNZ)) {
-        Ops<E, kMix>::update(W, ld, i, j, k, sm, threadIdx.x, BlockBarrier{});
+      if (word_max(prog[i * nb + k]) && tmax[k * nb + j]) {  // both operands hold a nonzero
+        tiles::tile_update(W, ld, i, j, k, sm, threadIdx.x, BlockBarrier{});
         ++done;
       }
     }
@@ -965,7 +1035,7 @@ __global__ void __launch_bounds__(512) wextract_kernel(const E* __restrict__ W, 
 // progress words, queue head, abort flag, and the relabeling.
 struct ClosureBufs {
   void* W;
-  uint32_t* prog;
+  uint32_t* prog;  // prog_words(nb): progress words, packed tiles' bounds, queue head, abort flag
   int32_t *rowflag, *perm, *inv, *warm;
   unsigned long long* counters;
   // optional: warm flags known from the tally, used when *hint_valid != 0
@@ -976,21 +1046,29 @@ struct ClosureBufs {
   bool margin = false;  // margin weights instead of winning votes
 };
 
+constexpr size_t prog_words(size_t nb) { return 4 * nb * nb + 2; }
+
 // Rowflags, relabel, pack, closure of the warm square, cold product, widen.
-// ctx may be null (no counting, no profiling). kMix: the min/max units of
-// the int32 tile updates (tiles::update2_s32).
-template <typename E, int kMix>
-int closure_pipeline_mix(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int64_t bound, int32_t* p,
-                         const ClosureBufs& bf, int32_t* status, cudaStream_t stream, int32_t* bb_out, bool side) {
+// ctx may be null (no counting, no profiling).
+template <typename E>
+int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int64_t bound, int32_t* p,
+                     const ClosureBufs& bf, int32_t* status, cudaStream_t stream, int32_t* bb_out = nullptr,
+                     bool side = false) {
   const int32_t mp = int32_t(align_up(size_t(m), kB));
   const int32_t nb = mp / kB;
   E* W = static_cast<E*>(bf.W);
-  uint32_t* head = bf.prog + size_t(nb) * size_t(nb);
+  const size_t tiles2 = size_t(nb) * size_t(nb);
+  unsigned long long* prog = reinterpret_cast<unsigned long long*>(bf.prog);
+  int32_t* tmax = reinterpret_cast<int32_t*>(bf.prog + 2 * tiles2);
+  int32_t* tmin = tmax + tiles2;
+  uint32_t* head = bf.prog + 4 * tiles2;
   uint32_t* abort_flag = head + 1;
+  int shift = 0;
+  while (((bound < INT32_MAX ? bound : int64_t(INT32_MAX)) >> shift) > int64_t(kBoundMax)) ++shift;
   {
-    // progress words, queue head and abort flag; row flags; the uniform count
+    // progress words, tile bounds, queue head and abort flag; row flags; the uniform count
     ZeroSpans z;
-    z.p[0] = bf.prog, z.words[0] = int64_t(nb) * nb + 2;
+    z.p[0] = bf.prog, z.words[0] = int64_t(prog_words(size_t(nb)));
     z.p[1] = reinterpret_cast<uint32_t*>(bf.rowflag), z.words[1] = m;
     z.p[2] = reinterpret_cast<uint32_t*>(bf.ucount), z.words[2] = 1;
     if (int rc = zero_async(ctx, z, stream)) return rc;
@@ -1016,13 +1094,14 @@ int closure_pipeline_mix(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m,
     const size_t smem = m <= kScanSmem ? size_t(m) * 4 : 0;
     cudaFuncSetAttribute(relabel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     launch_pdl(relabel_kernel, dim3(1), dim3(1024), smem, stream, false,
-               static_cast<const int32_t*>(bf.rowflag), m, bf.perm, bf.inv, bf.warm, bf.hint_valid);
+               static_cast<const int32_t*>(bf.rowflag), m, bf.perm, bf.inv, bf.warm, bf.hint, bf.hint_valid,
+               kClusterMaxWarm<E>);
   }
   {
     const int g = grid_for(reinterpret_cast<const void*>(pack_kernel<E>), 512, 0, mp);
     Launch L(ctx, stream, "closure_pack", 0.0);
     launch_pdl(pack_kernel<E>, dim3(g), dim3(512), 0, stream, false, d, m, mp,
-               static_cast<const int32_t*>(bf.perm), static_cast<const int32_t*>(bf.warm), W, bf.prog, nb, bf.hint,
+               static_cast<const int32_t*>(bf.perm), static_cast<const int32_t*>(bf.warm), W, tmax, tmin, nb, bf.hint,
                bf.hint_valid, bf.ucol, bf.margin ? 1 : 0);
   }
   if (int rc = check_launch()) return rc;
@@ -1030,20 +1109,18 @@ int closure_pipeline_mix(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m,
     const size_t smem = size_t(kClusterMaxWarm<E>) * kClusterMaxWarm<E> * sizeof(E);
     cudaFuncSetAttribute(closure_cluster_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     Launch L(ctx, stream, "closure_cluster", 0.0);
-    launch_pdl(closure_cluster_kernel<E>, dim3(kClusterCtas), dim3(kClusterThreads), smem, stream, false, W, mp, nb,
-               static_cast<const int32_t*>(bf.warm), bf.prog, bf.counters);
+    launch_pdl(closure_cluster_kernel<E>, dim3(kClusterCtas), dim3(kClusterThreads), smem, stream, false, W, mp,
+               static_cast<const int32_t*>(bf.warm), bf.counters);
   }
   if (int rc = check_launch()) return rc;
   {
     // persistent grid: every CTA resident (cooperative launch)
-    const int grid = grid_for(reinterpret_cast<const void*>(closure_persistent_kernel<E, kMix>), kThreads, 0,
+    const int grid = grid_for(reinterpret_cast<const void*>(closure_persistent_kernel<E>), kThreads, 0,
                               int64_t(nb) * nb * nb);
-    Sync sy{bf.prog, head, abort_flag, status, bf.warm, bf.counters,
-            ctx ? ctx->wait_limit_cycles : kSpinLimitCycles};
-    E* Wp = W;
-    int32_t ldp = mp, nbp = nb;
+    Sync sy{prog, tmax, tmin, head, abort_flag, status, bf.warm, bf.counters,
+            ctx ? ctx->wait_limit_cycles : kSpinLimitCycles, shift};
     Launch L(ctx, stream, "closure_persistent", double(m) * mm);
-    if (launch_pdl(closure_persistent_kernel<E, kMix>, dim3(grid), dim3(kThreads), 0, stream, true, Wp, ldp, nbp, sy) !=
+    if (launch_pdl(closure_persistent_kernel<E>, dim3(grid), dim3(kThreads), 0, stream, true, W, mp, m, nb, sy) !=
         cudaSuccess) {
       cudaGetLastError();
       return SCHULZE_ECUDA;
@@ -1058,11 +1135,11 @@ int closure_pipeline_mix(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m,
                static_cast<const int32_t*>(bf.warm), bf.counters, bf.hint_valid);
   }
   {
-    const int g = grid_for(reinterpret_cast<const void*>(cold_product_kernel<E, kMix>), kThreads, 0, int64_t(nb) * nb);
+    const int g = grid_for(reinterpret_cast<const void*>(cold_product_kernel<E>), kThreads, 0, int64_t(nb) * nb);
     Launch L(ctx, stream, "closure_cold", 0.0);
-    launch_pdl(cold_product_kernel<E, kMix>, dim3(g), dim3(kThreads), 0, stream, false, W, mp, nb, m,
-               static_cast<const int32_t*>(bf.warm), static_cast<const uint32_t*>(bf.prog), bf.counters,
-               bf.hint_valid);
+    launch_pdl(cold_product_kernel<E>, dim3(g), dim3(kThreads), 0, stream, false, W, mp, nb, m,
+               static_cast<const int32_t*>(bf.warm), static_cast<const unsigned long long*>(prog),
+               static_cast<const int32_t*>(tmax), bf.counters, bf.hint_valid);
   }
   if (bf.hint_valid) {
     Launch L(ctx, stream, "closure_cold_uniform", 0.0);
@@ -1101,20 +1178,6 @@ int closure_pipeline_mix(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m,
   return check_launch();
 }
 
-// The int32 tile updates share their work between the integer and the fp32
-// min/max units (the counts' bit patterns order alike on both) unless a
-// count could reach the fp32 infinity pattern 0x7F800000.
-template <typename E>
-int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int64_t bound, int32_t* p,
-                     const ClosureBufs& bf, int32_t* status, cudaStream_t stream, int32_t* bb_out = nullptr,
-                     bool side = false) {
-  if constexpr (sizeof(E) == 4 && tiles::kS32Mix != 0) {
-    if (bound < 0x7F800000LL)
-      return closure_pipeline_mix<E, tiles::kS32Mix>(ctx, sms, d, m, bound, p, bf, status, stream, bb_out, side);
-  }
-  return closure_pipeline_mix<E, 0>(ctx, sms, d, m, bound, p, bf, status, stream, bb_out, side);
-}
-
 template <typename E>
 int run_closure(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t bound, int32_t* p, void* ws,
                 cudaStream_t stream, int32_t* bb_out, int32_t* hint, const int32_t* hint_valid,
@@ -1124,7 +1187,7 @@ int run_closure(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t bound, in
   Carver cv(ws);
   ClosureBufs bf;
   bf.W = cv.take<E>(size_t(mp) * size_t(mp));
-  bf.prog = cv.take<uint32_t>(size_t(nb) * size_t(nb) + 2);
+  bf.prog = cv.take<uint32_t>(prog_words(size_t(nb)));
   bf.rowflag = cv.take<int32_t>(size_t(m));
   bf.perm = cv.take<int32_t>(size_t(m));
   bf.inv = cv.take<int32_t>(size_t(m));
@@ -1150,7 +1213,7 @@ int run_closure(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t bound, in
 size_t closure_workspace_bytes(int32_t m, int64_t bound, uint32_t flags) {
   size_t mp = align_up(size_t(m), kB);
   size_t nb = mp / kB;
-  return align_up(mp * mp * (use_s16(bound, flags) ? 2 : 4), 256) + align_up((nb * nb + 2) * 4, 256) +
+  return align_up(mp * mp * (use_s16(bound, flags) ? 2 : 4), 256) + align_up(prog_words(nb) * 4, 256) +
          6 * align_up(size_t(m) * 4, 256) + 4096;
 }
 
@@ -1179,7 +1242,7 @@ constexpr size_t kStaticNb = kStaticMp / kB;
 // byte offsets inside the array (each 256-aligned)
 constexpr size_t kStW = 0;                                            // W: up to kStaticMp^2 int32
 constexpr size_t kStProg = kStW + kStaticMp * kStaticMp * 4;          // progress words + head + abort
-constexpr size_t kStRowflag = kStProg + align_up((kStaticNb * kStaticNb + 2) * 4, 256);
+constexpr size_t kStRowflag = kStProg + align_up(prog_words(kStaticNb) * 4, 256);
 constexpr size_t kStPerm = kStRowflag + kStaticMaxM * 4;
 constexpr size_t kStInv = kStPerm + kStaticMaxM * 4;
 constexpr size_t kStWarm = kStInv + kStaticMaxM * 4;

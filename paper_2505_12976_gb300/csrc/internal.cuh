@@ -160,10 +160,11 @@ size_t tally_positions_workspace_bytes(int64_t n, int32_t m);
 // ws), a top-k tally also reports which candidates have an outgoing edge:
 // when some candidate is listed on no ballot, exactly the listed ones do
 // (each beats every unlisted one, and an unlisted one prefers nobody).
-// *hint_valid is set to 1 when hint holds them, else 0. Layout of hint:
-// flags [m], then the closure's warm-first relabeling of those flags, perm
-// [m] (new -> old), inv [m] (old -> new) and the warm count [1], which the
-// tally's plan pass writes so that the closure need not scan the flags.
+// *hint_valid is set to 1 when hint holds them, else 0. Layout of hint: the
+// number of ballots listing each candidate [m] (nonzero: it has an edge),
+// then the closure's warm-first relabeling, perm [m] (new -> old), inv [m]
+// (old -> new) and the warm count [1], which the tally's plan pass writes so
+// that the closure need not scan them.
 inline size_t hint_words(int32_t m) { return 3 * size_t(m) + 1; }
 int tally_launch(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, int32_t k, int32_t* d,
                  uint32_t flags, void* ws, cudaStream_t stream, int32_t* hint = nullptr,

@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(kPlanTile)
       // warm-first relabeling: listed c keeps rank f, unlisted c follows all
       // listed ones in id order
       const uint32_t nw = listed ? f : na + (uint32_t(c) - f);
-      hint[m + int64_t(nw)] = c, hint[2 * int64_t(m) + c] = int32_t(nw), hint[c] = listed ? 1 : 0;
+      hint[m + int64_t(nw)] = c, hint[2 * int64_t(m) + c] = int32_t(nw), hint[c] = x;
     }
     if (!compact) {
       slot[c] = listed ? int32_t(f) : -1;

@@ -1,0 +1,67 @@
+"""The persistent closure's tile bounds (skipped updates) and its relabeling
+by strength, against the oracle's widths bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from test_gpu_parity import cu, eq, host, lib  # noqa: F401 (the fixture builds the library)
+
+pytestmark = pytest.mark.gpu
+
+NT = 16
+
+
+def counts(kind, m, top, seed):
+    """A count matrix with zero diagonal and entries in [0, top]."""
+    rs = np.random.Generator(np.random.PCG64(seed))
+    u = np.arange(m)
+    if kind == "order":  # close to an order (few edges against it), shuffled
+        d = np.where(u[:, None] < u[None, :], top - (u[None, :] - u[:, None]) % max(1, top // 2), 0)
+        back = rs.random((m, m)) < 0.001
+        d = np.where(back & (u[:, None] > u[None, :]), rs.integers(1, top + 1, (m, m)), d)
+        s = rs.permutation(m)
+        d = d[np.ix_(s, s)]
+    elif kind == "ties":  # few distinct widths, dense: most updates change something
+        d = rs.integers(0, 4, (m, m)) * (top // 4)
+    elif kind == "chain":  # one heavy cycle through everyone over light random edges
+        d = rs.integers(0, max(2, top // 100), (m, m))
+        s = rs.permutation(m)
+        d[s, np.roll(s, -1)] = top - (u % 7)
+    else:  # "sparse": two thirds of the candidates have no edge at all (cold rows and columns)
+        d = rs.integers(0, top + 1, (m, m))
+        cold = rs.permutation(m)[: 2 * m // 3]
+        d[cold, :] = 0
+    d = d.astype(np.int32)
+    np.fill_diagonal(d, 0)
+    return d
+
+
+@pytest.mark.parametrize("top,flags", [(30000, 0), (30000, 1), (1 << 30, 0)])
+@pytest.mark.parametrize("kind,m", [("order", 257), ("order", 1000), ("ties", 320), ("ties", 705), ("chain", 449),
+                                    ("chain", 1089), ("sparse", 1200), ("order", 4300)])
+def test_closure_tile_bounds(kind, m, top, flags):
+    """Squares on both sides of whole tiles, with one tile and with several
+    tiles per work item (m = 4300), bounds that need rounding to the progress
+    word's 26 bits (2^30), cold rows and columns inside the last warm tile."""
+    import paper_2505_12976_gb300 as S
+    d = counts(kind, m, top, 7 * m + flags)
+    want = oracle.strongest_paths(d, nthreads=NT)
+    eq(host(S.schulze_strongest_paths(cu(d), top, flags=flags)), want, f"{kind} m={m} top={top} flags={flags}")
+    assert S.context().status() == S.OK
+
+
+def test_run_relabels_listed_candidates_by_ballots():
+    """More listed candidates than the cluster closure takes, some unlisted:
+    the closure sorts the tally's relabeling by ballots."""
+    import paper_2505_12976_gb300 as S
+    rs = np.random.Generator(np.random.PCG64(5))
+    m, n, k = 900, 4000, 12
+    w = np.zeros(m)
+    w[rs.permutation(m)[:600]] = (1 + np.arange(600)) ** -0.8
+    g = np.where(w > 0, np.log(np.maximum(w, 1e-300)), -1e9)[None, :] + rs.gumbel(size=(n, m))
+    r = np.argsort(-g, axis=1)[:, :k].astype(np.int32)
+    d, p, win, order, bb = oracle.schulze(r, m)
+    out = S.schulze_run(cu(r), m)
+    for key, want in (("d", d), ("p", p), ("winners", win), ("order", order), ("beaten_by", bb)):
+        eq(host(out[key]), want, key)

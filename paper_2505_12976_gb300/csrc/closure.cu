@@ -103,18 +103,51 @@ constexpr long long kSpinLimitCycles = 4000000000LL;  // ~2 s at 2 GHz, unless t
 
 // ------------------------------------------------------------ relabel
 
+// The weights in candidate order (w[i][j] as in pack_kernel, which permutes
+// their rows and columns), kept in the output p until the widths replace them:
+// rows of ldv entries of the closure's lane type, `vec` when each starts on a
+// 16-byte boundary.
+template <typename E>
+struct Weights {
+  E* v;
+  int64_t ldv;
+  int vec;
+};
+template <typename E>
+Weights<E> weights_in(int32_t* p, int32_t m) {
+  const size_t off = (16 - (reinterpret_cast<uintptr_t>(p) & 15u)) & 15u, room = size_t(m) * size_t(m) * 4;
+  const size_t ldv = align_up(size_t(m) * sizeof(E), 16) / sizeof(E);
+  if (off + size_t(m) * ldv * sizeof(E) <= room)
+    return Weights<E>{reinterpret_cast<E*>(reinterpret_cast<char*>(p) + off), int64_t(ldv), 1};
+  return Weights<E>{reinterpret_cast<E*>(p), int64_t(m), 0};
+}
+
+// With a valid hint the warm candidates are known. The weights are then
+// gathered from d straight away (pack_kernel) where the warm square is small
+// against the matrix: a gathered column costs a 32-byte sector per entry, so
+// that above half of the candidates the two streaming passes read less.
+__device__ __forceinline__ bool weigh_all(bool hv, int32_t nw, int32_t warm_max, int32_t m) {
+  return !hv || (nw > warm_max && 2 * int64_t(nw) > m);
+}
+
 // rowflag[i] = the number of outgoing edges of candidate i (the j with
-// d[i][j] > d[j][i]); also reports SCHULZE_EDATA for an entry outside
-// [0, bound]. Each CTA takes 64 x 64 block pairs (A, B), A <= B: thread
-// (r, c) holds d[A+r][B+c..c+3] and d[B+r][A+c..c+3] in registers (16-byte
-// loads when rows are 16-byte aligned), both tiles go to shared memory, and
-// each held entry is compared with its transposed partner from there.
+// d[i][j] > d[j][i]), and the weights in candidate order; also reports
+// SCHULZE_EDATA for an entry outside [0, bound]. Each CTA takes 64 x 64 block
+// pairs (A, B), A <= B: thread (r, c) holds d[A+r][B+c..c+3] and
+// d[B+r][A+c..c+3] in registers (16-byte loads when rows are 16-byte
+// aligned), both tiles go to shared memory, and each held entry is compared
+// with its transposed partner from there. Bound by HBM: d read and the
+// weights written once.
 constexpr int kFlagT = 64;
-__global__ void __launch_bounds__(256) rowflag_kernel(const int32_t* __restrict__ d, int32_t m, int64_t bound,
-                                                      int32_t* __restrict__ rowflag, int32_t* status,
-                                                      const int32_t* __restrict__ hint_valid, int vec4) {
+template <typename E>
+__global__ void __launch_bounds__(256) weigh_kernel(const int32_t* __restrict__ d, int32_t m, int64_t bound,
+                                                    int32_t* __restrict__ rowflag, int32_t* status,
+                                                    const int32_t* __restrict__ warm,
+                                                    const int32_t* __restrict__ hint_valid, int32_t warm_max, int vec4,
+                                                    Weights<E> V, int margin) {
   pdl_enter_early();
-  if (hint_valid && *hint_valid) return;  // the caller's tally already knows the flags
+  const bool hv = hint_valid && *hint_valid;
+  if (!weigh_all(hv, hv ? *warm : 0, warm_max, m)) return;
   __shared__ int32_t t1[kFlagT][kFlagT + 1], t2[kFlagT][kFlagT + 1];  // t1 = d[A.., B..], t2 = d[B.., A..]
   const int32_t nbt = (m + kFlagT - 1) / kFlagT;
   const int64_t npairs = int64_t(nbt) * (nbt + 1) / 2;
@@ -124,6 +157,20 @@ __global__ void __launch_bounds__(256) rowflag_kernel(const int32_t* __restrict_
   int32_t a = 0;           // pairs (a, b), a <= b, numbered row by row
   int64_t rowstart = 0;    // number of the pair (a, a)
   bool bad = false;
+  auto put = [&](int32_t i, int32_t j, const int32_t (&w)[4]) {  // weights of row i, columns j .. j + 3
+    if (i >= m || j >= m) return;
+    E* row = V.v + int64_t(i) * V.ldv + j;
+    if (V.vec && sizeof(E) == 4) {
+      *reinterpret_cast<int4*>(row) = make_int4(w[0], w[1], w[2], w[3]);
+    } else if (V.vec) {  // (two 16-bit lanes per word; the row's padding takes zeros)
+      *reinterpret_cast<uint2*>(row) = make_uint2((uint32_t(w[0]) & 0xFFFFu) | (uint32_t(w[1]) << 16),
+                                                  (uint32_t(w[2]) & 0xFFFFu) | (uint32_t(w[3]) << 16));
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (j + e < m) row[e] = E(w[e]);
+    }
+  };
   for (int64_t t = blockIdx.x; t < npairs; t += gridDim.x) {
     while (t >= rowstart + (nbt - a)) rowstart += nbt - a, ++a;
     const int32_t A = a * kFlagT, B = (a + int32_t(t - rowstart)) * kFlagT;
@@ -161,11 +208,24 @@ __global__ void __launch_bounds__(256) rowflag_kernel(const int32_t* __restrict_
     for (int q = 0; q < 4; ++q) {
       const int r = rq + 16 * q;
       uint32_t e = 0;  // side 0 in the low half, side 1 in the high half
+      int32_t w[4];
 #pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const int c = c4 + x;  // (on the diagonal both sides are the same entry: not counted)
-        e += x1[q][x] > T[c][r] ? 1u : 0u;
-        if (A != B) e += x2[q][x] > t1[c][r] ? 0x10000u : 0u;
+      for (int x = 0; x < 4; ++x) {  // (on the diagonal both sides are the same entry: no edge)
+        const int32_t u = T[c4 + x][r];
+        const bool edge = x1[q][x] > u;
+        e += edge ? 1u : 0u;
+        w[x] = edge ? x1[q][x] - (margin ? u : 0) : 0;
+      }
+      put(A + r, B + c4, w);
+      if (A != B) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          const int32_t u = t1[c4 + x][r];
+          const bool edge = x2[q][x] > u;
+          e += edge ? 0x10000u : 0u;
+          w[x] = edge ? x2[q][x] - (margin ? u : 0) : 0;
+        }
+        put(B + r, A + c4, w);
       }
       // padding entries are 0 on both sides, so they never count
 #pragma unroll
@@ -182,7 +242,7 @@ __global__ void __launch_bounds__(256) rowflag_kernel(const int32_t* __restrict_
 
 // perm[new] = old, inv[old] = new: candidates with edges first, strongest
 // first, then the others in id order. Strength is the number of outgoing
-// edges (rowflag_kernel), or, when the tally set *hint_valid, the number of
+// edges (weigh_kernel), or, when the tally set *hint_valid, the number of
 // ballots that list the candidate (hint). It is sorted by counting over
 // kStrengths classes (equal sizes for edge counts, relative steps of 1/128
 // for ballots; any order inside a class): the closure needs like candidates
@@ -237,17 +297,23 @@ __global__ void __launch_bounds__(1024) relabel_kernel(const int32_t* __restrict
 
 // W[a][b] = w[perm[a]][perm[b]] for the warm rows a < 64 * nbr (0 outside
 // m x m, on the diagonal and where d does not beat its transpose; w is d, or
-// the margin d - d^T with `margin`). One CTA
-// pass per row a: with x = perm[a], the threads walk b, reading d[x][perm b]
-// (along row x) and d[perm b][x] (down column x), and each warp adds its part
-// of the bounds of the 64 x 64 tile to tmax and tmin (tmin holds INT32_MAX -
-// min, so that both start at zero): the largest entry, and the smallest one
-// among the warm rows and the existing columns, off the diagonal.
+// the margin d - d^T with `margin`), with the bounds of the 64 x 64 tiles in
+// tmax and tmin (tmin holds INT32_MAX - min, so that both start at zero): the
+// largest entry, and the smallest one among the warm rows and the existing
+// columns, off the diagonal. With uniform cold columns only the square
+// (b < 64 nbr) is written, and ucol[a] receives the cold columns' common
+// value for row a.
 //
-// With the tally's flags (hint valid), a candidate y without edges is one no
-// ballot lists, so d[y][x] = 0 and that read is skipped.
-// With uniform cold columns only the square (b < 64 nbr) is written, and
-// ucol[a] receives the cold columns' common value for row a.
+// Two forms. After weigh_kernel, a CTA copies row perm[a] of the weights to
+// shared memory (when it fits, `rowbuf` bytes) and gathers its columns from
+// there, eight per thread: both passes over the matrix stay coalesced
+// whatever the order (gathering d's columns in strength order took 7.1 ms at
+// m = 16384, int32, a 32-byte sector per entry; weigh_kernel and this form
+// take 0.50 + 0.65 ms). Else (few warm
+// candidates) with x = perm[a] the threads read d[x][perm b] (along row x) and
+// d[perm b][x] (down column x); a candidate y without edges is one no ballot
+// lists, so d[y][x] = 0 and that read is skipped. `chunk` rows (of one tile
+// row) per CTA pass.
 template <typename E>
 __global__ void __launch_bounds__(512) pack_kernel(const int32_t* __restrict__ d, int32_t m, int32_t mp,
                                                    const int32_t* __restrict__ perm, const int32_t* __restrict__ warm,
@@ -255,19 +321,88 @@ __global__ void __launch_bounds__(512) pack_kernel(const int32_t* __restrict__ d
                                                    int32_t* __restrict__ tmin, int32_t nb,
                                                    const int32_t* __restrict__ hint,
                                                    const int32_t* __restrict__ hint_valid, int32_t* __restrict__ ucol,
-                                                   int margin) {
+                                                   int margin, int32_t warm_max, Weights<E> V, uint32_t rowbuf,
+                                                   int32_t chunk) {
   pdl_enter();
+  extern __shared__ __align__(16) unsigned char pack_smem[];
   const bool hv = hint_valid && *hint_valid;
-  const int32_t rows = (*warm + kB - 1) / kB * kB;  // W rows to write
+  const int32_t nw = *warm;
+  const int32_t rows = (nw + kB - 1) / kB * kB;  // W rows to write
   const bool uc = hv && rows < m;                    // uniform cold columns beyond the square
   const int32_t bend = uc ? rows : mp;
   const int lane = threadIdx.x & 31;
+  if (weigh_all(hv, nw, warm_max, m)) {
+    E* srow = reinterpret_cast<E*>(pack_smem);
+    int32_t* cmax = reinterpret_cast<int32_t*>(pack_smem + rowbuf);  // this chunk's bounds per tile column
+    int32_t* cmin = cmax + nb;
+    for (int t = threadIdx.x; t < 2 * nb; t += blockDim.x) cmax[t] = 0;
+    for (int32_t a0 = int32_t(blockIdx.x) * chunk; a0 < rows; a0 += int32_t(gridDim.x) * chunk) {
+      for (int32_t a = a0; a < a0 + chunk; ++a) {
+        E* wrow = W + int64_t(a) * mp;
+        __syncthreads();  // the row before is read
+        if (a >= nw) {    // rows without edges up to a whole tile
+          for (int32_t b = 8 * threadIdx.x; b < bend; b += 8 * blockDim.x) {
+#pragma unroll
+            for (int e = 0; e < int(sizeof(E)) / 2; ++e) reinterpret_cast<uint4*>(wrow + b)[e] = make_uint4(0, 0, 0, 0);
+          }
+          continue;
+        }
+        const int32_t x = perm[a];
+        if (uc && threadIdx.x == 0) ucol[a] = max(d[int64_t(x) * m + perm[rows]], 0);
+        const E* vrow = V.v + int64_t(x) * V.ldv;
+        if (rowbuf) {
+          if (V.vec) {
+            const int32_t n16 = int32_t((size_t(m) * sizeof(E) + 15) / 16);
+            for (int32_t t0 = threadIdx.x; t0 < n16; t0 += 4 * blockDim.x) {
+              uint4 v[4];
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                if (t0 + q * int32_t(blockDim.x) < n16) v[q] = __ldcs(reinterpret_cast<const uint4*>(vrow) + t0 + q * blockDim.x);
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                if (t0 + q * int32_t(blockDim.x) < n16) reinterpret_cast<uint4*>(srow)[t0 + q * blockDim.x] = v[q];
+            }
+          } else {
+            for (int32_t t = threadIdx.x; t < m; t += blockDim.x) srow[t] = vrow[t];
+          }
+          __syncthreads();
+          vrow = srow;
+        }
+        for (int32_t b = 8 * threadIdx.x; b < bend; b += 8 * blockDim.x) {
+          int32_t w[8], mx = 0, mn = INT32_MAX;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            w[e] = b + e < m ? int32_t(vrow[perm[b + e]]) : 0;
+            mx = max(mx, w[e]);
+            if (b + e < m && b + e != a) mn = min(mn, w[e]);
+          }
+          if (sizeof(E) == 2) {
+            uint32_t u[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) u[e] = (uint32_t(w[2 * e]) & 0xFFFFu) | (uint32_t(w[2 * e + 1]) << 16);
+            *reinterpret_cast<uint4*>(wrow + b) = make_uint4(u[0], u[1], u[2], u[3]);
+          } else {
+            reinterpret_cast<int4*>(wrow + b)[0] = make_int4(w[0], w[1], w[2], w[3]);
+            reinterpret_cast<int4*>(wrow + b)[1] = make_int4(w[4], w[5], w[6], w[7]);
+          }
+          if (mx > 0) atomicMax(&cmax[b / kB], mx);
+          if (mn < INT32_MAX) atomicMax(&cmin[b / kB], INT32_MAX - max(mn, 0));
+        }
+      }
+      __syncthreads();
+      for (int t = threadIdx.x; t < bend / kB; t += blockDim.x) {
+        if (cmax[t]) atomicMax(&tmax[(a0 / kB) * nb + t], cmax[t]), cmax[t] = 0;
+        if (cmin[t]) atomicMax(&tmin[(a0 / kB) * nb + t], cmin[t]), cmin[t] = 0;
+      }
+    }
+    return;
+  }
   constexpr int kU = 8;  // columns per thread and pass, their loads issued together
   for (int32_t a = blockIdx.x; a < rows; a += gridDim.x) {
     E* wrow = W + int64_t(a) * mp;
     const int32_t x = a < m ? perm[a] : -1;
     const int32_t* drow = x >= 0 ? d + int64_t(x) * m : nullptr;
-    if (uc && threadIdx.x == 0) ucol[a] = (x >= 0 && a < *warm) ? max(drow[perm[rows]], 0) : 0;
+    if (uc && threadIdx.x == 0) ucol[a] = (x >= 0 && a < nw) ? max(drow[perm[rows]], 0) : 0;
     for (int32_t b0 = 0; b0 < bend; b0 += kU * blockDim.x) {
       int32_t y[kU], v[kU], u[kU];
 #pragma unroll
@@ -286,7 +421,7 @@ __global__ void __launch_bounds__(512) pack_kernel(const int32_t* __restrict__ d
         const int32_t out = v[q] > u[q] ? (margin ? v[q] - u[q] : v[q]) : 0;
         if (b < bend) wrow[b] = E(out);
         const int32_t mx = __reduce_max_sync(0xFFFFFFFFu, out);
-        const int32_t mn = __reduce_min_sync(0xFFFFFFFFu, a < *warm && b < m && b != a ? out : INT32_MAX);
+        const int32_t mn = __reduce_min_sync(0xFFFFFFFFu, a < nw && b < m && b != a ? out : INT32_MAX);
         if (lane == 0 && b < bend) {
           const int32_t t = (a / kB) * nb + b / kB;
           if (mx > 0) atomicMax(&tmax[t], mx);
@@ -298,15 +433,21 @@ __global__ void __launch_bounds__(512) pack_kernel(const int32_t* __restrict__ d
 }
 
 // p[x][y] = W[inv[x]][inv[y]] for warm x and y != x; every other entry 0
-// (cold rows are written as zeros without reading W). One row per CTA pass.
+// (cold rows are written as zeros without reading W). A warm row of W is
+// copied to shared memory (when it fits, `rowbuf` bytes) and gathered from
+// there, so that W and p are both streamed whatever the order; bound by HBM
+// (m = 16384, int32: 0.61 ms for 2.1 GB, against 1.47 gathering from global
+// memory in strength order; m = 18407, int16: 0.64 against 2.05 ms).
+// With uniform cold columns (uc) every column outside the square is ucold.
 template <typename E>
-__global__ void __launch_bounds__(256) widen_kernel(const E* __restrict__ W, int32_t mp, int32_t m,
+__global__ void __launch_bounds__(512) widen_kernel(const E* __restrict__ W, int32_t mp, int32_t m,
                                                     const int32_t* __restrict__ inv,
                                                     const int32_t* __restrict__ perm,
                                                     const int32_t* __restrict__ warm, int32_t* __restrict__ p,
                                                     const int32_t* __restrict__ hint_valid,
-                                                    const int32_t* __restrict__ ucold, int vec4) {
+                                                    const int32_t* __restrict__ ucold, int vec4, uint32_t rowbuf) {
   pdl_enter();
+  extern __shared__ __align__(16) unsigned char widen_smem[];
   const int32_t nw = *warm;
   const int32_t rows = (nw + kB - 1) / kB * kB;
   const bool uc = hint_valid && *hint_valid && rows < m;  // cold columns beyond the square: ucold[ix]
@@ -322,10 +463,11 @@ __global__ void __launch_bounds__(256) widen_kernel(const E* __restrict__ W, int
       if (x >= m) break;
       const int32_t ix = __shfl_sync(0xFFFFFFFFu, ixl, r);
       int32_t* prow = p + int64_t(x) * m;
-      // a cold row is zero; with uniform cold columns a warm row is
-      // ucold[ix] outside the square, whose columns (relabeled b < rows,
-      // candidate perm[b]) come from W after the fill
-      if (ix >= nw || uc) {
+      const E* wrow = W + int64_t(ix) * mp;
+      // a cold row is zero; with uniform cold columns and a small square a
+      // warm row is ucold[ix] outside the square, whose columns (relabeled
+      // b < rows, candidate perm[b]) come from W after the fill
+      if (ix >= nw || (uc && 4 * rows < m)) {
         const int32_t fill = ix >= nw ? 0 : ucold[ix];
         if (vec4) {
           for (int32_t y = 4 * threadIdx.x; y < m; y += 4 * blockDim.x)
@@ -335,41 +477,38 @@ __global__ void __launch_bounds__(256) widen_kernel(const E* __restrict__ W, int
         }
         if (ix >= nw) continue;
         __syncthreads();  // the square's columns after the fill (the branch is the same in the whole CTA)
-        const E* wrow = W + int64_t(ix) * mp;
         for (int32_t b = threadIdx.x; b < rows; b += blockDim.x) prow[perm[b]] = b == ix ? 0 : int32_t(wrow[b]);
         continue;
       }
-      const E* wrow = W + int64_t(ix) * mp;
-      if (vec4) {
-        constexpr int kU = 4;  // int4 groups per thread and pass, loads issued together
-        for (int32_t y0 = 0; y0 < m; y0 += 4 * kU * blockDim.x) {
-          int4 iv[kU];
-  #pragma unroll
-          for (int q = 0; q < kU; ++q) {
-            const int32_t y = y0 + 4 * (q * blockDim.x + threadIdx.x);
-            iv[q] = y < m ? *reinterpret_cast<const int4*>(inv + y) : make_int4(0, 0, 0, 0);
-          }
-          int4 v[kU];
-          const int32_t uv = uc ? ucold[ix] : 0;
-          auto at = [&](int32_t iy) { return (uc && iy >= rows) ? uv : int32_t(wrow[iy]); };
-  #pragma unroll
-          for (int q = 0; q < kU; ++q) v[q] = make_int4(at(iv[q].x), at(iv[q].y), at(iv[q].z), at(iv[q].w));
-  #pragma unroll
-          for (int q = 0; q < kU; ++q) {
-            const int32_t y = y0 + 4 * (q * blockDim.x + threadIdx.x);
-            if (y >= m) continue;
-            if (x >= y && x < y + 4) {
-              const int32_t t = x - y;
-              v[q].x = t == 0 ? 0 : v[q].x, v[q].y = t == 1 ? 0 : v[q].y;
-              v[q].z = t == 2 ? 0 : v[q].z, v[q].w = t == 3 ? 0 : v[q].w;
-            }
-            *reinterpret_cast<int4*>(prow + y) = v[q];
-          }
+      const int32_t lim = uc ? rows : mp;  // columns of W to read
+      const int32_t uv = uc ? ucold[ix] : 0;
+      if (rowbuf) {
+        __syncthreads();  // the row before is read
+        E* srow = reinterpret_cast<E*>(widen_smem);
+        const int32_t n16 = lim * int32_t(sizeof(E)) / 16;  // (whole tiles)
+        for (int32_t t0 = threadIdx.x; t0 < n16; t0 += 4 * blockDim.x) {
+          uint4 v[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (t0 + q * int32_t(blockDim.x) < n16) v[q] = __ldcs(reinterpret_cast<const uint4*>(wrow) + t0 + q * blockDim.x);
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (t0 + q * int32_t(blockDim.x) < n16) reinterpret_cast<uint4*>(srow)[t0 + q * blockDim.x] = v[q];
         }
-      } else {
-        for (int32_t y = threadIdx.x; y < m; y += blockDim.x) {
-          const int32_t iy = inv[y];
-          prow[y] = (y == x) ? 0 : (uc && iy >= rows) ? ucold[ix] : int32_t(wrow[iy]);
+        __syncthreads();
+        wrow = srow;
+      }
+      constexpr int kU = 8;
+      for (int32_t y0 = threadIdx.x; y0 < m; y0 += kU * blockDim.x) {
+        int32_t iy[kU], v[kU];
+#pragma unroll
+        for (int q = 0; q < kU; ++q) iy[q] = y0 + q * int32_t(blockDim.x) < m ? inv[y0 + q * blockDim.x] : 0;
+#pragma unroll
+        for (int q = 0; q < kU; ++q) v[q] = iy[q] < lim ? int32_t(wrow[iy[q]]) : uv;
+#pragma unroll
+        for (int q = 0; q < kU; ++q) {
+          const int32_t y = y0 + q * int32_t(blockDim.x);
+          if (y < m) __stcs(prow + y, y == x ? 0 : v[q]);
         }
       }
     }
@@ -987,14 +1126,23 @@ __global__ void __launch_bounds__(kThreads) cold_product_kernel(E* __restrict__ 
 // beaten_by straight from the closed warm rows of W, for callers that need
 // the ranking but not a second pass over p: a cold candidate x (no outgoing
 // edge, p[x][*] = 0) is beaten by every warm j with p[j][x] > 0; a warm x by
-// every warm j with p[j][x] > p[x][j]; cold candidates beat nobody. CTA =
-// 32 relabeled columns x 8 row groups.
+// every warm j with p[j][x] > p[x][j]; cold candidates beat nobody.
+//
+// Squares of the persistent closure: CTA (J, c) counts, for the 64 columns of
+// tile column J, the rows of tile rows 32 c .. 32 c + 31 that beat them, and
+// adds the counts into bb (zeroed before). The tiles' bounds in the progress
+// words decide most pairs of tiles unread (every width of (I, J) above every
+// width of (J, I), or none): in strength order that is all but the ones near
+// the diagonal (m = 16384, int32: 0.086 ms, against 1.25 ms reading all of W).
+// Smaller squares: CTA = 32 relabeled columns x 16 row groups.
 template <typename E>
 __global__ void __launch_bounds__(512) wextract_kernel(const E* __restrict__ W, int32_t mp, int32_t m,
                                                        const int32_t* __restrict__ perm,
                                                        const int32_t* __restrict__ warm, int32_t* __restrict__ bb,
                                                        const int32_t* __restrict__ hint_valid,
-                                                       const int32_t* __restrict__ ucount) {
+                                                       const int32_t* __restrict__ ucount,
+                                                       const unsigned long long* __restrict__ prog, int32_t nb,
+                                                       int32_t warm_max) {
   pdl_enter();
   constexpr int kG = 16;  // row groups
   __shared__ int32_t part[kG][33];
@@ -1002,6 +1150,64 @@ __global__ void __launch_bounds__(512) wextract_kernel(const E* __restrict__ W, 
   const int32_t rows = (nw + kB - 1) / kB * kB;
   const bool uc = hint_valid && *hint_valid && rows < m;
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  if (nw > warm_max) {
+    __shared__ E tj[kB][kB + (sizeof(E) == 2 ? 2 : 1)];  // tile (J, I), rows an odd number of words apart
+    __shared__ int32_t cnt[kB];
+    __shared__ uint32_t s_read;
+    const int32_t nbr = rows / kB, nchunk = (nbr + 31) / 32;
+    for (int32_t t = blockIdx.x; t < nb * nchunk; t += gridDim.x) {
+      const int32_t J = t / nchunk, I0 = (t - J * nchunk) * 32;
+      if (uc && J >= nbr) {  // uniform cold columns: beaten by the warm rows with u > 0
+        if (I0 == 0 && threadIdx.x < kB && J * kB + int32_t(threadIdx.x) < m)
+          bb[perm[J * kB + threadIdx.x]] = *ucount;
+        continue;
+      }
+      if (threadIdx.x < kB) cnt[threadIdx.x] = 0;
+      if (g == 0) {
+        // all: every row of tile (I, J) with edges beats every column; none:
+        // no row beats any (cold columns, whose own rows are zero, need the
+        // tile itself to be zero)
+        const int32_t I = I0 + lane;
+        int32_t all = 0;
+        bool read = false;
+        if (I < nbr) {
+          const bool warm_j = J < nbr, cold_in_j = (J + 1) * kB > nw;
+          const uint64_t wij = warm_j ? prog[I * nb + J] : 0, wji = warm_j ? prog[J * nb + I] : 0;
+          if (I != J && warm_j && word_min(wij) > word_max(wji)) all = min(kB, nw - I * kB);
+          else read = !warm_j || I == J || (cold_in_j ? word_max(wij) > 0 : word_max(wij) > word_min(wji));
+        }
+        const uint32_t mask = __ballot_sync(0xFFFFFFFFu, read);
+        all = __reduce_add_sync(0xFFFFFFFFu, all);
+        if (lane == 0) s_read = mask;
+        __syncwarp();
+        cnt[lane] = all, cnt[lane + 32] = all;
+      }
+      __syncthreads();
+      int32_t c = 0;
+      const int col = threadIdx.x & (kB - 1), rg = threadIdx.x / kB;  // column, rows rg + 8 q
+      for (uint32_t mask = s_read; mask; mask &= mask - 1) {
+        const int32_t I = I0 + __ffs(int(mask)) - 1;
+        for (int e = threadIdx.x; e < kB * kB; e += blockDim.x) {  // (rows past the square are not in W)
+          const int32_t j = J * kB + e / kB;
+          tj[e / kB][e % kB] = j < rows ? W[int64_t(j) * mp + I * kB + e % kB] : E(0);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kB / 8; ++q) {
+          const int i = rg + 8 * q;
+          const bool in = I * kB + i < nw && J * kB + col < m && !(I == J && i == col);
+          if (in) c += int32_t(W[int64_t(I * kB + i) * mp + J * kB + col]) > int32_t(tj[col][i]);
+        }
+        __syncthreads();
+      }
+      if (c) atomicAdd(&cnt[col], c);
+      __syncthreads();
+      if (threadIdx.x < kB && J * kB + int32_t(threadIdx.x) < m && cnt[threadIdx.x])
+        atomicAdd(&bb[perm[J * kB + threadIdx.x]], cnt[threadIdx.x]);
+      __syncthreads();
+    }
+    return;
+  }
   for (int32_t b0 = blockIdx.x * 32; b0 < m; b0 += gridDim.x * 32) {
     if (uc && b0 >= rows) {  // uniform cold columns: beaten by the warm rows with u > 0
       if (g == 0 && b0 + lane < m) bb[perm[b0 + lane]] = *ucount;
@@ -1047,6 +1253,7 @@ struct ClosureBufs {
 };
 
 constexpr size_t prog_words(size_t nb) { return 4 * nb * nb + 2; }
+constexpr size_t kMaxRowBuf = 200 * 1024;  // larger rows (int32, m > 51200) are gathered from global memory
 
 // Rowflags, relabel, pack, closure of the warm square, cold product, widen.
 // ctx may be null (no counting, no profiling).
@@ -1057,6 +1264,7 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
   const int32_t mp = int32_t(align_up(size_t(m), kB));
   const int32_t nb = mp / kB;
   E* W = static_cast<E*>(bf.W);
+  const Weights<E> V = weights_in<E>(p, m);
   const size_t tiles2 = size_t(nb) * size_t(nb);
   unsigned long long* prog = reinterpret_cast<unsigned long long*>(bf.prog);
   int32_t* tmax = reinterpret_cast<int32_t*>(bf.prog + 2 * tiles2);
@@ -1071,6 +1279,7 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
     z.p[0] = bf.prog, z.words[0] = int64_t(prog_words(size_t(nb)));
     z.p[1] = reinterpret_cast<uint32_t*>(bf.rowflag), z.words[1] = m;
     z.p[2] = reinterpret_cast<uint32_t*>(bf.ucount), z.words[2] = 1;
+    z.p[3] = reinterpret_cast<uint32_t*>(bb_out), z.words[3] = bb_out ? m : 0;
     if (int rc = zero_async(ctx, z, stream)) return rc;
   }
   const double mm = double(m) * double(m);
@@ -1084,10 +1293,11 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
   };
   {
     const int64_t nbt = (m + kFlagT - 1) / kFlagT;
-    const int g = grid_for(reinterpret_cast<const void*>(rowflag_kernel), 256, 0, nbt * (nbt + 1) / 2);
+    const int g = grid_for(reinterpret_cast<const void*>(weigh_kernel<E>), 256, 0, nbt * (nbt + 1) / 2);
     Launch L(ctx, stream, "closure_rowflags", mm * 4.0);
-    launch_pdl(rowflag_kernel, dim3(g), dim3(256), 0, stream, false, d, m, bound, bf.rowflag, status, bf.hint_valid,
-               rows_vec16(d, m));
+    launch_pdl(weigh_kernel<E>, dim3(g), dim3(256), 0, stream, false, d, m, bound, bf.rowflag, status,
+               static_cast<const int32_t*>(bf.warm), bf.hint_valid, kClusterMaxWarm<E>, rows_vec16(d, m), V,
+               bf.margin ? 1 : 0);
   }
   {
     Launch L(ctx, stream, "closure_relabel", double(m) * 12.0);
@@ -1097,12 +1307,18 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
                static_cast<const int32_t*>(bf.rowflag), m, bf.perm, bf.inv, bf.warm, bf.hint, bf.hint_valid,
                kClusterMaxWarm<E>);
   }
+  // rows of the weights and of W in shared memory, up to what a CTA can have
+  const size_t rowbytes = align_up(size_t(mp) * sizeof(E), 16);
+  const uint32_t rowbuf = rowbytes <= kMaxRowBuf ? uint32_t(rowbytes) : 0u;
   {
-    const int g = grid_for(reinterpret_cast<const void*>(pack_kernel<E>), 512, 0, mp);
+    const size_t smem = rowbuf + 2 * size_t(nb) * 4;
+    const int32_t chunk = m >= 8192 ? 16 : m >= 2048 ? 4 : 1;
+    cudaFuncSetAttribute(pack_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    const int g = grid_for(reinterpret_cast<const void*>(pack_kernel<E>), 512, smem, mp);
     Launch L(ctx, stream, "closure_pack", 0.0);
-    launch_pdl(pack_kernel<E>, dim3(g), dim3(512), 0, stream, false, d, m, mp,
+    launch_pdl(pack_kernel<E>, dim3(g), dim3(512), smem, stream, false, d, m, mp,
                static_cast<const int32_t*>(bf.perm), static_cast<const int32_t*>(bf.warm), W, tmax, tmin, nb, bf.hint,
-               bf.hint_valid, bf.ucol, bf.margin ? 1 : 0);
+               bf.hint_valid, bf.ucol, bf.margin ? 1 : 0, kClusterMaxWarm<E>, V, rowbuf, chunk);
   }
   if (int rc = check_launch()) return rc;
   {
@@ -1153,27 +1369,29 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
     // stream, with at most four CTAs per SM so that those kernels find room
     const bool fork = side && bb_out && ctx && ctx->side_stream;
     cudaStream_t wst = stream;
-    int g = grid_for(reinterpret_cast<const void*>(widen_kernel<E>), 256, 0, m);
+    cudaFuncSetAttribute(widen_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(rowbuf));
+    int g = grid_for(reinterpret_cast<const void*>(widen_kernel<E>), 512, rowbuf, m);
     if (fork) {
       if (cudaEventRecord(ctx->side_fork, stream) != cudaSuccess ||
           cudaStreamWaitEvent(ctx->side_stream, ctx->side_fork, 0) != cudaSuccess)
         return SCHULZE_ECUDA;
       ctx->side_pending = true;  // joined by the caller, whatever happens next
       wst = ctx->side_stream;
-      g = std::min(g, 4 * sms);
+      g = std::min(g, 2 * sms);
     }
     Launch L(ctx, wst, "closure_widen", mm * 4.0);
-    launch_pdl(widen_kernel<E>, dim3(g), dim3(256), 0, wst, false, static_cast<const E*>(W), mp, m,
+    launch_pdl(widen_kernel<E>, dim3(g), dim3(512), rowbuf, wst, false, static_cast<const E*>(W), mp, m,
                static_cast<const int32_t*>(bf.inv), static_cast<const int32_t*>(bf.perm),
                static_cast<const int32_t*>(bf.warm), p, bf.hint_valid, static_cast<const int32_t*>(bf.ucold),
-               rows_vec16(p, m));
+               rows_vec16(p, m), rowbuf);
     if (fork && cudaEventRecord(ctx->side_join, wst) != cudaSuccess) return SCHULZE_ECUDA;
   }
   if (bb_out) {
     Launch L(ctx, stream, "closure_beaten_by", 0.0);
     launch_pdl(wextract_kernel<E>, dim3((m + 31) / 32), dim3(512), 0, stream, false, static_cast<const E*>(W), mp, m,
                static_cast<const int32_t*>(bf.perm), static_cast<const int32_t*>(bf.warm), bb_out, bf.hint_valid,
-               static_cast<const int32_t*>(bf.ucount));
+               static_cast<const int32_t*>(bf.ucount), static_cast<const unsigned long long*>(prog), nb,
+               kClusterMaxWarm<E>);
   }
   return check_launch();
 }

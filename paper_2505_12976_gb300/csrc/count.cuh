@@ -17,4 +17,12 @@ __device__ __forceinline__ uint32_t count_lt2(uint32_t acc, uint32_t a_guarded, 
   return acc + ((~(a_guarded - b) >> 15) & 0x00010001u);
 }
 
+// [a < b] on 32 ballots at once, one bit of two positions at a time from the
+// lowest up: lt' = (~a & b) | (~(a ^ b) & lt), one logic instruction.
+__device__ __forceinline__ uint32_t plane_lt(uint32_t a, uint32_t b, uint32_t lt) {
+  uint32_t r;
+  asm("lop3.b32 %0, %1, %2, %3, 0x8E;" : "=r"(r) : "r"(a), "r"(b), "r"(lt));
+  return r;
+}
+
 }  // namespace schulze

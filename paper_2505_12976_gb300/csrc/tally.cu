@@ -1,9 +1,10 @@
 // Pairwise tally: d[i][j] = number of ballots that prefer i to j (Sect. 2.1).
 //
 // Two exact kernels, chosen by cost:
-//  * dense  (position compare, O(n m^2)): ballots are turned into position
-//    rows pos[v][c] (unlisted = k) and every (i, j) tile counts
-//    pos[v][i] < pos[v][j] with packed 16-bit SIMD compares;
+//  * dense  (position compare, O(n m^2)): ballots are turned into bit planes
+//    of their positions (unlisted = k), a word per candidate holding one bit
+//    of its position on 32 ballots, and every (i, j) tile compares the
+//    positions of i and j on 32 ballots at once, bit by bit;
 //  * sparse (pair count, O(n k^2)): d[i][j] = cnt[i] - C[i][j], where cnt[i]
 //    is the number of ballots listing i and C[i][j] the number listing j
 //    above i. C vanishes outside A x A, A the set of listed candidates.
@@ -34,78 +35,143 @@ constexpr uint16_t kNoSlot = 0xFFFFu;
 
 // ------------------------------------------------------------------ dense
 
-constexpr int kDenseVoters = 32;  // ballots staged in shared memory per step
-constexpr int kMaxVoterChunk = 32768;  // 16-bit lane counters never overflow
+// Bit planes: planes[(g * bits + b) * ldp + c] holds bit b of candidate c's
+// position on ballots 32 g .. 32 g + 31 of the chunk (ballot v in bit v % 32).
+// Comparing two planes words bit by bit from the lowest bit up,
+//   lt = (~a & b) | (~(a ^ b) & lt),
+// is one three-input logic instruction per position bit for 32 ballots, so a
+// pair of candidates costs bits + 2 instructions (a population count and an
+// add) per 32 ballots: 0.37 a compare for positions below 1024, against 1.5
+// for packed 16-bit compares (count.cuh).
+constexpr int kPlaneVoters = 32;   // ballots per plane word
+constexpr int kPlaneCols = 2048;   // candidates whose positions a CTA turns at a time
+constexpr int kPlaneBits = 16;     // planes of weak orders (their largest position is not known ahead)
 
-// pos[v][c] for v in [v0, v0 + nv): position of c in ballot v, k if unlisted.
-// One warp per ballot. Out-of-range ids and repeated ids set EDATA.
-__global__ void pos_build_kernel(const int32_t* __restrict__ ranks, int64_t v0, int64_t nv, int32_t m, int32_t k,
-                                 int32_t ldp, uint16_t* __restrict__ pos, int32_t* status) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;
-  for (int64_t w = warp; w < nv; w += nwarps) {
-    const int32_t* row = ranks + (v0 + w) * k;
-    uint16_t* prow = pos + w * ldp;
-    for (int32_t c = lane; c < ldp; c += kWarp) prow[c] = uint16_t(k);
-    __syncwarp();
-    for (int32_t q = lane; q < k; q += kWarp) {
-      int32_t c = row[q];
-      if (c >= 0 && c < m)
-        prow[c] = uint16_t(q);
-      else
-        set_status(status, SCHULZE_EDATA);
+// planes [b0, b0 + 8) of the 32 positions at(v), written at out + b * ldp for b < bits
+template <class At>
+__device__ __forceinline__ void put_planes(At at, int b0, int bits, uint32_t* out, int32_t ldp) {
+  uint32_t w[8];
+#pragma unroll
+  for (int b = 0; b < 8; ++b) w[b] = 0u;
+#pragma unroll
+  for (int v = 0; v < kPlaneVoters; ++v) {
+    uint32_t y = at(v) >> b0;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) w[b] = __funnelshift_r(w[b], y, 1), y >>= 1;  // y's bit 0 into the top of w
+  }
+#pragma unroll
+  for (int b = 0; b < 8; ++b)
+    if (b0 + b < bits) out[int64_t(b0 + b) * ldp] = w[b];
+}
+
+// d zeroed by all CTAs of a launch (where the counts are added into it)
+__device__ __forceinline__ void zero_counts(int32_t* __restrict__ d, int64_t words, int64_t cta, int64_t ctas) {
+  if (!d) return;
+  for (int64_t t = cta * blockDim.x + threadIdx.x; t < words; t += ctas * blockDim.x) d[t] = 0;
+}
+
+// Ballots v0 .. v0 + nv - 1 into planes; CTA (g, y) turns its 32 ballots for
+// candidates kPlaneCols y .. through positions in shared memory (unlisted
+// candidates, and every candidate of the padding ballots, at k: equal, so
+// never counted). Out-of-range ids and repeated ids set EDATA.
+__global__ void __launch_bounds__(512) slice_ballots_kernel(const int32_t* __restrict__ ranks, int64_t v0, int64_t nv,
+                                                            int32_t m, int32_t k, int32_t ldp, int bits,
+                                                            uint32_t* __restrict__ planes, int32_t* status,
+                                                            int32_t* __restrict__ dzero) {
+  extern __shared__ __align__(16) uint16_t slice_pos[];  // [32][cols]
+  zero_counts(dzero, int64_t(m) * m, blockIdx.y * int64_t(gridDim.x) + blockIdx.x, int64_t(gridDim.x) * gridDim.y);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+  const int32_t c0 = int32_t(blockIdx.y) * kPlaneCols, cols = min(kPlaneCols, ldp - c0);  // cols: a multiple of 64
+  const int64_t vb = int64_t(blockIdx.x) * kPlaneVoters;
+  {
+    const uint32_t k2 = uint32_t(k & 0xFFFF) * 0x10001u;
+    uint32_t* pos2 = reinterpret_cast<uint32_t*>(slice_pos);
+    for (int t = threadIdx.x; t < kPlaneVoters * cols / 2; t += blockDim.x) pos2[t] = k2;
+  }
+  __syncthreads();
+  for (int v = wid; v < kPlaneVoters && vb + v < nv; v += nwarp) {
+    const int32_t* row = ranks + (v0 + vb + v) * k;
+    uint16_t* prow = slice_pos + v * cols;
+    constexpr int kU = 8;  // ids per lane and pass, their loads issued together
+    bool bad = false;
+    for (int32_t q0 = lane; q0 < k; q0 += kU * kWarp) {
+      int32_t c[kU];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) c[u] = q0 + u * kWarp < k ? row[q0 + u * kWarp] : 0;
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int32_t q = q0 + u * kWarp;
+        if (q >= k) break;
+        bad |= c[u] < 0 || c[u] >= m;
+        if (c[u] >= c0 && c[u] < c0 + cols) prow[c[u] - c0] = uint16_t(q);
+      }
     }
     __syncwarp();
     // a repeated id keeps only one of its positions: the other one sees it
-    for (int32_t q = lane; q < k; q += kWarp) {
-      int32_t c = row[q];
-      if (c >= 0 && c < m && prow[c] != uint16_t(q)) set_status(status, SCHULZE_EDATA);
+    for (int32_t q0 = lane; q0 < k; q0 += kU * kWarp) {
+      int32_t c[kU];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) c[u] = q0 + u * kWarp < k ? row[q0 + u * kWarp] : -1;
+#pragma unroll
+      for (int u = 0; u < kU; ++u)
+        bad |= c[u] >= c0 && c[u] < min(m, c0 + cols) && prow[c[u] - c0] != uint16_t(q0 + u * kWarp);
     }
-    __syncwarp();
+    if (bad) set_status(status, SCHULZE_EDATA);
   }
+  __syncthreads();
+  uint32_t* out = planes + int64_t(blockIdx.x) * bits * ldp + c0;
+  for (int32_t c = threadIdx.x; c < cols; c += blockDim.x)
+    for (int b0 = 0; b0 < bits; b0 += 8)
+      put_planes([&](int v) { return uint32_t(slice_pos[v * cols + c]); }, b0, bits, out + c, ldp);
 }
 
-// Weak orders in position form: pos[v][c] for v in [v0, v0 + nv) copied from
-// the caller's int32 positions (smaller is better, equal is tied) into the
-// 16-bit rows; a position outside [0, 65534] sets EDATA, one above 32767
-// sets *wide. Padding columns (c >= m) hold 0x7FFF; their counts are never
-// written.
-__global__ void pos_copy_kernel(const int32_t* __restrict__ src, int64_t v0, int64_t nv, int32_t m, int32_t ldp,
-                                uint16_t* __restrict__ pos, int32_t* status, int32_t* __restrict__ wide) {
-  const int64_t total = nv * ldp;
-  bool bad = false, big = false;
-  for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total; e += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t w = e / ldp;
-    const int32_t c = int32_t(e - w * ldp);
-    uint16_t v = 0x7FFFu;
-    if (c < m) {
-      const int32_t x = src[(v0 + w) * m + c];
-      bad |= x < 0 || x > 65534;
-      big |= x > 32767;
-      v = uint16_t(x < 0 ? 0 : (x > 65534 ? 65534 : x));
-    }
-    pos[e] = v;
+// Weak orders in position form: the caller's int32 positions (smaller is
+// better, equal is tied) into kPlaneBits planes; a position outside
+// [0, 65534] sets EDATA, and *used collects the bits that any position has.
+// Padding ballots and candidates (c >= m) are at position 0.
+__global__ void __launch_bounds__(256) slice_positions_kernel(const int32_t* __restrict__ src, int64_t v0, int64_t nv,
+                                                              int32_t m, int32_t ldp, uint32_t* __restrict__ planes,
+                                                              int32_t* status, uint32_t* __restrict__ used,
+                                                              int32_t* __restrict__ dzero) {
+  zero_counts(dzero, int64_t(m) * m, blockIdx.y * int64_t(gridDim.x) + blockIdx.x, int64_t(gridDim.x) * gridDim.y);
+  const int64_t vb = int64_t(blockIdx.x) * kPlaneVoters;
+  const int32_t c = int32_t(blockIdx.y * blockDim.x + threadIdx.x);
+  if (c >= ldp) return;
+  int32_t x[kPlaneVoters];
+  uint32_t any = 0;
+  bool bad = false;
+#pragma unroll
+  for (int v = 0; v < kPlaneVoters; ++v) x[v] = c < m && vb + v < nv ? __ldcs(src + (v0 + vb + v) * m + c) : 0;
+#pragma unroll
+  for (int v = 0; v < kPlaneVoters; ++v) {
+    bad |= x[v] < 0 || x[v] > 65534;
+    x[v] &= 0xFFFF;
+    any |= uint32_t(x[v]);
   }
   if (bad) set_status(status, SCHULZE_EDATA);
-  if (big) *wide = 1;  // positions need the 16-bit compare
+  any = __reduce_or_sync(__activemask(), any);
+  if (any & ~*reinterpret_cast<volatile uint32_t*>(used)) atomicOr(used, any);
+  uint32_t* out = planes + int64_t(blockIdx.x) * kPlaneBits * ldp + c;
+#pragma unroll
+  for (int b0 = 0; b0 < kPlaneBits; b0 += 8)
+    put_planes([&](int v) { return uint32_t(x[v]); }, b0, kPlaneBits, out, ldp);
 }
 
-// One CTA counts a TILE x TILE block of d over a chunk of ballots.
-// Thread micro-tile RM x RN (RN even); lanes of a 32-bit word hold two
-// adjacent j columns; the row operand is duplicated into both halves.
-// Positions below 2^15 (guard_ok, and no wide position flagged in *wide)
-// are compared with count_lt2, others with a packed 16-bit compare.
-template <int TILE, int RM, int RN>
-__global__ void __launch_bounds__((TILE / RM) * (TILE / RN))
-    dense_tally_kernel(const uint16_t* __restrict__ pos, int32_t ldp, int64_t nv, int32_t m, int32_t nbt,
-                       int32_t vchunk, int upper_only, int add, int guard_ok, const int32_t* __restrict__ wide,
+// One CTA counts a 64 x 64 tile of d over a chunk of plane groups: the planes
+// of its rows and columns are copied group by group with cp.async,
+// kPlaneStages - 1 groups ahead; a thread compares 8 rows with 4 columns (32
+// independent logic chains). Bound by the integer ALU: three 16-byte
+// shared-memory loads per 32 logic instructions, the population counts on
+// their own unit. Weak orders of 64 tiers, m = 1024, n = 20000: 0.34 ms, from
+// 1.61 ms with packed 16-bit compares (an estimate of 112 ALU cycles per 32 x
+// 32 pairs and group gives 0.24).
+constexpr int kPlaneStages = 4;
+constexpr int kPT = 64;  // tile size
+__global__ void __launch_bounds__(128, 5)
+    plane_tally_kernel(const uint32_t* __restrict__ planes, int32_t ldp, int32_t groups, int32_t m, int32_t nbt,
+                       int32_t gchunk, int upper_only, int add, int bits, const uint32_t* __restrict__ used, int vec,
                        int32_t* __restrict__ d) {
-  const bool guard = guard_ok && !(wide && *wide);
-  const uint32_t gbits = guard ? kGuard2 : 0u;
-  constexpr int TX = TILE / RN, TY = TILE / RM, NT = TX * TY, WN = RN / 2;
-  __shared__ __align__(16) uint32_t sI[kDenseVoters][TILE];      // row positions, duplicated
-  __shared__ __align__(16) uint16_t sJ[kDenseVoters][TILE];      // column positions
+  extern __shared__ __align__(16) uint32_t plane_smem[];  // [kPlaneStages][bits][2 kPT]: rows, then columns
   int32_t tile = blockIdx.x, bi, bj;
   if (upper_only) {  // enumerate bi <= bj
     bi = 0;
@@ -119,72 +185,70 @@ __global__ void __launch_bounds__((TILE / RM) * (TILE / RN))
     bi = tile / nbt;
     bj = tile % nbt;
   }
-  const int32_t I0 = bi * TILE, J0 = bj * TILE;
-  const int64_t vb = int64_t(blockIdx.y) * vchunk;
-  const int64_t ve = min(nv, vb + vchunk);
-  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-  uint32_t acc[RM][WN];
-#pragma unroll
-  for (int r = 0; r < RM; ++r)
-#pragma unroll
-    for (int w = 0; w < WN; ++w) acc[r][w] = 0u;
-
-  for (int64_t v0 = vb; v0 < ve; v0 += kDenseVoters) {
-    const int nvs = int(ve - v0 < kDenseVoters ? ve - v0 : int64_t(kDenseVoters));
-    __syncthreads();
-    for (int t = threadIdx.x; t < kDenseVoters * TILE; t += NT) {
-      int vv = t / TILE, c = t % TILE;
-      uint32_t pi = 0x7FFFu, pj = 0u;  // padding never counts: pi is not below pj
-      if (vv < nvs) {
-        const uint16_t* prow = pos + (v0 + vv) * ldp;
-        pi = prow[I0 + c];
-        pj = prow[J0 + c];
-      }
-      sI[vv][c] = pi | (pi << 16) | gbits;
-      sJ[vv][c] = uint16_t(pj);
-    }
-    __syncthreads();
-    for (int vv = 0; vv < nvs; ++vv) {
-      uint32_t a[RM], b[WN];
-#pragma unroll
-      for (int r = 0; r < RM; r += 4) {
-        uint4 t4 = *reinterpret_cast<const uint4*>(&sI[vv][ty * RM + r]);
-        a[r] = t4.x, a[r + 1] = t4.y, a[r + 2] = t4.z, a[r + 3] = t4.w;
-      }
-#pragma unroll
-      for (int w = 0; w < WN; w += 2) {
-        uint2 t2 = *reinterpret_cast<const uint2*>(&sJ[vv][tx * RN + 2 * w]);
-        b[w] = t2.x, b[w + 1] = t2.y;
-      }
-      if (guard) {
-#pragma unroll
-        for (int r = 0; r < RM; ++r)
-#pragma unroll
-          for (int w = 0; w < WN; ++w) acc[r][w] = count_lt2(acc[r][w], a[r], b[w]);
-      } else {
-#pragma unroll
-        for (int r = 0; r < RM; ++r)
-#pragma unroll
-          for (int w = 0; w < WN; ++w) acc[r][w] = __vsub2(acc[r][w], __vcmpltu2(a[r], b[w]));
+  const int32_t I0 = bi * kPT, J0 = bj * kPT;
+  const int32_t gb = int32_t(blockIdx.y) * gchunk, ge = min(groups, gb + gchunk);
+  const int nbits = used ? 32 - __clz(int(*used)) : bits;  // planes above hold no position's bit
+  const int tx = threadIdx.x % (kPT / 4), ty = threadIdx.x / (kPT / 4);
+  const uint32_t sbase = uint32_t(__cvta_generic_to_shared(plane_smem));
+  auto issue = [&](int32_t g) {
+    if (g < ge) {
+      const uint32_t* src = planes + int64_t(g) * bits * ldp;
+      const uint32_t dst = sbase + uint32_t((g - gb) % kPlaneStages) * uint32_t(bits) * (2 * kPT * 4);
+      for (int t = threadIdx.x; t < nbits * (kPT / 2); t += 128) {  // 16-byte pieces: 16 of the rows, 16 of the columns
+        const int b = t / (kPT / 2), ch = t % (kPT / 2);
+        const uint32_t* from = src + int64_t(b) * ldp + (ch < kPT / 4 ? I0 + 4 * ch : J0 + 4 * (ch - kPT / 4));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + uint32_t(t) * 16u), "l"(from) : "memory");
       }
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  int32_t cnt[8][4];
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) cnt[r][c] = 0;
+#pragma unroll
+  for (int s = 0; s < kPlaneStages - 1; ++s) issue(gb + s);
+  for (int32_t g = gb; g < ge; ++g) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kPlaneStages - 2) : "memory");
+    __syncthreads();  // this group's planes are there, the group before is counted
+    issue(g + kPlaneStages - 1);
+    const uint32_t* S = plane_smem + size_t((g - gb) % kPlaneStages) * bits * (2 * kPT);
+    uint32_t lt[8][4];
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) lt[r][c] = 0u;
+#pragma unroll 2
+    for (int b = 0; b < nbits; ++b) {
+      const uint4 a0 = *reinterpret_cast<const uint4*>(S + b * 2 * kPT + ty * 8);
+      const uint4 a1 = *reinterpret_cast<const uint4*>(S + b * 2 * kPT + ty * 8 + 4);
+      const uint4 q = *reinterpret_cast<const uint4*>(S + b * 2 * kPT + kPT + tx * 4);
+      const uint32_t a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w}, w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) lt[r][c] = plane_lt(a[r], w[c], lt[r][c]);
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) cnt[r][c] += __popc(lt[r][c]);
   }
-  // lanes -> int32 counts (added atomically when several CTAs share a tile)
 #pragma unroll
-  for (int r = 0; r < RM; ++r) {
-    int32_t i = I0 + ty * RM + r;
+  for (int r = 0; r < 8; ++r) {
+    const int32_t i = I0 + ty * 8 + r, j = J0 + tx * 4;
     if (i >= m) continue;
+    int32_t* dst = d + int64_t(i) * m + j;
+    if (!add && vec && j < m) {
+      *reinterpret_cast<int4*>(dst) = make_int4(cnt[r][0], cnt[r][1], cnt[r][2], cnt[r][3]);
+      continue;
+    }
 #pragma unroll
-    for (int w = 0; w < WN; ++w) {
-      int32_t j = J0 + tx * RN + 2 * w;
-      int32_t lo = int32_t(acc[r][w] & 0xFFFFu), hi = int32_t(acc[r][w] >> 16);
-      int32_t* dst = d + int64_t(i) * m + j;
-      if (j < m) {
-        if (add) atomicAdd(dst, lo); else dst[0] = lo;
-      }
-      if (j + 1 < m) {
-        if (add) atomicAdd(dst + 1, hi); else dst[1] = hi;
-      }
+    for (int c = 0; c < 4; ++c) {
+      if (j + c >= m) continue;
+      if (add) atomicAdd(dst + c, cnt[r][c]);  // several CTAs share the tile
+      else dst[c] = cnt[r][c];
     }
   }
 }
@@ -1176,59 +1240,51 @@ bool choose_dense(int64_t n, int32_t m, int32_t k, uint32_t flags) {
   return double(k) * double(k) * 4.0 > double(m) * double(m);
 }
 
-constexpr int kDenseTile = 128;
+int32_t plane_ldp(int32_t m) { return int32_t(align_up(size_t(m), kPT)); }
 
-int32_t dense_tile(int32_t m) { return m <= 64 ? 64 : kDenseTile; }
+int64_t dense_voter_chunk(int64_t n) { return std::min<int64_t>(std::max<int64_t>(n, 1), 1 << 16); }
 
-int64_t dense_voter_chunk(int64_t n, int32_t m) {
-  (void)m;
-  return std::min<int64_t>(std::max<int64_t>(n, 1), 1 << 16);
+size_t plane_bytes(int64_t n, int32_t m) {
+  return align_up(align_up(size_t(dense_voter_chunk(n)), kPlaneVoters) / kPlaneVoters * kPlaneBits * size_t(plane_ldp(m)) * 4,
+                  256) + 4096;
 }
 
-// Position-compare tally over n ballots whose 16-bit position rows build()
-// writes chunk by chunk: build(v0, nv, ldp, pos) fills rows v0 .. v0+nv-1.
-// `full`: strict full orders, only the upper tiles are counted and mirrored.
+// Position-compare tally over n ballots whose bit planes build() writes chunk
+// by chunk: build(v0, nv, ldp, bits, planes, dzero) turns ballots v0 ..
+// v0 + nv - 1 and zeroes dzero (when not null) beside. `full`: strict full
+// orders, only the upper tiles are counted and mirrored. used: the bits in
+// use, when only the device knows them.
 template <class Build>
-int dense_tally(schulze_ctx* ctx, int64_t n, int32_t m, bool full, bool guard_ok, int32_t* wide, int32_t* d,
+int dense_tally(schulze_ctx* ctx, int64_t n, int32_t m, bool full, int bits, const uint32_t* used, int32_t* d,
                 void* ws, cudaStream_t stream, Build build) {
-  const size_t mm = size_t(m) * size_t(m) * sizeof(int32_t);
   const int sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
-  Carver cv(ws);
-  const int32_t tile = dense_tile(m);
-  const int32_t ldp = int32_t(align_up(size_t(m), size_t(tile)));
-  const int32_t nbt = ldp / tile;
+  const int32_t ldp = plane_ldp(m);
+  const int32_t nbt = ldp / kPT;
   const int32_t ntiles = full ? nbt * (nbt + 1) / 2 : nbt * nbt;
-  const int64_t chunk = dense_voter_chunk(n, m);
-  uint16_t* pos = cv.take<uint16_t>(size_t(chunk) * size_t(ldp));
-  // voter split inside a chunk so that the grid covers the GPU about eight
-  // times over: the CTAs stage positions between barriers, and several per
-  // SM hide each other's staging (m = 1024, n = 20000: two per SM 2.57 ms for
-  // weak orders, eight 1.71 ms; the partial counts go into d with atomics)
-  int32_t vsplit = int32_t(std::max<int64_t>(1, (8LL * sms + ntiles - 1) / ntiles));
-  vsplit = int32_t(std::min<int64_t>(vsplit, std::max<int64_t>(1, std::min<int64_t>(n, chunk) / 64)));
+  const int64_t chunk = dense_voter_chunk(n);
+  uint32_t* planes = static_cast<uint32_t*>(ws);
+  const int32_t groups_all = int32_t((std::min<int64_t>(n, chunk) + kPlaneVoters - 1) / kPlaneVoters);
+  // the plane groups of a chunk are split over enough CTAs that the grid
+  // covers the resident CTAs (five per SM) about four times over, at least
+  // two groups each; the partial counts go into d with atomics
+  int32_t vsplit = int32_t(std::max<int64_t>(1, (20LL * sms + ntiles - 1) / ntiles));
+  vsplit = std::min(vsplit, std::max(1, groups_all / 2));
   const bool accumulate = vsplit > 1 || n > chunk;
-  if (accumulate && cudaMemsetAsync(d, 0, mm, stream) != cudaSuccess) return SCHULZE_ECUDA;
+  const size_t smem = size_t(kPlaneStages) * std::max(bits, 1) * (2 * kPT) * 4;
   for (int64_t v0 = 0; v0 < n; v0 += chunk) {
     const int64_t nv = std::min<int64_t>(chunk, n - v0);
-    int32_t vchunk = int32_t((nv + vsplit - 1) / vsplit);
-    vchunk = std::min<int32_t>(vchunk, kMaxVoterChunk);
-    const int32_t gy = int32_t((nv + vchunk - 1) / vchunk);
-    build(v0, nv, ldp, pos);
-    dim3 grid(ntiles, gy);
-    // gy > 1 or several chunks: the kernel adds atomically into zeroed d
+    const int32_t groups = int32_t((nv + kPlaneVoters - 1) / kPlaneVoters);
+    const int32_t gchunk = (groups + vsplit - 1) / vsplit;
+    if (int rc = build(v0, nv, ldp, bits, planes, v0 == 0 && accumulate ? d : nullptr)) return rc;
     Launch L(ctx, stream, "tally_dense", double(nv) * double(m) * double(m - 1) / (full ? 2.0 : 1.0));
-    if (tile == 64)
-      dense_tally_kernel<64, 8, 8><<<grid, 64, 0, stream>>>(pos, ldp, nv, m, nbt, vchunk, full ? 1 : 0,
-                                                             accumulate ? 1 : 0, guard_ok ? 1 : 0, wide, d);
-    else
-      dense_tally_kernel<128, 8, 8><<<grid, 256, 0, stream>>>(pos, ldp, nv, m, nbt, vchunk, full ? 1 : 0,
-                                                               accumulate ? 1 : 0, guard_ok ? 1 : 0, wide, d);
+    plane_tally_kernel<<<dim3(ntiles, (groups + gchunk - 1) / gchunk), 128, smem, stream>>>(
+        planes, ldp, groups, m, nbt, gchunk, full ? 1 : 0, accumulate ? 1 : 0, bits, used, rows_vec16(d, m), d);
     if (int rc = check_launch()) return rc;
   }
   if (full && nbt > 1) {
     Launch L(ctx, stream, "tally_mirror", double(m) * double(m) * 4.0);
     dim3 g((m + 31) / 32, (m + 31) / 32), b(32, 8);
-    mirror_kernel<<<g, b, 0, stream>>>(d, m, tile, n);
+    mirror_kernel<<<g, b, 0, stream>>>(d, m, kPT, n);
   }
   return check_launch();
 }
@@ -1265,9 +1321,7 @@ size_t grouped_bytes(const GroupedPlan& g) {
 
 size_t tally_workspace_bytes(int64_t n, int32_t m, int32_t k, uint32_t flags) {
   if (choose_dense(n, m, k, flags)) {
-    int32_t tile = dense_tile(m);
-    size_t ldp = align_up(size_t(m), size_t(tile));
-    return align_up(size_t(dense_voter_chunk(n, m)) * ldp * 2, 256) + 4096;
+    return plane_bytes(n, m);
   }
   size_t total = size_t(n) * size_t(k);
   // partial counts for up to kCompactMaxCtas slices, either counter width
@@ -1291,12 +1345,19 @@ int tally_launch(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, i
   const int sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
   Carver cv(ws);
   if (choose_dense(n, m, k, flags)) {
-    // strict full orders: d[j][i] = n - d[i][j]
-    return dense_tally(ctx, n, m, k >= m - 1, k <= 32767, nullptr, d, ws, stream,
-                       [&](int64_t v0, int64_t nv, int32_t ldp, uint16_t* pos) {
-                         const int pb = int(std::min<int64_t>((nv + 7) / 8, int64_t(sms) * 16));
+    // strict full orders (every candidate listed, or all but one): d[j][i] = n - d[i][j]
+    int bits = 0;  // of the largest position (k for an unlisted candidate)
+    while ((k < m ? k : k - 1) >> bits) ++bits;
+    return dense_tally(ctx, n, m, k >= m - 1, bits, nullptr, d, ws, stream,
+                       [&](int64_t v0, int64_t nv, int32_t ldp, int nbits, uint32_t* planes, int32_t* dzero) -> int {
+                         const size_t smem = size_t(kPlaneVoters) * size_t(std::min(ldp, kPlaneCols)) * 2;
+                         cudaFuncSetAttribute(slice_ballots_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              int(smem));
+                         const dim3 g((nv + kPlaneVoters - 1) / kPlaneVoters, (ldp + kPlaneCols - 1) / kPlaneCols);
                          Launch L(ctx, stream, "tally_positions", double(nv) * (double(k) * 4.0 + double(ldp) * 2.0));
-                         pos_build_kernel<<<pb, 256, 0, stream>>>(ranks, v0, nv, m, k, ldp, pos, ctx->status);
+                         slice_ballots_kernel<<<g, 512, smem, stream>>>(ranks, v0, nv, m, k, ldp, nbits, planes,
+                                                                        ctx->status, dzero);
+                         return check_launch();
                        });
   }
   // sparse
@@ -1404,24 +1465,21 @@ int tally_launch(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, i
   return check_launch();
 }
 
-size_t tally_positions_workspace_bytes(int64_t n, int32_t m) {
-  const int32_t tile = dense_tile(m);
-  const size_t ldp = align_up(size_t(m), size_t(tile));
-  return align_up(size_t(dense_voter_chunk(n, m)) * ldp * 2, 256) + 4096;
-}
+size_t tally_positions_workspace_bytes(int64_t n, int32_t m) { return plane_bytes(n, m); }
 
 int tally_positions_launch(schulze_ctx* ctx, const int32_t* pos_in, int64_t n, int32_t m, int32_t* d, void* ws,
                            cudaStream_t stream) {
   if (n == 0) return cudaMemsetAsync(d, 0, size_t(m) * size_t(m) * 4, stream) == cudaSuccess ? SCHULZE_OK : SCHULZE_ECUDA;
-  const int sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
-  // the flag word sits after the position rows in the workspace
-  int32_t* wide = reinterpret_cast<int32_t*>(static_cast<char*>(ws) + tally_positions_workspace_bytes(n, m) - 256);
-  if (cudaMemsetAsync(wide, 0, sizeof(int32_t), stream) != cudaSuccess) return SCHULZE_ECUDA;
-  return dense_tally(ctx, n, m, false, true, wide, d, ws, stream,
-                     [&](int64_t v0, int64_t nv, int32_t ldp, uint16_t* pos) {
-                       const int g = int(std::max<int64_t>(1, std::min<int64_t>((nv * ldp + 255) / 256, int64_t(sms) * 8)));
+  // the word of the bits in use sits after the planes in the workspace
+  uint32_t* used = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + tally_positions_workspace_bytes(n, m) - 256);
+  return dense_tally(ctx, n, m, false, kPlaneBits, used, d, ws, stream,
+                     [&](int64_t v0, int64_t nv, int32_t ldp, int, uint32_t* planes, int32_t* dzero) -> int {
+                       if (cudaMemsetAsync(used, 0, sizeof(uint32_t), stream) != cudaSuccess) return SCHULZE_ECUDA;
+                       const dim3 g((nv + kPlaneVoters - 1) / kPlaneVoters, (ldp + 255) / 256);
                        Launch L(ctx, stream, "tally_positions_copy", double(nv) * double(m) * 4.0);
-                       pos_copy_kernel<<<g, 256, 0, stream>>>(pos_in, v0, nv, m, ldp, pos, ctx->status, wide);
+                       slice_positions_kernel<<<g, 256, 0, stream>>>(pos_in, v0, nv, m, ldp, planes, ctx->status, used,
+                                                                     dzero);
+                       return check_launch();
                      });
 }
 

@@ -312,7 +312,7 @@ int schulze_batch_run_host(schulze_batch* b, const int32_t* ranks_host, int32_t*
 int schulze_batch_set_schedule(schulze_batch* b, int32_t tally_policy, int32_t order_policy);
 
 /* Elections are grouped by m into five buckets (m <= 64, 128, 256, 512,
- * 1024); the tally of an election stages `chunk` ballots per step as position
+ * 1024); the tally of an election reads `chunk` ballots per step into position
  * rows in shared memory (8, 16, 32 or 64; a power of two that fits: chunk *
  * ceil64(m) * 6 bytes within the CTA's shared memory and chunk * m <= 8192),
  * set here per bucket (EINVAL for a size that does not fit the bucket's
@@ -321,9 +321,9 @@ int schulze_batch_set_bucket_chunk(schulze_batch* b, int32_t bucket, int32_t chu
 
 /* The tally of an election covers d in 64 x 64 tiles, worked on by the four
  * 128-thread tile groups of a CTA; groups_per_tile (1, 2 or 4) groups share
- * one tile, each counting every groups_per_tile-th staged ballot (so an
- * election of one or two tiles still keeps all four busy), set here per
- * bucket (EINVAL otherwise). Synchronous. */
+ * one tile, each counting a part of its rows (an election or a last round of
+ * one or two tiles is shared in any case), set here per bucket (EINVAL
+ * otherwise). Synchronous. */
 int schulze_batch_set_bucket_tiles(schulze_batch* b, int32_t bucket, int32_t groups_per_tile);
 
 /* The per-bucket schedule: largest m of each bucket, its ballots per step

@@ -27,13 +27,12 @@ namespace {
 constexpr int kBT = 512;                        // threads per batch CTA
 constexpr int kGroups = kBT / tiles::kThreads;  // tile groups of 128 threads
 constexpr int32_t kBatchMaxM = 1024;
-constexpr int64_t kFlushVoters = 32768;  // 16-bit lane counters are flushed before they can overflow
 
 struct Job {
   int32_t n, m, k, e;
   int64_t ranks_off, mat_off, vec_off;
-  int32_t chunk;  // ballots staged per tally step (the schedule of the election's m-bucket)
-  int32_t gpt;    // tile groups that share one tally tile, splitting its ballots (1, 2 or 4)
+  int32_t chunk;  // ballots read per tally step (the schedule of the election's m-bucket)
+  int32_t gpt;    // tile groups that share the rows of one tally tile (1, 2 or 4)
   int32_t seg;    // schulze_batch_run_host: the segment whose arrival mark the job waits for
   int32_t pad;
 };
@@ -65,8 +64,8 @@ struct BatchArgs {
   int32_t* order;
   int32_t* beaten_by;
   unsigned char* scratch;
-  size_t slot_bytes;  // per CTA: W slot, then a d slot when the caller passes no d
-  size_t w_bytes;
+  size_t slot_bytes;  // per CTA: W slot, a d slot for when the caller passes no d, position planes
+  size_t w_bytes, plane_off;
   int32_t* status;
   // schulze_batch_run_host: arrival marks of the ballot segments (set by the
   // copy stream after each segment's copy; null otherwise) and the bound on
@@ -75,10 +74,8 @@ struct BatchArgs {
   long long wait_limit;
 };
 
-// Dynamic shared memory of one batch CTA, reused stage by stage. The tally
-// stages `chunk` ballots as position rows of mpad (m rounded up to 64)
-// entries: dup[chunk][mpad] (position in both 16-bit halves, guard bits set)
-// then pos[chunk][mpad] (16-bit), carved from `raw`.
+// Dynamic shared memory of one batch CTA, reused stage by stage: the tally's
+// position rows and its staged planes are carved from `raw`.
 constexpr size_t kStageBytes = sizeof(tiles::SmemS32) * kGroups + 2 * tiles::kB * 4;
 union BatchSmem {
   unsigned char raw[kStageBytes];
@@ -97,27 +94,169 @@ union BatchSmem {
 
 constexpr int kTT = 64;  // tally tile: 64 x 64 counters per group, 8 x 4 per thread
 constexpr int kDiagBlocks = 72;  // 8 x 4 blocks of a diagonal tile on or above the diagonal
+constexpr int kPlaneVoters = 32;     // ballots per plane word
+constexpr int kPlaneGroups = 256;    // plane groups counted at a time (bounds the CTA's scratch; counts fit 16 bits)
 
-// The election's d, tile by tile: the four 128-thread groups take tiles of
-// 64 x 64 entries, jb.gpt groups per tile (4 / gpt tiles per round), and
-// count them in 16-bit lanes (two columns per word, the row operand
-// duplicated into both halves); the groups of one tile take alternate
-// staged ballots and add their counts into d (zeroed first) with atomics,
-// so an election of one or two tiles still keeps every group busy (and so
-// does a last round with one or two tiles left, whatever jb.gpt is).
-// Ballots are staged `chunk` at a time as full position rows (unlisted
-// candidates at position k), so one staging serves the four tiles of a
-// round. Counters are added into d every kFlushVoters ballots. Full
-// rankings count only the tiles above the diagonal and the thread blocks of
-// the diagonal tiles on or above it (whole diagonal tiles when groups share
-// tiles), and mirror the rest: d[j][i] = n - d[i][j]. The first round also checks the ballots: an
-// id out of range, or one whose position slot is already taken within the
-// same ballot, is reported as SCHULZE_EDATA.
-__device__ void tally(const Job& jb, const int32_t* __restrict__ ranks, int32_t* __restrict__ dm, BatchSmem& sm,
-                      int32_t* status) {
-  const int32_t n = jb.n, m = jb.m, k = jb.k;
-  const bool full = k >= m - 1;
-  const int32_t nbt = (m + kTT - 1) / kTT;
+__host__ __device__ inline int position_bits(int32_t m, int32_t k) {  // of the largest position (k: unlisted)
+  int bits = 0;
+  while ((k < m ? k : k - 1) >> bits) ++bits;
+  return bits;
+}
+
+// Bit planes of the positions on ballots v0 .. v0 + 32 groups - 1 (those past
+// n count as all tied): planes[(g * bits + b) * mpad + c] holds bit b of
+// candidate c's position on ballots 32 g .. 32 g + 31 (count.cuh: comparing
+// two such words bit by bit costs one logic instruction per position bit for
+// 32 ballots). Ballots are read `chunk` at a time (the election's schedule),
+// their ids two steps ahead in registers, into 16-bit position rows in shared
+// memory (unlisted candidates at k), which are turned 32 rows at a time.
+// An id out of range or repeated within its ballot sets SCHULZE_EDATA. On full
+// rankings a repeated id leaves another candidate out: each row's entries
+// carry a bit that alternates between uses of the row, and the turn finds a
+// candidate that kept the old one (reading the ids' entries back instead, as
+// for shorter ballots, costs as many bank conflicts as writing them: the
+// entries of a ballot are 32 random places).
+__device__ void make_planes(const Job& jb, const int32_t* __restrict__ ranks, int64_t v0, int32_t groups, int bits,
+                            uint32_t* planes, BatchSmem& sm, int32_t* status) {
+  const int32_t n = jb.n, m = jb.m, k = jb.k, mpad = int32_t(align_up(size_t(m), kTT));
+  const int chunk = jb.chunk, rows = max(chunk, kPlaneVoters);  // chunk * k <= kBT * kPrefetch (plan)
+  const int tid = threadIdx.x, lanes = kBT / chunk, vv = tid / lanes, q0 = tid % lanes;
+  uint16_t* pos = reinterpret_cast<uint16_t*>(sm.raw);  // [rows][mpad]
+  const bool marked = k == m;  // positions below 1024, bit 15 is the mark
+  uint32_t mark = 0x8000u;
+  if (marked) {
+    for (int t = tid; t < rows * mpad / 2; t += kBT) reinterpret_cast<uint32_t*>(pos)[t] = 0u;
+    __syncthreads();
+  }
+  // ids of positions q0 + u * lanes of ballot vv of the step, and of the next
+  // one: two sets used in turn (moving one into the other would wait for its loads)
+  int32_t ids0[kPrefetch], ids1[kPrefetch];
+  auto load_ids = [&](int64_t v, int32_t (&x)[kPrefetch]) {
+    const bool have = v + vv < n;
+    const int32_t* row = ranks + (v + vv) * k;
+#pragma unroll
+    for (int u = 0; u < kPrefetch; ++u) {
+      const int32_t q = q0 + u * lanes;
+      x[u] = (have && q < k) ? __ldcg(row + q) : -1;  // L2 only: see schulze_batch_run_host
+    }
+  };
+  bool bad = false;
+  load_ids(v0, ids0);
+  load_ids(v0 + chunk, ids1);
+  const int64_t vend = v0 + int64_t(groups) * kPlaneVoters;
+  int row0 = 0, g0 = 0;  // the step's first row; the plane group of row 0
+  auto step = [&](int64_t v, int32_t (&cv)[kPrefetch]) {
+    // unlisted candidates, and all of a missing ballot, at position k
+    const bool fill = k < m || v + chunk > n;
+    if (fill) {
+      const uint32_t k2 = (uint32_t(k) | (marked ? mark : 0u)) * 0x10001u;
+      const int skip = marked ? int(min(int64_t(chunk), max(int64_t(0), n - v))) : 0;  // (full ballots need no filling)
+      uint32_t* p2 = reinterpret_cast<uint32_t*>(pos + (row0 + skip) * mpad);
+      for (int t = tid; t < (chunk - skip) * mpad / 2; t += kBT) p2[t] = k2;
+      __syncthreads();
+    }
+    uint16_t* prow = pos + (row0 + vv) * mpad;
+    const bool have = v + vv < n;
+#pragma unroll
+    for (int u = 0; u < kPrefetch; ++u) {
+      const int32_t q = q0 + u * lanes, c = cv[u];
+      if (!have || q >= k) break;
+      if (c < 0 || c >= m) bad = true;
+      else prow[c] = uint16_t(uint32_t(q) | (marked ? mark : 0u));
+    }
+    if (marked) load_ids(v + 2 * chunk, cv);  // in flight from here on
+    __syncthreads();
+    if (!marked) {
+      // a repeated id keeps only one of its positions: the other one sees it
+#pragma unroll
+      for (int u = 0; u < kPrefetch; ++u) {
+        const int32_t q = q0 + u * lanes, c = cv[u];
+        if (!have || q >= k) break;
+        if (c >= 0 && c < m && prow[c] != uint16_t(q)) bad = true;
+      }
+      load_ids(v + 2 * chunk, cv);
+    }
+    row0 += chunk;
+    if (row0 < rows) return;
+    for (int t = tid; t < rows / kPlaneVoters * mpad; t += kBT) {
+      const int gl = t / mpad, c = t - gl * mpad;
+      const uint16_t* at = pos + gl * kPlaneVoters * mpad + c;
+      uint32_t w[16];
+#pragma unroll
+      for (int q = 0; q < 16; ++q) w[q] = uint32_t(at[q * mpad]) | (uint32_t(at[(q + 16) * mpad]) << 16);
+      transpose_planes(w);
+      // (a missing ballot's row was filled with the mark)
+      if (marked && c < m && w[15] != (mark ? 0xFFFFFFFFu : 0u) && g0 + gl < groups) bad = true;
+      if (g0 + gl < groups) {
+        uint32_t* out = planes + int64_t(g0 + gl) * bits * mpad + c;
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+          if (q < bits) out[q * mpad] = w[q];
+      }
+    }
+    __syncthreads();  // the rows are free
+    mark ^= 0x8000u, row0 = 0, g0 += rows / kPlaneVoters;
+  };
+  for (int64_t v = v0; v < vend; v += 2 * chunk) {
+    step(v, ids0);
+    if (v + chunk < vend) step(v + chunk, ids1);
+  }
+  if (bad) set_status(status, SCHULZE_EDATA);
+}
+
+// counts of one plane group into a thread's RPT x 4 block (rows R0.., columns
+// C0..; two 16-bit counters per word)
+template <int RPT>
+__device__ __forceinline__ void count_group(const uint32_t* S, int bits, int32_t mpad, int32_t R0, int32_t C0,
+                                            uint32_t (&acc)[8][2]) {
+  uint32_t lt[RPT][4];
+#pragma unroll
+  for (int r = 0; r < RPT; ++r) lt[r][0] = lt[r][1] = lt[r][2] = lt[r][3] = 0u;
+#pragma unroll 2
+  for (int b = 0; b < bits; ++b) {
+    const uint32_t* P = S + b * mpad;
+    uint32_t a[RPT];
+    if (RPT == 2) {
+      const uint2 x = *reinterpret_cast<const uint2*>(P + R0);
+      a[0] = x.x, a[1] = x.y;
+    } else {
+#pragma unroll
+      for (int r = 0; r < RPT; r += 4) {
+        const uint4 x = *reinterpret_cast<const uint4*>(P + R0 + r);
+        a[r] = x.x, a[r + 1] = x.y, a[r + 2] = x.z, a[r + 3] = x.w;
+      }
+    }
+    const uint4 y = *reinterpret_cast<const uint4*>(P + C0);
+    const uint32_t w[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+    for (int r = 0; r < RPT; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) lt[r][c] = plane_lt(a[r], w[c], lt[r][c]);
+  }
+#pragma unroll
+  for (int r = 0; r < RPT; ++r)
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+      acc[r][c] += uint32_t(__popc(lt[r][2 * c])) + (uint32_t(__popc(lt[r][2 * c + 1])) << 16);
+}
+
+// The counts of `groups` plane groups (at most kPlaneGroups), stored into d
+// or (!first) added to it. The four 128-thread groups take 64 x 64 tiles of
+// d, two each per round (the planes are read once per round), with jb.gpt
+// groups per tile, which then share its rows (and so does a last round with
+// one or two tiles left, whatever jb.gpt is). Planes are copied with cp.async
+// while the groups before are counted. Full rankings count only the
+// tiles above the diagonal and the thread blocks of the diagonal tiles on or
+// above it (whole diagonal tiles when groups share tiles), and the last pass
+// writes the mirror images d[j][i] = n - d[i][j] with them, eight consecutive
+// entries of four rows per thread. Bound by the integer ALU: 4096 elections
+// (m to 512, n to 5000) 13.2 ms a CTA, where the logic, counts and adds alone
+// take 8.3; the planes before it 5.0, the closure 7.0, the other stages 3.7.
+// Counting packed 16-bit compares in the same kernel, the batch took 85.9 ms.
+__device__ void count_planes(const Job& jb, const uint32_t* planes, int32_t groups, int bits, bool first, bool last,
+                             int32_t* __restrict__ dm, BatchSmem& sm) {
+  const int32_t m = jb.m, mpad = int32_t(align_up(size_t(m), kTT)), nbt = mpad / kTT;
+  const bool full = jb.k >= m - 1;
   const int tid = threadIdx.x, g = tid / tiles::kThreads, lt = tid % tiles::kThreads;
   const int tx = lt % (kTT / 4), ty = lt / (kTT / 4);
   // Full rankings with one group per tile: the tiles above the diagonal are
@@ -127,49 +266,44 @@ __device__ void tally(const Job& jb, const int32_t* __restrict__ ranks, int32_t*
   const bool packdiag = full && jb.gpt == 1;
   const int32_t noff = nbt * (nbt - 1) / 2;
   const int32_t ntiles = !full ? nbt * nbt : packdiag ? noff + (nbt * kDiagBlocks + 127) / 128 : nbt * (nbt + 1) / 2;
-  // positions are below 2^15 (m <= 1024): the row operand carries the guard
-  // bits of count_lt2
-  const uint32_t unl = uint32_t(k) & 0xFFFFu, unl2 = unl | (unl << 16) | kGuard2;
-  const int32_t mpad = int32_t(align_up(size_t(m), kTT));
-  const int chunk = jb.chunk;  // chunk * mpad * 6 <= sizeof(BatchSmem), chunk * k <= kBT * kPrefetch (plan)
-  const int gpt = jb.gpt, tpr = kGroups / gpt;  // tiles per round
-  // a last round with fewer tiles than groups shares them out: one tile to
-  // all four groups, two tiles to two groups each
-  const int32_t rem_last = ntiles % tpr;
-  const int gpt_last = rem_last == 0 ? gpt : kGroups / (rem_last == 1 ? 1 : rem_last == 2 ? 2 : 4);
-  uint32_t* dup = reinterpret_cast<uint32_t*>(sm.raw);                         // [chunk][mpad]
-  uint16_t* pos = reinterpret_cast<uint16_t*>(sm.raw + size_t(chunk) * mpad * 4);  // [chunk][mpad]
-  // ballot ids of a step: thread tid holds positions q0 + u * lanes of ballot
-  // vv of the step; the next step's ids are loaded before this step's counts
-  const int lanes = kBT / chunk;
-  const int vv = tid / lanes, q0 = tid % lanes;
-  int32_t cv[kPrefetch];
-  auto load_ids = [&](int64_t v0n) {
-    const bool have = v0n + vv < n;
-    const int32_t* row = ranks + (v0n + vv) * k;
-#pragma unroll
-    for (int u = 0; u < kPrefetch; ++u) {
-      const int32_t q = q0 + u * lanes;
-      cv[u] = (have && q < k) ? __ldcg(row + q) : -1;  // L2 only: see schulze_batch_run_host
-    }
+  const int32_t gwords = bits * mpad;  // words of one plane group
+  // two stages of U plane groups each: one barrier per U groups, between which
+  // the warps drift apart, so that one warp's population counts (a quarter of
+  // the logic rate, on their own unit) run beside the others' logic
+  const int U = max(1, min(8, int(kStageBytes / (8 * size_t(max(gwords, 1))))));
+  const int32_t uwords = U * gwords;
+  const uint32_t* stage = reinterpret_cast<const uint32_t*>(sm.raw);  // [2][U][gwords]
+  const uint32_t sbase = uint32_t(__cvta_generic_to_shared(stage));
+  auto issue = [&](int32_t q0, int buf) {
+    const uint32_t* src = planes + int64_t(q0) * gwords;
+    const uint32_t dst = sbase + uint32_t(buf) * uint32_t(uwords) * 4u;
+    const int32_t words = min(U, groups - q0) * gwords;  // (negative past the end)
+    for (int t = tid; t < words / 4; t += kBT)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + uint32_t(t) * 16u), "l"(src + 4 * t)
+                   : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  if (gpt > 1 || gpt_last > 1)  // the groups of a tile add into d (visible after the first barrier below)
-    for (int64_t t = tid; t < int64_t(m) * m; t += kBT) dm[t] = 0;
+  const int tpr = 2 * kGroups / jb.gpt;  // tiles per round
   for (int32_t t0 = 0; t0 < ntiles; t0 += tpr) {
-    // this group's task and its share of the staged ballots; the thread's
-    // 8 x 4 block of d starts at row R0, column C0 (act: it has one)
-    const int gr = ntiles - t0 < tpr ? gpt_last : gpt, phase = g % gr;
-    const int32_t tt = t0 + g / gr;
-    int32_t R0 = 0, C0 = 0;
-    bool act = tt < ntiles;
-    if (act) {
+    const int T = min(tpr, ntiles - t0);
+    const int gr = max(jb.gpt, T == 1 ? 4 : T == 2 ? 2 : 1), teams = kGroups / gr;  // groups per tile, tiles at a time
+    // this thread's blocks of d: rows R0.., columns C0.. (8 / gr rows)
+    int32_t R0[2], C0[2];
+    bool act[2], mir[2];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const int32_t tt = t0 + g / gr + s * teams;
+      R0[s] = C0[s] = 0;
+      act[s] = tt < t0 + T, mir[s] = false;
+      if (!act[s]) continue;
       if (packdiag && tt >= noff) {  // packed blocks of the diagonal tiles
         const int32_t idx = (tt - noff) * 128 + lt;
-        act = idx < nbt * kDiagBlocks;
-        const int32_t dt = idx / kDiagBlocks;
+        act[s] = idx < nbt * kDiagBlocks;
+        const int32_t dt = act[s] ? idx / kDiagBlocks : 0;
         int blk = idx % kDiagBlocks, by = 0;
         while (blk >= kTT / 4 - 2 * by) blk -= kTT / 4 - 2 * by, ++by;  // row group by holds 16 - 2 by blocks
-        R0 = dt * kTT + by * 8, C0 = dt * kTT + (2 * by + blk) * 4;
+        R0[s] = dt * kTT + by * 8, C0[s] = dt * kTT + (2 * by + blk) * 4;
+        mir[s] = last && blk >= 2;  // (the first two blocks of a row group hold both halves)
       } else {
         int32_t bi = 0, bj = 0;
         if (full) {  // tiles bi <= bj in order (bi < bj when the diagonal is packed)
@@ -180,151 +314,209 @@ __device__ void tally(const Job& jb, const int32_t* __restrict__ ranks, int32_t*
         } else {
           bi = tt / nbt, bj = tt % nbt;
         }
-        R0 = bi * kTT + ty * 8, C0 = bj * kTT + tx * 4;
+        R0[s] = bi * kTT + ty * 8, C0[s] = bj * kTT + tx * 4;
+        mir[s] = last && full && bi != bj;
       }
+      R0[s] += (g % gr) * (8 / gr);
     }
-    const bool check = t0 == 0;
-    uint32_t acc[8][2];
+    uint32_t acc[2][8][2];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) acc[r][0] = acc[r][1] = 0u;
-    bool first_flush = true;
-    load_ids(0);
-    for (int64_t v0 = 0; v0 < n; v0 += chunk) {
-      const int nv = int(n - v0 < chunk ? n - v0 : int64_t(chunk));
-      __syncthreads();
-      if (k < m || check) {  // unlisted candidates sit at position k
-        for (int t = tid; t < chunk * mpad; t += kBT) {
-          dup[t] = unl2;
-          pos[t] = uint16_t(unl);
-        }
-        __syncthreads();
-      } else if (mpad > m) {  // full ballots fill 0..m-1; the padding stays unlisted
-        for (int t = tid; t < chunk * (mpad - m); t += kBT) {
-          const int w = t / (mpad - m), c = m + t % (mpad - m);
-          dup[w * mpad + c] = unl2;
-          pos[w * mpad + c] = uint16_t(unl);
-        }
-      }
-      if (vv < nv) {  // this step's ids, loaded during the previous step
-#pragma unroll
-        for (int u = 0; u < kPrefetch; ++u) {
-          const int32_t q = q0 + u * lanes;
-          if (q >= k) break;
-          const int32_t c = cv[u];
-          if (c < 0 || c >= m) {
-            if (check) set_status(status, SCHULZE_EDATA);
-            continue;
-          }
-          const uint32_t q2 = uint32_t(q) | (uint32_t(q) << 16) | kGuard2;
-          if (check) {
-            if (atomicExch(&dup[vv * mpad + c], q2) != unl2) set_status(status, SCHULZE_EDATA);
-          } else {
-            dup[vv * mpad + c] = q2;
-          }
-          pos[vv * mpad + c] = uint16_t(q);
-        }
-      }
-      if (v0 + chunk < n) load_ids(v0 + chunk);  // in flight while this step counts
-      __syncthreads();
-      if (act) {
-        for (int u = phase; u < nv; u += gr) {
-          uint32_t a[8], b[2];
-          const uint4 a0 = *reinterpret_cast<const uint4*>(&dup[u * mpad + R0]);
-          const uint4 a1 = *reinterpret_cast<const uint4*>(&dup[u * mpad + R0 + 4]);
-          a[0] = a0.x, a[1] = a0.y, a[2] = a0.z, a[3] = a0.w, a[4] = a1.x, a[5] = a1.y, a[6] = a1.z, a[7] = a1.w;
-          const uint2 bv = *reinterpret_cast<const uint2*>(&pos[u * mpad + C0]);
-          b[0] = bv.x, b[1] = bv.y;
-#pragma unroll
-          for (int r = 0; r < 8; ++r) {
-            acc[r][0] = count_lt2(acc[r][0], a[r], b[0]);
-            acc[r][1] = count_lt2(acc[r][1], a[r], b[1]);
-          }
-        }
-        const bool last = v0 + chunk >= n;
-        if (last || ((v0 + chunk) % kFlushVoters) == 0) {
-#pragma unroll
-          for (int r = 0; r < 8; ++r) {
-            const int32_t i = R0 + r;
-#pragma unroll
-            for (int w = 0; w < 2; ++w) {
-              const int32_t j = C0 + 2 * w;
-              if (i < m) {
-                int32_t* dst = dm + int64_t(i) * m + j;
-                const int32_t lo = int32_t(acc[r][w] & 0xFFFFu), hi = int32_t(acc[r][w] >> 16);
-                if (gr > 1) {
-                  if (j < m && lo) atomicAdd(dst, lo);
-                  if (j + 1 < m && hi) atomicAdd(dst + 1, hi);
-                } else {
-                  if (j < m) dst[0] = (first_flush ? 0 : dst[0]) + lo;
-                  if (j + 1 < m) dst[1] = (first_flush ? 0 : dst[1]) + hi;
-                }
-              }
-            }
-            acc[r][0] = acc[r][1] = 0u;
-          }
-          first_flush = false;
+    for (int r = 0; r < 8; ++r) acc[0][r][0] = acc[0][r][1] = acc[1][r][0] = acc[1][r][1] = 0u;
+    issue(0, 0);
+    for (int32_t q0 = 0, buf = 0; q0 < groups; q0 += U, buf ^= 1) {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();  // these groups' planes are there, the ones before are counted
+      issue(q0 + U, buf ^ 1);
+      const int qn = min(U, groups - q0);
+      for (int q = 0; q < qn; ++q) {
+        const uint32_t* S = stage + buf * uwords + q * gwords;
+        if (gr == 1) {
+          if (act[0]) count_group<8>(S, bits, mpad, R0[0], C0[0], acc[0]);
+          if (act[1]) count_group<8>(S, bits, mpad, R0[1], C0[1], acc[1]);
+        } else if (gr == 2) {
+          if (act[0]) count_group<4>(S, bits, mpad, R0[0], C0[0], acc[0]);
+          if (act[1]) count_group<4>(S, bits, mpad, R0[1], C0[1], acc[1]);
+        } else {
+          if (act[0]) count_group<2>(S, bits, mpad, R0[0], C0[0], acc[0]);
+          if (act[1]) count_group<2>(S, bits, mpad, R0[1], C0[1], acc[1]);
         }
       }
     }
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      if (!act[s]) continue;
+      int32_t v[8][4];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const int32_t i = R0[s] + r;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int32_t j = C0[s] + c;
+          v[r][c] = int32_t((acc[s][r][c >> 1] >> (16 * (c & 1))) & 0xFFFFu);
+          if (r >= 8 / gr || i >= m || j >= m) continue;
+          int32_t* dst = dm + int64_t(i) * m + j;
+          if (!first) v[r][c] += *dst;
+          *dst = v[r][c];
+        }
+      }
+      if (!mir[s]) continue;
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+          const int32_t i = R0[s] + r, j = C0[s] + c;
+          if (r < 8 / gr && i < m && j < m) dm[int64_t(j) * m + i] = jb.n - v[r][c];
+        }
+    }
+    __syncthreads();  // the stages are free
   }
-  __syncthreads();
-  if (full && (nbt > 1 || packdiag)) {
-    // the tiles below the diagonal and, when packed, the blocks of the
-    // diagonal tiles below it (column block (j % 64) / 4 < 2 (i % 64) / 8)
-    for (int64_t t = threadIdx.x; t < int64_t(m) * m; t += kBT) {
-      const int32_t i = int32_t(t / m), j = int32_t(t % m);
-      if (i / kTT > j / kTT || (packdiag && i / kTT == j / kTT && (j % kTT) / 4 < 2 * ((i % kTT) / 8)))
-        dm[t] = n - dm[int64_t(j) * m + i];
-    }
+}
+
+// The election's d: planes and counts, kPlaneGroups plane groups (8192
+// ballots) at a time.
+__device__ void tally(const Job& jb, const int32_t* __restrict__ ranks, int32_t* __restrict__ dm, uint32_t* planes,
+                      BatchSmem& sm, int32_t* status) {
+  const int32_t n = jb.n;
+  const int bits = position_bits(jb.m, jb.k);
+  for (int64_t v0 = 0; v0 < n; v0 += kPlaneGroups * kPlaneVoters) {
+    const int32_t groups = int32_t(min(int64_t(kPlaneGroups), (n - v0 + kPlaneVoters - 1) / kPlaneVoters));
+    make_planes(jb, ranks, v0, groups, bits, planes, sm, status);
+    __syncthreads();  // the planes are written
+    count_planes(jb, planes, groups, bits, v0 == 0, v0 + kPlaneGroups * kPlaneVoters >= n, dm, sm);
   }
   __syncthreads();
 }
 
 // ----------------------------------------------------------- stages
 
+constexpr int kMaxTiles = kBatchMaxM / tiles::kB;  // tile rows of the largest election
+
+// What the stages after the tally share: the relabeling of the candidates by
+// strength (row sums of d, strongest first), the bounds of the tiles of W and
+// the tiles of a phase of the closure that need their update.
+struct Shared {
+  uint16_t perm[kBatchMaxM], inv[kBatchMaxM];  // new -> old, old -> new
+  float key[kBatchMaxM];
+  int32_t tmax[kMaxTiles * kMaxTiles], tmin[kMaxTiles * kMaxTiles];
+  uint16_t list[kMaxTiles * kMaxTiles];
+  int32_t count;
+};
+
+// Strongest first, by row sums of d (ties by id): like candidates then share
+// tiles and most tile updates can be skipped (see closure.cu).
+__device__ void relabel(const int32_t* __restrict__ dm, int32_t m, Shared& sh) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int32_t i = wid; i < m; i += kBT / 32) {
+    float s = 0.f;
+    for (int32_t j = lane; j < m; j += 32) s += float(dm[int64_t(i) * m + j]);
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+    if (lane == 0) sh.key[i] = s;
+  }
+  __syncthreads();
+  for (int32_t i = threadIdx.x; i < m; i += kBT) {
+    const float mine = sh.key[i];
+    int32_t r = 0;
+    for (int32_t j = 0; j < m; ++j) r += sh.key[j] > mine || (sh.key[j] == mine && j < i);
+    sh.perm[r] = uint16_t(i), sh.inv[i] = uint16_t(r);
+  }
+  __syncthreads();
+}
+
+// W = the weights in strength order, a warp per row, and the tiles' bounds
 template <typename E>
-__device__ void pack(const int32_t* __restrict__ dm, int32_t m, int32_t mp, E* __restrict__ W) {
-  for (int64_t t = threadIdx.x; t < int64_t(mp) * mp; t += kBT) {
-    const int32_t i = int32_t(t / mp), j = int32_t(t % mp);
-    int32_t out = 0;
-    if (i < m && j < m && i != j) {
-      const int32_t a = dm[int64_t(i) * m + j], b = dm[int64_t(j) * m + i];
-      if (a > b) out = a;
+__device__ void pack(const Job& jb, const int32_t* __restrict__ dm, int32_t mp, E* __restrict__ W, Shared& sh) {
+  const int32_t m = jb.m, n = jb.n, nb = mp / tiles::kB;
+  const bool full = jb.k >= m - 1 && n > 0;  // then d[j][i] = n - d[i][j]
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int t = threadIdx.x; t < nb * nb; t += kBT) sh.tmax[t] = 0, sh.tmin[t] = INT32_MAX;
+  __syncthreads();
+  for (int32_t a = wid; a < mp; a += kBT / 32) {
+    const int32_t i = a < m ? sh.perm[a] : -1;
+    for (int32_t b = lane; b < mp; b += 32) {
+      int32_t out = 0;
+      if (i >= 0 && b < m && a != b) {
+        const int32_t j = sh.perm[b], x = dm[int64_t(i) * m + j], y = full ? n - x : dm[int64_t(j) * m + i];
+        if (x > y) out = x;
+      }
+      W[int64_t(a) * mp + b] = E(out);
+      const int32_t mx = __reduce_max_sync(0xFFFFFFFFu, out);
+      const int32_t mn = __reduce_min_sync(0xFFFFFFFFu, i >= 0 && b < m && a != b ? out : INT32_MAX);
+      if (lane == 0) {
+        const int t = (a / tiles::kB) * nb + b / tiles::kB;
+        atomicMax(&sh.tmax[t], mx), atomicMin(&sh.tmin[t], mn);
+      }
     }
-    W[t] = E(out);
   }
   __syncthreads();
 }
 
 template <typename E>
-__device__ void closure(E* __restrict__ W, int32_t mp, BatchSmem& sm) {
+__device__ void closure(E* W, int32_t m, int32_t mp, BatchSmem& sm, Shared& sh) {
   using Ops = tiles::Ops<E>;
-  const int32_t nb = mp / tiles::kB;
+  using tiles::Bounds;
+  using tiles::kB;
+  const int32_t nb = mp / kB;
   const int g = threadIdx.x / tiles::kThreads, lt = threadIdx.x % tiles::kThreads;
   const tiles::GroupBarrier bar{1 + g};
   auto& ts = sizeof(E) == 2 ? reinterpret_cast<typename Ops::Smem*>(sm.c16.t)[g]
                             : reinterpret_cast<typename Ops::Smem*>(sm.c32.t)[g];
-  int32_t(*rowbuf)[tiles::kB] = sizeof(E) == 2 ? sm.c16.rowbuf : sm.c32.rowbuf;
+  int32_t(*rowbuf)[kB] = sizeof(E) == 2 ? sm.c16.rowbuf : sm.c32.rowbuf;
+  // the group's part of tile t's bounds after its update (reset before it)
+  auto bounds = [&](int t, const Bounds& bd) {
+    const int32_t mx = __reduce_max_sync(0xFFFFFFFFu, bd.mx), mn = __reduce_min_sync(0xFFFFFFFFu, bd.mn);
+    if ((lt & 31) == 0) atomicMax(&sh.tmax[t], mx), atomicMin(&sh.tmin[t], mn);
+  };
+  // tiles with min(max A, max B) <= min X cannot change; the others of the
+  // phase's `total`, at(t) = tile row * nb + tile column, go to sh.list
+  auto select = [&](int32_t r, int32_t total, auto at) {
+    if (threadIdx.x == 0) sh.count = 0;
+    __syncthreads();
+    for (int32_t t = threadIdx.x; t < total; t += kBT) {
+      const int32_t x = at(t), i = x / nb, j = x % nb;
+      if (min(sh.tmax[i * nb + r], sh.tmax[r * nb + j]) > sh.tmin[x]) sh.list[atomicAdd(&sh.count, 1)] = uint16_t(x);
+    }
+    __syncthreads();
+  };
+  auto update = [&](int32_t r) {
+    for (int32_t t = g; t < sh.count; t += kGroups) {
+      const int32_t x = sh.list[t], i = x / nb, j = x % nb, vr = m - i * kB, vc = m - j * kB;
+      Ops::load_a(W + int64_t(i) * kB * mp + int64_t(r) * kB, mp, ts, lt);
+      Ops::load_b(W + int64_t(r) * kB * mp + int64_t(j) * kB, mp, ts, lt);
+      if (lt == 0) sh.tmax[x] = 0, sh.tmin[x] = INT32_MAX;  // (this group's alone until the phase ends)
+      Bounds bd;
+      Ops::template multiply<true>(W + int64_t(i) * kB * mp + int64_t(j) * kB, mp, ts, lt, bar, bd,
+                                   i == j || vr < kB || vc < kB, i == j, vr, vc);
+      bounds(x, bd);
+      bar.sync();  // the operands are free
+    }
+    __syncthreads();
+  };
   for (int32_t r = 0; r < nb; ++r) {
-    if (g == 0) tiles::diag_closure<E>(W, mp, r, rowbuf, lt, bar);
-    __syncthreads();
-    for (int32_t t = g; t < 2 * (nb - 1); t += kGroups) {  // row, then column panel tiles
-      if (t < nb - 1)
-        tiles::tile_update(W, mp, r, t + (t >= r), r, ts, lt, bar);
-      else
-        tiles::tile_update(W, mp, (t - (nb - 1)) + ((t - (nb - 1)) >= r), r, r, ts, lt, bar);
+    const bool close = sh.tmax[r * nb + r] > 0;  // a zero diagonal tile is closed
+    __syncthreads();                             // (read by all before its bounds are reset)
+    if (g == 0 && close) {
+      if (lt == 0) sh.tmax[r * nb + r] = 0, sh.tmin[r * nb + r] = INT32_MAX;
+      Bounds bd;
+      tiles::diag_closure_local<E>(W, mp, r, m - r * kB, m - r * kB, rowbuf, lt, bar, bd);
+      bounds(r * nb + r, bd);
     }
     __syncthreads();
-    for (int32_t t = g; t < (nb - 1) * (nb - 1); t += kGroups) {
-      int32_t i = t / (nb - 1), j = t % (nb - 1);
-      tiles::tile_update(W, mp, i + (i >= r), j + (j >= r), r, ts, lt, bar);
-    }
-    __syncthreads();
+    select(r, 2 * (nb - 1), [&](int32_t t) {  // row, then column panel tiles
+      const int32_t v = t < nb - 1 ? t : t - (nb - 1), x = v + (v >= r);
+      return t < nb - 1 ? r * nb + x : x * nb + r;
+    });
+    update(r);
+    select(r, (nb - 1) * (nb - 1), [&](int32_t t) {
+      const int32_t i = t / (nb - 1), j = t % (nb - 1);
+      return (i + (i >= r)) * nb + j + (j >= r);
+    });
+    update(r);
   }
 }
 
 template <typename E>
-__device__ void extract(const Job& jb, const E* __restrict__ W, int32_t mp, const BatchArgs& a, BatchSmem& sm) {
+__device__ void extract(const Job& jb, const E* __restrict__ W, int32_t mp, const BatchArgs& a, BatchSmem& sm,
+                        const Shared& sh) {
   const int32_t m = jb.m;
   int32_t* bb = sm.bb;
   for (int32_t i = threadIdx.x; i < m; i += kBT) bb[i] = 0;
@@ -350,24 +542,24 @@ __device__ void extract(const Job& jb, const E* __restrict__ W, int32_t mp, cons
     if (lane == 0 && beaten_i) atomicAdd(&bb[i], beaten_i);
   }
   __syncthreads();
-  for (int32_t i = threadIdx.x; i < m; i += kBT) {
-    const int32_t mine = bb[i];
-    if (a.winners) a.winners[jb.vec_off + i] = mine == 0;
-    if (a.beaten_by) a.beaten_by[jb.vec_off + i] = mine;
+  for (int32_t i = threadIdx.x; i < m; i += kBT) {  // relabeled index i, candidate sh.perm[i]
+    const int32_t mine = bb[i], id = sh.perm[i];
+    if (a.winners) a.winners[jb.vec_off + id] = mine == 0;
+    if (a.beaten_by) a.beaten_by[jb.vec_off + id] = mine;
     if (a.order) {
       int32_t pos = 0;
       for (int32_t j = 0; j < m; ++j) {
         const int32_t o = bb[j];
-        pos += (o < mine) || (o == mine && j < i);
+        pos += (o < mine) || (o == mine && sh.perm[j] < id);
       }
-      a.order[jb.vec_off + pos] = i;
+      a.order[jb.vec_off + pos] = id;
     }
   }
   if (a.p) {
     int32_t* pm = a.p + jb.mat_off;
     for (int64_t t = threadIdx.x; t < int64_t(m) * m; t += kBT) {
       const int32_t i = int32_t(t / m), j = int32_t(t % m);
-      pm[t] = (i == j) ? 0 : int32_t(W[int64_t(i) * mp + j]);
+      pm[t] = (i == j) ? 0 : int32_t(W[int64_t(sh.inv[i]) * mp + sh.inv[j]]);
     }
   }
   __syncthreads();
@@ -378,9 +570,11 @@ __global__ void __launch_bounds__(kBT, 1) batch_kernel(BatchArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   BatchSmem& sm = *reinterpret_cast<BatchSmem*>(smem_raw);
   __shared__ int32_t s_job;
+  __shared__ Shared sh;
   unsigned char* slot = a.scratch + size_t(blockIdx.x) * a.slot_bytes;
   E* W = reinterpret_cast<E*>(slot);
   int32_t* dslot = reinterpret_cast<int32_t*>(slot + a.w_bytes);
+  uint32_t* planes = reinterpret_cast<uint32_t*>(slot + a.plane_off);
   for (;;) {
     if (threadIdx.x == 0) s_job = int32_t(atomicAdd(a.head, 1u));
     __syncthreads();
@@ -416,12 +610,13 @@ __global__ void __launch_bounds__(kBT, 1) batch_kernel(BatchArgs a) {
       for (int64_t t = threadIdx.x; t < int64_t(m) * m; t += kBT) dm[t] = 0;
       __syncthreads();
     } else {
-      tally(jb, ranks, dm, sm, a.status);
+      tally(jb, ranks, dm, planes, sm, a.status);
     }
     const int32_t mp = int32_t(align_up(size_t(m), tiles::kB));
-    pack<E>(dm, m, mp, W);
-    closure<E>(W, mp, sm);
-    extract<E>(jb, W, mp, a, sm);
+    relabel(dm, m, sh);
+    pack<E>(jb, dm, mp, W, sh);
+    closure<E>(W, m, mp, sm, sh);
+    extract<E>(jb, W, mp, a, sm, sh);
   }
 }
 
@@ -439,7 +634,7 @@ struct schulze_batch {
   schulze::Job* jobs_dev = nullptr;
   uint32_t* head = nullptr;
   unsigned char* scratch = nullptr;
-  size_t slot_bytes = 0, w_bytes = 0;
+  size_t slot_bytes = 0, w_bytes = 0, plane_off = 0;
   int grid = 0;
   int32_t tally_policy = 0;  // 0: each m-bucket's ballots per step; 1: eight everywhere
   int32_t order_policy = 0;  // 0 longest first, 1 the caller's order
@@ -526,6 +721,7 @@ int launch_jobs(schulze_batch* b, int32_t njobs, const int32_t* ranks, int32_t* 
   a.scratch = b->scratch;
   a.slot_bytes = b->slot_bytes;
   a.w_bytes = b->w_bytes;
+  a.plane_off = b->plane_off;
   a.status = b->ctx->status;
   Launch L(b->ctx, stream, "batch_elections", double(njobs));
   if (b->s16)
@@ -588,7 +784,13 @@ int schulze_batch_create(schulze_ctx* ctx, int32_t E, const int32_t* n, const in
   b->grid = int(std::max<int64_t>(1, std::min<int64_t>(int64_t(per_sm) * ctx->sm_count, std::max(E, 1))));
   const size_t mp = align_up(size_t(std::max(b->m_max, 1)), tiles::kB);
   b->w_bytes = align_up(mp * mp * (b->s16 ? 2 : 4), 256);
-  b->slot_bytes = b->w_bytes + align_up(size_t(b->m_max) * size_t(b->m_max) * 4, 256);
+  b->plane_off = b->w_bytes + align_up(size_t(b->m_max) * size_t(b->m_max) * 4, 256);
+  size_t plane_words = 0;  // of the largest election's plane groups counted at a time
+  for (int32_t e = 0; e < E; ++e) {
+    const size_t groups = std::min<size_t>(kPlaneGroups, (size_t(n[e]) + kPlaneVoters - 1) / kPlaneVoters);
+    if (k[e] > 0) plane_words = std::max(plane_words, groups * position_bits(m[e], k[e]) * align_up(size_t(m[e]), kTT));
+  }
+  b->slot_bytes = b->plane_off + align_up(plane_words * 4, 256);
   if (cudaMalloc(&b->jobs_dev, sizeof(Job) * size_t(std::max(E, 1))) != cudaSuccess ||
       cudaMalloc(&b->head, 256) != cudaSuccess ||
       cudaMalloc(&b->scratch, b->slot_bytes * size_t(b->grid)) != cudaSuccess) {

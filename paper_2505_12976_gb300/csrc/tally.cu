@@ -47,21 +47,16 @@ constexpr int kPlaneVoters = 32;   // ballots per plane word
 constexpr int kPlaneCols = 2048;   // candidates whose positions a CTA turns at a time
 constexpr int kPlaneBits = 16;     // planes of weak orders (their largest position is not known ahead)
 
-// planes [b0, b0 + 8) of the 32 positions at(v), written at out + b * ldp for b < bits
+// the planes of the 32 positions at(v), plane b < bits at out + b * ldp
 template <class At>
-__device__ __forceinline__ void put_planes(At at, int b0, int bits, uint32_t* out, int32_t ldp) {
-  uint32_t w[8];
+__device__ __forceinline__ void put_planes(At at, int bits, uint32_t* out, int32_t ldp) {
+  uint32_t w[16];
 #pragma unroll
-  for (int b = 0; b < 8; ++b) w[b] = 0u;
+  for (int v = 0; v < 16; ++v) w[v] = at(v) | (at(v + 16) << 16);
+  transpose_planes(w);
 #pragma unroll
-  for (int v = 0; v < kPlaneVoters; ++v) {
-    uint32_t y = at(v) >> b0;
-#pragma unroll
-    for (int b = 0; b < 8; ++b) w[b] = __funnelshift_r(w[b], y, 1), y >>= 1;  // y's bit 0 into the top of w
-  }
-#pragma unroll
-  for (int b = 0; b < 8; ++b)
-    if (b0 + b < bits) out[int64_t(b0 + b) * ldp] = w[b];
+  for (int b = 0; b < 16; ++b)
+    if (b < bits) out[int64_t(b) * ldp] = w[b];
 }
 
 // d zeroed by all CTAs of a launch (where the counts are added into it)
@@ -121,8 +116,7 @@ __global__ void __launch_bounds__(512) slice_ballots_kernel(const int32_t* __res
   __syncthreads();
   uint32_t* out = planes + int64_t(blockIdx.x) * bits * ldp + c0;
   for (int32_t c = threadIdx.x; c < cols; c += blockDim.x)
-    for (int b0 = 0; b0 < bits; b0 += 8)
-      put_planes([&](int v) { return uint32_t(slice_pos[v * cols + c]); }, b0, bits, out + c, ldp);
+    put_planes([&](int v) { return uint32_t(slice_pos[v * cols + c]); }, bits, out + c, ldp);
 }
 
 // Weak orders in position form: the caller's int32 positions (smaller is
@@ -152,9 +146,7 @@ __global__ void __launch_bounds__(256) slice_positions_kernel(const int32_t* __r
   any = __reduce_or_sync(__activemask(), any);
   if (any & ~*reinterpret_cast<volatile uint32_t*>(used)) atomicOr(used, any);
   uint32_t* out = planes + int64_t(blockIdx.x) * kPlaneBits * ldp + c;
-#pragma unroll
-  for (int b0 = 0; b0 < kPlaneBits; b0 += 8)
-    put_planes([&](int v) { return uint32_t(x[v]); }, b0, kPlaneBits, out, ldp);
+  put_planes([&](int v) { return uint32_t(x[v]); }, kPlaneBits, out, ldp);
 }
 
 // One CTA counts a 64 x 64 tile of d over a chunk of plane groups: the planes

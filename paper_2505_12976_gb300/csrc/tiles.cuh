@@ -43,88 +43,57 @@ struct Bounds {
 // Row k and column k do not change during step k (min(x, y) <= x). The
 // tile's diagonal may pick up cycle widths; it never changes an off-diagonal
 // entry and is zeroed on output. The caller's barrier has to follow.
+// 16-bit lanes stay packed two to a word (two lane updates per min and max).
 template <typename E, class Bar>
 __device__ void diag_closure_local(E* __restrict__ W, int32_t ld, int32_t r, int32_t vr, int32_t vc,
                                    int32_t (*rowbuf)[kB], int tid, const Bar& bar, Bounds& bd) {
+  constexpr int kPer = 4 / int(sizeof(E));  // entries per word
+  constexpr int kWords = 32 / kPer;         // words of a thread's half row
   const int i = tid >> 1, half = tid & 1;
   E* base = W + (int64_t(r) * kB + i) * ld + int64_t(r) * kB + half * 32;
-  int32_t v[32];
-  if (sizeof(E) == 2) {
-    const uint4* src = reinterpret_cast<const uint4*>(base);
+  uint32_t v[kWords];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      uint4 x = __ldcg(src + q);
-      const uint32_t w4[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        v[8 * q + 2 * h] = int32_t(int16_t(w4[h] & 0xFFFFu));
-        v[8 * q + 2 * h + 1] = int32_t(int16_t(w4[h] >> 16));
-      }
-    }
-  } else {
-    const int4* src = reinterpret_cast<const int4*>(base);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      int4 x = __ldcg(src + q);
-      v[4 * q] = x.x, v[4 * q + 1] = x.y, v[4 * q + 2] = x.z, v[4 * q + 3] = x.w;
-    }
+  for (int q = 0; q < kWords / 4; ++q) {
+    const uint4 x = __ldcg(reinterpret_cast<const uint4*>(base) + q);
+    v[4 * q] = x.x, v[4 * q + 1] = x.y, v[4 * q + 2] = x.z, v[4 * q + 3] = x.w;
   }
 #pragma unroll
   for (int k = 0; k < kB; ++k) {
-    int32_t* rb = rowbuf[k & 1];
+    uint32_t* rb = reinterpret_cast<uint32_t*>(rowbuf[k & 1]) + half * kWords;
     if (i == k) {
 #pragma unroll
-      for (int c = 0; c < 32; c += 4)
-        *reinterpret_cast<int4*>(&rb[half * 32 + c]) = make_int4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+      for (int c = 0; c < kWords; c += 4)
+        *reinterpret_cast<uint4*>(&rb[c]) = make_uint4(v[c], v[c + 1], v[c + 2], v[c + 3]);
     }
     bar.sync();
-    const int32_t mine = v[k & 31];
-    const int32_t other = __shfl_xor_sync(0xFFFFFFFFu, mine, 1);
-    const int32_t a = ((k >> 5) == half) ? mine : other;  // p[i][k]
+    const int kk = k & 31;
+    uint32_t mine = v[kk / kPer];
+    if (sizeof(E) == 2) mine = __byte_perm(mine, 0, (kk & 1) ? 0x3232 : 0x1010);
+    const uint32_t other = __shfl_xor_sync(0xFFFFFFFFu, mine, 1);
+    const uint32_t a = ((k >> 5) == half) ? mine : other;  // p[i][k] (in both lanes)
 #pragma unroll
-    for (int c = 0; c < 32; c += 4) {
-      int4 b = *reinterpret_cast<const int4*>(&rb[half * 32 + c]);
-      v[c] = max(v[c], min(a, b.x));
-      v[c + 1] = max(v[c + 1], min(a, b.y));
-      v[c + 2] = max(v[c + 2], min(a, b.z));
-      v[c + 3] = max(v[c + 3], min(a, b.w));
+    for (int c = 0; c < kWords; c += 4) {
+      const uint4 b = *reinterpret_cast<const uint4*>(&rb[c]);
+      auto step = [&](uint32_t& x, uint32_t y) {
+        if (sizeof(E) == 2) x = __vmaxs2(x, __vmins2(a, y));
+        else x = uint32_t(max(int32_t(x), min(int32_t(a), int32_t(y))));
+      };
+      step(v[c], b.x), step(v[c + 1], b.y), step(v[c + 2], b.z), step(v[c + 3], b.w);
     }
   }
-  if (sizeof(E) == 2) {
-    uint4* dst = reinterpret_cast<uint4*>(base);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      uint32_t w4[4];
-#pragma unroll
-      for (int h = 0; h < 4; ++h)
-        w4[h] = (uint32_t(v[8 * q + 2 * h]) & 0xFFFFu) | (uint32_t(v[8 * q + 2 * h + 1]) << 16);
-      __stcg(dst + q, make_uint4(w4[0], w4[1], w4[2], w4[3]));
-    }
-  } else {
-    int4* dst = reinterpret_cast<int4*>(base);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      __stcg(dst + q, make_int4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
-    }
-  }
+  for (int q = 0; q < kWords / 4; ++q)
+    __stcg(reinterpret_cast<uint4*>(base) + q, make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
   // this thread's part of the tile's bounds
   bd = Bounds{0, INT32_MAX};
 #pragma unroll
   for (int c = 0; c < 32; ++c) {
     const int j = half * 32 + c;
+    const int32_t x = sizeof(E) == 2 ? int32_t(int16_t(v[c / kPer] >> (16 * (c & 1)))) : int32_t(v[c / kPer]);
     if (j == i) continue;
-    bd.mx = max(bd.mx, v[c]);
-    if (i < vr && j < vc) bd.mn = min(bd.mn, v[c]);
+    bd.mx = max(bd.mx, x);
+    if (i < vr && j < vc) bd.mn = min(bd.mn, x);
   }
-}
-
-// The closure above, then one barrier.
-template <typename E, class Bar>
-__device__ void diag_closure(E* __restrict__ W, int32_t ld, int32_t r, int32_t (*rowbuf)[kB], int tid,
-                             const Bar& bar) {
-  Bounds bd;
-  diag_closure_local<E>(W, ld, r, kB, kB, rowbuf, tid, bar, bd);
-  bar.sync();
 }
 
 // Shared-memory operand layouts of one tile update.

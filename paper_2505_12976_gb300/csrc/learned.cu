@@ -976,6 +976,7 @@ LearnedWs carve_learned(void* ws, int32_t m) {
   return w;
 }
 
+// The statistics of every candidate, and with feat the features made of them.
 int features_into(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t n, float* feat, const LearnedWs& w,
                   cudaStream_t stream) {
   const int g = std::max(1, std::min((m + 255) / 256, 1024));
@@ -997,6 +998,7 @@ int features_into(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t n, floa
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFSmem));
     kern<<<grid, 256, kFSmem, stream>>>(d, m, w.acc);
   }
+  if (!feat) return check_launch();
   {
     Launch L(ctx, stream, "learn_features_finalize", double(m) * kNF * 4.0);
     features_finalize_kernel<<<(m + 63) / 64, 64, 0, stream>>>(w.acc, m, n, feat);
@@ -1109,14 +1111,13 @@ int schulze_certify(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t n, co
       ncand > kMaxProposals)
     return SCHULZE_EINVAL;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return SCHULZE_ECUDA;
-  const size_t need = learned_ws_bytes(m) + align_up(size_t(m) * kNF * 4, 256) + 2 * align_up(size_t(m) * 4, 256);
+  const size_t need = learned_ws_bytes(m) + 2 * align_up(size_t(m) * 4, 256);
   if (int rc = ensure_workspace(ctx, need, stream)) return rc;
   const LearnedWs w = carve_learned(ctx->ws.base, m);
   Carver cv(static_cast<char*>(ctx->ws.base) + learned_ws_bytes(m));
-  float* feat = cv.take<float>(size_t(m) * kNF);
   int32_t* fwd = cv.take<int32_t>(m);
   int32_t* bwd = cv.take<int32_t>(m);
-  if (int rc = features_into(ctx, d, m, n, feat, w, stream)) return rc;  // wins / losses for the warm set
+  if (int rc = features_into(ctx, d, m, n, nullptr, w, stream)) return rc;  // wins / losses for the warm set
   return certify_launch(ctx, d, m, cand, ncand, winners, result, w, fwd, bwd, stream);
 }
 
@@ -1126,14 +1127,16 @@ int schulze_winners_fast(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t 
   if (!ctx || !d || !winners || m < 1 || m > kMaxM || n < 0 || top < 1 || top > kMaxProposals) return SCHULZE_EINVAL;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return SCHULZE_ECUDA;
   const size_t lw = learned_ws_bytes(m);
-  const size_t need = lw + align_up(size_t(m) * kNF * 4, 256) + 2 * align_up(size_t(m) * 4, 256) + 4096;
+  // (the propagation's scratch after the statistics, whose heaviest edges it takes)
+  const size_t pws = lw + align_up(size_t(m) * kNF * 4, 256) + 2 * align_up(size_t(m) * 4, 256) + 4096;
+  const size_t need = pws + (m > kCertifyMaxWarm ? propagation_workspace_bytes(m) : 0);
   if (int rc = ensure_workspace(ctx, need, stream)) return rc;
   const LearnedWs w = carve_learned(ctx->ws.base, m);
   Carver cv(static_cast<char*>(ctx->ws.base) + lw);
   float* feat = cv.take<float>(size_t(m) * kNF);
   int32_t* fwd = cv.take<int32_t>(m);
   int32_t* bwd = cv.take<int32_t>(m);
-  if (int rc = features_into(ctx, d, m, n, feat, w, stream)) return rc;
+  if (int rc = features_into(ctx, d, m, n, params ? feat : nullptr, w, stream)) return rc;
   {
     Launch L(ctx, stream, "proposal_scores", double(m) * 5248.0 * 2.0);
     if (params)
@@ -1161,9 +1164,10 @@ int schulze_winners_fast(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t 
     // paper's propagation (Alg. 1-4) decides exactly, with O(m^2) passes
     // per round instead of the closure's O(nw^3)
     fallback = 2;
-    if (int rc = ensure_workspace(ctx, propagation_workspace_bytes(m), stream)) return rc;
     int32_t ps[2] = {0, 0};
-    if (int rc = winners_propagation_launch(ctx, d, m, false, winners, ps, ctx->ws.base, stream)) return rc;
+    if (int rc = winners_propagation_launch(ctx, d, m, false, winners, ps, static_cast<char*>(ctx->ws.base) + pws, stream,
+                                            w.acc.maxw_in, w.acc.maxw_out))
+      return rc;
   } else if (!res[0]) {
     // no proposal certified (or too many ties): the full closure decides,
     // on workspace memory after the certification data

@@ -843,6 +843,7 @@ __global__ void SCHULZE_PERSIST_BOUNDS closure_persistent_kernel(E* W, int32_t l
 constexpr int kClusterCtas = 8;
 constexpr int kClusterThreads = 512;
 constexpr int kMaxSweeps = 40;  // > ceil(log2 256) + 1: never reached
+constexpr int32_t kSmallMax = 256;  // candidates of closure_small_kernel (kClusterMaxWarm of either lane type)
 
 // acc (16 bytes of a row) = max(acc, min(a(k), b0), min(a(k + 1), b1)) with
 // b0, b1 the same 16 bytes of rows k and k + 1 and a the row's entries k,
@@ -869,18 +870,76 @@ __device__ __forceinline__ bool differs(const uint4& a, const uint4& b) {
 }
 
 template <typename E>
+using RowPair = typename std::conditional<sizeof(E) == 2, uint32_t, int2>::type;  // a row's entries k, k + 1
+
+// The sweeps over the square S4 (rows of Qs 16-byte pieces, Q of them in
+// use), rows 0 .. nw - 1 (row nw zero when nw is odd), every copy loaded and
+// every flag clear. Returns the number of sweeps.
+template <typename E>
+__device__ int sweep_square(cooperative_groups::cluster_group& cl, uint4* S4, int32_t Qs, int32_t Q, int32_t nw,
+                            uint32_t (*flags)[kClusterCtas]) {
+  using AW = RowPair<E>;
+  const AW* A = reinterpret_cast<const AW*>(S4);
+  const int32_t ra = Qs * 16 / int32_t(sizeof(AW));  // row stride of A
+  const int32_t nwe = (nw + 1) & ~1;                 // pivots, in pairs
+  const int t = threadIdx.x;
+  const unsigned q = cl.block_rank();
+  const int32_t own = int32_t(q) < nw ? (nw - int32_t(q) + kClusterCtas - 1) / kClusterCtas : 0;
+  const int32_t items = (own + 1) / 2 * Q;  // (pair of owned rows, piece)
+  int sweeps = 0;
+  while (sweeps < kMaxSweeps) {
+    bool changed = false;
+    for (int32_t it = t; it < items; it += kClusterThreads) {
+      const int32_t rp = it / Q, c = it % Q;
+      const int32_t i0 = int32_t(q) + kClusterCtas * (2 * rp), i1 = i0 + kClusterCtas;
+      const bool has1 = i1 < nw;
+      const uint4 x0 = S4[i0 * Qs + c], x1 = has1 ? S4[i1 * Qs + c] : x0;
+      uint4 acc0 = x0, acc1 = x1;
+      const AW* a0p = A + i0 * ra;
+      const AW* a1p = A + (has1 ? i1 : i0) * ra;
+#pragma unroll 4
+      for (int32_t k = 0; k < nwe; k += 2) {
+        const uint4 b0 = S4[k * Qs + c], b1 = S4[(k + 1) * Qs + c];
+        sweep_step(acc0, a0p[k >> 1], b0, b1);
+        sweep_step(acc1, a1p[k >> 1], b0, b1);
+      }
+      if (differs(acc0, x0)) {
+        changed = true;
+        S4[i0 * Qs + c] = acc0;
+#pragma unroll
+        for (int o = 1; o < kClusterCtas; ++o)
+          *cl.map_shared_rank(S4 + i0 * Qs + c, (q + o) % kClusterCtas) = acc0;
+      }
+      if (has1 && differs(acc1, x1)) {
+        changed = true;
+        S4[i1 * Qs + c] = acc1;
+#pragma unroll
+        for (int o = 1; o < kClusterCtas; ++o)
+          *cl.map_shared_rank(S4 + i1 * Qs + c, (q + o) % kClusterCtas) = acc1;
+      }
+    }
+    ++sweeps;
+    const int any = __syncthreads_or(changed);
+    if (any && t < kClusterCtas) *cl.map_shared_rank(&flags[sweeps & 1][q], unsigned(t)) = 1u;
+    cl.sync();  // this sweep's copies and flags visible everywhere
+    const int more = __syncthreads_or(t < kClusterCtas && flags[sweeps & 1][t] != 0u);
+    if (t < kClusterCtas) flags[sweeps & 1][t] = 0u;  // rewritten two sweeps on, after the next barrier
+    if (!more) break;  // the same decision in every CTA
+  }
+  return sweeps;
+}
+
+template <typename E>
 __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterThreads, 1)
     closure_cluster_kernel(E* __restrict__ W, int32_t ld, const int32_t* __restrict__ warm,
                            unsigned long long* counters) {
   pdl_enter();
-  using AW = typename std::conditional<sizeof(E) == 2, uint32_t, int2>::type;  // a row's entries k, k + 1
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   const int32_t nw = *warm;
   if (nw == 0 || nw > kClusterMaxWarm<E>) return;  // the same branch in every CTA
   extern __shared__ __align__(16) unsigned char cluster_smem[];
   uint4* S4 = reinterpret_cast<uint4*>(cluster_smem);
-  const AW* A = reinterpret_cast<const AW*>(cluster_smem);  // row i, entries k, k + 1: A[i * n / 2 + k / 2]
   __shared__ uint32_t flags[2][kClusterCtas];     // CTA o changed something in the sweep (two buffers)
   const int32_t n = (nw + kB - 1) / kB * kB;      // square side: whole 64-wide tiles
   constexpr int kPer16 = 16 / sizeof(E);          // entries per 16-byte piece
@@ -909,47 +968,7 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
   if (t < 2 * kClusterCtas) flags[t / kClusterCtas][t % kClusterCtas] = 0u;
   cl.sync();  // every copy loaded, every flag clear, before any remote write
   const int32_t own = int32_t(q) < nw ? (nw - int32_t(q) + kClusterCtas - 1) / kClusterCtas : 0;
-  const int32_t items = (own + 1) / 2 * Q;  // (pair of owned rows, piece)
-  int sweeps = 0;
-  while (sweeps < kMaxSweeps) {
-    bool changed = false;
-    for (int32_t it = t; it < items; it += kClusterThreads) {
-      const int32_t rp = it / Q, c = it % Q;
-      const int32_t i0 = int32_t(q) + kClusterCtas * (2 * rp), i1 = i0 + kClusterCtas;
-      const bool has1 = i1 < nw;
-      const uint4 x0 = S4[i0 * Q + c], x1 = has1 ? S4[i1 * Q + c] : x0;
-      uint4 acc0 = x0, acc1 = x1;
-      const AW* a0p = A + i0 * (n / 2);
-      const AW* a1p = A + (has1 ? i1 : i0) * (n / 2);
-#pragma unroll 4
-      for (int32_t k = 0; k < nwe; k += 2) {
-        const uint4 b0 = S4[k * Q + c], b1 = S4[(k + 1) * Q + c];
-        sweep_step(acc0, a0p[k >> 1], b0, b1);
-        sweep_step(acc1, a1p[k >> 1], b0, b1);
-      }
-      if (differs(acc0, x0)) {
-        changed = true;
-        S4[i0 * Q + c] = acc0;
-#pragma unroll
-        for (int o = 1; o < kClusterCtas; ++o)
-          *cl.map_shared_rank(S4 + i0 * Q + c, (q + o) % kClusterCtas) = acc0;
-      }
-      if (has1 && differs(acc1, x1)) {
-        changed = true;
-        S4[i1 * Q + c] = acc1;
-#pragma unroll
-        for (int o = 1; o < kClusterCtas; ++o)
-          *cl.map_shared_rank(S4 + i1 * Q + c, (q + o) % kClusterCtas) = acc1;
-      }
-    }
-    ++sweeps;
-    const int any = __syncthreads_or(changed);
-    if (any && t < kClusterCtas) *cl.map_shared_rank(&flags[sweeps & 1][q], unsigned(t)) = 1u;
-    cl.sync();  // this sweep's copies and flags visible everywhere
-    const int more = __syncthreads_or(t < kClusterCtas && flags[sweeps & 1][t] != 0u);
-    if (t < kClusterCtas) flags[sweeps & 1][t] = 0u;  // rewritten two sweeps on, after the next barrier
-    if (!more) break;  // the same decision in every CTA
-  }
+  const int sweeps = sweep_square<E>(cl, S4, Q, Q, nw, flags);
   // each CTA writes its rows back with a zero diagonal. No CTA writes into
   // another any more.
   for (int32_t it = t; it < own * Q; it += kClusterThreads) {
@@ -969,6 +988,89 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
   }
   if (t == 0 && q == 0)  // entry updates, in 64 x 64 x 64 tile units
     atomicAdd(&counters[0], (unsigned long long)sweeps * uint64_t(nw) * uint64_t(nw) * uint64_t(n) / 262144ull);
+}
+
+// Elections of at most kClusterMaxWarm candidates: the whole way from d to p,
+// beaten_by, winners and order in one launch of the cluster (each of bb,
+// winners and order may be null). CTA q makes the weights of rows q, q + 8,
+// ... (eight entries per thread: 32 bytes of the row, and the transposed
+// column) and copies them into every CTA's square, rows one 16-byte piece
+// longer than they need so that a column's entries spread over the banks;
+// after the sweeps it writes its rows of p, counts who beats its candidates,
+// hands the counts to the other CTAs and ranks its candidates. Bound by
+// latency: it replaces a chain of eleven launches (m = 64: 10 us).
+template <typename E>
+__global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterThreads, 1)
+    closure_small_kernel(const int32_t* __restrict__ d, int32_t m, int64_t bound, int margin, int32_t* __restrict__ p,
+                         int32_t* __restrict__ bb, int32_t* __restrict__ winners, int32_t* __restrict__ order,
+                         int32_t* status, unsigned long long* counters) {
+  pdl_enter();
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  extern __shared__ __align__(16) unsigned char small_smem[];
+  constexpr int kPer16 = 16 / sizeof(E);
+  const int32_t Q = (m + kPer16 - 1) / kPer16, Qs = Q + 1;
+  uint4* S4 = reinterpret_cast<uint4*>(small_smem);
+  const E* S = reinterpret_cast<const E*>(small_smem);  // entry (i, j): S[i * ls + j]
+  const int32_t ls = Qs * kPer16;
+  __shared__ uint32_t flags[2][kClusterCtas];
+  __shared__ int32_t beaten[kSmallMax];
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  const unsigned q = cl.block_rank();
+  const int32_t own = int32_t(q) < m ? (m - int32_t(q) + kClusterCtas - 1) / kClusterCtas : 0;
+  if (t < 2 * kClusterCtas) flags[t / kClusterCtas][t % kClusterCtas] = 0u;
+  if (m & 1)  // the row past the last one, which a pair of pivots reads
+    for (int32_t c = t; c < Q; c += kClusterThreads) S4[m * Qs + c] = make_uint4(0u, 0u, 0u, 0u);
+  cl.sync();  // every CTA has started before any remote write
+  bool bad = false;
+  for (int32_t it = t; it < own * Q; it += kClusterThreads) {
+    const int32_t c = it / own, i = int32_t(q) + kClusterCtas * (it - c * own), j0 = c * kPer16;
+    int32_t x[kPer16], y[kPer16];
+#pragma unroll
+    for (int e = 0; e < kPer16; ++e) {
+      x[e] = j0 + e < m ? d[int64_t(i) * m + j0 + e] : 0;
+      y[e] = j0 + e < m ? d[int64_t(j0 + e) * m + i] : 0;
+    }
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int e = 0; e < kPer16; ++e) {
+      bad |= x[e] < 0 || int64_t(x[e]) > bound;
+      const int32_t out = x[e] > y[e] ? x[e] - (margin ? y[e] : 0) : 0;
+      if (sizeof(E) == 2) w[e >> 1] |= (uint32_t(out) & 0xFFFFu) << (16 * (e & 1));
+      else w[e & 3] = uint32_t(out);
+    }
+    const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
+#pragma unroll
+    for (int o = 0; o < kClusterCtas; ++o) *cl.map_shared_rank(S4 + i * Qs + c, unsigned(o)) = v;
+  }
+  if (bad) set_status(status, SCHULZE_EDATA);
+  cl.sync();  // every square complete
+  const int sweeps = sweep_square<E>(cl, S4, Qs, Q, m, flags);
+  for (int32_t r = wid; r < own; r += kClusterThreads / 32) {
+    const int32_t i = int32_t(q) + kClusterCtas * r;
+    int32_t c = 0;
+    for (int32_t j = lane; j < m; j += 32) {
+      const int32_t x = j == i ? 0 : int32_t(S[i * ls + j]);
+      p[int64_t(i) * m + j] = x;
+      c += j != i && int32_t(S[j * ls + i]) > x;
+    }
+    c = __reduce_add_sync(0xFFFFFFFFu, c);
+    if (lane < kClusterCtas) *cl.map_shared_rank(beaten + i, unsigned(lane)) = c;
+  }
+  cl.sync();  // every count everywhere
+  for (int32_t r = wid; r < own; r += kClusterThreads / 32) {
+    const int32_t i = int32_t(q) + kClusterCtas * r, mine = beaten[i];
+    int32_t pos = 0;  // candidates ahead of i by (beaten_by, id)
+    for (int32_t j = lane; j < m; j += 32) pos += beaten[j] < mine || (beaten[j] == mine && j < i);
+    pos = __reduce_add_sync(0xFFFFFFFFu, pos);
+    if (lane == 0) {
+      if (bb) bb[i] = mine;
+      if (winners) winners[i] = mine == 0;
+      if (order) order[pos] = i;
+    }
+  }
+  if (t == 0 && q == 0)  // entry updates, in 64 x 64 x 64 tile units
+    atomicAdd(&counters[0], (unsigned long long)sweeps * uint64_t(m) * uint64_t(m) * uint64_t(m) / 262144ull);
 }
 
 // Uniform cold columns: u[i] = max(ucol[i], max_x min(W[i][x], ucol[x]))
@@ -1260,7 +1362,16 @@ constexpr size_t kMaxRowBuf = 200 * 1024;  // larger rows (int32, m > 51200) are
 template <typename E>
 int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int64_t bound, int32_t* p,
                      const ClosureBufs& bf, int32_t* status, cudaStream_t stream, int32_t* bb_out = nullptr,
-                     bool side = false) {
+                     bool side = false, int32_t* winners = nullptr, int32_t* order = nullptr) {
+  if (m <= kClusterMaxWarm<E>) {
+    constexpr int kPer16 = 16 / int(sizeof(E));
+    const size_t Q = size_t(m + kPer16 - 1) / kPer16, smem = size_t(m + 1) * (Q + 1) * 16;
+    cudaFuncSetAttribute(closure_small_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    Launch L(ctx, stream, "closure_small", double(m) * double(m) * double(m));
+    launch_pdl(closure_small_kernel<E>, dim3(kClusterCtas), dim3(kClusterThreads), smem, stream, false, d, m, bound,
+               bf.margin ? 1 : 0, p, bb_out, winners, order, status, bf.counters);
+    return check_launch();
+  }
   const int32_t mp = int32_t(align_up(size_t(m), kB));
   const int32_t nb = mp / kB;
   E* W = static_cast<E*>(bf.W);
@@ -1399,7 +1510,7 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
 template <typename E>
 int run_closure(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t bound, int32_t* p, void* ws,
                 cudaStream_t stream, int32_t* bb_out, int32_t* hint, const int32_t* hint_valid,
-                bool margin, bool side) {
+                bool margin, bool side, int32_t* winners, int32_t* order) {
   const int32_t mp = int32_t(align_up(size_t(m), kB));
   const int32_t nb = mp / kB;
   Carver cv(ws);
@@ -1423,7 +1534,7 @@ int run_closure(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t bound, in
   bf.hint_valid = hint_valid;
   bf.margin = margin;
   const int sms = ctx->sm_count > 0 ? ctx->sm_count : 1;
-  return closure_pipeline<E>(ctx, sms, d, m, bound, p, bf, ctx->status, stream, bb_out, side);
+  return closure_pipeline<E>(ctx, sms, d, m, bound, p, bf, ctx->status, stream, bb_out, side, winners, order);
 }
 
 }  // namespace
@@ -1435,13 +1546,19 @@ size_t closure_workspace_bytes(int32_t m, int64_t bound, uint32_t flags) {
          6 * align_up(size_t(m) * 4, 256) + 4096;
 }
 
+bool closure_small(int32_t m, int64_t bound, uint32_t flags) {
+  return m <= (use_s16(bound, flags) ? kClusterMaxWarm<int16_t> : kClusterMaxWarm<int32_t>);
+}
+
 int closure_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t bound, int32_t* p, uint32_t flags,
                    void* ws, cudaStream_t stream, int32_t* beaten_by, int32_t* hint,
-                   const int32_t* hint_valid, bool side) {
+                   const int32_t* hint_valid, bool side, int32_t* winners, int32_t* order) {
   const bool margin = (flags & SCHULZE_F_MARGIN) != 0;
   if (use_s16(bound, flags))
-    return run_closure<int16_t>(ctx, d, m, bound, p, ws, stream, beaten_by, hint, hint_valid, margin, side);
-  return run_closure<int32_t>(ctx, d, m, bound, p, ws, stream, beaten_by, hint, hint_valid, margin, side);
+    return run_closure<int16_t>(ctx, d, m, bound, p, ws, stream, beaten_by, hint, hint_valid, margin, side, winners,
+                                order);
+  return run_closure<int32_t>(ctx, d, m, bound, p, ws, stream, beaten_by, hint, hint_valid, margin, side, winners,
+                                order);
 }
 
 // ------------------------------------------------- allocation-free variant

@@ -344,10 +344,13 @@ int schulze_run(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, in
   int32_t* hint_valid = reinterpret_cast<int32_t*>(tail + hv);
   int32_t* bb = beaten_by ? beaten_by : reinterpret_cast<int32_t*>(tail + hv + 256);
   void* xws = static_cast<char*>(ctx->ws.base) + xoff;
+  const bool small = closure_small(m, n, flags);  // one launch for the closure, the winners and the ranking
+  if (small) hint = hint_valid = nullptr;         // (which needs no warm flags)
   if (int rc = tally_launch(ctx, ranks, n, m, k, d, flags, ctx->ws.base, stream, hint, hint_valid)) return rc;
   const bool ext = winners || order || beaten_by;
-  int rc = closure_launch(ctx, d, m, n, p, flags, ctx->ws.base, stream, ext ? bb : nullptr, hint, hint_valid, true);
-  if (!rc && ext && (winners || order)) rc = extract_from_beaten_by(ctx, bb, m, winners, order, xws, stream);
+  int rc = closure_launch(ctx, d, m, n, p, flags, ctx->ws.base, stream, ext ? bb : nullptr, hint, hint_valid, true,
+                          winners, order);
+  if (!rc && !small && (winners || order)) rc = extract_from_beaten_by(ctx, bb, m, winners, order, xws, stream);
   const int rj = side_join(ctx, stream);  // also after an error: a capture must end with the fork joined
   return rc ? rc : rj;
 }
@@ -383,10 +386,14 @@ int schulze_run_host(schulze_ctx* ctx, const int32_t* ranks_host, int64_t n, int
   auto enqueue = [&](cudaStream_t s, int32_t* st) -> int {
     if (rbytes && cudaMemcpyAsync(ranks, ranks_host, rbytes, cudaMemcpyHostToDevice, s) != cudaSuccess)
       return SCHULZE_ECUDA;
-    if (int rc = tally_launch(ctx, ranks, n, m, k, d, flags, rest, s, hint, hint_valid)) return rc;
+    const bool small = closure_small(m, n, flags);
+    if (int rc = tally_launch(ctx, ranks, n, m, k, d, flags, rest, s, small ? nullptr : hint,
+                              small ? nullptr : hint_valid))
+      return rc;
     const bool ext = winners_host || order_host;
-    int rc = closure_launch(ctx, d, m, n, p, flags, rest, s, ext ? bb : nullptr, hint, hint_valid, true);
-    if (!rc && ext) rc = extract_from_beaten_by(ctx, bb, m, win, ord, xrest, s);
+    int rc = closure_launch(ctx, d, m, n, p, flags, rest, s, ext ? bb : nullptr, hint, hint_valid, true,
+                            winners_host ? win : nullptr, order_host ? ord : nullptr);
+    if (!rc && ext && !small) rc = extract_from_beaten_by(ctx, bb, m, win, ord, xrest, s);
     const int rj = side_join(ctx, s);
     if (rc || rj) return rc ? rc : rj;
     if (winners_host && cudaMemcpyAsync(winners_host, win, size_t(m) * 4, cudaMemcpyDeviceToHost, s) != cudaSuccess)

@@ -185,7 +185,12 @@ int tally_positions_launch(schulze_ctx* ctx, const int32_t* pos, int64_t n, int3
 // on stream reuses the closure's scratch).
 int closure_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t bound, int32_t* p, uint32_t flags,
                    void* ws, cudaStream_t stream, int32_t* beaten_by = nullptr, int32_t* hint = nullptr,
-                   const int32_t* hint_valid = nullptr, bool side = false);
+                   const int32_t* hint_valid = nullptr, bool side = false, int32_t* winners = nullptr,
+                   int32_t* order = nullptr);
+// Whether closure_launch takes such an election in one launch, which then
+// also fills winners and order when given (it ignores them otherwise, and
+// needs neither hint nor side stream).
+bool closure_small(int32_t m, int64_t bound, uint32_t flags);
 // stream waits for the side stream's work if closure_launch forked any
 int side_join(schulze_ctx* ctx, cudaStream_t stream);
 int extract_launch(schulze_ctx* ctx, const int32_t* p, int32_t m, int32_t* winners, int32_t* order,

@@ -775,7 +775,7 @@ int schulze_batch_create(schulze_ctx* ctx, int32_t E, const int32_t* n, const in
   int per_sm = 0;
   const void* fn = b->s16 ? reinterpret_cast<const void*>(batch_kernel<int16_t>)
                           : reinterpret_cast<const void*>(batch_kernel<int32_t>);
-  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(b->smem));
+  raise_smem(ctx, fn);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBT, b->smem) != cudaSuccess || per_sm < 1) {
     cudaGetLastError();
     delete b;

@@ -1366,7 +1366,7 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
   if (m <= kClusterMaxWarm<E>) {
     constexpr int kPer16 = 16 / int(sizeof(E));
     const size_t Q = size_t(m + kPer16 - 1) / kPer16, smem = size_t(m + 1) * (Q + 1) * 16;
-    cudaFuncSetAttribute(closure_small_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    raise_smem(ctx, reinterpret_cast<const void*>(closure_small_kernel<E>));
     Launch L(ctx, stream, "closure_small", double(m) * double(m) * double(m));
     launch_pdl(closure_small_kernel<E>, dim3(kClusterCtas), dim3(kClusterThreads), smem, stream, false, d, m, bound,
                bf.margin ? 1 : 0, p, bb_out, winners, order, status, bf.counters);
@@ -1395,11 +1395,7 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
   }
   const double mm = double(m) * double(m);
   auto grid_for = [&](const void* fn, int threads, size_t smem, int64_t cap) {
-    int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess || per_sm < 1) {
-      cudaGetLastError();
-      per_sm = 1;
-    }
+    const int per_sm = blocks_per_sm(ctx, fn, threads, smem);
     return int(std::max<int64_t>(1, std::min<int64_t>(int64_t(per_sm) * sms, cap)));
   };
   {
@@ -1413,7 +1409,7 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
   {
     Launch L(ctx, stream, "closure_relabel", double(m) * 12.0);
     const size_t smem = m <= kScanSmem ? size_t(m) * 4 : 0;
-    cudaFuncSetAttribute(relabel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    raise_smem(ctx, reinterpret_cast<const void*>(relabel_kernel));
     launch_pdl(relabel_kernel, dim3(1), dim3(1024), smem, stream, false,
                static_cast<const int32_t*>(bf.rowflag), m, bf.perm, bf.inv, bf.warm, bf.hint, bf.hint_valid,
                kClusterMaxWarm<E>);
@@ -1424,7 +1420,7 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
   {
     const size_t smem = rowbuf + 2 * size_t(nb) * 4;
     const int32_t chunk = m >= 8192 ? 16 : m >= 2048 ? 4 : 1;
-    cudaFuncSetAttribute(pack_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    raise_smem(ctx, reinterpret_cast<const void*>(pack_kernel<E>));
     const int g = grid_for(reinterpret_cast<const void*>(pack_kernel<E>), 512, smem, mp);
     Launch L(ctx, stream, "closure_pack", 0.0);
     launch_pdl(pack_kernel<E>, dim3(g), dim3(512), smem, stream, false, d, m, mp,
@@ -1434,7 +1430,7 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
   if (int rc = check_launch()) return rc;
   {
     const size_t smem = size_t(kClusterMaxWarm<E>) * kClusterMaxWarm<E> * sizeof(E);
-    cudaFuncSetAttribute(closure_cluster_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    raise_smem(ctx, reinterpret_cast<const void*>(closure_cluster_kernel<E>));
     Launch L(ctx, stream, "closure_cluster", 0.0);
     launch_pdl(closure_cluster_kernel<E>, dim3(kClusterCtas), dim3(kClusterThreads), smem, stream, false, W, mp,
                static_cast<const int32_t*>(bf.warm), bf.counters);
@@ -1456,7 +1452,7 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
   {
     const size_t cw = size_t(kClusterMaxWarm<E>);
     const size_t smem = (cw * (cw * sizeof(E) / 4 + 1) + cw * kStripWords) * 4;
-    cudaFuncSetAttribute(cold_strip_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    raise_smem(ctx, reinterpret_cast<const void*>(cold_strip_kernel<E>));
     Launch L(ctx, stream, "closure_cold_strips", 0.0);
     launch_pdl(cold_strip_kernel<E>, dim3(sms), dim3(512), smem, stream, false, W, mp, m,
                static_cast<const int32_t*>(bf.warm), bf.counters, bf.hint_valid);
@@ -1480,7 +1476,7 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
     // stream, with at most four CTAs per SM so that those kernels find room
     const bool fork = side && bb_out && ctx && ctx->side_stream;
     cudaStream_t wst = stream;
-    cudaFuncSetAttribute(widen_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(rowbuf));
+    raise_smem(ctx, reinterpret_cast<const void*>(widen_kernel<E>));
     int g = grid_for(reinterpret_cast<const void*>(widen_kernel<E>), 512, rowbuf, m);
     if (fork) {
       if (cudaEventRecord(ctx->side_fork, stream) != cudaSuccess ||

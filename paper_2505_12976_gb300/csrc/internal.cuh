@@ -67,6 +67,13 @@ struct ProfRecord {
   cudaEvent_t start, stop;
   double work;
 };
+// Resident CTAs per SM of a kernel at a block size and dynamic shared memory.
+struct Residency {
+  const void* fn;
+  int threads;
+  size_t smem;
+  int per_sm;
+};
 struct ProfClass {
   std::string name;
   int64_t launches = 0;
@@ -86,6 +93,11 @@ struct schulze_ctx {
   // bound on each device-side wait of the persistent closure, in SM clock
   // cycles (schulze_set_wait_limit)
   long long wait_limit_cycles = 4000000000LL;
+  // kernels allowed the device's largest dynamic shared memory, and
+  // occupancies asked for so far: each costs a runtime call of about a
+  // microsecond, a dozen of them per election otherwise
+  std::vector<const void*> raised;
+  std::vector<schulze::Residency> residency;
   std::vector<schulze::ProfRecord> prof_pending;
   std::vector<schulze::ProfClass> prof_classes;
   std::vector<cudaEvent_t> prof_free_events;
@@ -211,6 +223,13 @@ int iterated_level(schulze_ctx* ctx, const int32_t* bb, int32_t m, int32_t t, in
 // Winners (beaten_by == 0) and the ranking from a filled beaten_by.
 int extract_from_beaten_by(schulze_ctx* ctx, const int32_t* beaten_by, int32_t m, int32_t* winners, int32_t* order,
                            void* ws, cudaStream_t stream);
+
+// Lets kernel fn use as much dynamic shared memory as the device has for a
+// CTA (one value for every caller, so that no context lowers it for another).
+// Once per context and kernel; ctx may be null (then at every call).
+void raise_smem(schulze_ctx* ctx, const void* fn);
+// Resident CTAs per SM of fn, at least 1; remembered in the context.
+int blocks_per_sm(schulze_ctx* ctx, const void* fn, int threads, size_t smem);
 
 // Brackets one kernel launch: counts it and, when profiling is on, records
 // CUDA events around it on `stream`, filed under `name` with `work` units.

@@ -995,7 +995,7 @@ int features_into(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t n, floa
                     : (mode == kFPacked   ? features_pass_kernel<false, kFPacked>
                        : mode == kFNarrow ? features_pass_kernel<false, kFNarrow>
                                           : features_pass_kernel<false, kFWide>);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFSmem));
+    raise_smem(ctx, reinterpret_cast<const void*>(kern));
     kern<<<grid, 256, kFSmem, stream>>>(d, m, w.acc);
   }
   if (!feat) return check_launch();
@@ -1092,8 +1092,7 @@ int schulze_mlp_train_step(schulze_ctx* ctx, float* params, float* adam_m, float
   }
   {
     Launch L(ctx, stream, "mlp_train_backward", double(N) * 5248.0 * 4.0);
-    cudaFuncSetAttribute(mlp_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         int(sizeof(BackwardSmem)));
+    raise_smem(ctx, reinterpret_cast<const void*>(mlp_backward_kernel));
     mlp_backward_kernel<<<nchunks, 256, sizeof(BackwardSmem), stream>>>(params, feat, h1, h2, ds, N, partial);
     mlp_reduce_kernel<<<(kNP + 255) / 256, 256, 0, stream>>>(partial, nchunks, seg_loss, nseg, g, loss);
   }

@@ -57,6 +57,39 @@ Launch::~Launch() {
   if (rec_ >= 0) cudaEventRecord(ctx_->prof_pending[rec_].stop, stream_);
 }
 
+void raise_smem(schulze_ctx* ctx, const void* fn) {
+  if (ctx)
+    for (const void* f : ctx->raised)
+      if (f == fn) return;
+  int device = 0, optin = 0;
+  cudaFuncAttributes fa;
+  if (cudaGetDevice(&device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
+      cudaFuncGetAttributes(&fa, fn) != cudaSuccess ||
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - int(fa.sharedSizeBytes)) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    return;  // a launch that needs more than the default reports it
+  }
+  if (ctx) ctx->raised.push_back(fn);
+}
+
+int blocks_per_sm(schulze_ctx* ctx, const void* fn, int threads, size_t smem) {
+  if (ctx)
+    for (const Residency& r : ctx->residency)
+      if (r.fn == fn && r.threads == threads && r.smem == smem) return r.per_sm;
+  int per_sm = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess || per_sm < 1) {
+    cudaGetLastError();
+    per_sm = 1;
+  }
+  if (ctx) {
+    if (ctx->residency.size() >= 64) ctx->residency.clear();  // sizes keep changing: start over
+    ctx->residency.push_back(Residency{fn, threads, smem, per_sm});
+  }
+  return per_sm;
+}
+
 static void drain(schulze_ctx* ctx) {
   for (ProfRecord& r : ctx->prof_pending) {
     float ms = 0.f;

@@ -1343,8 +1343,7 @@ int tally_launch(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, i
     return dense_tally(ctx, n, m, k >= m - 1, bits, nullptr, d, ws, stream,
                        [&](int64_t v0, int64_t nv, int32_t ldp, int nbits, uint32_t* planes, int32_t* dzero) -> int {
                          const size_t smem = size_t(kPlaneVoters) * size_t(std::min(ldp, kPlaneCols)) * 2;
-                         cudaFuncSetAttribute(slice_ballots_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              int(smem));
+                         raise_smem(ctx, reinterpret_cast<const void*>(slice_ballots_kernel));
                          const dim3 g((nv + kPlaneVoters - 1) / kPlaneVoters, (ldp + kPlaneCols - 1) / kPlaneCols);
                          Launch L(ctx, stream, "tally_positions", double(nv) * (double(k) * 4.0 + double(ldp) * 2.0));
                          slice_ballots_kernel<<<g, 512, smem, stream>>>(ranks, v0, nv, m, k, ldp, nbits, planes,
@@ -1383,10 +1382,8 @@ int tally_launch(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, i
     const int threads = 512;
     const size_t smem = (local_hist ? size_t(m) * 4 : 0) + size_t(threads / 32) * size_t((m + 31) / 32) * 4;
     auto kern = local_hist ? sparse_count_kernel<true> : sparse_count_kernel<false>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1)
-      per_sm = 1;
+    raise_smem(ctx, reinterpret_cast<const void*>(kern));
+    const int per_sm = blocks_per_sm(ctx, reinterpret_cast<const void*>(kern), threads, smem);
     // about one ballot per warp: the pass is bound by load latency
     const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((n + 15) / 16, int64_t(sms) * per_sm)));
     Launch L(ctx, stream, "tally_count", double(total) * 4.0);
@@ -1407,7 +1404,7 @@ int tally_launch(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, i
   if (cp.cmax > 0) {
     Launch L(ctx, stream, "tally_compact_pairs", double(m) * double(m) * 4.0 + double(total) * 4.0);
     auto kern = cp.packed ? compact_pairs_kernel<true> : compact_pairs_kernel<false>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(cp.smem));
+    raise_smem(ctx, reinterpret_cast<const void*>(kern));
     launch_pdl(kern, dim3(cp.G), dim3(kCompactThreads), cp.smem, stream, false, ranks, n, m, k,
                static_cast<const int32_t*>(cnt), static_cast<const int32_t*>(slot), static_cast<const int32_t*>(meta),
                partial, int32_t(cp.stage), d, rows_vec16(d, m));
@@ -1424,7 +1421,7 @@ int tally_launch(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, i
     if (local_hist) {
       const size_t smem = size_t(m) * 8;
       const int blocks = int(std::min<uint64_t>((uint64_t(total) + 4095) / 4096, uint64_t(sms)));
-      cudaFuncSetAttribute(sparse_scatter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+      raise_smem(ctx, reinterpret_cast<const void*>(sparse_scatter_kernel<true>));
       launch_pdl(sparse_scatter_kernel<true>, dim3(blocks), dim3(kScatterThreads), smem, stream, false, ranks, total, m, cursor,
                  entries, static_cast<const int32_t*>(meta), static_cast<const int32_t*>(gmeta), hacc, hdone);
     } else {
@@ -1437,15 +1434,14 @@ int tally_launch(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, i
   {
     // persistent rows kernel: every CTA resident, rows from the plan's queue
     const size_t smem = align_up(size_t((m + 1) / 2) * 4, 16);
-    cudaFuncSetAttribute(grouped_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    cudaFuncSetAttribute(grouped_rows_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                         int(cudaSharedmemCarveoutMaxShared));
-    int per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, grouped_rows_kernel, kRowsThreads, smem) !=
-            cudaSuccess || per_sm < 1) {
-      cudaGetLastError();
-      per_sm = 1;
-    }
+    const void* fn = reinterpret_cast<const void*>(grouped_rows_kernel);
+    bool known = false;
+    for (const void* f : ctx->raised) known = known || f == fn;
+    if (!known)
+      cudaFuncSetAttribute(grouped_rows_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                           int(cudaSharedmemCarveoutMaxShared));
+    raise_smem(ctx, fn);
+    const int per_sm = blocks_per_sm(ctx, fn, kRowsThreads, smem);
     const int grid = int(std::min<int64_t>(int64_t(per_sm) * sms, m));
     Launch L(ctx, stream, "tally_rows", double(m) * double(m) * 4.0 + double(total) * 4.0);
     launch_pdl(grouped_rows_kernel, dim3(grid), dim3(kRowsThreads), smem, stream, false, ranks, m, k,

@@ -482,23 +482,29 @@ __global__ void __launch_bounds__(256) mlp_forward_kernel(const float* __restric
   float out = p[kOffB3];
   // four outputs at a time: their sums are independent chains that hide
   // each other's latency (each sum still runs in the parameters' order)
-#pragma unroll 4
-  for (int o = 0; o < kH; ++o) {
-    float s = p[kOffB2 + o];
-    const float4* w = reinterpret_cast<const float4*>(p + kOffW2 + o * kH);
+#pragma unroll 1
+  for (int o = 0; o < kH; o += 4) {
+    float h[4];
 #pragma unroll
-    for (int q4 = 0; q4 < kH / 4; ++q4) {
-      const float4 v = w[q4];
-      s = fmaf(v.x, h1[4 * q4], s), s = fmaf(v.y, h1[4 * q4 + 1], s);
-      s = fmaf(v.z, h1[4 * q4 + 2], s), s = fmaf(v.w, h1[4 * q4 + 3], s);
+    for (int e = 0; e < 4; ++e) {
+      float s = p[kOffB2 + o + e];
+      const float4* w = reinterpret_cast<const float4*>(p + kOffW2 + (o + e) * kH);
+#pragma unroll
+      for (int q4 = 0; q4 < kH / 4; ++q4) {
+        const float4 v = w[q4];
+        s = fmaf(v.x, h1[4 * q4], s), s = fmaf(v.y, h1[4 * q4 + 1], s);
+        s = fmaf(v.z, h1[4 * q4 + 2], s), s = fmaf(v.w, h1[4 * q4 + 3], s);
+      }
+      h[e] = fmaxf(s, 0.f);
+      out = fmaf(p[kOffW3 + o + e], h[e], out);
     }
-    const float h = fmaxf(s, 0.f);
-    if (h2out) h2out[int64_t(c) * kH + o] = h;
-    out = fmaf(p[kOffW3 + o], h, out);
+    // (16-byte stores: a thread's outputs are a row of their own)
+    if (h2out) *reinterpret_cast<float4*>(h2out + int64_t(c) * kH + o) = make_float4(h[0], h[1], h[2], h[3]);
   }
   if (h1out) {
 #pragma unroll
-    for (int q = 0; q < kH; ++q) h1out[int64_t(c) * kH + q] = h1[q];
+    for (int q = 0; q < kH; q += 4)
+      *reinterpret_cast<float4*>(h1out + int64_t(c) * kH + q) = make_float4(h1[q], h1[q + 1], h1[q + 2], h1[q + 3]);
   }
   score[c] = out;
 }
@@ -563,10 +569,17 @@ __global__ void __launch_bounds__(256) mlp_loss_kernel(const float* __restrict__
 constexpr int kChunk = 64;  // candidates per backward CTA
 
 // Backward over a chunk of kChunk candidates: dh2, dh1 per candidate, then
-// this chunk's sum of every parameter gradient into partial[chunk][kNP].
+// this chunk's sum of every parameter gradient into partial[chunk][kNP]. The
+// three products run on 4 x 4 (W1: 1 x 4) outputs per thread from 16-byte
+// reads of shared memory, 8 of them for 64 fused multiply-adds; one output
+// per thread read two words for each, and the pass was bound by those (with
+// the reduction 200 us for 73,000 candidates, now 72). Every sum still runs
+// over its terms in order.
 struct BackwardSmem {
-  float W2[kH * kH], W3[kH];
-  float sx[kChunk][kNF], sh1[kChunk][kH + 1], sh2[kChunk][kH + 1], sd2[kChunk][kH + 1], sd1[kChunk][kH + 1];
+  float W2[kH][kH], W3[kH];
+  float sx[kChunk][kNF];
+  // rows 16-byte aligned, four words longer than they need (fewer bank conflicts)
+  float sh1[kChunk][kH + 4], sh2[kChunk][kH + 4], sd2[kChunk][kH + 4], sd1[kChunk][kH + 4];
   float sds[kChunk];
 };
 
@@ -577,81 +590,143 @@ __global__ void __launch_bounds__(256) mlp_backward_kernel(const float* __restri
                                                            float* __restrict__ partial) {
   extern __shared__ __align__(16) unsigned char bw_raw[];
   BackwardSmem& S = *reinterpret_cast<BackwardSmem*>(bw_raw);
-  float* W2 = S.W2;
-  float* W3 = S.W3;
-  auto& sx = S.sx;
-  auto& sh1 = S.sh1;
-  auto& sh2 = S.sh2;
-  auto& sd2 = S.sd2;
-  auto& sd1 = S.sd1;
-  float* sds = S.sds;
   const int32_t c0 = blockIdx.x * kChunk;
   const int nc = min(kChunk, N - c0);
-  for (int t = threadIdx.x; t < kH * kH; t += blockDim.x) W2[t] = theta[kOffW2 + t];
-  for (int t = threadIdx.x; t < kH; t += blockDim.x) W3[t] = theta[kOffW3 + t];
-  for (int t = threadIdx.x; t < kChunk * kH; t += blockDim.x) {
-    const int r = t / kH, q = t % kH;
-    sh1[r][q] = r < nc ? h1g[int64_t(c0 + r) * kH + q] : 0.f;
-    sh2[r][q] = r < nc ? h2g[int64_t(c0 + r) * kH + q] : 0.f;
+  const int tid = threadIdx.x;
+  for (int t = tid; t < kH * kH; t += blockDim.x) S.W2[t / kH][t % kH] = theta[kOffW2 + t];
+  for (int t = tid; t < kH; t += blockDim.x) S.W3[t] = theta[kOffW3 + t];
+  for (int t = tid; t < kChunk; t += blockDim.x) S.sds[t] = t < nc ? ds[c0 + t] : 0.f;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int t = tid; t < kChunk * kH / 4; t += blockDim.x) {  // (h1, h2 are the pass's own 256-byte aligned rows)
+    const int r = t / (kH / 4), q = 4 * (t % (kH / 4));
+    *reinterpret_cast<float4*>(&S.sh1[r][q]) =
+        r < nc ? *reinterpret_cast<const float4*>(h1g + int64_t(c0 + r) * kH + q) : zero;
+    *reinterpret_cast<float4*>(&S.sh2[r][q]) =
+        r < nc ? *reinterpret_cast<const float4*>(h2g + int64_t(c0 + r) * kH + q) : zero;
   }
-  for (int t = threadIdx.x; t < kChunk * kNF; t += blockDim.x) {
+  for (int t = tid; t < kChunk * kNF; t += blockDim.x) {
     const int r = t / kNF, q = t % kNF;
-    sx[r][q] = r < nc ? feat[int64_t(c0 + r) * kNF + q] : 0.f;
+    S.sx[r][q] = r < nc ? feat[int64_t(c0 + r) * kNF + q] : 0.f;
   }
-  for (int t = threadIdx.x; t < kChunk; t += blockDim.x) sds[t] = t < nc ? ds[c0 + t] : 0.f;
   __syncthreads();
   // dh2[r][o] = ds_r * W3[o] * [h2 > 0]
-  for (int t = threadIdx.x; t < kChunk * kH; t += blockDim.x) {
+  for (int t = tid; t < kChunk * kH; t += blockDim.x) {
     const int r = t / kH, o = t % kH;
-    sd2[r][o] = sh2[r][o] > 0.f ? sds[r] * W3[o] : 0.f;
+    S.sd2[r][o] = S.sh2[r][o] > 0.f ? S.sds[r] * S.W3[o] : 0.f;
   }
   __syncthreads();
-  // dh1[r][q] = sum_o W2[o][q] dh2[r][o] * [h1 > 0]
-  for (int t = threadIdx.x; t < kChunk * kH; t += blockDim.x) {
-    const int r = t / kH, q = t % kH;
-    float s = 0.f;
-    for (int o = 0; o < kH; ++o) s = fmaf(W2[o * kH + q], sd2[r][o], s);
-    sd1[r][q] = sh1[r][q] > 0.f ? s : 0.f;
-  }
-  __syncthreads();
+  const int a0 = 4 * (tid / 16), b0 = 4 * (tid % 16);  // this thread's 4 x 4 block
   float* out = partial + int64_t(blockIdx.x) * kNP;
-  for (int t = threadIdx.x; t < kNP; t += blockDim.x) {
-    float g = 0.f;
-    if (t < kOffB1) {  // W1[o][q]: sum_r dh1[r][o] x[r][q]
-      const int o = t / kNF, q = t % kNF;
-      for (int r = 0; r < kChunk; ++r) g = fmaf(sd1[r][o], sx[r][q], g);
-    } else if (t < kOffW2) {
-      const int o = t - kOffB1;
-      for (int r = 0; r < kChunk; ++r) g += sd1[r][o];
-    } else if (t < kOffB2) {  // W2[o][q]: sum_r dh2[r][o] h1[r][q]
-      const int o = (t - kOffW2) / kH, q = (t - kOffW2) % kH;
-      for (int r = 0; r < kChunk; ++r) g = fmaf(sd2[r][o], sh1[r][q], g);
-    } else if (t < kOffW3) {
-      const int o = t - kOffB2;
-      for (int r = 0; r < kChunk; ++r) g += sd2[r][o];
-    } else if (t < kOffB3) {  // W3[o]: sum_r ds_r h2[r][o]
-      const int o = t - kOffW3;
-      for (int r = 0; r < kChunk; ++r) g = fmaf(sds[r], sh2[r][o], g);
-    } else {
-      for (int r = 0; r < kChunk; ++r) g += sds[r];
+  auto at = [](const float4& v, int e) { return e == 0 ? v.x : e == 1 ? v.y : e == 2 ? v.z : v.w; };
+  {
+    // dh1[r][q] = sum_o W2[o][q] dh2[r][o] * [h1 > 0], rows a0.., columns b0..
+    float s[4][4] = {};
+#pragma unroll 2
+    for (int o = 0; o < kH; o += 4) {
+      float4 x[4], w[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        x[e] = *reinterpret_cast<const float4*>(&S.sd2[a0 + e][o]);
+        w[e] = *reinterpret_cast<const float4*>(&S.W2[o + e][b0]);
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) s[i][j] = fmaf(at(w[e], j), at(x[i], e), s[i][j]);
     }
-    out[t] = g;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) S.sd1[a0 + i][b0 + j] = S.sh1[a0 + i][b0 + j] > 0.f ? s[i][j] : 0.f;
+  }
+  {
+    // W2[o][q]: sum_r dh2[r][o] h1[r][q], o from a0, q from b0
+    float s[4][4] = {};
+#pragma unroll 4
+    for (int r = 0; r < kChunk; ++r) {
+      const float4 x = *reinterpret_cast<const float4*>(&S.sd2[r][a0]);
+      const float4 h = *reinterpret_cast<const float4*>(&S.sh1[r][b0]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s[i][j] = fmaf(at(x, i), at(h, j), s[i][j]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) out[kOffW2 + (a0 + i) * kH + b0 + j] = s[i][j];
+  }
+  __syncthreads();
+  {
+    // W1[o][q]: sum_r dh1[r][o] x[r][q], o = tid / 4, four q
+    const int o = tid / 4, q0 = 4 * (tid % 4);
+    float s[4] = {};
+#pragma unroll 4
+    for (int r = 0; r < kChunk; ++r) {
+      const float x = S.sd1[r][o];
+      const float4 f = *reinterpret_cast<const float4*>(&S.sx[r][q0]);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s[j] = fmaf(x, at(f, j), s[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) out[kOffW1 + o * kNF + q0 + j] = s[j];
+  }
+  // the biases and W3, one output per thread
+  if (tid < kH) {
+    float g = 0.f;
+    for (int r = 0; r < kChunk; ++r) g += S.sd1[r][tid];
+    out[kOffB1 + tid] = g;
+  } else if (tid < 2 * kH) {
+    float g = 0.f;
+    for (int r = 0; r < kChunk; ++r) g += S.sd2[r][tid - kH];
+    out[kOffB2 + tid - kH] = g;
+  } else if (tid < 3 * kH) {
+    float g = 0.f;
+    for (int r = 0; r < kChunk; ++r) g = fmaf(S.sds[r], S.sh2[r][tid - 2 * kH], g);
+    out[kOffW3 + tid - 2 * kH] = g;
+  } else if (tid == 3 * kH) {
+    float g = 0.f;
+    for (int r = 0; r < kChunk; ++r) g += S.sds[r];
+    out[kOffB3] = g;
   }
 }
 
-// grad[t] = sum over chunks of partial[chunk][t], in chunk order; loss =
-// sum of the segment losses / nseg. Deterministic.
-__global__ void mlp_reduce_kernel(const float* __restrict__ partial, int32_t nchunks, const float* __restrict__ seg_loss,
-                                  int32_t nseg, float* __restrict__ grad, float* __restrict__ loss) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+// grad[t] = sum over chunks of partial[chunk][t]: kRedSegs threads per
+// parameter sum a run of chunks each, in chunk order, with eight loads in
+// flight, and their sums are added in run order; loss = sum of the segment
+// losses / nseg. Deterministic. (One thread per parameter left 5313 threads
+// with a chain of loads over all chunks each.)
+constexpr int kRedSegs = 16;
+__global__ void __launch_bounds__(32 * kRedSegs) mlp_reduce_kernel(const float* __restrict__ partial, int32_t nchunks,
+                                                                   const float* __restrict__ seg_loss, int32_t nseg,
+                                                                   float* __restrict__ grad, float* __restrict__ loss) {
+  __shared__ float part[kRedSegs][32];
+  const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+  const int t = blockIdx.x * 32 + lane;
+  const int32_t per = (nchunks + kRedSegs - 1) / kRedSegs;
+  const int32_t b = min(nchunks, seg * per), e = min(nchunks, b + per);
+  float g = 0.f;
   if (t < kNP) {
-    float g = 0.f;
-    for (int32_t c = 0; c < nchunks; ++c) g += partial[int64_t(c) * kNP + t];
+    for (int32_t c = b; c < e; c += 8) {
+      float x[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = c + u < e ? partial[int64_t(c + u) * kNP + t] : 0.f;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) g += x[u];
+    }
+  }
+  part[seg][lane] = g;
+  __syncthreads();
+  if (seg == 0 && t < kNP) {
+#pragma unroll
+    for (int s = 1; s < kRedSegs; ++s) g += part[s][lane];
     grad[t] = g;
   }
-  if (t == 0 && loss) {
+  if (blockIdx.x == 0 && threadIdx.x == 0 && loss) {
     float l = 0.f;
-    for (int32_t e = 0; e < nseg; ++e) l += seg_loss[e];
+    for (int32_t e2 = 0; e2 < nseg; ++e2) l += seg_loss[e2];
     *loss = l / float(nseg);
   }
 }
@@ -1094,7 +1169,7 @@ int schulze_mlp_train_step(schulze_ctx* ctx, float* params, float* adam_m, float
     Launch L(ctx, stream, "mlp_train_backward", double(N) * 5248.0 * 4.0);
     raise_smem(ctx, reinterpret_cast<const void*>(mlp_backward_kernel));
     mlp_backward_kernel<<<nchunks, 256, sizeof(BackwardSmem), stream>>>(params, feat, h1, h2, ds, N, partial);
-    mlp_reduce_kernel<<<(kNP + 255) / 256, 256, 0, stream>>>(partial, nchunks, seg_loss, nseg, g, loss);
+    mlp_reduce_kernel<<<(kNP + 31) / 32, 32 * kRedSegs, 0, stream>>>(partial, nchunks, seg_loss, nseg, g, loss);
   }
   {
     Launch L(ctx, stream, "mlp_train_adam", double(kNP) * 16.0);

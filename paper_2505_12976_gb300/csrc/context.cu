@@ -53,27 +53,15 @@ static int set_device(schulze_ctx* ctx) {
 
 using namespace schulze;
 
-// Page-locked host memory (or no buffer): graph copy nodes need it; calls
-// with pageable buffers run eagerly.
-static bool pinned(const void* ptr) {
-  if (!ptr) return true;
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return a.type == cudaMemoryTypeHost;
-}
-
-// Makes ctx->host_exec the graph of schulze_run_host's work for `key`,
-// capturing enqueue(cap_stream, host_status) when the key changed; false
-// when the call cannot be a graph (pageable host buffers, a failed capture)
-// and must run eagerly.
+// Makes ctx->host_exec the graph of schulze_run_host's kernels for `key`,
+// capturing enqueue(cap_stream) when the key changed; false when the capture
+// failed and the call must run eagerly. The graph works on the workspace
+// alone (the copies from and to the caller's buffers stay outside), so calls
+// with other buffers of the same sizes replay it.
 template <class Enqueue>
 static bool host_graph(schulze_ctx* ctx, const schulze_ctx::HostKey& key, Enqueue&& enqueue) {
-  if (!ctx->cap_stream || !ctx->host_status) return false;
+  if (!ctx->cap_stream) return false;
   if (ctx->host_exec && ctx->host_key == key) return true;
-  if (!pinned(key.ranks) || !pinned(key.winners) || !pinned(key.order)) return false;
   if (ctx->host_exec) {
     cudaGraphExecDestroy(ctx->host_exec);
     ctx->host_exec = nullptr;
@@ -83,7 +71,7 @@ static bool host_graph(schulze_ctx* ctx, const schulze_ctx::HostKey& key, Enqueu
     cudaGetLastError();
     return false;
   }
-  const int rc = enqueue(ctx->cap_stream, ctx->host_status);
+  const int rc = enqueue(ctx->cap_stream);
   cudaGraph_t g = nullptr;
   const cudaError_t ec = cudaStreamEndCapture(ctx->cap_stream, &g);
   cudaGraphExec_t exec = nullptr;
@@ -382,10 +370,8 @@ int schulze_run_host(schulze_ctx* ctx, const int32_t* ranks_host, int64_t n, int
   void* rest = cv.take<char>(0);
   void* xrest = static_cast<char*>(rest) +
                 align_up(std::max(tally_workspace_bytes(n, m, k, flags), closure_workspace_bytes(m, n, flags)), 256);
-  // the call's work on stream s, the status word copied to *st
-  auto enqueue = [&](cudaStream_t s, int32_t* st) -> int {
-    if (rbytes && cudaMemcpyAsync(ranks, ranks_host, rbytes, cudaMemcpyHostToDevice, s) != cudaSuccess)
-      return SCHULZE_ECUDA;
+  // the kernels, on stream s
+  auto enqueue = [&](cudaStream_t s) -> int {
     const bool small = closure_small(m, n, flags);
     if (int rc = tally_launch(ctx, ranks, n, m, k, d, flags, rest, s, small ? nullptr : hint,
                               small ? nullptr : hint_valid))
@@ -395,24 +381,23 @@ int schulze_run_host(schulze_ctx* ctx, const int32_t* ranks_host, int64_t n, int
                             winners_host ? win : nullptr, order_host ? ord : nullptr);
     if (!rc && ext && !small) rc = extract_from_beaten_by(ctx, bb, m, win, ord, xrest, s);
     const int rj = side_join(ctx, s);
-    if (rc || rj) return rc ? rc : rj;
-    if (winners_host && cudaMemcpyAsync(winners_host, win, size_t(m) * 4, cudaMemcpyDeviceToHost, s) != cudaSuccess)
-      return SCHULZE_ECUDA;
-    if (order_host && cudaMemcpyAsync(order_host, ord, size_t(m) * 4, cudaMemcpyDeviceToHost, s) != cudaSuccess)
-      return SCHULZE_ECUDA;
-    if (cudaMemcpyAsync(st, ctx->status, sizeof(int32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-      return SCHULZE_ECUDA;
-    return SCHULZE_OK;
+    return rc ? rc : rj;
   };
-  int32_t st = 0;
-  if (host_graph(ctx, {ranks_host, winners_host, order_host, ctx->ws.base, n, m, k, flags}, enqueue)) {
-    if (cudaGraphLaunch(ctx->host_exec, stream) != cudaSuccess || cudaStreamSynchronize(stream) != cudaSuccess)
-      return SCHULZE_ECUDA;
-    st = *ctx->host_status;
-  } else {
-    if (int rc = enqueue(stream, &st)) return rc;
-    if (cudaStreamSynchronize(stream) != cudaSuccess) return SCHULZE_ECUDA;
+  if (rbytes && cudaMemcpyAsync(ranks, ranks_host, rbytes, cudaMemcpyHostToDevice, stream) != cudaSuccess)
+    return SCHULZE_ECUDA;
+  if (host_graph(ctx, {ctx->ws.base, n, m, k, flags, winners_host != nullptr, order_host != nullptr}, enqueue)) {
+    if (cudaGraphLaunch(ctx->host_exec, stream) != cudaSuccess) return SCHULZE_ECUDA;
+  } else if (int rc = enqueue(stream)) {
+    return rc;
   }
+  int32_t st = 0;
+  int32_t* const hst = ctx->host_status ? ctx->host_status : &st;  // (page-locked: the copy does not wait for the stream)
+  if ((winners_host && cudaMemcpyAsync(winners_host, win, size_t(m) * 4, cudaMemcpyDeviceToHost, stream) != cudaSuccess) ||
+      (order_host && cudaMemcpyAsync(order_host, ord, size_t(m) * 4, cudaMemcpyDeviceToHost, stream) != cudaSuccess) ||
+      cudaMemcpyAsync(hst, ctx->status, sizeof(int32_t), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+      cudaStreamSynchronize(stream) != cudaSuccess)
+    return SCHULZE_ECUDA;
+  st = *hst;
   if (st != 0) {
     cudaMemsetAsync(ctx->status, 0, sizeof(int32_t), stream);
     cudaStreamSynchronize(stream);

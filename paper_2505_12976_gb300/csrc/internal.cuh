@@ -101,9 +101,9 @@ struct schulze_ctx {
   std::vector<schulze::ProfRecord> prof_pending;
   std::vector<schulze::ProfClass> prof_classes;
   std::vector<cudaEvent_t> prof_free_events;
-  // schulze_run_host: the whole call (copies in, path, copies out) captured
-  // once as a CUDA graph on cap_stream and replayed while the arguments,
-  // the workspace and the host buffers (page-locked) stay the same
+  // schulze_run_host: the path's kernels on workspace memory captured once as
+  // a CUDA graph on cap_stream and replayed while the sizes, the flags and the
+  // workspace stay the same
   cudaStream_t cap_stream = nullptr;
   // schulze_run / schulze_run_host: the closure writes p on side_stream
   // (forked from the call's stream with side_fork) while the winners and
@@ -115,16 +115,14 @@ struct schulze_ctx {
   cudaGraphExec_t host_exec = nullptr;
   int32_t* host_status = nullptr;  // page-locked word receiving the device status
   struct HostKey {
-    const void* ranks = nullptr;
-    const void* winners = nullptr;
-    const void* order = nullptr;
     const void* ws = nullptr;
     int64_t n = -1;
     int32_t m = -1, k = -1;
     uint32_t flags = 0;
+    bool winners = false, order = false;  // which results are computed
     bool operator==(const HostKey& o) const {
-      return ranks == o.ranks && winners == o.winners && order == o.order && ws == o.ws && n == o.n && m == o.m &&
-             k == o.k && flags == o.flags;
+      return ws == o.ws && n == o.n && m == o.m && k == o.k && flags == o.flags && winners == o.winners &&
+             order == o.order;
     }
   } host_key;
 };

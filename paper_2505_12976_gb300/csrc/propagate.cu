@@ -25,7 +25,7 @@
 // starts at a few unknown candidates touches their rows and columns only, and
 // one in which everything changed reads d once. On m = 18407 (top-200 lists)
 // the two iterations took 6.3 ms with a transposed copy of d and two rows
-// per candidate read in every pass, 2.6 ms in this form.
+// per candidate read in every pass, 1.4 ms in this form.
 #include <algorithm>
 
 #include "internal.cuh"
@@ -64,6 +64,7 @@ struct PassArgs {
   Key *fn, *bn;             // kPropagate: the next round's (start as f and b)
   int32_t* changed;         // kPropagate: cleared here, set by commit_kernel
   const int32_t* asked;     // kMarks: candidates asked about
+  const int4* label;        // kMarks: per block its first candidate's ids (x, y), z: all share them
   int32_t *lose, *scc_lose;  // kMarks
 };
 
@@ -76,8 +77,8 @@ __global__ void __launch_bounds__(256) pair_kernel(PassArgs g) {
   int32_t a = 0;
   int64_t rem = blockIdx.x;  // pair (a, a + rem), numbered row by row
   {
-    const double x = double(nbt) + 0.5;  // a from the triangular numbering, then corrected
-    a = max(0, min(nbt - 1, int32_t(x - sqrt(max(0.0, x * x - 2.0 * double(rem))))));
+    const float x = float(nbt) + 0.5f;  // a from the triangular numbering, then corrected (FP64 is slow here)
+    a = max(0, min(nbt - 1, int32_t(x - sqrtf(max(0.f, x * x - 2.f * float(rem))))));
     auto first = [&](int64_t r) { return r * nbt - r * (r - 1) / 2; };
     while (a > 0 && first(a) > rem) --a;
     while (a + 1 < nbt && first(a + 1) <= rem) ++a;
@@ -87,7 +88,11 @@ __global__ void __launch_bounds__(256) pair_kernel(PassArgs g) {
   // side 0: targets in A, sources in B; side 1: the other way round
   bool s0 = true, s1 = A != B;
   if (kPass == kPropagate) s0 = g.flag[bt] != 0, s1 = s1 && g.flag[a] != 0;
-  if (kPass == kMarks) s0 = g.flag[a] != 0, s1 = s1 && g.flag[bt] != 0;
+  if (kPass == kMarks) {
+    // blocks of one and the same label hold no edge from another SCC
+    const bool same = g.label[a].z && g.label[bt].z && g.label[a].x == g.label[bt].x && g.label[a].y == g.label[bt].y;
+    s0 = g.flag[a] != 0 && !same, s1 = s1 && g.flag[bt] != 0 && !same;
+  }
   if (!s0 && !s1) return;
   __shared__ int32_t t1[kPT][kPT + 1], t2[kPT][kPT + 1];  // t1 = d[A.., B..], t2 = d[B.., A..]
   __shared__ Key sf[2][kPT], sb[2][kPT];                  // keys of A, of B
@@ -125,6 +130,11 @@ __global__ void __launch_bounds__(256) pair_kernel(PassArgs g) {
   __syncthreads();
   // targets T + r of tile side ts (their d rows in x), sources S + c (their d rows in `other`)
   auto serve = [&](int32_t T, int ts, int ss, const int32_t (&x)[4][4], const int32_t(*other)[kPT + 1]) {
+    Key uf[4], ub[4];  // the keys of this thread's sources
+    if (kPass != kInit) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) uf[e] = sf[ss][c4 + e], ub[e] = sb[ss][c4 + e];
+    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int r = rq + 16 * q;
@@ -147,14 +157,23 @@ __global__ void __launch_bounds__(256) pair_kernel(PassArgs g) {
         }
       } else if (kPass == kPropagate) {
         const Key mf = sf[ts][r], mb = sb[ts][r];
-        Key bf = mf, bb = mb;
+        // along (u, c) from u's source, against (c, u) from u's target; most
+        // of the pass finds nothing better, so that is all that it asks first
+        bool better = false;
+        int32_t wi[4], wo[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const int32_t o = other[c4 + e][r], wi = edge(o, x[q][e], g.margin), wo = edge(x[q][e], o, g.margin);
-          if (wi) bf = min(bf, along(sf[ss][c4 + e], wi));  // along (u, c)
-          if (wo) bb = min(bb, along(sb[ss][c4 + e], wo));  // against (c, u)
+          const int32_t o = other[c4 + e][r];
+          wi[e] = edge(o, x[q][e], g.margin), wo[e] = edge(x[q][e], o, g.margin);
+          better |= (o > x[q][e] && along(uf[e], wi[e]) < mf) || (x[q][e] > o && along(ub[e], wo[e]) < mb);
         }
-        if (__any_sync(0xFFFFFFFFu, bf < mf || bb < mb)) {
+        if (__any_sync(0xFFFFFFFFu, better)) {
+          Key bf = mf, bb = mb;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            if (wi[e]) bf = min(bf, along(uf[e], wi[e]));
+            if (wo[e]) bb = min(bb, along(ub[e], wo[e]));
+          }
 #pragma unroll
           for (int o = 8; o; o >>= 1) {
             bf = min(bf, __shfl_xor_sync(0xFFFFFFFFu, bf, o));
@@ -171,7 +190,7 @@ __global__ void __launch_bounds__(256) pair_kernel(PassArgs g) {
         bool other_scc = false;
 #pragma unroll
         for (int e = 0; e < 4; ++e)
-          other_scc |= other[c4 + e][r] > x[q][e] && (key_id(sf[ss][c4 + e]) != ms || key_id(sb[ss][c4 + e]) != mt);
+          other_scc |= other[c4 + e][r] > x[q][e] && (key_id(uf[e]) != ms || key_id(ub[e]) != mt);
         const uint32_t any = __ballot_sync(0xFFFFFFFFu, other_scc) >> (lane & 16) & 0xFFFFu;
         if ((lane & 15) == 0 && any && c < m && g.asked[c]) {
           if (ms == mt) g.scc_lose[ms == kNone ? m : ms] = 1;
@@ -235,11 +254,14 @@ __global__ void __launch_bounds__(kPT) commit_kernel(int32_t m, Key* __restrict_
 // unknown candidate's. A CTA per block of 64.
 __global__ void __launch_bounds__(kPT) label_kernel(const Key* __restrict__ f, const Key* __restrict__ b, int32_t m,
                                                     const int32_t* __restrict__ status, int32_t* __restrict__ lose,
-                                                    int32_t* __restrict__ asked, int32_t* __restrict__ flag) {
+                                                    int32_t* __restrict__ asked, int32_t* __restrict__ flag,
+                                                    int4* __restrict__ label) {
   const int32_t c = blockIdx.x * kPT + threadIdx.x;
-  bool ask = false;
+  const int32_t s0 = key_id(f[blockIdx.x * kPT]), t0 = key_id(b[blockIdx.x * kPT]);
+  bool ask = false, same = true;
   if (c < m) {
     const int32_t s = key_id(f[c]), t = key_id(b[c]);
+    same = s == s0 && t == t0;
     if (s < t) {
       lose[c] = 1;
     } else if (s > t) {
@@ -252,8 +274,8 @@ __global__ void __launch_bounds__(kPT) label_kernel(const Key* __restrict__ f, c
     ask = status[c] == kUnknown || (s == t && s != kNone);
     asked[c] = ask;
   }
-  const int any = __syncthreads_or(ask);
-  if (threadIdx.x == 0) flag[blockIdx.x] = any;
+  const int any = __syncthreads_or(ask), one = __syncthreads_and(same);
+  if (threadIdx.x == 0) flag[blockIdx.x] = any, label[blockIdx.x] = make_int4(s0, t0, one, 0);
 }
 
 // Postprocessing, applied: unknown candidates marked (or in a marked SCC)
@@ -307,12 +329,13 @@ int winners_propagation_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, bo
   int32_t* words = cv.take<int32_t>(3);                  // [0] changed, [1] decided, [2] unknown
   const int32_t nbt = (m + kPT - 1) / kPT;
   int32_t* flag = cv.take<int32_t>(size_t(nbt));
+  int4* label = cv.take<int4>(size_t(nbt));
   const unsigned pairs = unsigned(int64_t(nbt) * (nbt + 1) / 2);
   const int g = std::max(1, std::min((m + 255) / 256, 1024));
   PassArgs pa{};
   pa.d = d, pa.m = m, pa.margin = margin ? 1 : 0, pa.vec4 = rows_vec16(d, m);
   pa.in = inout, pa.out = inout + m, pa.flag = flag, pa.f = f, pa.b = b, pa.fn = fn, pa.bn = bn, pa.changed = words;
-  pa.asked = asked, pa.lose = lose, pa.scc_lose = scc_lose;
+  pa.asked = asked, pa.label = label, pa.lose = lose, pa.scc_lose = scc_lose;
   {
     Launch L(ctx, stream, "propagation_init", double(m) * double(m) * 4.0);
     if (!max_in) {
@@ -350,7 +373,7 @@ int winners_propagation_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, bo
     }
     {
       Launch L(ctx, stream, "propagation_marks", double(m) * double(m) * 4.0);
-      label_kernel<<<nbt, kPT, 0, stream>>>(f, b, m, status, lose, asked, flag);
+      label_kernel<<<nbt, kPT, 0, stream>>>(f, b, m, status, lose, asked, flag, label);
       pair_kernel<kMarks><<<pairs, 256, 0, stream>>>(pa);
     }
     apply_kernel<<<g, 256, 0, stream>>>(f, b, m, lose, scc_lose, status, words + 1);

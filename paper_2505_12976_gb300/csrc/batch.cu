@@ -79,14 +79,8 @@ struct BatchArgs {
 constexpr size_t kStageBytes = sizeof(tiles::SmemS32) * kGroups + 2 * tiles::kB * 4;
 union BatchSmem {
   unsigned char raw[kStageBytes];
-  struct {
-    tiles::SmemS32 t[kGroups];
-    int32_t rowbuf[2][tiles::kB];
-  } c32;
-  struct {
-    tiles::SmemS16 t[kGroups];
-    int32_t rowbuf[2][tiles::kB];
-  } c16;
+  tiles::SmemS32 t32[kGroups];
+  tiles::SmemS16 t16[kGroups];
   int32_t bb[kBatchMaxM];
 };
 
@@ -399,6 +393,7 @@ struct Shared {
   float key[kBatchMaxM];
   int32_t tmax[kMaxTiles * kMaxTiles], tmin[kMaxTiles * kMaxTiles];
   uint16_t list[kMaxTiles * kMaxTiles];
+  alignas(16) int32_t rowbuf[2][tiles::kB];  // the diagonal tile's pivot rows
   int32_t count;
 };
 
@@ -458,9 +453,8 @@ __device__ void closure(E* W, int32_t m, int32_t mp, BatchSmem& sm, Shared& sh) 
   const int32_t nb = mp / kB;
   const int g = threadIdx.x / tiles::kThreads, lt = threadIdx.x % tiles::kThreads;
   const tiles::GroupBarrier bar{1 + g};
-  auto& ts = sizeof(E) == 2 ? reinterpret_cast<typename Ops::Smem*>(sm.c16.t)[g]
-                            : reinterpret_cast<typename Ops::Smem*>(sm.c32.t)[g];
-  int32_t(*rowbuf)[kB] = sizeof(E) == 2 ? sm.c16.rowbuf : sm.c32.rowbuf;
+  auto& ts = sizeof(E) == 2 ? reinterpret_cast<typename Ops::Smem*>(sm.t16)[g]
+                            : reinterpret_cast<typename Ops::Smem*>(sm.t32)[g];
   // the group's part of tile t's bounds after its update (reset before it)
   auto bounds = [&](int t, const Bounds& bd) {
     const int32_t mx = __reduce_max_sync(0xFFFFFFFFu, bd.mx), mn = __reduce_min_sync(0xFFFFFFFFu, bd.mn);
@@ -497,7 +491,7 @@ __device__ void closure(E* W, int32_t m, int32_t mp, BatchSmem& sm, Shared& sh) 
     if (g == 0 && close) {
       if (lt == 0) sh.tmax[r * nb + r] = 0, sh.tmin[r * nb + r] = INT32_MAX;
       Bounds bd;
-      tiles::diag_closure_local<E>(W, mp, r, m - r * kB, m - r * kB, rowbuf, lt, bar, bd);
+      tiles::diag_closure_local<E>(W, mp, r, m - r * kB, m - r * kB, sh.rowbuf, lt, bar, bd);
       bounds(r * nb + r, bd);
     }
     __syncthreads();

@@ -47,11 +47,11 @@
 // CPU, blocked Floyd-Warshall): 0.9% for Plackett-Luce Zipf(1.1) top-20 lists
 // at m = 8192, 3.7% at m = 2048, 4.6% for top-200 lists at m = 2048, 2.1% for
 // Mallows(0.98) full rankings and 92% for impartial culture at m = 1024. The
-// closure went from 390 to 10.8 ms at m = 16384 (int32, top-20, 0.7% of the
-// updates left) and from 309 to 13.0 ms at m = 18407 (int16, top-200, 4%); it
-// is now bound by the chain diagonal tile - panels - next diagonal tile of
-// its 256 to 288 rounds, about 40 us each. Where every update is needed
-// (uniform random d, m = 8192) the tests and bounds cost 5%.
+// closure went from 390 to 8.4 ms at m = 16384 (int32, top-20, 0.7% of the
+// updates left) and from 309 to 9.7 ms at m = 18407 (int16, top-200, 4%); it
+// is now bound by the chain diagonal tile - panel - next diagonal tile of
+// its 256 to 288 rounds (33 us each; 16 us where nothing else runs). Where every update is needed
+// (uniform random d, m = 8192) the tests and bounds cost up to 4%.
 //
 // All rounds run in ONE persistent cooperative launch: the CTAs take work
 // items from a global queue in a fixed order in which the next round's
@@ -523,6 +523,7 @@ enum ItemKind : int32_t { kDiag = 0, kPanel = 1, kTile = 2, kStop = 3 };
 // for tile t. The index runs along tile row or column fix, or (kGrid) over
 // the n x n tiles of R(r) row by row; tile indices are counted without the
 // `skip` indices r, r + 1, ...
+constexpr int kItemTiles = 32;  // one per lane
 enum ItemShape : int32_t { kRow = 0, kColumn = 1, kGrid = 2 };
 struct Item {
   int32_t kind, r, shape, fix, v0, stride, cnt, skip, n;
@@ -541,108 +542,96 @@ struct Item {
 // the cold columns.
 //
 // Queue order, stage by stage:
-//   stage 0:             D(0) P(0) L(0)
-//   stage s (1..nbr-2):  D(s) P(s) X(s-1) R(s-1) L(s)
-//   stage nbr-1:         D(s) P(s) R(s-1)
+//   stage 0:             D(0) P(0) D(1) L(0)
+//   stage s (1..nbr-2):  P(s) X(s-1) D(s+1) L(s) R(s-1)
+//   stage nbr-1:         P(s) R(s-1)
 //   stage nbr:           R(nbr-1)
-// D(r): diagonal tile; P(r): the panel tiles (r, r+1) and (r+1, r) the next
-// diagonal tile waits for, then the rest of row panel r and of column panel
-// r; L(r): round-r tiles that the next round's panels are made of, the next
-// diagonal tile (r+1, r+1) first, then tile row r+1, then tile column r+1;
-// X(r): the round-r tiles of tile row and column r+2, which L(r+1) is made
-// of, ahead of R(r): the other round-r tiles. P, L and X come in items of at
-// most gp tiles, R in items of at most gr: about two items per CTA and round,
-// or 16 where most tiles need their update (a round then ends with CTAs
-// waiting for its last items). One tile per item costs nothing at few tiles
-// and keeps the chain of the panels short; at many tiles the tests of 32
+// D(r): the diagonal tile: its round r-1 update, then its closure; P(r): the
+// panel tiles (r, r+1) and (r+1, r) that D(r+1) waits for, then the rest of
+// row panel r and of column panel r; L(r): the round-r tiles of tile row and
+// column r+1, which the next round's panels are made of; X(r): those of tile
+// row and column r+2, which L(r+1) is made of; R(r): the other round-r tiles.
+// So the chain from one diagonal tile to the next (D, P, D, ...) never waits
+// for R, and D(r+1) runs beside R(r-1). P, L and X come tile by tile, which
+// keeps the chain of the panels short, R in items of at most gr tiles: about
+// two items per CTA and round, or 16 where most tiles need their update (a
+// round then ends with CTAs waiting for its last items). The tests of 32
 // tiles, a lane each, cost one round trip to the progress words instead of 32
-// (a skipped tile by itself would take its CTA about a microsecond). The
+// (a skipped tile by itself would take its CTA about a microsecond); 64 left
+// the items with too much work (m = 18407 top-200: 12.9 ms against 9.7). The
 // tiles of an item are spread evenly over their range: those that need an
 // update lie next to each other (m = 16384 top-20: 480 of 65536 in a round),
 // and items of neighbours left some CTAs with most of them (the closure took
 // 28.5 ms, 10.8 ms spread).
 struct Shape {
-  int32_t nbr, gp, gr;
-  int32_t sp, sp_last;  // items per panel side, r < nbr - 1 and r = nbr - 1 (no r + 1 to leave out)
-  int32_t xc;           // items of the column side of X (its row side has sp)
+  int32_t nbr, gr;
   int32_t P, L;         // items of P(r), L(r), r < nbr - 1
   int32_t X, R;         // items of X(r), R(r), r < nbr - 2
   int32_t P_last, R_pen, R_last;  // P(nbr - 1), R(nbr - 2), R(nbr - 1)
+  uint32_t first, mid, total;     // items of stage 0, of a stage 1 .. nbr - 2, of the queue
 };
 
-__device__ __forceinline__ Shape make_shape(int32_t nbr, int32_t grid, bool dense) {  // nbr >= 3
+__device__ Shape make_shape(int32_t nbr, int32_t grid, bool dense) {  // nbr >= 3
   Shape sh;
   sh.nbr = nbr;
-  sh.gr = min(32, max(1, nbr * nbr / ((dense ? 16 : 2) * grid)));
-  sh.gp = min(4, max(1, nbr / 64));
-  const int32_t q = nbr - 2;
-  sh.sp = (q + sh.gp - 1) / sh.gp, sh.sp_last = (q + sh.gp) / sh.gp;
-  sh.xc = (q - 1 + sh.gp - 1) / sh.gp;
-  sh.P = 2 + 2 * sh.sp, sh.L = 1 + 2 * sh.sp, sh.P_last = 2 * sh.sp_last;
-  sh.X = sh.sp + sh.xc, sh.R = ((q - 1) * (q - 1) + sh.gr - 1) / sh.gr;
+  sh.gr = min(kItemTiles, max(1, nbr * nbr / ((dense ? 16 : 2) * grid)));
+  const int32_t q = nbr - 2;  // tile indices without r and r + 1
+  sh.P = 2 + 2 * q, sh.L = 2 * q, sh.P_last = 2 * (q + 1);
+  sh.X = q + (q - 1), sh.R = ((q - 1) * (q - 1) + sh.gr - 1) / sh.gr;
   sh.R_pen = (q * q + sh.gr - 1) / sh.gr, sh.R_last = ((q + 1) * (q + 1) + sh.gr - 1) / sh.gr;
+  sh.first = 2 + sh.P + sh.L, sh.mid = 1 + sh.P + sh.X + sh.L + sh.R;
+  sh.total = sh.first + uint32_t(q) * sh.mid + uint32_t(sh.P_last + sh.R_pen + sh.R_last);
   return sh;
 }
 
-__device__ __forceinline__ uint32_t queue_items(const Shape& sh) {
-  return uint32_t(sh.nbr) + uint32_t(sh.nbr - 1) * uint32_t(sh.P + sh.L) +
-         uint32_t(sh.nbr - 2) * uint32_t(sh.X + sh.R) + uint32_t(sh.P_last + sh.R_pen + sh.R_last);
-}
-
-// item t of the queue, t < queue_items(sh)
+// item t of the queue, t < sh.total
 __device__ Item decode_item(uint32_t t, const Shape& sh) {
   const int32_t nbr = sh.nbr, q = nbr - 2;
-  const uint32_t first = 1 + sh.P + sh.L, mid = first + sh.X + sh.R;
   int32_t s = 0;
-  if (t >= first) {
-    t -= first;
-    if (t < uint32_t(q) * mid) {
-      s = 1 + int32_t(t / mid);
-      t -= uint32_t(s - 1) * mid;
+  if (t >= sh.first) {
+    t -= sh.first;
+    if (t < uint32_t(q) * sh.mid) {
+      s = 1 + int32_t(t / sh.mid);
+      t -= uint32_t(s - 1) * sh.mid;
     } else {
-      t -= uint32_t(q) * mid;
+      t -= uint32_t(q) * sh.mid;
       s = nbr - 1;
-      const uint32_t z = 1 + sh.P_last + sh.R_pen;
+      const uint32_t z = sh.P_last + sh.R_pen;
       if (t >= z) t -= z, s = nbr;
     }
   }
-  const bool last = s == nbr - 1;
   auto one = [](int32_t kind, int32_t r, int32_t i, int32_t j) { return Item{kind, r, kRow, i, j, 0, 1, 0, 0}; };
   // item a of the `items` that share the n tiles (or n x n) of a range
   auto part = [](int32_t kind, int32_t r, int32_t shape, int32_t fix, int32_t a, int32_t items, int32_t n, int32_t skip) {
     const int32_t range = shape == kGrid ? n * n : n;
     return Item{kind, r, shape, fix, a, items, (range - a + items - 1) / items, skip, n};
   };
-  if (s < nbr) {
-    if (t == 0) return one(kDiag, s, s, s);
-    t -= 1;
-    const uint32_t P = last ? sh.P_last : sh.P;
-    if (t < P) {
-      if (!last) {
-        if (t < 2) return t == 0 ? one(kPanel, s, s, s + 1) : one(kPanel, s, s + 1, s);
-        t -= 2;
-      }
-      const int32_t sp = last ? sh.sp_last : sh.sp, a = int32_t(t);
-      return part(kPanel, s, a < sp ? kRow : kColumn, s, a < sp ? a : a - sp, sp, last ? q + 1 : q, last ? 1 : 2);
-    }
-    t -= P;
+  int32_t a = int32_t(t);
+  if (s == nbr) return part(kTile, nbr - 1, kGrid, 0, a, sh.R_last, q + 1, 1);
+  if (s == nbr - 1) {
+    if (a < sh.P_last)
+      return part(kPanel, s, a <= q ? kRow : kColumn, s, a <= q ? a : a - (q + 1), q + 1, q + 1, 1);
+    return part(kTile, s - 1, kGrid, 0, a - sh.P_last, sh.R_pen, q, 2);
   }
+  if (s == 0) {
+    if (a == 0) return one(kDiag, 0, 0, 0);
+    a -= 1;
+  }
+  if (a < 2) return a == 0 ? one(kPanel, s, s, s + 1) : one(kPanel, s, s + 1, s);
+  if (a < sh.P) {
+    a -= 2;
+    return part(kPanel, s, a < q ? kRow : kColumn, s, a < q ? a : a - q, q, q, 2);
+  }
+  a -= sh.P;
   if (s >= 1) {
-    const int32_t r = s - 1, skip = s == nbr ? 1 : last ? 2 : 3;
-    if (skip == 3) {
-      const int32_t a = int32_t(t);
-      if (a < sh.sp) return part(kTile, r, kRow, r + 2, a, sh.sp, q, 2);
-      if (a < sh.X) return part(kTile, r, kColumn, r + 2, a - sh.sp, sh.xc, q - 1, 3);
-      t -= sh.X;
-    }
-    const int32_t R = skip == 1 ? sh.R_last : skip == 2 ? sh.R_pen : sh.R;
-    if (int32_t(t) < R) return part(kTile, r, kGrid, 0, int32_t(t), R, nbr - skip, skip);
-    t -= R;
+    if (a < q) return part(kTile, s - 1, kRow, s + 1, a, q, q, 2);
+    if (a < sh.X) return part(kTile, s - 1, kColumn, s + 1, a - q, q - 1, q - 1, 3);
+    a -= sh.X;
   }
-  // L(s)
-  if (t == 0) return one(kTile, s, s + 1, s + 1);
-  const int32_t a = int32_t(t) - 1;
-  return part(kTile, s, a < sh.sp ? kRow : kColumn, s + 1, a < sh.sp ? a : a - sh.sp, sh.sp, q, 2);
+  if (a == 0) return one(kDiag, s + 1, s + 1, s + 1);
+  a -= 1;
+  if (a < sh.L) return part(kTile, s, a < q ? kRow : kColumn, s + 1, a < q ? a : a - q, q, q, 2);
+  return part(kTile, s - 1, kGrid, 0, a - sh.L, sh.R, q - 1, 3);
 }
 
 struct Sync {
@@ -667,6 +656,8 @@ __device__ __forceinline__ uint64_t load_word(const unsigned long long* p) {
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
+// (__threadfence() would be the stronger, slower fence.sc)
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 __device__ __forceinline__ void store_word(unsigned long long* p, uint64_t v) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
@@ -684,44 +675,51 @@ constexpr int32_t kClusterMaxWarm = sizeof(E) == 2 ? 256 : 192;
 #define SCHULZE_PERSIST_BOUNDS __launch_bounds__(kThreads, sizeof(E) == 2 ? 6 : 5)
 
 // Warp 1 runs the schedule: it claims the CTA's next queue slot while the CTA
-// works on the current item, and between items its lane t waits for the
-// words tile t of the new item depends on (own tile: the rounds before;
-// panel: the closed diagonal; tile: both panels) and tests its bounds: a tile
-// that cannot change is passed on to the next round at once, the others are
-// computed one after another by the CTA and published by thread 0 as they are
-// done (the last one while warp 1 is at the next item already). The schedule
-// stays deadlock-free: every wait is on an item earlier in the queue, and a
-// CTA holds at most one claimed, unstarted item, later in the queue than its
-// current one, so the earliest unfinished item is always being worked on.
-struct Slot {  // an item and its tiles to compute
+// works on the current item, and between items its lanes wait for the words
+// the new item's tiles depend on (own tile: the rounds before; panel: the
+// closed diagonal; tile: both panels; diagonal: both panels of the round
+// before) and test their bounds: a tile that cannot change is passed on to
+// the next round at once, the others are computed one after another by the
+// CTA and published by thread 0 as they are done (the last one while warp 1 is
+// at the next item already). The schedule stays deadlock-free: every wait is
+// on an item earlier in the queue, and a CTA holds at most one claimed,
+// unstarted item, later in the queue than its current one, so the earliest
+// unfinished item is always being worked on.
+struct Slot {  // an item and its tiles to compute; diagonal: whether its update of the round before is needed
   Item it;
-  uint32_t mask;
+  uint32_t mask, update;
 };
 
 // warp 1: the item of queue slot t into *s (kStop at the end of the queue or
 // after a failed wait); out of line, as the tile update needs the registers
-__device__ __noinline__ void next_item(const Sync& sy, uint32_t t, int32_t nbr, int32_t nb, bool dense, Slot* s) {
+__device__ __noinline__ void next_item(const Sync& sy, uint32_t t, const Shape& sh, int32_t nb, Slot* s) {
   const int lane = threadIdx.x & 31;
   if (lane == 0) {
-    const Shape sh = make_shape(nbr, int32_t(gridDim.x), dense);
-    if (t >= queue_items(sh) || *reinterpret_cast<volatile uint32_t*>(sy.abort_flag)) s->it.kind = kStop;
+    if (t >= sh.total || *reinterpret_cast<volatile uint32_t*>(sy.abort_flag)) s->it = Item{kStop, 0, kRow, 0, 0, 0, 0, 0, 0};
     else s->it = decode_item(t, sh);
   }
   __syncwarp();
   const Item it = s->it;
   const uint32_t r = uint32_t(it.r);
-  bool ok = true, need = false;
-  if (it.kind != kStop && lane < it.cnt) {
+  const bool diag = it.kind == kDiag;
+  // rounds the own word and the operands' words need to have; a diagonal
+  // tile's own update is that of round r - 1
+  const uint32_t n0 = diag && r ? r - 1 : r, nd = diag ? r : r + 1;
+  const int32_t rr = diag ? it.r - 1 : it.r;  // the round whose operands are read
+  const bool two = it.kind == kTile || (diag && r);  // operands (i, rr) and (rr, j)
+  bool ok = true, need = false, update = false;
+  if (lane < it.cnt) {
     int32_t i, j;
     it.tile(lane, i, j);
     const int32_t own = i * nb + j;
-    const bool ta = it.kind != kDiag, tb = it.kind == kTile;
-    const int32_t da = it.kind == kTile ? i * nb + it.r : it.r * nb + it.r, db = it.r * nb + j;
-    uint64_t w0 = r ? load_word(sy.prog + own) : 0, w1 = ta ? load_word(sy.prog + da) : 0,
-             w2 = tb ? load_word(sy.prog + db) : 0;
+    const int32_t da = it.kind == kPanel ? it.r * nb + it.r : i * nb + rr, db = rr * nb + j;
+    constexpr uint64_t kThere = ~uint64_t(0);  // (no word to wait for)
+    uint64_t w0 = n0 ? load_word(sy.prog + own) : kThere;
+    uint64_t w1 = two || it.kind == kPanel ? load_word(sy.prog + da) : kThere;
+    uint64_t w2 = two ? load_word(sy.prog + db) : kThere;
     const long long t0 = clock64();
     for (;;) {
-      const bool m0 = word_rounds(w0) < r, m1 = ta && word_rounds(w1) <= r, m2 = tb && word_rounds(w2) <= r;
+      const bool m0 = word_rounds(w0) < n0, m1 = word_rounds(w1) < nd, m2 = word_rounds(w2) < nd;
       if (!(m0 || m1 || m2)) break;
       if (*reinterpret_cast<volatile uint32_t*>(sy.abort_flag)) ok = false;
       if (ok && clock64() - t0 > sy.spin_limit) {
@@ -735,18 +733,20 @@ __device__ __noinline__ void next_item(const Sync& sy, uint32_t t, int32_t nbr, 
       if (m1) w1 = load_word(sy.prog + da);
       if (m2) w2 = load_word(sy.prog + db);
     }
-    __threadfence();
-    if (r == 0) w0 = make_word(0, Bounds{sy.tmax[own], INT32_MAX - sy.tmin[own]}, sy.shift);
+    fence_gpu();
+    if (n0 == 0) w0 = make_word(0, Bounds{sy.tmax[own], INT32_MAX - sy.tmin[own]}, sy.shift);
     // what the update can offer at most, against the tile's smallest entry
-    const uint32_t offer = it.kind == kDiag    ? word_max(w0)
-                           : it.kind == kPanel ? min(word_max(w1), word_max(w0))
-                                               : min(word_max(w1), word_max(w2));
-    need = offer > (it.kind == kDiag ? 0u : word_min(w0));
+    const uint32_t offer = min(word_max(w1), two ? word_max(w2) : word_max(w0));
+    need = offer > word_min(w0);
+    if (diag) {
+      update = two && need;
+      need = update || word_max(w0) > 0;  // a zero tile is closed
+    }
     if (ok && !need) store_word(sy.prog + own, word_at(w0, r + 1));
   }
   const uint32_t mask = __ballot_sync(0xFFFFFFFFu, need), fail = __ballot_sync(0xFFFFFFFFu, !ok);
   if (lane == 0) {
-    s->mask = mask;
+    s->mask = mask, s->update = update ? 1u : 0u;
     if (fail) s->it.kind = kStop;
   }
 }
@@ -771,6 +771,7 @@ __global__ void SCHULZE_PERSIST_BOUNDS closure_persistent_kernel(E* W, int32_t l
   pdl_enter_early();
   __shared__ __align__(16) typename Ops<E>::Smem sm;
   __shared__ __align__(16) int32_t rowbuf[2][kB];
+  __shared__ Shape s_shape;
   // two slots: warp 1 writes the next one while the others read the current
   __shared__ Slot s_slot[2];
   __shared__ uint32_t s_done[3];  // tile updates, diagonal closures, items
@@ -781,10 +782,12 @@ __global__ void SCHULZE_PERSIST_BOUNDS closure_persistent_kernel(E* W, int32_t l
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const bool dense = sample_dense(sy, nbr, nb);
   if (tid < 3) s_done[tid] = 0u;
+  if (tid == 32) s_shape = make_shape(nbr, int32_t(gridDim.x), dense);  // (warp 1 alone reads it)
+  __syncwarp();
   uint32_t next = 0;  // warp 1, lane 0: the claimed queue slot
   if (tid == 32) next = atomicAdd(sy.head, 1u);
   for (int buf = 0, par = 0;; buf ^= 1) {
-    if (wid == 1) next_item(sy, next, nbr, nb, dense, &s_slot[buf]);
+    if (wid == 1) next_item(sy, next, s_shape, nb, &s_slot[buf]);
     __syncthreads();
     const Slot& sl = s_slot[buf];
     const int32_t kind = sl.it.kind, r = sl.it.r;
@@ -798,6 +801,12 @@ __global__ void SCHULZE_PERSIST_BOUNDS closure_persistent_kernel(E* W, int32_t l
       const int32_t vr = nw - i * kB, vc = m - j * kB;  // candidates with edges / candidates from the tile's corner on
       E* Cg = W + int64_t(i) * kB * ld + int64_t(j) * kB;
       if (kind == kDiag) {
+        if (sl.update) {  // its update of the round before
+          Ops<E>::load_a(Cg - kB, ld, sm, tid);
+          Ops<E>::load_b(Cg - int64_t(kB) * ld, ld, sm, tid);
+          Ops<E>::template multiply<false>(Cg, ld, sm, tid, BlockBarrier{}, bd);
+          __syncthreads();
+        }
         diag_closure_local<E>(W, ld, r, vr, vc, rowbuf, tid, BlockBarrier{}, bd);
       } else {
         // the tiles of a panel side share an operand
@@ -814,7 +823,7 @@ __global__ void SCHULZE_PERSIST_BOUNDS closure_persistent_kernel(E* W, int32_t l
         Bounds b = s_bd[par][0];
 #pragma unroll
         for (int w = 1; w < kThreads / 32; ++w) b.mx = max(b.mx, s_bd[par][w].mx), b.mn = min(b.mn, s_bd[par][w].mn);
-        __threadfence();
+        fence_gpu();
         store_word(sy.prog + (i * nb + j), make_word(r + 1, b, sy.shift));
         ++s_done[kind == kDiag ? 1 : 0];
       }

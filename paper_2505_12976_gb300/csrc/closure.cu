@@ -1361,6 +1361,7 @@ struct ClosureBufs {
   // uniform cold columns (used only with a valid hint): ucol, u [m], ucount
   int32_t *ucol = nullptr, *ucold = nullptr, *ucount = nullptr;
   bool margin = false;  // margin weights instead of winning votes
+  bool zeroed = false;  // prog, rowflag, ucount and beaten_by are zero already
 };
 
 constexpr size_t prog_words(size_t nb) { return 4 * nb * nb + 2; }
@@ -1393,13 +1394,10 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
   uint32_t* abort_flag = head + 1;
   int shift = 0;
   while (((bound < INT32_MAX ? bound : int64_t(INT32_MAX)) >> shift) > int64_t(kBoundMax)) ++shift;
-  {
+  if (!bf.zeroed) {
     // progress words, tile bounds, queue head and abort flag; row flags; the uniform count
     ZeroSpans z;
-    z.p[0] = bf.prog, z.words[0] = int64_t(prog_words(size_t(nb)));
-    z.p[1] = reinterpret_cast<uint32_t*>(bf.rowflag), z.words[1] = m;
-    z.p[2] = reinterpret_cast<uint32_t*>(bf.ucount), z.words[2] = 1;
-    z.p[3] = reinterpret_cast<uint32_t*>(bb_out), z.words[3] = bb_out ? m : 0;
+    z.add(bf.prog, int64_t(prog_words(size_t(nb)))), z.add(bf.rowflag, m), z.add(bf.ucount, 1), z.add(bb_out, m);
     if (int rc = zero_async(ctx, z, stream)) return rc;
   }
   const double mm = double(m) * double(m);
@@ -1515,7 +1513,7 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
 template <typename E>
 int run_closure(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t bound, int32_t* p, void* ws,
                 cudaStream_t stream, int32_t* bb_out, int32_t* hint, const int32_t* hint_valid,
-                bool margin, bool side, int32_t* winners, int32_t* order) {
+                bool margin, bool side, int32_t* winners, int32_t* order, uint32_t* control) {
   const int32_t mp = int32_t(align_up(size_t(m), kB));
   const int32_t nb = mp / kB;
   Carver cv(ws);
@@ -1534,6 +1532,12 @@ int run_closure(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t bound, in
   bf.ucol = cv.take<int32_t>(size_t(m));
   bf.ucold = cv.take<int32_t>(size_t(m));
   bf.ucount = cv.take<int32_t>(1);
+  if (control) {  // (closure_control_words)
+    bf.prog = control;
+    bf.rowflag = reinterpret_cast<int32_t*>(control + prog_words(size_t(nb)));
+    bf.ucount = bf.rowflag + m;
+    bf.zeroed = true;
+  }
   bf.counters = ctx->counters;
   bf.hint = hint;
   bf.hint_valid = hint_valid;
@@ -1551,19 +1555,23 @@ size_t closure_workspace_bytes(int32_t m, int64_t bound, uint32_t flags) {
          6 * align_up(size_t(m) * 4, 256) + 4096;
 }
 
+size_t closure_control_words(int32_t m) {
+  return prog_words((size_t(m) + kB - 1) / kB) + size_t(m) + 1;
+}
+
 bool closure_small(int32_t m, int64_t bound, uint32_t flags) {
   return m <= (use_s16(bound, flags) ? kClusterMaxWarm<int16_t> : kClusterMaxWarm<int32_t>);
 }
 
 int closure_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t bound, int32_t* p, uint32_t flags,
                    void* ws, cudaStream_t stream, int32_t* beaten_by, int32_t* hint,
-                   const int32_t* hint_valid, bool side, int32_t* winners, int32_t* order) {
+                   const int32_t* hint_valid, bool side, int32_t* winners, int32_t* order, uint32_t* control) {
   const bool margin = (flags & SCHULZE_F_MARGIN) != 0;
   if (use_s16(bound, flags))
     return run_closure<int16_t>(ctx, d, m, bound, p, ws, stream, beaten_by, hint, hint_valid, margin, side, winners,
-                                order);
+                                order, control);
   return run_closure<int32_t>(ctx, d, m, bound, p, ws, stream, beaten_by, hint, hint_valid, margin, side, winners,
-                                order);
+                                order, control);
 }
 
 // ------------------------------------------------- allocation-free variant

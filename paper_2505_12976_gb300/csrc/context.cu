@@ -53,6 +53,28 @@ static int set_device(schulze_ctx* ctx) {
 
 using namespace schulze;
 
+// The kernels of schulze_run: tally, closure, winners and ranking. ws: the
+// stages' scratch; control: closure_control_words(m) words and xws: m words
+// outside it, zeroed in the tally's first launch with bb (one zeroing launch
+// instead of three); hint, hint_valid: outside ws too.
+static int run_path(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, int32_t k, int32_t* d, int32_t* p,
+                    int32_t* winners, int32_t* order, int32_t* bb, uint32_t flags, void* ws, uint32_t* control,
+                    int32_t* hint, int32_t* hint_valid, void* xws, cudaStream_t stream) {
+  if (closure_small(m, n, flags)) {  // one launch for the closure, the winners and the ranking
+    if (int rc = tally_launch(ctx, ranks, n, m, k, d, flags, ws, stream)) return rc;
+    return closure_launch(ctx, d, m, n, p, flags, ws, stream, bb, nullptr, nullptr, false, winners, order);
+  }
+  if (!tally_gives_hint(n, m, k, flags)) hint = hint_valid = nullptr;
+  ZeroSpans more;
+  more.add(control, int64_t(closure_control_words(m)));
+  more.add(bb, m);
+  if (order) more.add(xws, m);
+  if (int rc = tally_launch(ctx, ranks, n, m, k, d, flags, ws, stream, hint, hint_valid, &more)) return rc;
+  int rc = closure_launch(ctx, d, m, n, p, flags, ws, stream, bb, hint, hint_valid, true, nullptr, nullptr, control);
+  if (!rc && (winners || order)) rc = extract_from_beaten_by(ctx, bb, m, winners, order, xws, stream, true);
+  return rc;
+}
+
 // Makes ctx->host_exec the graph of schulze_run_host's kernels for `key`,
 // capturing enqueue(cap_stream) when the key changed; false when the capture
 // failed and the call must run eagerly. The graph works on the workspace
@@ -191,11 +213,12 @@ int schulze_reserve(schulze_ctx* ctx, int32_t m_max, int64_t n_max, int32_t k_ma
   // schulze_run keeps the tally's warm flags (with their relabeling) and
   // beaten_by after the stages, then the extraction's scratch
   const size_t mv = align_up(size_t(m_max) * 4, 256), hv = align_up(hint_words(m_max) * 4, 256);
-  size_t need = align_up(std::max(t, c), 256) + hv + mv + 256 + x;
+  const size_t cw = align_up(closure_control_words(m_max) * 4, 256);
+  size_t need = align_up(std::max(t, c), 256) + cw + hv + mv + 256 + x;
   // schulze_run_host keeps ranks, d, p, three vectors and the hint words
   // next to the stages
   size_t host_path = align_up(size_t(n_max) * size_t(k_max) * 4, 256) +
-                     2 * align_up(size_t(m_max) * size_t(m_max) * 4, 256) + 3 * mv + hv + 512 + need + 4096;
+                     2 * align_up(size_t(m_max) * size_t(m_max) * 4, 256) + 3 * mv + hv + cw + 512 + need + 4096;
   need = std::max(need, host_path);
   int rc = ensure_workspace(ctx, need, nullptr);
   if (rc) return rc;
@@ -325,20 +348,18 @@ int schulze_run(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, in
   const size_t mv = align_up(size_t(m) * 4, 256), hv = align_up(hint_words(m) * 4, 256);
   const size_t keep = std::max(align_up(tally_workspace_bytes(n, m, k, flags), 256),
                                align_up(closure_workspace_bytes(m, n, flags), 256));
-  const size_t xoff = keep + hv + mv + 256;
+  const size_t cv = align_up(closure_control_words(m) * 4, 256);
+  const size_t xoff = keep + cv + hv + mv + 256;
   if (int rc = ensure_workspace(ctx, xoff + extract_workspace_bytes(m), stream)) return rc;
-  char* tail = static_cast<char*>(ctx->ws.base) + keep;
+  uint32_t* control = reinterpret_cast<uint32_t*>(static_cast<char*>(ctx->ws.base) + keep);
+  char* tail = static_cast<char*>(ctx->ws.base) + keep + cv;
   int32_t* hint = reinterpret_cast<int32_t*>(tail);
   int32_t* hint_valid = reinterpret_cast<int32_t*>(tail + hv);
   int32_t* bb = beaten_by ? beaten_by : reinterpret_cast<int32_t*>(tail + hv + 256);
   void* xws = static_cast<char*>(ctx->ws.base) + xoff;
-  const bool small = closure_small(m, n, flags);  // one launch for the closure, the winners and the ranking
-  if (small) hint = hint_valid = nullptr;         // (which needs no warm flags)
-  if (int rc = tally_launch(ctx, ranks, n, m, k, d, flags, ctx->ws.base, stream, hint, hint_valid)) return rc;
   const bool ext = winners || order || beaten_by;
-  int rc = closure_launch(ctx, d, m, n, p, flags, ctx->ws.base, stream, ext ? bb : nullptr, hint, hint_valid, true,
-                          winners, order);
-  if (!rc && !small && (winners || order)) rc = extract_from_beaten_by(ctx, bb, m, winners, order, xws, stream);
+  int rc = run_path(ctx, ranks, n, m, k, d, p, winners, order, ext ? bb : nullptr, flags, ctx->ws.base, control, hint,
+                    hint_valid, xws, stream);
   const int rj = side_join(ctx, stream);  // also after an error: a capture must end with the fork joined
   return rc ? rc : rj;
 }
@@ -356,7 +377,7 @@ int schulze_run_host(schulze_ctx* ctx, const int32_t* ranks_host, int64_t n, int
   size_t stage = align_up(std::max(tally_workspace_bytes(n, m, k, flags), closure_workspace_bytes(m, n, flags)), 256) +
                  extract_workspace_bytes(m);
   size_t head = align_up(rbytes, 256) + 2 * align_up(mm, 256) + 3 * align_up(size_t(m) * 4, 256) +
-                align_up(hint_words(m) * 4, 256) + 512;
+                align_up(hint_words(m) * 4, 256) + align_up(closure_control_words(m) * 4, 256) + 512;
   if (int rc = ensure_workspace(ctx, head + stage + 4096, stream)) return rc;
   Carver cv(ctx->ws.base);
   int32_t* ranks = cv.take<int32_t>(size_t(n) * size_t(k));
@@ -367,19 +388,15 @@ int schulze_run_host(schulze_ctx* ctx, const int32_t* ranks_host, int64_t n, int
   int32_t* bb = cv.take<int32_t>(size_t(m));
   int32_t* hint = cv.take<int32_t>(hint_words(m));
   int32_t* hint_valid = cv.take<int32_t>(1);
+  uint32_t* control = cv.take<uint32_t>(closure_control_words(m));
   void* rest = cv.take<char>(0);
   void* xrest = static_cast<char*>(rest) +
                 align_up(std::max(tally_workspace_bytes(n, m, k, flags), closure_workspace_bytes(m, n, flags)), 256);
   // the kernels, on stream s
   auto enqueue = [&](cudaStream_t s) -> int {
-    const bool small = closure_small(m, n, flags);
-    if (int rc = tally_launch(ctx, ranks, n, m, k, d, flags, rest, s, small ? nullptr : hint,
-                              small ? nullptr : hint_valid))
-      return rc;
     const bool ext = winners_host || order_host;
-    int rc = closure_launch(ctx, d, m, n, p, flags, rest, s, ext ? bb : nullptr, hint, hint_valid, true,
-                            winners_host ? win : nullptr, order_host ? ord : nullptr);
-    if (!rc && ext && !small) rc = extract_from_beaten_by(ctx, bb, m, win, ord, xrest, s);
+    int rc = run_path(ctx, ranks, n, m, k, d, p, winners_host ? win : nullptr, order_host ? ord : nullptr,
+                      ext ? bb : nullptr, flags, rest, control, hint, hint_valid, xrest, s);
     const int rj = side_join(ctx, s);
     return rc ? rc : rj;
   };

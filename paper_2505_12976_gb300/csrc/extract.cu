@@ -17,6 +17,7 @@ constexpr int kRankChunk = 256;  // keys per shared-memory chunk of the rank pas
 // both blocks is counted by four threads and added with one atomic per row.
 __global__ void __launch_bounds__(256) beaten_by_kernel(const int32_t* __restrict__ p, int32_t m,
                                                         int32_t* __restrict__ bb) {
+  pdl_enter();
   const int32_t I = blockIdx.y * kT, J = blockIdx.x * kT;
   if (I > J) return;
   __shared__ int32_t a[kT][kT + 1];  // a[r][c] = p[I + r][J + c]
@@ -86,12 +87,14 @@ __global__ void rank_scatter_kernel(const int32_t* __restrict__ pos, const int32
 
 // winners and ranking from beaten_by; pos is scratch [m]
 int finish(schulze_ctx* ctx, const int32_t* bb, int32_t* pos, int32_t m, int32_t* winners, int32_t* order,
-           cudaStream_t stream) {
+           cudaStream_t stream, bool zeroed = false) {
   const int g = (m + 255) / 256;
   if (order) {
-    ZeroSpans z;
-    z.p[0] = reinterpret_cast<uint32_t*>(pos), z.words[0] = m;
-    if (int rc = zero_async(ctx, z, stream)) return rc;
+    if (!zeroed) {
+      ZeroSpans z;
+      z.add(pos, m);
+      if (int rc = zero_async(ctx, z, stream)) return rc;
+    }
     {
       Launch L(ctx, stream, "extract_rank", double(m) * 8.0);
       launch_pdl(rank_count_kernel, dim3(g, (m + kRankChunk - 1) / kRankChunk), dim3(256), 0, stream, false, bb, m,
@@ -144,17 +147,17 @@ int extract_launch(schulze_ctx* ctx, const int32_t* p, int32_t m, int32_t* winne
   const int32_t nbt = (m + kT - 1) / kT;
   {
     Launch L(ctx, stream, "extract_beaten_by", double(m) * double(m) * 4.0);
-    beaten_by_kernel<<<dim3(nbt, nbt), 256, 0, stream>>>(p, m, bb);
+    launch_pdl(beaten_by_kernel, dim3(nbt, nbt), dim3(256), 0, stream, false, p, m, bb);
   }
   if (int rc = check_launch()) return rc;
   return finish(ctx, bb, pos, m, winners, order, stream);
 }
 
 int extract_from_beaten_by(schulze_ctx* ctx, const int32_t* beaten_by, int32_t m, int32_t* winners, int32_t* order,
-                           void* ws, cudaStream_t stream) {
+                           void* ws, cudaStream_t stream, bool zeroed) {
   Carver cv(ws);
   int32_t* pos = cv.take<int32_t>(size_t(m));
-  return finish(ctx, beaten_by, pos, m, winners, order, stream);
+  return finish(ctx, beaten_by, pos, m, winners, order, stream, zeroed);
 }
 
 int iterated_level(schulze_ctx* ctx, const int32_t* bb, int32_t m, int32_t t, int32_t* level, int32_t* placed,

@@ -176,9 +176,12 @@ size_t tally_positions_workspace_bytes(int64_t n, int32_t m);
 // (old -> new) and the warm count [1], which the tally's plan pass writes so
 // that the closure need not scan them.
 inline size_t hint_words(int32_t m) { return 3 * size_t(m) + 1; }
+// With more (at most three spans, outside ws) the tally zeroes those with its
+// own counters, in one launch where it has one.
+struct ZeroSpans;
 int tally_launch(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, int32_t k, int32_t* d,
                  uint32_t flags, void* ws, cudaStream_t stream, int32_t* hint = nullptr,
-                 int32_t* hint_valid = nullptr);
+                 int32_t* hint_valid = nullptr, const ZeroSpans* more = nullptr);
 // Tally of weak-order ballots given as int32 positions [n, m].
 int tally_positions_launch(schulze_ctx* ctx, const int32_t* pos, int64_t n, int32_t m, int32_t* d, void* ws,
                            cudaStream_t stream);
@@ -196,7 +199,13 @@ int tally_positions_launch(schulze_ctx* ctx, const int32_t* pos, int64_t n, int3
 int closure_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t bound, int32_t* p, uint32_t flags,
                    void* ws, cudaStream_t stream, int32_t* beaten_by = nullptr, int32_t* hint = nullptr,
                    const int32_t* hint_valid = nullptr, bool side = false, int32_t* winners = nullptr,
-                   int32_t* order = nullptr);
+                   int32_t* order = nullptr, uint32_t* control = nullptr);
+// Words of the closure that must start at zero (progress words, tile bounds,
+// row flags): closure_launch zeroes its own, with beaten_by, unless the
+// caller passes such an area (outside ws, zeroed already, as beaten_by is).
+size_t closure_control_words(int32_t m);
+// Whether tally_launch can report the warm candidates (hint).
+bool tally_gives_hint(int64_t n, int32_t m, int32_t k, uint32_t flags);
 // Whether closure_launch takes such an election in one launch, which then
 // also fills winners and order when given (it ignores them otherwise, and
 // needs neither hint nor side stream).
@@ -219,8 +228,9 @@ int winners_propagation_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, bo
 int iterated_level(schulze_ctx* ctx, const int32_t* bb, int32_t m, int32_t t, int32_t* level, int32_t* placed,
                    int32_t* dw, cudaStream_t stream);
 // Winners (beaten_by == 0) and the ranking from a filled beaten_by.
+// With zeroed the first m words of ws are zero already.
 int extract_from_beaten_by(schulze_ctx* ctx, const int32_t* beaten_by, int32_t m, int32_t* winners, int32_t* order,
-                           void* ws, cudaStream_t stream);
+                           void* ws, cudaStream_t stream, bool zeroed = false);
 
 // Lets kernel fn use as much dynamic shared memory as the device has for a
 // CTA (one value for every caller, so that no context lowers it for another).
@@ -278,12 +288,18 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// Zeroes up to four spans of 32-bit words in one kernel launched with
+// Zeroes up to kZeroSpans spans of 32-bit words in one kernel launched with
 // launch_pdl (where a memset would end the programmatic chain); spans with a
 // null pointer or no words are skipped.
+constexpr int kZeroSpans = 6;
 struct ZeroSpans {
-  uint32_t* p[4] = {nullptr, nullptr, nullptr, nullptr};
-  int64_t words[4] = {0, 0, 0, 0};
+  uint32_t* p[kZeroSpans] = {};
+  int64_t words[kZeroSpans] = {};
+  void add(void* ptr, int64_t n) {
+    int q = 0;
+    while (q < kZeroSpans && words[q]) ++q;
+    if (q < kZeroSpans && ptr && n > 0) p[q] = static_cast<uint32_t*>(ptr), words[q] = n;
+  }
 };
 int zero_async(schulze_ctx* ctx, const ZeroSpans& z, cudaStream_t stream);
 

@@ -52,6 +52,7 @@ struct Acc {  // per-candidate accumulators of the features pass
 // The accumulators of the features pass and the rank counters (one launch
 // instead of a kernel and two memsets).
 __global__ void acc_init_kernel(Acc a, int32_t m, int32_t* __restrict__ cnt14, int32_t* __restrict__ cnt15) {
+  pdl_enter();
   for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < m; c += gridDim.x * blockDim.x) {
     cnt14[c] = cnt15[c] = 0;
     a.wins[c] = a.losses[c] = 0;
@@ -163,6 +164,7 @@ constexpr int kFPacked = 0, kFNarrow = 1, kFWide = 2;
 
 template <bool kVec, int kMode>
 __global__ void __launch_bounds__(256, kFMinBlocks) features_pass_kernel(const int32_t* __restrict__ d, int32_t m, Acc a) {
+  pdl_enter();
   using Part = typename std::conditional<kMode == kFWide, unsigned long long, uint32_t>::type;
   extern __shared__ __align__(16) int32_t fsm[];
   // stage b: x = d[i][j] (kFR rows of kFXL), then y = d[j][i] (kFC rows: of
@@ -332,6 +334,7 @@ __global__ void __launch_bounds__(256, kFMinBlocks) features_pass_kernel(const i
 
 // f[c][0..13] from the accumulators; ranks (14, 15) are counted afterwards.
 __global__ void features_finalize_kernel(Acc a, int32_t m, int64_t n, float* __restrict__ feat) {
+  pdl_enter();
   const double nn = double(n > 0 ? n : 1), mm = double(m > 1 ? m - 1 : 1);
   const double inv_m = 1.0 / mm, inv_n = 1.0 / nn, inv_nm = 1.0 / (nn * mm);  // FP64 divides are slow
   for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < m; c += gridDim.x * blockDim.x) {
@@ -370,6 +373,7 @@ __global__ void features_finalize_kernel(Acc a, int32_t m, int64_t n, float* __r
 constexpr int kRankChunk = 1024;
 __global__ void __launch_bounds__(kRankChunk / 2) features_rank_kernel(Acc a, int32_t m, int32_t* __restrict__ cnt14,
                                                                        int32_t* __restrict__ cnt15) {
+  pdl_enter();
   __shared__ unsigned long long ks[kRankChunk];
   const bool by_row = blockIdx.z == 0;
   auto key = [&](int32_t c) -> unsigned long long {
@@ -402,6 +406,7 @@ __global__ void __launch_bounds__(kRankChunk / 2) features_rank_kernel(Acc a, in
 
 __global__ void features_rank_finalize_kernel(const int32_t* __restrict__ cnt14, const int32_t* __restrict__ cnt15,
                                               int32_t m, float* __restrict__ feat) {
+  pdl_enter();
   const double inv_m = 1.0 / double(m > 1 ? m - 1 : 1);
   for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < m; c += gridDim.x * blockDim.x) {
     if (m < 2) continue;
@@ -423,6 +428,7 @@ __global__ void __launch_bounds__(256) mlp_forward_kernel(const float* __restric
                                                           const float* __restrict__ feat, int32_t N,
                                                           float* __restrict__ score, float* __restrict__ h1out,
                                                           float* __restrict__ h2out) {
+  pdl_enter();
   __shared__ __align__(16) float p[kNP + 3];
   // stage the parameters with eight loads in flight per thread (16-byte
   // loads when the caller's array is 16-byte aligned)
@@ -516,6 +522,7 @@ __global__ void __launch_bounds__(256) mlp_loss_kernel(const float* __restrict__
                                                        const int32_t* __restrict__ label,
                                                        const int32_t* __restrict__ seg_off, int32_t nseg,
                                                        float* __restrict__ ds, float* __restrict__ seg_loss) {
+  pdl_enter();
   __shared__ float red[256];
   __shared__ int32_t redi[256];
   const int32_t e = blockIdx.x;
@@ -588,6 +595,7 @@ __global__ void __launch_bounds__(256) mlp_backward_kernel(const float* __restri
                                                            const float* __restrict__ h1g, const float* __restrict__ h2g,
                                                            const float* __restrict__ ds, int32_t N,
                                                            float* __restrict__ partial) {
+  pdl_enter();
   extern __shared__ __align__(16) unsigned char bw_raw[];
   BackwardSmem& S = *reinterpret_cast<BackwardSmem*>(bw_raw);
   const int32_t c0 = blockIdx.x * kChunk;
@@ -702,6 +710,7 @@ constexpr int kRedSegs = 16;
 __global__ void __launch_bounds__(32 * kRedSegs) mlp_reduce_kernel(const float* __restrict__ partial, int32_t nchunks,
                                                                    const float* __restrict__ seg_loss, int32_t nseg,
                                                                    float* __restrict__ grad, float* __restrict__ loss) {
+  pdl_enter();
   __shared__ float part[kRedSegs][32];
   const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
   const int t = blockIdx.x * 32 + lane;
@@ -734,6 +743,7 @@ __global__ void __launch_bounds__(32 * kRedSegs) mlp_reduce_kernel(const float* 
 // Adam (Kingma and Ba, 2015), 1-based step.
 __global__ void adam_kernel(float* __restrict__ theta, float* __restrict__ m1, float* __restrict__ m2,
                             const float* __restrict__ grad, int64_t step, float lr, float b1, float b2, float eps) {
+  pdl_enter();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= kNP) return;
   const float g = grad[t];
@@ -819,6 +829,7 @@ __device__ void topk_body(const float* __restrict__ score, int32_t m, int32_t to
 
 // Copeland score wins - losses as a non-learned proposer.
 __global__ void copeland_score_kernel(Acc a, int32_t m, float* __restrict__ score) {
+  pdl_enter();
   for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < m; c += gridDim.x * blockDim.x)
     score[c] = float(a.wins[c] - a.losses[c]);
 }
@@ -858,6 +869,7 @@ __device__ void warm_list_body(const int32_t* __restrict__ wins, int32_t m, int3
 __global__ void __launch_bounds__(1024) warm_list_kernel(const int32_t* __restrict__ wins, int32_t m,
                                                          int32_t* __restrict__ warm, int32_t* __restrict__ slot,
                                                          int32_t* __restrict__ nwarm) {
+  pdl_enter();
   warm_list_body(wins, m, warm, slot, nwarm);
 }
 
@@ -868,6 +880,7 @@ __global__ void __launch_bounds__(1024) propose_kernel(const float* __restrict__
                                                        int32_t* __restrict__ out, const int32_t* __restrict__ wins,
                                                        int32_t* __restrict__ warm, int32_t* __restrict__ slot,
                                                        int32_t* __restrict__ nwarm) {
+  pdl_enter();
   if (blockIdx.x == 0)
     topk_body(score, m, top, out);
   else
@@ -877,6 +890,7 @@ __global__ void __launch_bounds__(1024) propose_kernel(const float* __restrict__
 // Ww[a][b] = w(warm[a], warm[b]) and Wt[b][a] = the same (winning votes).
 __global__ void warm_pack_kernel(const int32_t* __restrict__ d, int32_t m, const int32_t* __restrict__ warm,
                                  const int32_t* __restrict__ nwarm, int32_t* __restrict__ Ww, int32_t* __restrict__ Wt) {
+  pdl_enter();
   const int32_t nw = *nwarm;
   if (nw > kCertifyMaxWarm) return;
   const int64_t total = int64_t(nw) * nw;
@@ -940,6 +954,7 @@ __global__ void __launch_bounds__(1024) certify_kernel(const int32_t* __restrict
                                                        const int32_t* __restrict__ cand, int32_t ncand,
                                                        int32_t* __restrict__ fwd, int32_t* __restrict__ bwd,
                                                        int32_t* __restrict__ winners, int32_t* __restrict__ res) {
+  pdl_enter();
   __shared__ int32_t s_ok, s_ties[kMaxTies], s_nties, s_overflow;
   const int32_t nw = *nwarm_p;
   for (int32_t c = threadIdx.x; c < m; c += blockDim.x) winners[c] = 0;
@@ -1057,7 +1072,7 @@ int features_into(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t n, floa
   const int g = std::max(1, std::min((m + 255) / 256, 1024));
   {
     Launch L(ctx, stream, "learn_features_init", double(m) * 64.0);
-    acc_init_kernel<<<g, 256, 0, stream>>>(w.acc, m, w.cnt14, w.cnt15);
+    launch_pdl(acc_init_kernel, dim3(g), dim3(256), 0, stream, false, w.acc, m, w.cnt14, w.cnt15);
   }
   {
     Launch L(ctx, stream, "learn_features", double(m) * double(m) * 4.0);
@@ -1071,18 +1086,18 @@ int features_into(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t n, floa
                        : mode == kFNarrow ? features_pass_kernel<false, kFNarrow>
                                           : features_pass_kernel<false, kFWide>);
     raise_smem(ctx, reinterpret_cast<const void*>(kern));
-    kern<<<grid, 256, kFSmem, stream>>>(d, m, w.acc);
+    launch_pdl(kern, dim3(grid), dim3(256), kFSmem, stream, false, d, m, w.acc);
   }
   if (!feat) return check_launch();
   {
     Launch L(ctx, stream, "learn_features_finalize", double(m) * kNF * 4.0);
-    features_finalize_kernel<<<(m + 63) / 64, 64, 0, stream>>>(w.acc, m, n, feat);
+    launch_pdl(features_finalize_kernel, dim3((m + 63) / 64), dim3(64), 0, stream, false, w.acc, m, n, feat);
   }
   {
     Launch L(ctx, stream, "learn_feature_ranks", double(m) * 16.0);
     const unsigned nch = unsigned((m + kRankChunk - 1) / kRankChunk);
-    features_rank_kernel<<<dim3(nch, nch, 2), kRankChunk / 2, 0, stream>>>(w.acc, m, w.cnt14, w.cnt15);
-    features_rank_finalize_kernel<<<(m + 63) / 64, 64, 0, stream>>>(w.cnt14, w.cnt15, m, feat);
+    launch_pdl(features_rank_kernel, dim3(nch, nch, 2), dim3(kRankChunk / 2), 0, stream, false, w.acc, m, w.cnt14, w.cnt15);
+    launch_pdl(features_rank_finalize_kernel, dim3((m + 63) / 64), dim3(64), 0, stream, false, w.cnt14, w.cnt15, m, feat);
   }
   return check_launch();
 }
@@ -1092,17 +1107,17 @@ int certify_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, const int32_t*
                    cudaStream_t stream, bool warm_listed = false) {
   if (!warm_listed) {
     Launch L(ctx, stream, "certify_warm_list", double(m) * 8.0);
-    warm_list_kernel<<<1, 1024, 0, stream>>>(w.acc.wins, m, w.warm, w.slot, w.nwarm);
+    launch_pdl(warm_list_kernel, dim3(1), dim3(1024), 0, stream, false, w.acc.wins, m, w.warm, w.slot, w.nwarm);
   }
   {
     const int64_t cw = std::min<int32_t>(m, kCertifyMaxWarm);
     const int blocks = int(std::max<int64_t>(1, std::min<int64_t>((cw * cw + 255) / 256, 4096)));
     Launch L(ctx, stream, "certify_warm_pack", double(cw) * double(cw) * 16.0);
-    warm_pack_kernel<<<blocks, 256, 0, stream>>>(d, m, w.warm, w.nwarm, w.Ww, w.Wt);
+    launch_pdl(warm_pack_kernel, dim3(blocks), dim3(256), 0, stream, false, d, m, w.warm, w.nwarm, w.Ww, w.Wt);
   }
   {
     Launch L(ctx, stream, "certify_paths", 0.0);
-    certify_kernel<<<1, 1024, 0, stream>>>(w.Ww, w.Wt, w.nwarm, w.warm, w.slot, w.acc.losses, m, cand, ncand, fwd,
+    launch_pdl(certify_kernel, dim3(1), dim3(1024), 0, stream, false, w.Ww, w.Wt, w.nwarm, w.warm, w.slot, w.acc.losses, m, cand, ncand, fwd,
                                            bwd, winners, res);
   }
   return check_launch();
@@ -1131,7 +1146,7 @@ int schulze_mlp_forward(schulze_ctx* ctx, const float* params, const float* feat
   if (N == 0) return SCHULZE_OK;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return SCHULZE_ECUDA;
   Launch L(ctx, stream, "mlp_forward", double(N) * 5248.0 * 2.0);
-  mlp_forward_kernel<<<(N + kMlpThreads - 1) / kMlpThreads, kMlpThreads, 0, stream>>>(params, feat, N, score, nullptr,
+  launch_pdl(mlp_forward_kernel, dim3((N + kMlpThreads - 1) / kMlpThreads), dim3(kMlpThreads), 0, stream, false, params, feat, N, score, nullptr,
                                                                                         nullptr);
   return check_launch();
 }
@@ -1159,21 +1174,21 @@ int schulze_mlp_train_step(schulze_ctx* ctx, float* params, float* adam_m, float
   float* g = grad ? grad : cv.take<float>(kNP);
   {
     Launch L(ctx, stream, "mlp_train_forward", double(N) * 5248.0 * 2.0);
-    mlp_forward_kernel<<<(N + kMlpThreads - 1) / kMlpThreads, kMlpThreads, 0, stream>>>(params, feat, N, score, h1, h2);
+    launch_pdl(mlp_forward_kernel, dim3((N + kMlpThreads - 1) / kMlpThreads), dim3(kMlpThreads), 0, stream, false, params, feat, N, score, h1, h2);
   }
   {
     Launch L(ctx, stream, "mlp_train_loss", double(N) * 8.0);
-    mlp_loss_kernel<<<nseg, 256, 0, stream>>>(score, label, seg_off, nseg, ds, seg_loss);
+    launch_pdl(mlp_loss_kernel, dim3(nseg), dim3(256), 0, stream, false, score, label, seg_off, nseg, ds, seg_loss);
   }
   {
     Launch L(ctx, stream, "mlp_train_backward", double(N) * 5248.0 * 4.0);
     raise_smem(ctx, reinterpret_cast<const void*>(mlp_backward_kernel));
-    mlp_backward_kernel<<<nchunks, 256, sizeof(BackwardSmem), stream>>>(params, feat, h1, h2, ds, N, partial);
-    mlp_reduce_kernel<<<(kNP + 31) / 32, 32 * kRedSegs, 0, stream>>>(partial, nchunks, seg_loss, nseg, g, loss);
+    launch_pdl(mlp_backward_kernel, dim3(nchunks), dim3(256), sizeof(BackwardSmem), stream, false, params, feat, h1, h2, ds, N, partial);
+    launch_pdl(mlp_reduce_kernel, dim3((kNP + 31) / 32), dim3(32 * kRedSegs), 0, stream, false, partial, nchunks, seg_loss, nseg, g, loss);
   }
   {
     Launch L(ctx, stream, "mlp_train_adam", double(kNP) * 16.0);
-    adam_kernel<<<(kNP + 255) / 256, 256, 0, stream>>>(params, adam_m, adam_v, g, step, lr, 0.9f, 0.999f, 1e-8f);
+    launch_pdl(adam_kernel, dim3((kNP + 255) / 256), dim3(256), 0, stream, false, params, adam_m, adam_v, g, step, lr, 0.9f, 0.999f, 1e-8f);
   }
   return check_launch();
 }
@@ -1214,14 +1229,14 @@ int schulze_winners_fast(schulze_ctx* ctx, const int32_t* d, int32_t m, int64_t 
   {
     Launch L(ctx, stream, "proposal_scores", double(m) * 5248.0 * 2.0);
     if (params)
-      mlp_forward_kernel<<<(m + kMlpThreads - 1) / kMlpThreads, kMlpThreads, 0, stream>>>(params, feat, m, w.score,
+      launch_pdl(mlp_forward_kernel, dim3((m + kMlpThreads - 1) / kMlpThreads), dim3(kMlpThreads), 0, stream, false, params, feat, m, w.score,
                                                                                           nullptr, nullptr);
     else
-      copeland_score_kernel<<<std::max(1, std::min((m + 255) / 256, 1024)), 256, 0, stream>>>(w.acc, m, w.score);
+      launch_pdl(copeland_score_kernel, dim3(std::max(1, std::min((m + 255) / 256, 1024))), dim3(256), 0, stream, false, w.acc, m, w.score);
   }
   {
     Launch L(ctx, stream, "proposal_topk", double(m) * 4.0);  // and the warm list
-    propose_kernel<<<2, 1024, 0, stream>>>(w.score, m, std::min(top, m), w.cand, w.acc.wins, w.warm, w.slot,
+    launch_pdl(propose_kernel, dim3(2), dim3(1024), 0, stream, false, w.score, m, std::min(top, m), w.cand, w.acc.wins, w.warm, w.slot,
                                           w.nwarm);
   }
   if (int rc = certify_launch(ctx, d, m, w.cand, std::min(top, m), winners, w.res, w, fwd, bwd, stream, true))

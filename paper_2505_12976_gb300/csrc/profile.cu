@@ -114,20 +114,20 @@ __global__ void __launch_bounds__(256) zero_kernel(ZeroSpans z) {
   pdl_enter();
   const int64_t stride = int64_t(gridDim.x) * blockDim.x;
 #pragma unroll
-  for (int s = 0; s < 4; ++s)
+  for (int s = 0; s < kZeroSpans; ++s)
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < z.words[s]; i += stride) z.p[s][i] = 0u;
 }
 }  // namespace
 
 int zero_async(schulze_ctx* ctx, const ZeroSpans& z, cudaStream_t stream) {
   int64_t most = 0;
-  for (int s = 0; s < 4; ++s)
+  for (int s = 0; s < kZeroSpans; ++s)
     if (z.p[s]) most = std::max(most, z.words[s]);
   if (most == 0) return SCHULZE_OK;
   const int sms = ctx && ctx->sm_count > 0 ? ctx->sm_count : 148;
   const int grid = int(std::max<int64_t>(1, std::min<int64_t>((most + 255) / 256, int64_t(sms) * 4)));
   ZeroSpans zz = z;
-  for (int s = 0; s < 4; ++s)
+  for (int s = 0; s < kZeroSpans; ++s)
     if (!zz.p[s]) zz.words[s] = 0;
   Launch L(ctx, stream, "zero", double(most) * 4.0);
   if (launch_pdl(zero_kernel, dim3(grid), dim3(256), 0, stream, false, zz) != cudaSuccess) {

@@ -73,6 +73,7 @@ __global__ void __launch_bounds__(512) slice_ballots_kernel(const int32_t* __res
                                                             int32_t m, int32_t k, int32_t ldp, int bits,
                                                             uint32_t* __restrict__ planes, int32_t* status,
                                                             int32_t* __restrict__ dzero) {
+  pdl_enter();
   extern __shared__ __align__(16) uint16_t slice_pos[];  // [32][cols]
   zero_counts(dzero, int64_t(m) * m, blockIdx.y * int64_t(gridDim.x) + blockIdx.x, int64_t(gridDim.x) * gridDim.y);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
@@ -127,6 +128,7 @@ __global__ void __launch_bounds__(256) slice_positions_kernel(const int32_t* __r
                                                               int32_t m, int32_t ldp, uint32_t* __restrict__ planes,
                                                               int32_t* status, uint32_t* __restrict__ used,
                                                               int32_t* __restrict__ dzero) {
+  pdl_enter();
   zero_counts(dzero, int64_t(m) * m, blockIdx.y * int64_t(gridDim.x) + blockIdx.x, int64_t(gridDim.x) * gridDim.y);
   const int64_t vb = int64_t(blockIdx.x) * kPlaneVoters;
   const int32_t c = int32_t(blockIdx.y * blockDim.x + threadIdx.x);
@@ -163,6 +165,7 @@ __global__ void __launch_bounds__(128, 5)
     plane_tally_kernel(const uint32_t* __restrict__ planes, int32_t ldp, int32_t groups, int32_t m, int32_t nbt,
                        int32_t gchunk, int upper_only, int add, int bits, const uint32_t* __restrict__ used, int vec,
                        int32_t* __restrict__ d) {
+  pdl_enter();
   extern __shared__ __align__(16) uint32_t plane_smem[];  // [kPlaneStages][bits][2 kPT]: rows, then columns
   int32_t tile = blockIdx.x, bi, bj;
   if (upper_only) {  // enumerate bi <= bj
@@ -248,6 +251,7 @@ __global__ void __launch_bounds__(128, 5)
 // Full rankings: d[j][i] = n - d[i][j]. Fills the strictly lower tiles from
 // the upper ones (tiles of size TILE; the diagonal tiles are complete).
 __global__ void mirror_kernel(int32_t* __restrict__ d, int32_t m, int32_t tile, int64_t n) {
+  pdl_enter();
   __shared__ int32_t s[32][33];
   const int32_t bi = blockIdx.y * 32, bj = blockIdx.x * 32;  // source block (rows bi.., cols bj..), bi < bj tile
   if ((bi / tile) >= (bj / tile)) return;  // only blocks inside strictly upper tiles
@@ -1269,14 +1273,15 @@ int dense_tally(schulze_ctx* ctx, int64_t n, int32_t m, bool full, int bits, con
     const int32_t gchunk = (groups + vsplit - 1) / vsplit;
     if (int rc = build(v0, nv, ldp, bits, planes, v0 == 0 && accumulate ? d : nullptr)) return rc;
     Launch L(ctx, stream, "tally_dense", double(nv) * double(m) * double(m - 1) / (full ? 2.0 : 1.0));
-    plane_tally_kernel<<<dim3(ntiles, (groups + gchunk - 1) / gchunk), 128, smem, stream>>>(
-        planes, ldp, groups, m, nbt, gchunk, full ? 1 : 0, accumulate ? 1 : 0, bits, used, rows_vec16(d, m), d);
+    launch_pdl(plane_tally_kernel, dim3(ntiles, (groups + gchunk - 1) / gchunk), dim3(128), smem, stream, false,
+               static_cast<const uint32_t*>(planes), ldp, groups, m, nbt, gchunk, full ? 1 : 0, accumulate ? 1 : 0, bits,
+               used, rows_vec16(d, m), d);
     if (int rc = check_launch()) return rc;
   }
   if (full && nbt > 1) {
     Launch L(ctx, stream, "tally_mirror", double(m) * double(m) * 4.0);
     dim3 g((m + 31) / 32, (m + 31) / 32), b(32, 8);
-    mirror_kernel<<<g, b, 0, stream>>>(d, m, kPT, n);
+    launch_pdl(mirror_kernel, g, b, 0, stream, false, d, m, kPT, n);
   }
   return check_launch();
 }
@@ -1324,13 +1329,20 @@ size_t tally_workspace_bytes(int64_t n, int32_t m, int32_t k, uint32_t flags) {
          grouped_bytes(grouped_plan(n, m, k, kSmsForSizing)) + 4096;
 }
 
+bool tally_gives_hint(int64_t n, int32_t m, int32_t k, uint32_t flags) {
+  return n > 0 && k > 0 && !choose_dense(n, m, k, flags);
+}
+
 int tally_launch(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, int32_t k, int32_t* d,
-                 uint32_t flags, void* ws, cudaStream_t stream, int32_t* hint, int32_t* hint_valid) {
+                 uint32_t flags, void* ws, cudaStream_t stream, int32_t* hint, int32_t* hint_valid,
+                 const ZeroSpans* more) {
   const size_t mm = size_t(m) * size_t(m) * sizeof(int32_t);
-  const bool sparse_path = n > 0 && k > 0 && !choose_dense(n, m, k, flags);
-  // (the sparse path clears hint_valid with its counters)
-  if (hint && !sparse_path && cudaMemsetAsync(hint_valid, 0, sizeof(int32_t), stream) != cudaSuccess)
-    return SCHULZE_ECUDA;
+  const bool sparse_path = tally_gives_hint(n, m, k, flags);
+  ZeroSpans z;
+  if (more) z = *more;
+  if (hint) z.add(hint_valid, 1);
+  if (!sparse_path && (hint || more))
+    if (int rc = zero_async(ctx, z, stream)) return rc;
   if (n == 0 || k == 0) {
     return cudaMemsetAsync(d, 0, mm, stream) == cudaSuccess ? SCHULZE_OK : SCHULZE_ECUDA;
   }
@@ -1346,8 +1358,8 @@ int tally_launch(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, i
                          raise_smem(ctx, reinterpret_cast<const void*>(slice_ballots_kernel));
                          const dim3 g((nv + kPlaneVoters - 1) / kPlaneVoters, (ldp + kPlaneCols - 1) / kPlaneCols);
                          Launch L(ctx, stream, "tally_positions", double(nv) * (double(k) * 4.0 + double(ldp) * 2.0));
-                         slice_ballots_kernel<<<g, 512, smem, stream>>>(ranks, v0, nv, m, k, ldp, nbits, planes,
-                                                                        ctx->status, dzero);
+                         launch_pdl(slice_ballots_kernel, g, dim3(512), smem, stream, false, ranks, v0, nv, m, k, ldp,
+                                    nbits, planes, ctx->status, dzero);
                          return check_launch();
                        });
   }
@@ -1370,13 +1382,8 @@ int tally_launch(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, i
   uint32_t* agg = cv.take<uint32_t>(size_t((m + kPlanTile - 1) / kPlanTile) * kAggWords);
   int32_t* hacc = cv.take<int32_t>(size_t(gp.hcap) * size_t(gp.hld));
   uint32_t* hdone = cv.take<uint32_t>(size_t(gp.hcap));
-  {
-    ZeroSpans z;
-    z.p[0] = reinterpret_cast<uint32_t*>(cnt), z.words[0] = m;
-    z.p[1] = reinterpret_cast<uint32_t*>(hint_valid), z.words[1] = hint ? 1 : 0;
-    z.p[2] = queue, z.words[2] = 1;
-    if (int rc = zero_async(ctx, z, stream)) return rc;
-  }
+  z.add(cnt, m), z.add(queue, 1);
+  if (int rc = zero_async(ctx, z, stream)) return rc;
   const bool local_hist = m <= kLocalHistMax;
   {
     const int threads = 512;
@@ -1465,8 +1472,8 @@ int tally_positions_launch(schulze_ctx* ctx, const int32_t* pos_in, int64_t n, i
                        if (cudaMemsetAsync(used, 0, sizeof(uint32_t), stream) != cudaSuccess) return SCHULZE_ECUDA;
                        const dim3 g((nv + kPlaneVoters - 1) / kPlaneVoters, (ldp + 255) / 256);
                        Launch L(ctx, stream, "tally_positions_copy", double(nv) * double(m) * 4.0);
-                       slice_positions_kernel<<<g, 256, 0, stream>>>(pos_in, v0, nv, m, ldp, planes, ctx->status, used,
-                                                                     dzero);
+                       launch_pdl(slice_positions_kernel, g, dim3(256), 0, stream, false, pos_in, v0, nv, m, ldp, planes,
+                                  ctx->status, used, dzero);
                        return check_launch();
                      });
 }

@@ -350,8 +350,9 @@ def run_weak(args, world, rank, local):
         t = torch.tensor([ms], dtype=torch.float64, device=dev)
         dist.all_reduce(t, op=dist.ReduceOp.MAX)
         ms = float(t.item())
-    # dense tally: n m (m - 1) position compares, ALU-bound; 16-bit packed
-    # compare + subtract = one instruction per compare and lane pair
+    # dense tally: n m (m - 1) position compares, ALU-bound: on bit planes 32
+    # ballots of a pair cost one logic instruction per position bit, a
+    # population count and an add
     top = max(prof.items(), key=lambda kv: kv[1]["ms"])
     tally = prof.get("tally_dense")
     roof = None
@@ -359,11 +360,13 @@ def run_weak(args, world, rank, local):
         per = tally["ms"] / max(1, tally["launches"])
         cmp_per_launch = float(n) * m * (m - 1) / max(1, tally["launches"] // args.steps)
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
-        peak = sms * 64 * 2 * 2.07e9  # 64 lanes/clk/SM x 2 lanes per packed op; a compare takes vsub + vcmp
+        sec, upd = S.probe_minmax(0, sms * 8, 4096, local)
+        peak = 2 * upd / sec * 32 / (int(pos_h.max()).bit_length() + 2)
         roof = {"bound": "alu", "kernel": "tally_dense", "achieved": cmp_per_launch / (per * 1e-3) / 1e9,
-                "peak": peak / 2 / 1e9, "unit": "Gcompares/s", "frac": cmp_per_launch / (per * 1e-3) / (peak / 2),
+                "peak": peak / 1e9, "unit": "Gcompares/s", "frac": cmp_per_launch / (per * 1e-3) / peak,
                 "traffic": None, "per_launch_ms": per,
-                "peak_source": "152 SMs x 64 int lanes/clk x 2 lanes per 16-bit op x 2.07 GHz / 2 ops per compare"}
+                "peak_source": "integer lane rate of schulze_probe_minmax kind 0 (two instructions per update) measured "
+                               "in this run x 32 ballots per (position bits + 2) instructions"}
     # end to end: host positions (pinned) in, winners and order out, through the same calls
     pos_pin = torch.from_numpy(pos_h).pin_memory()
     win_h = torch.empty(m, dtype=torch.int32).pin_memory()
@@ -604,15 +607,21 @@ def run_batch(args, world, rank, local):
     # roofline of the one batch kernel: its algorithmic work is the tally's
     # position compares (n m (m - 1) / 2 per full-ranking election, n m (m - 1)
     # otherwise) and the closure's m^3 (max, min) updates, each at the rate the
-    # probes measure on this GPU (guard-bit compare; packed 16-bit min/max with
-    # a three-input max, or int32 when an election has more than 32767 ballots)
+    # probes measure on this GPU (bit-plane compares: 32 ballots per position
+    # bits + 2 integer instructions; packed 16-bit min/max with a three-input
+    # max, or int32 when an election has more than 32767 ballots). The closure
+    # skips tile updates that cannot change anything; its count here is
+    # Floyd-Warshall's all the same.
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    sec_c, cmp_c = S.probe_minmax(12, sms * 8, 4096, local)
+    sec_c, upd_c = S.probe_minmax(0, sms * 8, 4096, local)
     s16_batch = bool(np.all(bw.n <= 32767))
     sec_u, upd_u = S.probe_minmax(2 if s16_batch else 3, sms * 8, 4096, local)
-    cmp_peak, upd_peak = cmp_c / sec_c, upd_u / sec_u
     mf, nf, kf = (x.astype(np.float64) for x in (bw.m, bw.n, bw.k))
-    compares = float(np.sum(np.where(kf >= mf - 1, 0.5, 1.0) * nf * mf * (mf - 1)))
+    per_e = np.where(kf >= mf - 1, 0.5, 1.0) * nf * mf * (mf - 1)
+    compares = float(np.sum(per_e))
+    bits = np.ceil(np.log2(np.maximum(np.where(kf < mf, kf + 1, kf), 1)))  # of the largest position
+    cmp_peak = 2 * upd_c / sec_c * 32 * compares / float(np.sum(per_e * (bits + 2)))
+    upd_peak = upd_u / sec_u
     at_peak = compares / cmp_peak + cubes / upd_peak  # seconds of ALU work at the measured rates
     roof = {"bound": "alu", "kernel": "batch_elections (tally compares + closure updates)",
             "achieved": (compares + cubes * cmp_peak / upd_peak) / (ms * 1e-3) / 1e9, "peak": cmp_peak / 1e9,
@@ -620,7 +629,8 @@ def run_batch(args, world, rank, local):
             "frac": at_peak / (ms * 1e-3), "traffic": None,
             "work": {"tally_compares": compares, "closure_updates": cubes,
                      "tally_ms_at_peak": compares / cmp_peak * 1e3, "closure_ms_at_peak": cubes / upd_peak * 1e3},
-            "peak_source": "schulze_probe_minmax kinds 12 (compare) and 2/3 (min/max) measured in this run"}
+            "peak_source": "schulze_probe_minmax kinds 0 (integer lane rate, for the compares) and 2/3 (min/max) "
+                           "measured in this run"}
     sched = plan.bucket_schedule()
     # one launch sequence per election on a sample of the same batch
     sample = list(range(0, E, max(1, E // 256)))[:256]
@@ -1059,14 +1069,15 @@ def main():
         "tally_rows": ("hbm", mm4 + float(n) * k * 4, "d written once, ballots read once"),
         "tally_dense": ("alu", float(n) * m * (m - 1) / 2, "pair compares"),
         "tally_count": ("hbm", float(n) * k * 4, "ballots read once"),
-        "closure_rowflags": ("hbm", mm4, "d read once"),
-        "closure_widen": ("hbm", mm4, "p written once"),
-        "closure_pack": ("hbm", float(nwp) * m * (8 + esz), "warm rows of d and d^T read, W written"),
+        "closure_rowflags": ("hbm", mm4 + float(m) * m * esz, "d read and the weights written once"),
+        "closure_widen": ("hbm", mm4 + float(nwp) * m * esz, "W read and p written once"),
+        "closure_pack": ("hbm", 2.0 * nwp * m * esz, "weights read and W written, warm rows"),
         "closure_cluster": ("alu", float(nw) ** 3, "(max, min) updates of the warm square"),
         "closure_cold": ("alu", float(nw) ** 2 * (m - nw), "(max, min) updates of the cold columns"),
-        "closure_persistent": ("alu", float(nw) ** 3, "(max, min) updates of the warm square, nw^3 (Floyd-Warshall "
-                               "count; executed: 64^3 per tile update, reported beside it)"),
-        "closure_beaten_by": ("hbm", 2.0 * nw * nw * esz, "warm square of W read along rows and columns"),
+        "closure_persistent": ("alu", (executed["tile_updates"] + executed["diag_closures"]) * 64.0 ** 3,
+                               "(max, min) updates executed, 64^3 per tile update (those that cannot change anything "
+                               "are skipped; the Floyd-Warshall count nw^3 is reported beside it)"),
+        "closure_beaten_by": ("hbm", 0.0, "only the tile pairs that their bounds leave open are read"),
         "extract_beaten_by": ("hbm", 2 * mm4, "p and p^T read"),
     }
 
@@ -1091,7 +1102,7 @@ def main():
     ranked = sorted(prof.items(), key=lambda kv: -kv[1]["ms"])
     roof = roofline(*ranked[0]) if ranked else None
     if roof and roof["kernel"] == "closure_persistent":
-        roof["executed_updates_per_launch"] = (executed["tile_updates"] + executed["diag_closures"]) * 64.0 ** 3
+        roof["floyd_warshall_updates_per_launch"] = float(nw) ** 3
     # kernels whose case the device decided against return at once: no work,
     # no roofline
     roof_all = {name: {key: r[key] for key in ("bound", "frac", "achieved", "unit", "per_launch_ms")}

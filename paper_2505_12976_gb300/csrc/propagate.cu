@@ -25,7 +25,7 @@
 // starts at a few unknown candidates touches their rows and columns only, and
 // one in which everything changed reads d once. On m = 18407 (top-200 lists)
 // the two iterations took 6.3 ms with a transposed copy of d and two rows
-// per candidate read in every pass, 1.4 ms in this form.
+// per candidate read in every pass, 1.2 ms in this form.
 #include <algorithm>
 
 #include "internal.cuh"
@@ -57,7 +57,7 @@ __device__ __forceinline__ Key along(Key k, int32_t w) {
 enum Pass : int { kInit = 0, kPropagate = 1, kMarks = 2 };
 struct PassArgs {
   const int32_t* d;
-  int32_t m, margin, vec4;
+  int32_t m, margin;
   int32_t *in, *out;        // kInit: heaviest incoming / outgoing edge (zeroed before)
   const int32_t* flag;      // per block of 64: kPropagate: a key changed; kMarks: asked about
   const Key *f, *b;         // keys
@@ -68,10 +68,17 @@ struct PassArgs {
   int32_t *lose, *scc_lose;  // kMarks
 };
 
-// One pass over the pairs of blocks; thread (r, c) holds d[A+r][B+c..c+3] and
-// d[B+r][A+c..c+3] for four r, their transposed partners are in shared memory.
-template <int kPass>
-__global__ void __launch_bounds__(256) pair_kernel(PassArgs g) {
+// One pass over the pairs of blocks; a thread holds four columns of four rows
+// of d[A..][B..] and of d[B..][A..], their transposed partners are in shared
+// memory. kVec (rows on 16-byte boundaries): the columns are neighbours, one
+// 16-byte load. Else they lie 16 apart, so that each 4-byte load of a
+// half-warp covers 64 neighbouring bytes: with neighbours there too, every
+// sector went through L1 four times (m = 18407, a full round 318 -> 309 us).
+// A round is bound by its compares as much as by d: one 64-bit compare per
+// entry instead of two 309 -> 276 us, four CTAs per SM instead of three (at
+// the price of a few spilled words) 256 us.
+template <int kPass, bool kVec>
+__global__ void __launch_bounds__(256, 4) pair_kernel(PassArgs g) {
   if (kPass == kPropagate && blockIdx.x == 0 && threadIdx.x == 0) *g.changed = 0;
   const int32_t m = g.m, nbt = (m + kPT - 1) / kPT;
   int32_t a = 0;
@@ -97,24 +104,30 @@ __global__ void __launch_bounds__(256) pair_kernel(PassArgs g) {
   __shared__ int32_t t1[kPT][kPT + 1], t2[kPT][kPT + 1];  // t1 = d[A.., B..], t2 = d[B.., A..]
   __shared__ Key sf[2][kPT], sb[2][kPT];                  // keys of A, of B
   const int lane = threadIdx.x & 31;
-  const int rq = threadIdx.x >> 4, c4 = (threadIdx.x & 15) * 4;  // rows rq + 16 q, columns c4 .. c4 + 3
+  constexpr int kCs = kVec ? 1 : 16;
+  const int rq = threadIdx.x >> 4, c0 = (threadIdx.x & 15) * (kVec ? 4 : 1);  // rows rq + 16 q, columns c0 + kCs e
   int32_t x1[4][4], x2[4][4];
   auto load = [&](int32_t R, int32_t C, int32_t (&x)[4][4]) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int32_t i = R + rq + 16 * q, j = C + c4;
-      if (g.vec4) {
+      const int32_t i = R + rq + 16 * q, j = C + c0;
+      if (kVec) {
         int4 v = make_int4(0, 0, 0, 0);
         if (i < m && j < m) v = __ldcs(reinterpret_cast<const int4*>(g.d + int64_t(i) * m + j));
         x[q][0] = v.x, x[q][1] = v.y, x[q][2] = v.z, x[q][3] = v.w;
       } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) x[q][e] = (i < m && j + e < m) ? __ldcs(g.d + int64_t(i) * m + j + e) : 0;
+        for (int e = 0; e < 4; ++e) x[q][e] = (i < m && j + kCs * e < m) ? __ldcs(g.d + int64_t(i) * m + j + kCs * e) : 0;
       }
     }
   };
   load(A, B, x1);
   if (A != B) load(B, A, x2);
+  if (kPass == kInit && threadIdx.x < 2 * kPT) {  // what the candidates have by now (it only grows)
+    const int side = threadIdx.x / kPT, t = threadIdx.x % kPT;
+    const int32_t c = (side ? B : A) + t;
+    sf[side][t] = c < m ? Key(__ldcg(g.in + c)) : 0, sb[side][t] = c < m ? Key(__ldcg(g.out + c)) : 0;
+  }
   if (kPass != kInit && threadIdx.x < 2 * kPT) {
     const int side = threadIdx.x / kPT, t = threadIdx.x % kPT;
     const int32_t c = (side ? B : A) + t;
@@ -124,8 +137,8 @@ __global__ void __launch_bounds__(256) pair_kernel(PassArgs g) {
   for (int q = 0; q < 4; ++q)
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      t1[rq + 16 * q][c4 + e] = x1[q][e];
-      if (A != B) t2[rq + 16 * q][c4 + e] = x2[q][e];
+      t1[rq + 16 * q][c0 + kCs * e] = x1[q][e];
+      if (A != B) t2[rq + 16 * q][c0 + kCs * e] = x2[q][e];
     }
   __syncthreads();
   // targets T + r of tile side ts (their d rows in x), sources S + c (their d rows in `other`)
@@ -133,7 +146,7 @@ __global__ void __launch_bounds__(256) pair_kernel(PassArgs g) {
     Key uf[4], ub[4];  // the keys of this thread's sources
     if (kPass != kInit) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) uf[e] = sf[ss][c4 + e], ub[e] = sb[ss][c4 + e];
+      for (int e = 0; e < 4; ++e) uf[e] = sf[ss][c0 + kCs * e], ub[e] = sb[ss][c0 + kCs * e];
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -143,41 +156,50 @@ __global__ void __launch_bounds__(256) pair_kernel(PassArgs g) {
         int32_t in = 0, out = 0;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const int32_t o = other[c4 + e][r];
+          const int32_t o = other[c0 + kCs * e][r];
           out = max(out, edge(x[q][e], o, g.margin)), in = max(in, edge(o, x[q][e], g.margin));
         }
+        const int32_t had_in = int32_t(sf[ts][r]), had_out = int32_t(sb[ts][r]);
+        // seldom, once the heavy edges were met (m = 18407: 494 -> 320 us for
+        // the pass, which every pair's shuffles and atomics bounded)
+        if (__any_sync(0xFFFFFFFFu, in > had_in || out > had_out)) {
 #pragma unroll
-        for (int o = 8; o; o >>= 1) {
-          in = max(in, __shfl_xor_sync(0xFFFFFFFFu, in, o));
-          out = max(out, __shfl_xor_sync(0xFFFFFFFFu, out, o));
-        }
-        if ((lane & 15) == 0 && c < m) {
-          if (in) atomicMax(&g.in[c], in);
-          if (out) atomicMax(&g.out[c], out);
+          for (int o = 8; o; o >>= 1) {
+            in = max(in, __shfl_xor_sync(0xFFFFFFFFu, in, o));
+            out = max(out, __shfl_xor_sync(0xFFFFFFFFu, out, o));
+          }
+          if ((lane & 15) == 0 && c < m) {
+            if (in > had_in) atomicMax(&g.in[c], in);
+            if (out > had_out) atomicMax(&g.out[c], out);
+          }
         }
       } else if (kPass == kPropagate) {
         const Key mf = sf[ts][r], mb = sb[ts][r];
         // along (u, c) from u's source, against (c, u) from u's target; most
         // of the pass finds nothing better, so that is all that it asks first
+        // (of the two edges between them one at most is there: its side's keys
+        // are picked first, then compared once)
         bool better = false;
-        int32_t wi[4], wo[4];
+        int32_t o[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const int32_t o = other[c4 + e][r];
-          wi[e] = edge(o, x[q][e], g.margin), wo[e] = edge(x[q][e], o, g.margin);
-          better |= (o > x[q][e] && along(uf[e], wi[e]) < mf) || (x[q][e] > o && along(ub[e], wo[e]) < mb);
+          o[e] = other[c0 + kCs * e][r];
+          const bool in = o[e] > x[q][e];
+          const int32_t w = g.margin ? abs(o[e] - x[q][e]) : max(o[e], x[q][e]);
+          better |= o[e] != x[q][e] && along(in ? uf[e] : ub[e], w) < (in ? mf : mb);
         }
         if (__any_sync(0xFFFFFFFFu, better)) {
           Key bf = mf, bb = mb;
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            if (wi[e]) bf = min(bf, along(uf[e], wi[e]));
-            if (wo[e]) bb = min(bb, along(ub[e], wo[e]));
+            const int32_t wi = edge(o[e], x[q][e], g.margin), wo = edge(x[q][e], o[e], g.margin);
+            if (wi) bf = min(bf, along(uf[e], wi));
+            if (wo) bb = min(bb, along(ub[e], wo));
           }
 #pragma unroll
-          for (int o = 8; o; o >>= 1) {
-            bf = min(bf, __shfl_xor_sync(0xFFFFFFFFu, bf, o));
-            bb = min(bb, __shfl_xor_sync(0xFFFFFFFFu, bb, o));
+          for (int h = 8; h; h >>= 1) {
+            bf = min(bf, __shfl_xor_sync(0xFFFFFFFFu, bf, h));
+            bb = min(bb, __shfl_xor_sync(0xFFFFFFFFu, bb, h));
           }
           if ((lane & 15) == 0 && c < m) {
             if (bf < mf) atomicMin(&g.fn[c], bf);
@@ -190,7 +212,7 @@ __global__ void __launch_bounds__(256) pair_kernel(PassArgs g) {
         bool other_scc = false;
 #pragma unroll
         for (int e = 0; e < 4; ++e)
-          other_scc |= other[c4 + e][r] > x[q][e] && (key_id(uf[e]) != ms || key_id(ub[e]) != mt);
+          other_scc |= other[c0 + kCs * e][r] > x[q][e] && (key_id(uf[e]) != ms || key_id(ub[e]) != mt);
         const uint32_t any = __ballot_sync(0xFFFFFFFFu, other_scc) >> (lane & 16) & 0xFFFFu;
         if ((lane & 15) == 0 && any && c < m && g.asked[c]) {
           if (ms == mt) g.scc_lose[ms == kNone ? m : ms] = 1;
@@ -333,14 +355,15 @@ int winners_propagation_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, bo
   const unsigned pairs = unsigned(int64_t(nbt) * (nbt + 1) / 2);
   const int g = std::max(1, std::min((m + 255) / 256, 1024));
   PassArgs pa{};
-  pa.d = d, pa.m = m, pa.margin = margin ? 1 : 0, pa.vec4 = rows_vec16(d, m);
+  pa.d = d, pa.m = m, pa.margin = margin ? 1 : 0;
+  const bool vec = rows_vec16(d, m);
   pa.in = inout, pa.out = inout + m, pa.flag = flag, pa.f = f, pa.b = b, pa.fn = fn, pa.bn = bn, pa.changed = words;
   pa.asked = asked, pa.label = label, pa.lose = lose, pa.scc_lose = scc_lose;
   {
     Launch L(ctx, stream, "propagation_init", double(m) * double(m) * 4.0);
     if (!max_in) {
       if (cudaMemsetAsync(inout, 0, 2 * size_t(m) * 4, stream) != cudaSuccess) return SCHULZE_ECUDA;
-      pair_kernel<kInit><<<pairs, 256, 0, stream>>>(pa);
+      (vec ? pair_kernel<kInit, true> : pair_kernel<kInit, false>)<<<pairs, 256, 0, stream>>>(pa);
     }
     init_status_kernel<<<g, 256, 0, stream>>>(max_in ? max_in : pa.in, max_in ? max_out : pa.out, m, status);
   }
@@ -362,7 +385,7 @@ int winners_propagation_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, bo
       int32_t changed = 0;
       {
         Launch L(ctx, stream, "propagation_round", double(m) * double(m) * 4.0);
-        pair_kernel<kPropagate><<<pairs, 256, 0, stream>>>(pa);
+        (vec ? pair_kernel<kPropagate, true> : pair_kernel<kPropagate, false>)<<<pairs, 256, 0, stream>>>(pa);
         commit_kernel<<<nbt, kPT, 0, stream>>>(m, f, b, fn, bn, flag, words);
       }
       ++rounds;
@@ -374,7 +397,7 @@ int winners_propagation_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, bo
     {
       Launch L(ctx, stream, "propagation_marks", double(m) * double(m) * 4.0);
       label_kernel<<<nbt, kPT, 0, stream>>>(f, b, m, status, lose, asked, flag, label);
-      pair_kernel<kMarks><<<pairs, 256, 0, stream>>>(pa);
+      (vec ? pair_kernel<kMarks, true> : pair_kernel<kMarks, false>)<<<pairs, 256, 0, stream>>>(pa);
     }
     apply_kernel<<<g, 256, 0, stream>>>(f, b, m, lose, scc_lose, status, words + 1);
     int32_t decided = 0;

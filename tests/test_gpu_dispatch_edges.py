@@ -200,3 +200,33 @@ def test_host_call_replays_on_any_buffers(m, n, k):
         S.schulze_run_host(bad, m)
     got, _ = S.schulze_run_host(r, m)
     eq(got, win, "after a refused call")
+
+
+# ------------------------------------ winners when the warm set is too large
+
+@pytest.mark.parametrize("m,warm,answer", [(2049, 2048, (0, 1)), (2049, 2049, (2,)), (6001, 2048, (0, 1)),
+                                           (6001, 2049, (2,)), (6000, 6000, (2,)), (9001, 9001, (2,))])
+def test_winners_fast_around_the_warm_limit(m, warm, answer):
+    """Candidates with an outgoing edge around the certification's 2048, few
+    and many to either side: the features pass may stop once it has seen too
+    many, and the propagation then decides, as it does by itself."""
+    import paper_2505_12976_gb300 as S
+    rs = np.random.Generator(np.random.PCG64(m + warm))
+    s = rs.permutation(m)[:warm]  # the warm ones: near an order, and a cycle at the top
+    d = np.zeros((m, m), np.int32)
+    back = rs.random((warm, warm)) < 1e-4
+    base = np.where(np.arange(warm)[:, None] < np.arange(warm)[None, :], rs.integers(600, 900, (warm, warm)), 100)
+    d[np.ix_(s, s)] = np.where(back, 950, base)
+    d[s[0], s[1]], d[s[1], s[2]], d[s[2], s[0]] = 700, 700, 700
+    d[s[1], s[0]] = d[s[2], s[1]] = d[s[0], s[2]] = 100
+    if warm < m:
+        d[s, [c for c in range(m) if c not in set(s.tolist())][0]] = 500  # the last one has an edge too
+    else:
+        d[s[-1], s[0]], d[s[0], s[-1]] = 400, 300
+    np.fill_diagonal(d, 0)
+    dev = cu(d)
+    assert int(((dev > dev.T).sum(1) > 0).sum()) == warm
+    for params in (None, torch.from_numpy(W.mlp_init(5)).cuda()):
+        got, stats = S.schulze_winners_fast(dev, 1000, params)
+        assert stats[1] in answer, stats
+        eq(host(got), host(S.schulze_winners(S.schulze_strongest_paths(dev, 1000))), f"m={m} warm={warm}")

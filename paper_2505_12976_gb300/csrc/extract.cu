@@ -97,8 +97,16 @@ int finish(schulze_ctx* ctx, const int32_t* bb, int32_t* pos, int32_t m, int32_t
     }
     {
       Launch L(ctx, stream, "extract_rank", double(m) * 8.0);
-      launch_pdl(rank_count_kernel, dim3(g, (m + kRankChunk - 1) / kRankChunk), dim3(256), 0, stream, false, bb, m,
-                 pos);
+      const dim3 grid(g, (m + kRankChunk - 1) / kRankChunk);
+      // A programmatic launch lets the CTAs wait on the SMs for beaten_by. From
+      // about one per SM on they take the room of p's writing on the side
+      // stream (schulze_run, m = 8192, 144 listed: 154 against 147 us; m =
+      // 16384 430 against 410); below, the early launch is worth more (m =
+      // 4096: 84 against 87 us).
+      if (int64_t(grid.x) * grid.y < (ctx ? ctx->sm_count : 0))
+        launch_pdl(rank_count_kernel, grid, dim3(256), 0, stream, false, bb, m, pos);
+      else
+        rank_count_kernel<<<grid, 256, 0, stream>>>(bb, m, pos);
     }
     Launch L(ctx, stream, "extract_order", double(m) * 8.0);
     launch_pdl(rank_scatter_kernel, dim3(g), dim3(256), 0, stream, false, static_cast<const int32_t*>(pos), bb, m,

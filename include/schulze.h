@@ -139,7 +139,8 @@ int schulze_tally_positions(schulze_ctx* ctx, const int32_t* pos, int64_t n, int
  *          it selects the 16-bit packed closure when <= 32767. A d entry
  *          above it, or below 0, is reported as SCHULZE_EDATA.
  *   p      [m, m] int32 device output: p[i][j] = widest-path width from i to
- *          j, 0 if j is unreachable, p[i][i] = 0. May not alias d.
+ *          j, 0 if j is unreachable, p[i][i] = 0. May not alias d. Holds
+ *          the edge weights on the way, so it is valid at the call's end only.
  *   flags  SCHULZE_F_AUTO, SCHULZE_F_FORCE_S32 or SCHULZE_F_FORCE_S16, plus
  *          SCHULZE_F_MARGIN for the paper's margin weights
  *          w[i][j] = d[i][j] - d[j][i] when positive (same edges).

@@ -1280,8 +1280,7 @@ __global__ void __launch_bounds__(512) wextract_kernel(const E* __restrict__ W, 
           bb[perm[J * kB + threadIdx.x]] = *ucount;
         continue;
       }
-      if (threadIdx.x < kB) cnt[threadIdx.x] = 0;
-      if (g == 0) {
+      if (g == 0) {  // warp 0 alone starts every counter, before the barrier
         // all: every row of tile (I, J) with edges beats every column; none:
         // no row beats any (cold columns, whose own rows are zero, need the
         // tile itself to be zero)

@@ -85,6 +85,30 @@ def test_general_path_beaten_by_with_cold_columns(m, odd):
     eq(host(S.schulze_winners(pg)), oracle.winners(p), "winners")
 
 
+@pytest.mark.parametrize("listed,unlisted", [(300, 0), (257, 63), (257, 64), (320, 1), (321, 127), (321, 200),
+                                             (449, 300), (2113, 70)])
+@pytest.mark.parametrize("lanes", [1, 2])
+def test_run_beaten_by_of_large_squares_without_hint(listed, unlisted, lanes):
+    """beaten_by as the closure counts it from its tiles and their bounds: a
+    dense tally of short lists gives no hint, so the unlisted candidates are
+    general cold columns, inside the last warm tile, beyond it, or both;
+    popular and unpopular candidates far apart, so that whole tiles beat whole
+    tiles; more than 32 tile rows at the last size."""
+    import paper_2505_12976_gb300 as S
+    m, n, k = listed + unlisted, min(40 * listed, 30000), 6
+    rs = np.random.Generator(np.random.PCG64(7 * listed + unlisted))
+    ids = rs.permutation(m)[:listed]
+    # ballots around an order of the listed candidates: windows of neighbours, popular ones first
+    start = np.minimum((listed - k) * rs.random(n) ** 1.5, listed - k).astype(np.int64)
+    start[: listed - k + 1] = np.arange(listed - k + 1)  # everyone is on a ballot
+    r = ids[start[:, None] + np.argsort(np.arange(k)[None, :] + rs.gumbel(size=(n, k)), axis=1)].astype(np.int32)
+    d, p, win, order, bb = oracle.schulze(r, m, nthreads=16)
+    out = S.schulze_run(cu(r), m, flags=S.F_TALLY_DENSE | lanes)
+    for key, want in (("d", d), ("p", p), ("beaten_by", bb), ("order", order), ("winners", win)):
+        eq(host(out[key]), want, f"{key} listed={listed} unlisted={unlisted} lanes={lanes}")
+    assert S.context().status() == S.OK
+
+
 # ------------------------------------------------------ blocks of propagation
 
 @pytest.mark.parametrize("m", [1, 2, 31, 32, 33, 63, 64, 65, 127, 128, 129, 200])

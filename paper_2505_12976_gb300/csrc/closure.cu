@@ -83,11 +83,22 @@ using tiles::diag_closure_local;
 
 // Progress word of a tile: rounds applied (12 bits), then the largest entry
 // (rounded up) and the smallest (rounded down) as 26-bit values of
-// 2^shift each, shift chosen so that the bound on the counts fits.
+// 2^shift each.
 constexpr int kBoundBits = 26;
 constexpr uint32_t kBoundMax = (1u << kBoundBits) - 1u;
 
+// The least shift at which the bound on the counts fits even rounded up: a
+// clamped maximum could equal the rounded-down minimum of a tile that an
+// update would still raise (bound 2^27 - 1: shift 2, not 1).
+inline int word_shift(int64_t bound) {
+  const int64_t top = bound < INT32_MAX ? bound : int64_t(INT32_MAX);
+  int shift = 0;
+  while ((top + (int64_t(1) << shift) - 1) >> shift > int64_t(kBoundMax)) ++shift;
+  return shift;
+}
+
 __device__ __forceinline__ uint64_t make_word(uint32_t rounds, Bounds b, int shift) {
+  // (the clamps act on entries above the bound alone, which are reported as SCHULZE_EDATA)
   const uint32_t mx = min((uint32_t(max(b.mx, 0)) + ((1u << shift) - 1u)) >> shift, kBoundMax);
   const uint32_t mn = min(uint32_t(max(b.mn, 0)) >> shift, kBoundMax);
   return (uint64_t(rounds) << (2 * kBoundBits)) | (uint64_t(mx) << kBoundBits) | mn;
@@ -1398,8 +1409,7 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
   int32_t* tmin = tmax + tiles2;
   uint32_t* head = bf.prog + 4 * tiles2;
   uint32_t* abort_flag = head + 1;
-  int shift = 0;
-  while (((bound < INT32_MAX ? bound : int64_t(INT32_MAX)) >> shift) > int64_t(kBoundMax)) ++shift;
+  const int shift = word_shift(bound);
   if (!bf.zeroed) {
     // progress words, tile bounds, queue head and abort flag; row flags; the uniform count
     ZeroSpans z;

@@ -65,3 +65,51 @@ def test_run_relabels_listed_candidates_by_ballots():
     out = S.schulze_run(cu(r), m)
     for key, want in (("d", d), ("p", p), ("winners", win), ("order", order), ("beaten_by", bb)):
         eq(host(out[key]), want, key)
+
+
+def near_top(m, top, seed):
+    """Widths of top - 1 between everyone, and of top along a few heavy
+    chains over several tiles: what the heavy edges add shows only in the last
+    bit below the bound."""
+    rs = np.random.Generator(np.random.PCG64(seed))
+    u = np.arange(m)
+    ahead = (u[None, :] - u[:, None]) % m
+    d = np.where((ahead > 0) & (ahead <= (m - 1) // 2), top - 1, 0)  # the next half of the circle: a tournament
+    for _ in range(4):
+        a = rs.permutation(m)[:9]
+        d[a[:-1], a[1:]], d[a[1:], a[:-1]] = top, 0
+    np.fill_diagonal(d, 0)
+    return d.astype(np.int32)
+
+
+NEAR_TOP = [(1 << 26) - 1, 1 << 26, (1 << 27) - 1, 1 << 27, (1 << 28) - 3, (1 << 30) - 1, (1 << 31) - 1]
+
+
+@pytest.mark.parametrize("top", NEAR_TOP)
+@pytest.mark.parametrize("m", [257, 513])
+def test_closure_bounds_at_the_top_of_the_range(m, top):
+    """Entries in the last few values below a power of two, the largest int32
+    included: the progress word's rounded maximum must not pass for less."""
+    import paper_2505_12976_gb300 as S
+    d = near_top(m, top, m)
+    got = host(S.schulze_strongest_paths(cu(d), top))
+    eq(got, oracle.strongest_paths(d, nthreads=NT), f"m={m} top={top}")
+    if m == 257:  # one pair of heavy edges over three tiles
+        d = np.triu(np.full((m, m), top - 1, np.int64), 1).astype(np.int32)
+        d[0, 70] = d[70, 200] = top
+        got = host(S.schulze_strongest_paths(cu(d), top))
+        assert got[0, 200] == top
+        eq(got, oracle.strongest_paths(d, nthreads=NT), f"three tiles, top={top}")
+    assert S.context().status() == S.OK
+
+
+@pytest.mark.parametrize("top", NEAR_TOP)
+def test_beaten_by_at_the_top_of_the_range(top):
+    """The closure's own beaten_by, which decides whole tiles by the same
+    bounds: the levels of the iterated ranking on widths one apart."""
+    import paper_2505_12976_gb300 as S
+    d = near_top(300, top, 11)
+    want, nlevels = oracle.ranking_iterated(d)
+    got, n = S.schulze_ranking_iterated(cu(d), top)
+    eq(host(got), want, f"levels, top={top}")
+    assert n == nlevels and S.context().status() == S.OK

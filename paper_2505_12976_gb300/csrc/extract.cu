@@ -98,12 +98,13 @@ int finish(schulze_ctx* ctx, const int32_t* bb, int32_t* pos, int32_t m, int32_t
     {
       Launch L(ctx, stream, "extract_rank", double(m) * 8.0);
       const dim3 grid(g, (m + kRankChunk - 1) / kRankChunk);
-      // A programmatic launch lets the CTAs wait on the SMs for beaten_by. From
-      // about one per SM on they take the room of p's writing on the side
-      // stream (schulze_run, m = 8192, 144 listed: 154 against 147 us; m =
-      // 16384 430 against 410); below, the early launch is worth more (m =
-      // 4096: 84 against 87 us).
-      if (int64_t(grid.x) * grid.y < (ctx ? ctx->sm_count : 0))
+      // A programmatic launch lets the CTAs wait on the SMs for beaten_by; when
+      // there are many they take the room of p's writing on the side stream.
+      // schulze_run, top-50 lists, 144 listed, early launch against plain one:
+      // m = 3328 86.4 against 90.2 us, m = 4096 90.6 against 94.5, m = 5632
+      // (3.2 CTAs per SM) 109.3 against 109.7, m = 6144 117.1 against 115.0,
+      // m = 8192 154 against 147 (m = 16384 430 against 410).
+      if (int64_t(grid.x) * grid.y < 3 * (ctx ? ctx->sm_count : 0))
         launch_pdl(rank_count_kernel, grid, dim3(256), 0, stream, false, bb, m, pos);
       else
         rank_count_kernel<<<grid, 256, 0, stream>>>(bb, m, pos);

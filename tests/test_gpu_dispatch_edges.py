@@ -109,6 +109,21 @@ def test_run_beaten_by_of_large_squares_without_hint(listed, unlisted, lanes):
     assert S.context().status() == S.OK
 
 
+@pytest.mark.parametrize("m", [4096, 5376, 5377, 6400])
+def test_run_ranking_on_both_sides_of_its_launch_rule(m):
+    """order, winners and beaten_by against p on the host, with the counting
+    launched early (m up to 5376 on 152 SMs) and plainly, twice in a row on
+    other ballots."""
+    import paper_2505_12976_gb300 as S
+    for seed in (1, 2):
+        out = S.schulze_run(cu(W.mallows(seed, 500, m, 20, phi=0.9)), m)
+        p = host(out["p"])
+        bb = (p.T > p).sum(1).astype(np.int32)
+        eq(host(out["beaten_by"]), bb, f"beaten_by m={m}")
+        eq(host(out["order"]), np.lexsort((np.arange(m), bb)).astype(np.int32), f"order m={m}")
+        eq(host(out["winners"]), (bb == 0).astype(np.int32), f"winners m={m}")
+
+
 # ------------------------------------------------------ blocks of propagation
 
 @pytest.mark.parametrize("m", [1, 2, 31, 32, 33, 63, 64, 65, 127, 128, 129, 200])

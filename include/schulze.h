@@ -248,9 +248,10 @@ int schulze_run(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, in
  * path on workspace memory and copies winners and order (each may be NULL)
  * back to the host. Synchronous on `stream`. Device d and p stay inside the
  * context. Returns SCHULZE_EDATA directly when the ballots are invalid.
- * The kernels between the copies are captured once as a CUDA graph and
- * replayed by later calls of the same sizes and flags, whatever their
- * buffers; page-locked buffers copy fastest.
+ * The kernels between the copies are captured as a CUDA graph at the second
+ * call in a row of the same sizes and flags, and replayed by later ones,
+ * whatever their buffers; other calls launch them one by one. Page-locked
+ * buffers copy fastest.
  */
 int schulze_run_host(schulze_ctx* ctx, const int32_t* ranks_host, int64_t n, int32_t m, int32_t k,
                      int32_t* winners_host, int32_t* order_host, uint32_t flags, schulze_stream_t stream);

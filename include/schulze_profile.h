@@ -37,6 +37,9 @@ int schulze_profile_read(schulze_ctx* ctx, schulze_kernel_stats* out, int max, i
 /* Kernel launches issued by this context since it was created. */
 int64_t schulze_launch_count(const schulze_ctx* ctx);
 
+/* CUDA graphs that schulze_run_host has captured on this context. */
+int64_t schulze_graph_captures(const schulze_ctx* ctx);
+
 /* Work the widest-path closure kernel actually executed on this context
  * since it was created (synchronizes the device): 64 x 64 x 64 tile updates
  * computed (skipped all-zero updates not counted), 64 x 64 diagonal-tile

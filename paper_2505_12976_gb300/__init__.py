@@ -76,6 +76,7 @@ SIGNATURES = [
     ("schulze_profile_enable", _c.c_int, [_vp, _c.c_int]),
     ("schulze_profile_read", _c.c_int, [_vp, _vp, _c.c_int, _c.POINTER(_c.c_int)]),
     ("schulze_launch_count", _i64, [_vp]),
+    ("schulze_graph_captures", _i64, [_vp]),
     ("schulze_closure_counters", _c.c_int, [_vp, _c.POINTER(_i64), _c.POINTER(_i64), _c.POINTER(_i64)]),
     ("schulze_probe_minmax", _c.c_int, [_c.c_int, _c.c_int, _c.c_int, _c.c_int, _c.POINTER(_c.c_double),
                                         _c.POINTER(_c.c_double)]),
@@ -153,6 +154,10 @@ class Context:
 
     def launch_count(self) -> int:
         return int(self._lib.schulze_launch_count(self.handle))
+
+    def graph_captures(self) -> int:
+        """CUDA graphs captured by schulze_run_host on this context."""
+        return int(self._lib.schulze_graph_captures(self.handle))
 
     def closure_counters(self) -> dict:
         """Cumulative closure work: tile updates, diagonal closures, queue items."""

@@ -101,9 +101,9 @@ struct schulze_ctx {
   std::vector<schulze::ProfRecord> prof_pending;
   std::vector<schulze::ProfClass> prof_classes;
   std::vector<cudaEvent_t> prof_free_events;
-  // schulze_run_host: the path's kernels on workspace memory captured once as
-  // a CUDA graph on cap_stream and replayed while the sizes, the flags and the
-  // workspace stay the same
+  // schulze_run_host: the path's kernels on workspace memory captured as a
+  // CUDA graph on cap_stream when sizes, flags and workspace are those of the
+  // call before, and replayed for calls that share them
   cudaStream_t cap_stream = nullptr;
   // schulze_run / schulze_run_host: the closure writes p on side_stream
   // (forked from the call's stream with side_fork) while the winners and
@@ -124,7 +124,8 @@ struct schulze_ctx {
       return ws == o.ws && n == o.n && m == o.m && k == o.k && flags == o.flags && winners == o.winners &&
              order == o.order;
     }
-  } host_key;
+  } host_key, host_last;  // of host_exec, of the latest call
+  int64_t host_captures = 0;
 };
 
 namespace schulze {

@@ -309,6 +309,8 @@ int schulze_profile_read(schulze_ctx* ctx, schulze_kernel_stats* out, int max, i
 
 int64_t schulze_launch_count(const schulze_ctx* ctx) { return ctx ? ctx->launches : -1; }
 
+int64_t schulze_graph_captures(const schulze_ctx* ctx) { return ctx ? ctx->host_captures : -1; }
+
 int schulze_closure_counters(schulze_ctx* ctx, int64_t* tile_updates, int64_t* diag_closures, int64_t* items) {
   if (!ctx || !tile_updates || !diag_closures || !items) return SCHULZE_EINVAL;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return SCHULZE_ECUDA;

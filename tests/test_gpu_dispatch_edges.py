@@ -241,6 +241,27 @@ def test_host_call_replays_on_any_buffers(m, n, k):
     eq(got, win, "after a refused call")
 
 
+def test_host_call_captures_a_size_that_comes_back():
+    """A graph is made at the second call in a row of one size, never for
+    sizes that take turns; the one at hand serves its size in between. Every
+    call answers for its own ballots."""
+    import paper_2505_12976_gb300 as S
+    ctx, m, k = S.context(), 391, 30
+    ballots = {n: W.impartial(n, n, m, k) for n in (901, 902, 903)}
+    want = {n: oracle.schulze(r, m, 8) for n, r in ballots.items()}
+
+    def call(n, flags=0):
+        before = ctx.graph_captures()
+        win, order = S.schulze_run_host(ballots[n], m, flags=flags)
+        eq(win, want[n][2], f"winners n={n}")
+        eq(order, want[n][3], f"order n={n}")
+        return ctx.graph_captures() - before
+
+    call(903, flags=1), call(903, flags=1)  # workspace grown, another graph at hand
+    got = [call(n) for n in (901, 902, 901, 902, 903, 903, 901, 903, 902, 902, 902)]
+    assert got == [0, 0, 0, 0, 0, 1, 0, 0, 0, 1, 0]
+
+
 # ------------------------------------ winners when the warm set is too large
 
 @pytest.mark.parametrize("m,warm,answer", [(2049, 2048, (0, 1)), (2049, 2049, (2,)), (6001, 2048, (0, 1)),

@@ -34,7 +34,9 @@ int schulze_profile_enable(schulze_ctx* ctx, int enable);
  * their number to *count. Statistics keep accumulating until re-enabled. */
 int schulze_profile_read(schulze_ctx* ctx, schulze_kernel_stats* out, int max, int* count);
 
-/* Kernel launches issued by this context since it was created. */
+/* Kernel launches issued by this context since it was created, those in the
+ * graphs that schulze_run_host replays included. (While profiling is enabled
+ * that call launches its kernels one by one.) */
 int64_t schulze_launch_count(const schulze_ctx* ctx);
 
 /* CUDA graphs that schulze_run_host has captured on this context. */

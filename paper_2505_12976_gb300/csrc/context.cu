@@ -89,7 +89,11 @@ static bool host_graph(schulze_ctx* ctx, const schulze_ctx::HostKey& key, Enqueu
   if (!ctx->cap_stream) return false;
   const bool again = ctx->host_last == key;
   ctx->host_last = key;
-  if (ctx->host_exec && ctx->host_key == key) return true;
+  if (ctx->profiling) return false;  // events around every launch
+  if (ctx->host_exec && ctx->host_key == key) {
+    ctx->launches += ctx->host_launches;
+    return true;
+  }
   if (!again) return false;
   if (ctx->host_exec) {
     cudaGraphExecDestroy(ctx->host_exec);
@@ -100,6 +104,7 @@ static bool host_graph(schulze_ctx* ctx, const schulze_ctx::HostKey& key, Enqueu
     cudaGetLastError();
     return false;
   }
+  const int64_t before = ctx->launches;
   const int rc = enqueue(ctx->cap_stream);
   cudaGraph_t g = nullptr;
   const cudaError_t ec = cudaStreamEndCapture(ctx->cap_stream, &g);
@@ -113,6 +118,7 @@ static bool host_graph(schulze_ctx* ctx, const schulze_ctx::HostKey& key, Enqueu
   }
   ctx->host_exec = exec;
   ctx->host_key = key;
+  ctx->host_launches = ctx->launches - before;
   ctx->host_captures += 1;
   return true;
 }

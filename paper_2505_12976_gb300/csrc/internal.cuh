@@ -125,7 +125,7 @@ struct schulze_ctx {
              order == o.order;
     }
   } host_key, host_last;  // of host_exec, of the latest call
-  int64_t host_captures = 0;
+  int64_t host_captures = 0, host_launches = 0;  // graphs made; launches in host_exec
 };
 
 namespace schulze {

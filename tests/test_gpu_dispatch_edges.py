@@ -262,6 +262,30 @@ def test_host_call_captures_a_size_that_comes_back():
     assert got == [0, 0, 0, 0, 0, 1, 0, 0, 0, 1, 0]
 
 
+@pytest.mark.parametrize("pinned", [False, True])
+def test_host_call_counts_and_times_its_launches(pinned):
+    """Launch counts and kernel times of the host call do not depend on
+    whether a graph serves it."""
+    import paper_2505_12976_gb300 as S
+    ctx, m, n, k = S.context(), 333, 800, 25
+    src = torch.from_numpy(W.impartial(5, n, m, k).copy())
+    if pinned:
+        src = src.pin_memory()
+    counts = []
+    for _ in range(4):
+        before = ctx.launch_count()
+        S.schulze_run_host(src, m)
+        counts.append(ctx.launch_count() - before)
+    assert counts[0] > 0 and counts == [counts[0]] * 4
+    ctx.profile(True)
+    for _ in range(3):
+        S.schulze_run_host(src, m)
+    seen = ctx.profile_read()
+    ctx.profile(False)
+    assert sum(v["launches"] for v in seen.values()) == 3 * counts[0], seen
+    assert seen["closure_persistent"]["launches"] == 3 and seen["closure_persistent"]["ms"] > 0
+
+
 # ------------------------------------ winners when the warm set is too large
 
 @pytest.mark.parametrize("m,warm,answer", [(2049, 2048, (0, 1)), (2049, 2049, (2,)), (6001, 2048, (0, 1)),

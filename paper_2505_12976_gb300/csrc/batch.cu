@@ -47,6 +47,9 @@ inline int bucket_of(int32_t m) {
   while (b + 1 < kBuckets && m > kBucketMax[b]) ++b;
   return b;
 }
+// In the autotuner's cache keys: changed with the kernel, so that choices timed
+// on an earlier one (packed compares had no such word) are timed again.
+constexpr const char* kTuneKernel = "planes1";
 constexpr int kChunkChoices[4] = {8, 16, 32, 64};
 constexpr int kGptChoices[3] = {1, 2, 4};
 // ballot ids a thread holds for the next step (16: the kernel then fits 128
@@ -660,11 +663,12 @@ double job_cost(const Job& j) {
 }
 
 // Whether `chunk` ballots of an election with m candidates can be staged:
-// the position rows fit the shared memory, and a thread holds at most
-// kPrefetch ids of a step (chunk * m <= kBT * kPrefetch, as k <= m).
+// the position rows (16-bit, at least kPlaneVoters of them) fit the shared
+// memory, and a thread holds at most kPrefetch ids of a step (chunk * m <=
+// kBT * kPrefetch, as k <= m).
 bool chunk_fits(int32_t m, int32_t chunk) {
-  const size_t mpad = align_up(size_t(m), 64);
-  return chunk >= 1 && chunk <= kBT && size_t(chunk) * mpad * 6 <= kStageBytes &&
+  const size_t mpad = align_up(size_t(m), kTT);
+  return chunk >= 1 && chunk <= kBT && size_t(std::max(chunk, kPlaneVoters)) * mpad * 2 <= kStageBytes &&
          int64_t(chunk) * m <= int64_t(kBT) * kPrefetch;
 }
 
@@ -984,8 +988,9 @@ int schulze_batch_autotune(schulze_batch* b, const int32_t* ranks, const char* c
   AbiRange abi_range("schulze_batch_autotune");
   if (!b || (b->ranks_elems > 0 && !ranks)) return SCHULZE_EINVAL;
   if (cudaSetDevice(b->ctx->device) != cudaSuccess) return SCHULZE_ECUDA;
-  // cache keys: GPU, counter width, then per m-bucket its election count and
-  // mean ballot count (the tally schedule), per batch its totals (the order)
+  // cache keys: GPU, kernel, counter width, then per m-bucket its election
+  // count and mean ballot count (the tally schedule), per batch its totals
+  // (the order)
   cudaDeviceProp prop;
   cudaGetDeviceProperties(&prop, b->ctx->device);
   auto clean = [](char* key) {
@@ -1039,8 +1044,8 @@ int schulze_batch_autotune(schulze_batch* b, const int32_t* ranks, const char* c
     if (sub.empty()) continue;
     // the cached value is chunk * 8 + groups per tile
     char key[400];
-    snprintf(key, sizeof(key), "%.100s|s16=%d|bucket<=%d|chunk_gpt|elections=%zu|mean_n=%lld", prop.name,
-             b->s16 ? 1 : 0, kBucketMax[q], sub.size(), (long long)(nsum / double(sub.size())));
+    snprintf(key, sizeof(key), "%.100s|%s|s16=%d|bucket<=%d|chunk_gpt|elections=%zu|mean_n=%lld", prop.name,
+             kTuneKernel, b->s16 ? 1 : 0, kBucketMax[q], sub.size(), (long long)(nsum / double(sub.size())));
     clean(key);
     int best_v = lookup(key);
     if (best_v < 0 || !chunk_fits(kBucketMax[q], best_v / 8) || !gpt_valid(best_v % 8)) {
@@ -1071,7 +1076,7 @@ int schulze_batch_autotune(schulze_batch* b, const int32_t* ranks, const char* c
   int32_t bo = -1;
   if (rc == SCHULZE_OK) {
     char key[400];
-    snprintf(key, sizeof(key), "%.100s|s16=%d|order|E=%d|R=%lld|M=%lld|mmax=%d", prop.name, b->s16 ? 1 : 0, b->E,
+    snprintf(key, sizeof(key), "%.100s|%s|s16=%d|order|E=%d|R=%lld|M=%lld|mmax=%d", prop.name, kTuneKernel, b->s16 ? 1 : 0, b->E,
              (long long)b->ranks_elems, (long long)b->mat_elems, b->m_max);
     clean(key);
     bo = lookup(key);

@@ -157,6 +157,23 @@ def test_batch_autotune_keeps_results_exact(tmp_path):
     _check(b, [(bw.election(e).ranks, int(bw.m[e])) for e in range(bw.E)], outs)
 
 
+def test_batch_autotune_times_choices_of_an_earlier_kernel_again(tmp_path):
+    """A cache file of the earlier kernel (keys without the kernel's word)
+    does not decide the schedule: every choice is timed and recorded."""
+    bw = W.batch_mixed(E=24, seed=6, m_range=(8, 300), n_range=(50, 400))
+    ranks = torch.from_numpy(bw.ranks).cuda()
+    first, second = str(tmp_path / "first.txt"), str(tmp_path / "second.txt")
+    S.SchulzeBatch(bw.n, bw.m, bw.k).autotune(ranks, first)
+    lines = open(first).read().splitlines()
+    with open(second, "w") as f:
+        f.writelines(ln.replace("|planes1|", "|") + "\n" for ln in lines)
+    earlier = open(second).read().splitlines()
+    assert len(earlier) == len(lines) and all(a.split("|")[1].startswith("s16=") for a in earlier)
+    S.SchulzeBatch(bw.n, bw.m, bw.k).autotune(ranks, second)
+    now = open(second).read().splitlines()
+    assert now[:len(lines)] == earlier and [x.split()[0] for x in now[len(lines):]] == [x.split()[0] for x in lines]
+
+
 def test_batch_every_bucket_schedule_is_exact():
     """Every ballots-per-step size each m-bucket accepts (8 to 64 where the
     position rows fit) and every number of tile groups per tally tile (1, 2,

@@ -662,14 +662,16 @@ double job_cost(const Job& j) {
   return tally + 1.5 * mp * mp * mp;
 }
 
-// Whether `chunk` ballots of an election with m candidates can be staged:
-// the position rows (16-bit, at least kPlaneVoters of them) fit the shared
+// Whether `chunk` ballots of an election with m candidates can be staged: a
+// power of two (the CTA's threads divide evenly over the ballots of a step, and
+// steps fill whole groups of kPlaneVoters rows or the other way round), the
+// position rows (16-bit, at least kPlaneVoters of them) fit the shared
 // memory, and a thread holds at most kPrefetch ids of a step (chunk * m <=
 // kBT * kPrefetch, as k <= m).
 bool chunk_fits(int32_t m, int32_t chunk) {
   const size_t mpad = align_up(size_t(m), kTT);
-  return chunk >= 1 && chunk <= kBT && size_t(std::max(chunk, kPlaneVoters)) * mpad * 2 <= kStageBytes &&
-         int64_t(chunk) * m <= int64_t(kBT) * kPrefetch;
+  return chunk >= 1 && chunk <= kBT && (chunk & (chunk - 1)) == 0 &&
+         size_t(std::max(chunk, kPlaneVoters)) * mpad * 2 <= kStageBytes && int64_t(chunk) * m <= int64_t(kBT) * kPrefetch;
 }
 
 int32_t job_chunk(const schulze_batch* b, int32_t m) {
@@ -946,7 +948,7 @@ int schulze_batch_set_schedule(schulze_batch* b, int32_t tally_policy, int32_t o
 }
 
 int schulze_batch_set_bucket_chunk(schulze_batch* b, int32_t bucket, int32_t chunk) {
-  if (!b || bucket < 0 || bucket >= kBuckets || !chunk_fits(kBucketMax[bucket], chunk) || (chunk & (chunk - 1)))
+  if (!b || bucket < 0 || bucket >= kBuckets || !chunk_fits(kBucketMax[bucket], chunk))
     return SCHULZE_EINVAL;
   if (cudaSetDevice(b->ctx->device) != cudaSuccess) return SCHULZE_ECUDA;
   if (cudaDeviceSynchronize() != cudaSuccess) return SCHULZE_ECUDA;

@@ -174,6 +174,28 @@ def test_batch_autotune_times_choices_of_an_earlier_kernel_again(tmp_path):
     assert now[:len(lines)] == earlier and [x.split()[0] for x in now[len(lines):]] == [x.split()[0] for x in lines]
 
 
+@pytest.mark.parametrize("value", [24 * 8 + 1, 3 * 8 + 2, 100 * 8 + 1, 16 * 8 + 3, 0, 5])
+def test_batch_autotune_ignores_choices_that_cannot_be(tmp_path, value):
+    """A damaged cache entry (ballots per step that are no power of two or do
+    not fit, a number of groups that does not exist) is timed again instead
+    of taken, and the tuned plan stays exact."""
+    bw = W.batch_mixed(E=24, seed=9, m_range=(8, 300), n_range=(50, 400))
+    ranks = torch.from_numpy(bw.ranks).cuda()
+    first, second = str(tmp_path / "first.txt"), str(tmp_path / "second.txt")
+    S.SchulzeBatch(bw.n, bw.m, bw.k).autotune(ranks, first)
+    keys = [ln.split()[0] for ln in open(first) if "chunk_gpt" in ln]
+    with open(second, "w") as f:
+        f.writelines(f"{key} {value}\n" for key in keys)
+    b = S.SchulzeBatch(bw.n, bw.m, bw.k)
+    b.autotune(ranks, second)
+    assert all(ch in (8, 16, 32, 64) for _, ch, _ in b.bucket_schedule())
+    assert [ln.split()[0] for ln in open(second) if "chunk_gpt" in ln] == 2 * keys
+    outs = _outputs(b)
+    b.run(ranks, *outs)
+    torch.cuda.synchronize()
+    _check(b, [(bw.election(e).ranks, int(bw.m[e])) for e in range(bw.E)], outs)
+
+
 def test_batch_every_bucket_schedule_is_exact():
     """Every ballots-per-step size each m-bucket accepts (8 to 64 where the
     position rows fit) and every number of tile groups per tally tile (1, 2,

@@ -291,15 +291,19 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 
 // Zeroes up to kZeroSpans spans of 32-bit words in one kernel launched with
 // launch_pdl (where a memset would end the programmatic chain); spans with a
-// null pointer or no words are skipped.
+// null pointer or no words are skipped. A span that finds no place is not
+// dropped: zero_async then refuses the whole call (SCHULZE_EINVAL).
 constexpr int kZeroSpans = 6;
 struct ZeroSpans {
   uint32_t* p[kZeroSpans] = {};
   int64_t words[kZeroSpans] = {};
+  bool overflow = false;
   void add(void* ptr, int64_t n) {
+    if (!ptr || n <= 0) return;
     int q = 0;
     while (q < kZeroSpans && words[q]) ++q;
-    if (q < kZeroSpans && ptr && n > 0) p[q] = static_cast<uint32_t*>(ptr), words[q] = n;
+    if (q == kZeroSpans) overflow = true;
+    else p[q] = static_cast<uint32_t*>(ptr), words[q] = n;
   }
 };
 int zero_async(schulze_ctx* ctx, const ZeroSpans& z, cudaStream_t stream);

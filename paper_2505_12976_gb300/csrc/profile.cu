@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(256) zero_kernel(ZeroSpans z) {
 }  // namespace
 
 int zero_async(schulze_ctx* ctx, const ZeroSpans& z, cudaStream_t stream) {
+  if (z.overflow) return SCHULZE_EINVAL;
   int64_t most = 0;
   for (int s = 0; s < kZeroSpans; ++s)
     if (z.p[s]) most = std::max(most, z.words[s]);

@@ -94,3 +94,37 @@ def test_product_path_has_no_cpu_fallback():
     for f in glob.glob(os.path.join(pkg, "**", "*.py"), recursive=True):
         src = open(f).read()
         assert "import oracle" not in src and "from oracle" not in src, f
+
+
+ZERO_SPANS_PROBE = r"""
+#include "internal.cuh"
+// spans with nothing to zero take no place; one too many is reported
+int main() {
+  using namespace schulze;
+  uint32_t w[16] = {};
+  ZeroSpans z;
+  z.add(nullptr, 4), z.add(w, 0);
+  for (int q = 0; q < kZeroSpans; ++q) z.add(w + q, 1);
+  for (int q = 0; q < kZeroSpans; ++q)
+    if (z.p[q] != w + q || z.words[q] != 1) return 1;
+  z.add(nullptr, 4), z.add(w, 0);
+  if (z.overflow) return 2;
+  z.add(w + kZeroSpans, 1);
+  if (!z.overflow) return 3;
+  return zero_async(nullptr, z, nullptr) == SCHULZE_EINVAL ? 0 : 4;
+}
+"""
+
+
+def test_zero_spans_refuse_one_too_many(lib, tmp_path):
+    """A span that finds no place makes the zeroing fail instead of being
+    left out (host code: no launch is made)."""
+    import subprocess
+
+    from paper_2505_12976_gb300 import _build
+    src, exe = tmp_path / "spans.cu", tmp_path / "spans"
+    src.write_text(ZERO_SPANS_PROBE)
+    subprocess.run([_build._nvcc(), *_build.ARCH, "-std=c++17", "--expt-relaxed-constexpr",
+                    "-I", os.path.join(ROOT, "include"), "-I", _build.CSRC, str(src),
+                    *sorted(glob.glob(os.path.join(_build.BUILD, "*.o"))), "-o", str(exe)], check=True)
+    assert subprocess.run([str(exe)]).returncode == 0

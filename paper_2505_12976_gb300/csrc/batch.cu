@@ -67,8 +67,8 @@ struct BatchArgs {
   int32_t* order;
   int32_t* beaten_by;
   unsigned char* scratch;
-  size_t slot_bytes;  // per CTA: W slot, a d slot for when the caller passes no d, position planes
-  size_t w_bytes, plane_off;
+  size_t slot_bytes;   // per CTA: position planes (the tally), then W over them (the rest), and
+  size_t plane_bytes;  // behind these bytes a d slot for when the caller passes no d
   int32_t* status;
   // schulze_batch_run_host: arrival marks of the ballot segments (set by the
   // copy stream after each segment's copy; null otherwise) and the bound on
@@ -92,7 +92,7 @@ union BatchSmem {
 constexpr int kTT = 64;  // tally tile: 64 x 64 counters per group, 8 x 4 per thread
 constexpr int kDiagBlocks = 72;  // 8 x 4 blocks of a diagonal tile on or above the diagonal
 constexpr int kPlaneVoters = 32;     // ballots per plane word
-constexpr int kPlaneGroups = 256;    // plane groups counted at a time (bounds the CTA's scratch; counts fit 16 bits)
+constexpr int kPlaneGroups = 256;    // plane groups counted at a time at most (bounds the CTA's scratch; counts fit 16 bits)
 
 __host__ __device__ inline int position_bits(int32_t m, int32_t k) {  // of the largest position (k: unlisted)
   int bits = 0;
@@ -369,17 +369,20 @@ __device__ void count_planes(const Job& jb, const uint32_t* planes, int32_t grou
   }
 }
 
-// The election's d: planes and counts, kPlaneGroups plane groups (8192
-// ballots) at a time.
+// The election's d: planes and counts, as many plane groups at a time as the
+// scratch holds (kPlaneGroups, 8192 ballots, unless the plan had to do with less
+// memory).
 __device__ void tally(const Job& jb, const int32_t* __restrict__ ranks, int32_t* __restrict__ dm, uint32_t* planes,
-                      BatchSmem& sm, int32_t* status) {
+                      size_t plane_bytes, BatchSmem& sm, int32_t* status) {
   const int32_t n = jb.n;
   const int bits = position_bits(jb.m, jb.k);
-  for (int64_t v0 = 0; v0 < n; v0 += kPlaneGroups * kPlaneVoters) {
-    const int32_t groups = int32_t(min(int64_t(kPlaneGroups), (n - v0 + kPlaneVoters - 1) / kPlaneVoters));
+  const size_t group_bytes = size_t(max(bits, 1)) * align_up(size_t(jb.m), kTT) * 4;
+  const int32_t most = int32_t(min(size_t(kPlaneGroups), plane_bytes / group_bytes));  // at least 1: W is larger
+  for (int64_t v0 = 0; v0 < n; v0 += int64_t(most) * kPlaneVoters) {
+    const int32_t groups = int32_t(min(int64_t(most), (n - v0 + kPlaneVoters - 1) / kPlaneVoters));
     make_planes(jb, ranks, v0, groups, bits, planes, sm, status);
     __syncthreads();  // the planes are written
-    count_planes(jb, planes, groups, bits, v0 == 0, v0 + kPlaneGroups * kPlaneVoters >= n, dm, sm);
+    count_planes(jb, planes, groups, bits, v0 == 0, v0 + int64_t(most) * kPlaneVoters >= n, dm, sm);
   }
   __syncthreads();
 }
@@ -570,8 +573,8 @@ __global__ void __launch_bounds__(kBT, 1) batch_kernel(BatchArgs a) {
   __shared__ Shared sh;
   unsigned char* slot = a.scratch + size_t(blockIdx.x) * a.slot_bytes;
   E* W = reinterpret_cast<E*>(slot);
-  int32_t* dslot = reinterpret_cast<int32_t*>(slot + a.w_bytes);
-  uint32_t* planes = reinterpret_cast<uint32_t*>(slot + a.plane_off);
+  uint32_t* planes = reinterpret_cast<uint32_t*>(slot);  // done with before W is packed
+  int32_t* dslot = reinterpret_cast<int32_t*>(slot + a.plane_bytes);
   for (;;) {
     if (threadIdx.x == 0) s_job = int32_t(atomicAdd(a.head, 1u));
     __syncthreads();
@@ -607,7 +610,7 @@ __global__ void __launch_bounds__(kBT, 1) batch_kernel(BatchArgs a) {
       for (int64_t t = threadIdx.x; t < int64_t(m) * m; t += kBT) dm[t] = 0;
       __syncthreads();
     } else {
-      tally(jb, ranks, dm, planes, sm, a.status);
+      tally(jb, ranks, dm, planes, a.plane_bytes, sm, a.status);
     }
     const int32_t mp = int32_t(align_up(size_t(m), tiles::kB));
     relabel(dm, m, sh);
@@ -631,7 +634,7 @@ struct schulze_batch {
   schulze::Job* jobs_dev = nullptr;
   uint32_t* head = nullptr;
   unsigned char* scratch = nullptr;
-  size_t slot_bytes = 0, w_bytes = 0, plane_off = 0;
+  size_t slot_bytes = 0, plane_bytes = 0;
   int grid = 0;
   int32_t tally_policy = 0;  // 0: each m-bucket's ballots per step; 1: eight everywhere
   int32_t order_policy = 0;  // 0 longest first, 1 the caller's order
@@ -720,8 +723,7 @@ int launch_jobs(schulze_batch* b, int32_t njobs, const int32_t* ranks, int32_t* 
   a.d = d, a.p = p, a.winners = winners, a.order = order, a.beaten_by = beaten_by;
   a.scratch = b->scratch;
   a.slot_bytes = b->slot_bytes;
-  a.w_bytes = b->w_bytes;
-  a.plane_off = b->plane_off;
+  a.plane_bytes = b->plane_bytes;
   a.status = b->ctx->status;
   Launch L(b->ctx, stream, "batch_elections", double(njobs));
   if (b->s16)
@@ -783,21 +785,28 @@ int schulze_batch_create(schulze_ctx* ctx, int32_t E, const int32_t* n, const in
   }
   b->grid = int(std::max<int64_t>(1, std::min<int64_t>(int64_t(per_sm) * ctx->sm_count, std::max(E, 1))));
   const size_t mp = align_up(size_t(std::max(b->m_max, 1)), tiles::kB);
-  b->w_bytes = align_up(mp * mp * (b->s16 ? 2 : 4), 256);
-  b->plane_off = b->w_bytes + align_up(size_t(b->m_max) * size_t(b->m_max) * 4, 256);
+  const size_t w_bytes = align_up(mp * mp * (b->s16 ? 2 : 4), 256);
+  const size_t d_bytes = align_up(size_t(b->m_max) * size_t(b->m_max) * 4, 256);
   size_t plane_words = 0;  // of the largest election's plane groups counted at a time
   for (int32_t e = 0; e < E; ++e) {
     const size_t groups = std::min<size_t>(kPlaneGroups, (size_t(n[e]) + kPlaneVoters - 1) / kPlaneVoters);
     if (k[e] > 0) plane_words = std::max(plane_words, groups * position_bits(m[e], k[e]) * align_up(size_t(m[e]), kTT));
   }
-  b->slot_bytes = b->plane_off + align_up(plane_words * 4, 256);
+  // planes over W, with room for every plane group of a pass (m = 1024: 10 MB
+  // a CTA against W's 2 or 4); where that is not to be had, in W's room alone,
+  // in more passes (it holds 5 groups at m = 64 and 51 at m = 1024)
+  auto slots = [&](size_t planes) {
+    b->plane_bytes = std::max(w_bytes, planes);
+    b->slot_bytes = b->plane_bytes + d_bytes;
+    const bool ok = cudaMalloc(&b->scratch, b->slot_bytes * size_t(b->grid)) == cudaSuccess;
+    if (!ok) cudaGetLastError(), b->scratch = nullptr;
+    return ok;
+  };
   if (cudaMalloc(&b->jobs_dev, sizeof(Job) * size_t(std::max(E, 1))) != cudaSuccess ||
-      cudaMalloc(&b->head, 256) != cudaSuccess ||
-      cudaMalloc(&b->scratch, b->slot_bytes * size_t(b->grid)) != cudaSuccess) {
+      cudaMalloc(&b->head, 256) != cudaSuccess || !(slots(align_up(plane_words * 4, 256)) || slots(0))) {
     cudaGetLastError();
     if (b->jobs_dev) cudaFree(b->jobs_dev);
     if (b->head) cudaFree(b->head);
-    if (b->scratch) cudaFree(b->scratch);
     delete b;
     return SCHULZE_ENOMEM;
   }

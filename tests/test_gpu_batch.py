@@ -288,3 +288,28 @@ def test_batch_reports_bad_ballots():
     b = S.SchulzeBatch(n, m, k)
     b.run(torch.from_numpy(flat).cuda(), *_outputs(b))
     assert ctx.status() == S.EDATA
+
+
+def test_batch_plan_with_little_memory_left():
+    """A plan whose position planes find no room of their own counts in more
+    passes over the closure's scratch: 0.91 GB of scratch here, 2.2 GB with
+    planes for 8192 ballots, and 1.4 GB left on the device."""
+    n, m, k = [8200, 8191, 3000] + [40] * 200, [1024, 1000, 130] + [9] * 200, [513, 17, 129] + [4] * 200
+    els = [(W.impartial(70 + e, n[e], m[e], k[e]), m[e]) for e in range(len(n))]
+    flat = torch.from_numpy(np.concatenate([r.reshape(-1) for r, _ in els])).cuda()
+    S.SchulzeBatch([5], [4], [4])  # the kernels loaded before memory gets short
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    b = None
+    hog = None
+    try:
+        hog = torch.empty(torch.cuda.mem_get_info()[0] - 1400 * 2**20, dtype=torch.uint8, device="cuda")
+        b = S.SchulzeBatch(n, m, k)
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    outs = _outputs(b)
+    b.run(flat, *outs)
+    torch.cuda.synchronize()
+    _check(b, els, outs)
+    assert S.context().status() == S.OK

@@ -96,8 +96,11 @@ struct schulze_ctx {
   // kernels allowed the device's largest dynamic shared memory, and
   // occupancies asked for so far: each costs a runtime call of about a
   // microsecond, a dozen of them per election otherwise
-  std::vector<const void*> raised;
-  std::vector<schulze::Residency> residency;
+  // (plain arrays: nothing that can throw on the way out of a C entry; past
+  // their end `raised` is asked for again at every call, `residency` starts over)
+  const void* raised[48] = {};
+  schulze::Residency residency[64] = {};
+  int raised_count = 0, residency_count = 0;
   std::vector<schulze::ProfRecord> prof_pending;
   std::vector<schulze::ProfClass> prof_classes;
   std::vector<cudaEvent_t> prof_free_events;
@@ -237,8 +240,10 @@ int extract_from_beaten_by(schulze_ctx* ctx, const int32_t* beaten_by, int32_t m
 // CTA (one value for every caller, so that no context lowers it for another).
 // Once per context and kernel; ctx may be null (then at every call).
 void raise_smem(schulze_ctx* ctx, const void* fn);
+bool smem_raised(const schulze_ctx* ctx, const void* fn);  // whether this context did so already
 // Resident CTAs per SM of fn, at least 1; remembered in the context.
 int blocks_per_sm(schulze_ctx* ctx, const void* fn, int threads, size_t smem);
+void remember(schulze_ctx* ctx, const Residency& r);
 
 // Brackets one kernel launch: counts it and, when profiling is on, records
 // CUDA events around it on `stream`, filed under `name` with `work` units.

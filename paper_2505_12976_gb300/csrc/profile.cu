@@ -57,10 +57,15 @@ Launch::~Launch() {
   if (rec_ >= 0) cudaEventRecord(ctx_->prof_pending[rec_].stop, stream_);
 }
 
-void raise_smem(schulze_ctx* ctx, const void* fn) {
+bool smem_raised(const schulze_ctx* ctx, const void* fn) {
   if (ctx)
-    for (const void* f : ctx->raised)
-      if (f == fn) return;
+    for (int q = 0; q < ctx->raised_count; ++q)
+      if (ctx->raised[q] == fn) return true;
+  return false;
+}
+
+void raise_smem(schulze_ctx* ctx, const void* fn) {
+  if (smem_raised(ctx, fn)) return;
   int device = 0, optin = 0;
   cudaFuncAttributes fa;
   if (cudaGetDevice(&device) != cudaSuccess ||
@@ -71,22 +76,28 @@ void raise_smem(schulze_ctx* ctx, const void* fn) {
     cudaGetLastError();
     return;  // a launch that needs more than the default reports it
   }
-  if (ctx) ctx->raised.push_back(fn);
+  if (ctx && ctx->raised_count < int(sizeof(ctx->raised) / sizeof(ctx->raised[0])))
+    ctx->raised[ctx->raised_count++] = fn;
+}
+
+void remember(schulze_ctx* ctx, const Residency& r) {
+  constexpr int kMost = int(sizeof(ctx->residency) / sizeof(ctx->residency[0]));
+  if (ctx->residency_count == kMost) ctx->residency_count = 0;  // sizes keep changing: start over
+  ctx->residency[ctx->residency_count++] = r;
 }
 
 int blocks_per_sm(schulze_ctx* ctx, const void* fn, int threads, size_t smem) {
   if (ctx)
-    for (const Residency& r : ctx->residency)
+    for (int q = 0; q < ctx->residency_count; ++q) {
+      const Residency& r = ctx->residency[q];
       if (r.fn == fn && r.threads == threads && r.smem == smem) return r.per_sm;
+    }
   int per_sm = 1;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess || per_sm < 1) {
     cudaGetLastError();
-    per_sm = 1;
+    return 1;  // (not remembered)
   }
-  if (ctx) {
-    if (ctx->residency.size() >= 64) ctx->residency.clear();  // sizes keep changing: start over
-    ctx->residency.push_back(Residency{fn, threads, smem, per_sm});
-  }
+  if (ctx) remember(ctx, Residency{fn, threads, smem, per_sm});
   return per_sm;
 }
 

@@ -1442,9 +1442,7 @@ int tally_launch(schulze_ctx* ctx, const int32_t* ranks, int64_t n, int32_t m, i
     // persistent rows kernel: every CTA resident, rows from the plan's queue
     const size_t smem = align_up(size_t((m + 1) / 2) * 4, 16);
     const void* fn = reinterpret_cast<const void*>(grouped_rows_kernel);
-    bool known = false;
-    for (const void* f : ctx->raised) known = known || f == fn;
-    if (!known)
+    if (!smem_raised(ctx, fn))
       cudaFuncSetAttribute(grouped_rows_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                            int(cudaSharedmemCarveoutMaxShared));
     raise_smem(ctx, fn);

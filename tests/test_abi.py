@@ -96,6 +96,20 @@ def test_product_path_has_no_cpu_fallback():
         assert "import oracle" not in src and "from oracle" not in src, f
 
 
+def run_probe(tmp_path, text):
+    """Compiles host code against the internal header and the library's
+    objects, runs it and returns its exit code."""
+    import subprocess
+
+    from paper_2505_12976_gb300 import _build
+    src, exe = tmp_path / "probe.cu", tmp_path / "probe"
+    src.write_text(text)
+    subprocess.run([_build._nvcc(), *_build.ARCH, "-std=c++17", "--expt-relaxed-constexpr",
+                    "-I", os.path.join(ROOT, "include"), "-I", _build.CSRC, str(src),
+                    *sorted(glob.glob(os.path.join(_build.BUILD, "*.o"))), "-o", str(exe)], check=True)
+    return subprocess.run([str(exe)]).returncode
+
+
 ZERO_SPANS_PROBE = r"""
 #include "internal.cuh"
 // spans with nothing to zero take no place; one too many is reported
@@ -119,12 +133,42 @@ int main() {
 def test_zero_spans_refuse_one_too_many(lib, tmp_path):
     """A span that finds no place makes the zeroing fail instead of being
     left out (host code: no launch is made)."""
-    import subprocess
+    assert run_probe(tmp_path, ZERO_SPANS_PROBE) == 0
 
-    from paper_2505_12976_gb300 import _build
-    src, exe = tmp_path / "spans.cu", tmp_path / "spans"
-    src.write_text(ZERO_SPANS_PROBE)
-    subprocess.run([_build._nvcc(), *_build.ARCH, "-std=c++17", "--expt-relaxed-constexpr",
-                    "-I", os.path.join(ROOT, "include"), "-I", _build.CSRC, str(src),
-                    *sorted(glob.glob(os.path.join(_build.BUILD, "*.o"))), "-o", str(exe)], check=True)
-    assert subprocess.run([str(exe)]).returncode == 0
+
+NO_MEMORY_PROBE = r"""
+#include <stdlib.h>
+
+#include "internal.cuh"
+static bool deny = false;
+void* operator new(size_t n) {
+#ifndef __CUDA_ARCH__
+  if (deny) exit(9);  // an allocation, which could have thrown
+#endif
+  return malloc(n ? n : 1);
+}
+void operator delete(void* p) noexcept { free(p); }
+void operator delete(void* p, size_t) noexcept { free(p); }
+__global__ void some_kernel() {}
+// the launch helpers remember what they asked for without allocating, also
+// past what they can hold
+int main() {
+  using namespace schulze;
+  schulze_ctx* ctx = new schulze_ctx();
+  deny = true;
+  const void* fn = reinterpret_cast<const void*>(some_kernel);
+  for (int q = 0; q < 200; ++q) {
+    raise_smem(ctx, q % 2 ? fn : static_cast<const char*>(fn) + q);
+    if (blocks_per_sm(ctx, fn, 32, size_t(q)) < 1) return 2;
+    remember(ctx, Residency{fn, 32, size_t(q), 3});
+    if (blocks_per_sm(ctx, fn, 32, size_t(q)) != 3) return 3;
+  }
+  return 0;
+}
+"""
+
+
+def test_launch_helpers_do_not_allocate(lib, tmp_path):
+    """No exception can leave a C entry from the launch helpers (host code: no
+    launch is made)."""
+    assert run_probe(tmp_path, NO_MEMORY_PROBE) == 0

@@ -50,8 +50,10 @@
 // closure went from 390 to 8.4 ms at m = 16384 (int32, top-20, 0.7% of the
 // updates left) and from 309 to 9.7 ms at m = 18407 (int16, top-200, 4%); it
 // is now bound by the chain diagonal tile - panel - next diagonal tile of
-// its 256 to 288 rounds (33 us each; 16 us where nothing else runs). Where every update is needed
-// (uniform random d, m = 8192) the tests and bounds cost up to 4%.
+// its 256 to 288 rounds (33 us each; 16 us where nothing else runs). Where
+// every update is needed (uniform random d, int32) the tests and bounds cost
+// 1% at m = 4096 (6.55 -> 6.62 ms without and with them), and larger squares
+// gain from the shared operands of neighbouring tiles (m = 8192: 49.9 -> 48.5).
 //
 // All rounds run in ONE persistent cooperative launch: the CTAs take work
 // items from a global queue in a fixed order in which the next round's
@@ -572,8 +574,7 @@ struct Item {
 // So the chain from one diagonal tile to the next (D, P, D, ...) never waits
 // for R, and D(r+1) runs beside R(r-1). P, L and X come tile by tile, which
 // keeps the chain of the panels short, R in items of at most gr tiles: about
-// two items per CTA and round, or 16 where most tiles need their update (a
-// round then ends with CTAs waiting for its last items). The tests of 32
+// two items per CTA and round. The tests of 32
 // tiles, a lane each, cost one round trip to the progress words instead of 32
 // (a skipped tile by itself would take its CTA about a microsecond); 64 left
 // the items with too much work (m = 18407 top-200: 12.9 ms against 9.7). The
@@ -581,8 +582,17 @@ struct Item {
 // update lie next to each other (m = 16384 top-20: 480 of 65536 in a round),
 // and items of neighbours left some CTAs with most of them (the closure took
 // 28.5 ms, 10.8 ms spread).
+// Where most tiles need their update (run) none of that holds: the tiles of an
+// item are then neighbours along a tile row, which share their operand (i, r),
+// and there are about eight items per CTA and round (fewer tiles, and the tests
+// cost too much; more, and a round ends with CTAs waiting for its last items),
+// at least pairs of tiles from four tiles per CTA on. Uniform random d, int32,
+// spread and one tile per item up to m = 8192 against this: m = 4096 6.69 -> 6.62
+// ms, m = 5000 12.42 -> 11.99, m = 8192 51.7 -> 48.5, m = 12288 167.5 -> 159.6;
+// int16, m = 8192: 27.7 -> 25.6.
 struct Shape {
   int32_t nbr, gr;
+  bool run;
   int32_t P, L;         // items of P(r), L(r), r < nbr - 1
   int32_t X, R;         // items of X(r), R(r), r < nbr - 2
   int32_t P_last, R_pen, R_last;  // P(nbr - 1), R(nbr - 2), R(nbr - 1)
@@ -591,8 +601,9 @@ struct Shape {
 
 __device__ Shape make_shape(int32_t nbr, int32_t grid, bool dense) {  // nbr >= 3
   Shape sh;
-  sh.nbr = nbr;
-  sh.gr = min(kItemTiles, max(1, nbr * nbr / ((dense ? 16 : 2) * grid)));
+  sh.nbr = nbr, sh.run = dense;
+  const int32_t per = nbr * nbr / grid;  // tiles per CTA and round
+  sh.gr = min(kItemTiles, !dense ? max(1, per / 2) : per >= 4 ? max(2, per / 8) : 1);
   const int32_t q = nbr - 2;  // tile indices without r and r + 1
   sh.P = 2 + 2 * q, sh.L = 2 * q, sh.P_last = 2 * (q + 1);
   sh.X = q + (q - 1), sh.R = ((q - 1) * (q - 1) + sh.gr - 1) / sh.gr;
@@ -619,17 +630,19 @@ __device__ Item decode_item(uint32_t t, const Shape& sh) {
     }
   }
   auto one = [](int32_t kind, int32_t r, int32_t i, int32_t j) { return Item{kind, r, kRow, i, j, 0, 1, 0, 0}; };
-  // item a of the `items` that share the n tiles (or n x n) of a range
-  auto part = [](int32_t kind, int32_t r, int32_t shape, int32_t fix, int32_t a, int32_t items, int32_t n, int32_t skip) {
-    const int32_t range = shape == kGrid ? n * n : n;
-    return Item{kind, r, shape, fix, a, items, (range - a + items - 1) / items, skip, n};
+  // item a of a tile row's or column's; item a of the `items` of a grid
+  auto side = [](int32_t kind, int32_t r, int32_t shape, int32_t fix, int32_t a, int32_t skip) {
+    return Item{kind, r, shape, fix, a, 0, 1, skip, 0};
+  };
+  auto grid = [&](int32_t r, int32_t a, int32_t items, int32_t n, int32_t skip) {
+    return Item{kTile, r, kGrid, 0, sh.run ? a * sh.gr : a, sh.run ? 1 : items, sh.gr, skip, n};
   };
   int32_t a = int32_t(t);
-  if (s == nbr) return part(kTile, nbr - 1, kGrid, 0, a, sh.R_last, q + 1, 1);
+  if (s == nbr) return grid(nbr - 1, a, sh.R_last, q + 1, 1);
   if (s == nbr - 1) {
     if (a < sh.P_last)
-      return part(kPanel, s, a <= q ? kRow : kColumn, s, a <= q ? a : a - (q + 1), q + 1, q + 1, 1);
-    return part(kTile, s - 1, kGrid, 0, a - sh.P_last, sh.R_pen, q, 2);
+      return side(kPanel, s, a <= q ? kRow : kColumn, s, a <= q ? a : a - (q + 1), 1);
+    return grid(s - 1, a - sh.P_last, sh.R_pen, q, 2);
   }
   if (s == 0) {
     if (a == 0) return one(kDiag, 0, 0, 0);
@@ -638,18 +651,18 @@ __device__ Item decode_item(uint32_t t, const Shape& sh) {
   if (a < 2) return a == 0 ? one(kPanel, s, s, s + 1) : one(kPanel, s, s + 1, s);
   if (a < sh.P) {
     a -= 2;
-    return part(kPanel, s, a < q ? kRow : kColumn, s, a < q ? a : a - q, q, q, 2);
+    return side(kPanel, s, a < q ? kRow : kColumn, s, a < q ? a : a - q, 2);
   }
   a -= sh.P;
   if (s >= 1) {
-    if (a < q) return part(kTile, s - 1, kRow, s + 1, a, q, q, 2);
-    if (a < sh.X) return part(kTile, s - 1, kColumn, s + 1, a - q, q - 1, q - 1, 3);
+    if (a < q) return side(kTile, s - 1, kRow, s + 1, a, 2);
+    if (a < sh.X) return side(kTile, s - 1, kColumn, s + 1, a - q, 3);
     a -= sh.X;
   }
   if (a == 0) return one(kDiag, s + 1, s + 1, s + 1);
   a -= 1;
-  if (a < sh.L) return part(kTile, s, a < q ? kRow : kColumn, s + 1, a < q ? a : a - q, q, q, 2);
-  return part(kTile, s - 1, kGrid, 0, a - sh.L, sh.R, q - 1, 3);
+  if (a < sh.L) return side(kTile, s, a < q ? kRow : kColumn, s + 1, a < q ? a : a - q, 2);
+  return grid(s - 1, a - sh.L, sh.R, q - 1, 3);
 }
 
 struct Sync {
@@ -726,7 +739,7 @@ __device__ __noinline__ void next_item(const Sync& sy, uint32_t t, const Shape& 
   const int32_t rr = diag ? it.r - 1 : it.r;  // the round whose operands are read
   const bool two = it.kind == kTile || (diag && r);  // operands (i, rr) and (rr, j)
   bool ok = true, need = false, update = false;
-  if (lane < it.cnt) {
+  if (lane < it.cnt && (it.shape != kGrid || it.v0 + lane * it.stride < it.n * it.n)) {
     int32_t i, j;
     it.tile(lane, i, j);
     const int32_t own = i * nb + j;

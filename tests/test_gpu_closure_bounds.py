@@ -51,6 +51,24 @@ def test_closure_tile_bounds(kind, m, top, flags):
     assert S.context().status() == S.OK
 
 
+def test_closure_runs_of_neighbouring_tiles():
+    """A square in which nearly every update is needed, large enough that a
+    work item is a run of neighbouring tiles (two here, the last item of a
+    round shorter), in both lane formats, with and without bounds that need
+    rounding."""
+    import paper_2505_12976_gb300 as S
+    m = 3905
+    rs = np.random.Generator(np.random.PCG64(m))
+    d = rs.integers(0, 30001, (m, m)).astype(np.int32)
+    np.fill_diagonal(d, 0)
+    want = oracle.strongest_paths(d, nthreads=NT)
+    for flags in (0, S.F_FORCE_S32):
+        eq(host(S.schulze_strongest_paths(cu(d), 30000, flags=flags)), want, f"flags={flags}")
+    big = 1 << 15  # the same order of widths above 2^26
+    eq(host(S.schulze_strongest_paths(cu(d * big), 30000 * big)), want * big, "scaled")
+    assert S.context().status() == S.OK
+
+
 def test_run_relabels_listed_candidates_by_ballots():
     """More listed candidates than the cluster closure takes, some unlisted:
     the closure sorts the tally's relabeling by ballots."""

@@ -149,15 +149,19 @@ __device__ __forceinline__ bool weigh_all(bool hv, int32_t nw, int32_t warm_max,
 // pairs (A, B), A <= B: thread (r, c) holds d[A+r][B+c..c+3] and
 // d[B+r][A+c..c+3] in registers (16-byte loads when rows are 16-byte
 // aligned), both tiles go to shared memory, and each held entry is compared
-// with its transposed partner from there. Bound by HBM: d read and the
-// weights written once.
+// with its transposed partner from there. Bound by HBM (d read and the
+// weights written once) as far as the instructions per entry allow: with a
+// 64-bit test of every entry against the bound, the choice of weights made per
+// entry and a shuffle sum per row it took 440 us at m = 16384 with 16-bit lanes
+// and 479 with 32-bit ones, with one maximum per thread, kMargin and two rows
+// per shuffle sum 300 and 343 (1.6 and 2.1 GB, 0.79 and 0.92 of HBM).
 constexpr int kFlagT = 64;
-template <typename E>
+template <typename E, bool kMargin>
 __global__ void __launch_bounds__(256) weigh_kernel(const int32_t* __restrict__ d, int32_t m, int64_t bound,
                                                     int32_t* __restrict__ rowflag, int32_t* status,
                                                     const int32_t* __restrict__ warm,
                                                     const int32_t* __restrict__ hint_valid, int32_t warm_max, int vec4,
-                                                    Weights<E> V, int margin) {
+                                                    Weights<E> V) {
   pdl_enter_early();
   const bool hv = hint_valid && *hint_valid;
   if (!weigh_all(hv, hv ? *warm : 0, warm_max, m)) return;
@@ -169,7 +173,7 @@ __global__ void __launch_bounds__(256) weigh_kernel(const int32_t* __restrict__ 
   const bool vec = vec4 != 0;  // rows of d start on 16-byte boundaries
   int32_t a = 0;           // pairs (a, b), a <= b, numbered row by row
   int64_t rowstart = 0;    // number of the pair (a, a)
-  bool bad = false;
+  uint32_t largest = 0;  // entry met, negative ones above every bound
   auto put = [&](int32_t i, int32_t j, const int32_t (&w)[4]) {  // weights of row i, columns j .. j + 3
     if (i >= m || j >= m) return;
     E* row = V.v + int64_t(i) * V.ldv + j;
@@ -200,8 +204,7 @@ __global__ void __launch_bounds__(256) weigh_kernel(const int32_t* __restrict__ 
 #pragma unroll
           for (int e = 0; e < 4; ++e) x[q][e] = (i < m && j + e < m) ? d[int64_t(i) * m + j + e] : 0;
         }
-#pragma unroll
-        for (int e = 0; e < 4; ++e) bad |= x[q][e] < 0 || int64_t(x[q][e]) > bound;
+        largest = max(largest, max(max(uint32_t(x[q][0]), uint32_t(x[q][1])), max(uint32_t(x[q][2]), uint32_t(x[q][3]))));
       }
     };
     load(A, B, x1);
@@ -218,39 +221,44 @@ __global__ void __launch_bounds__(256) weigh_kernel(const int32_t* __restrict__ 
     // side 1: row B + r, columns A + c: edge when t2[r][c] > t1[c][r]
     const int32_t(*T)[kFlagT + 1] = A == B ? t1 : t2;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = rq + 16 * q;
-      uint32_t e = 0;  // side 0 in the low half, side 1 in the high half
-      int32_t w[4];
+    for (int h = 0; h < 2; ++h) {
+      uint32_t e = 0;  // edges of rows 2 h and 2 h + 1 of side 0, then of side 1 (64 at most each), a byte each
 #pragma unroll
-      for (int x = 0; x < 4; ++x) {  // (on the diagonal both sides are the same entry: no edge)
-        const int32_t u = T[c4 + x][r];
-        const bool edge = x1[q][x] > u;
-        e += edge ? 1u : 0u;
-        w[x] = edge ? x1[q][x] - (margin ? u : 0) : 0;
-      }
-      put(A + r, B + c4, w);
-      if (A != B) {
+      for (int q = 2 * h; q < 2 * h + 2; ++q) {
+        const int r = rq + 16 * q;
+        const uint32_t one = q & 1 ? 0x100u : 1u;
+        int32_t w[4];
 #pragma unroll
-        for (int x = 0; x < 4; ++x) {
-          const int32_t u = t1[c4 + x][r];
-          const bool edge = x2[q][x] > u;
-          e += edge ? 0x10000u : 0u;
-          w[x] = edge ? x2[q][x] - (margin ? u : 0) : 0;
+        for (int x = 0; x < 4; ++x) {  // (on the diagonal both sides are the same entry: no edge)
+          const int32_t u = T[c4 + x][r];
+          const bool edge = x1[q][x] > u;
+          e += edge ? one : 0u;
+          w[x] = edge ? x1[q][x] - (kMargin ? u : 0) : 0;
         }
-        put(B + r, A + c4, w);
+        put(A + r, B + c4, w);
+        if (A != B) {
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const int32_t u = t1[c4 + x][r];
+            const bool edge = x2[q][x] > u;
+            e += edge ? one << 16 : 0u;
+            w[x] = edge ? x2[q][x] - (kMargin ? u : 0) : 0;
+          }
+          put(B + r, A + c4, w);
+        }
       }
       // padding entries are 0 on both sides, so they never count
 #pragma unroll
       for (int o = 8; o; o >>= 1) e += __shfl_xor_sync(0xFFFFFFFFu, e, o);
-      if ((lane & 15) == 0) {
-        if (e & 0xFFFFu) atomicAdd(&rowflag[A + r], int32_t(e & 0xFFFFu));
-        if (e >> 16) atomicAdd(&rowflag[B + r], int32_t(e >> 16));
+      const int r = rq + 32 * h + (lane & 1) * 16, f = int(e >> (lane & 1) * 8);
+      if ((lane & 15) < 2) {
+        if (f & 0xFF) atomicAdd(&rowflag[A + r], f & 0xFF);
+        if ((f >> 16) & 0xFF) atomicAdd(&rowflag[B + r], (f >> 16) & 0xFF);
       }
     }
     __syncthreads();
   }
-  if (bad) set_status(status, SCHULZE_EDATA);
+  if (largest > uint32_t(min(bound, int64_t(INT32_MAX)))) set_status(status, SCHULZE_EDATA);
 }
 
 // perm[new] = old, inv[old] = new: candidates with edges first, strongest
@@ -1436,11 +1444,11 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
   };
   {
     const int64_t nbt = (m + kFlagT - 1) / kFlagT;
-    const int g = grid_for(reinterpret_cast<const void*>(weigh_kernel<E>), 256, 0, nbt * (nbt + 1) / 2);
+    auto kern = bf.margin ? weigh_kernel<E, true> : weigh_kernel<E, false>;
+    const int g = grid_for(reinterpret_cast<const void*>(kern), 256, 0, nbt * (nbt + 1) / 2);
     Launch L(ctx, stream, "closure_rowflags", mm * 4.0);
-    launch_pdl(weigh_kernel<E>, dim3(g), dim3(256), 0, stream, false, d, m, bound, bf.rowflag, status,
-               static_cast<const int32_t*>(bf.warm), bf.hint_valid, kClusterMaxWarm<E>, rows_vec16(d, m), V,
-               bf.margin ? 1 : 0);
+    launch_pdl(kern, dim3(g), dim3(256), 0, stream, false, d, m, bound, bf.rowflag, status,
+               static_cast<const int32_t*>(bf.warm), bf.hint_valid, kClusterMaxWarm<E>, rows_vec16(d, m), V);
   }
   {
     Launch L(ctx, stream, "closure_relabel", double(m) * 12.0);

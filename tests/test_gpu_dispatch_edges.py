@@ -68,6 +68,26 @@ def test_small_closure_reports_counts_out_of_range(m, wrong):
     assert S.context().status() == S.OK
 
 
+@pytest.mark.parametrize("m", [257, 300, 705])
+@pytest.mark.parametrize("bound,wrong", [(100, -1), (100, 101), (100, -2**31), (40000, 40001), (2**31 - 1, -1),
+                                         (2**40, -5), (0, 1)])
+def test_large_closure_reports_counts_out_of_range(m, bound, wrong):
+    """One entry below 0 or above the bound is reported, wherever it lies and
+    whatever the bound (beyond 31 bits too); the largest allowed one is not."""
+    import paper_2505_12976_gb300 as S
+    ok = min(bound, 2**31 - 1)
+    d = np.minimum(counts("ties", m, 100, 3), ok).astype(np.int32)
+    for i, j in ((0, m - 1), (m - 1, 0), (m // 2, m // 2 + 1), (m - 1, m - 1)):
+        for flags in (0, S.F_MARGIN):
+            e = d.copy()
+            e[i, j] = wrong
+            S.schulze_strongest_paths(cu(e), bound, flags=flags)
+            assert S.context().status() == S.EDATA, (i, j, flags)
+            e[i, j] = ok
+            S.schulze_strongest_paths(shifted(e), bound, flags=flags)
+            assert S.context().status() == S.OK, (i, j, flags)
+
+
 @pytest.mark.parametrize("m,odd", [(701, 0), (704, 1), (1000, 0)])
 def test_general_path_beaten_by_with_cold_columns(m, odd):
     """winners, order and beaten_by of the general path with candidates that

@@ -920,52 +920,60 @@ __device__ __forceinline__ bool differs(const uint4& a, const uint4& b) {
 template <typename E>
 using RowPair = typename std::conditional<sizeof(E) == 2, uint32_t, int2>::type;  // a row's entries k, k + 1
 
-// The sweeps over the square S4 (rows of Qs 16-byte pieces, Q of them in
-// use), rows 0 .. nw - 1 (row nw zero when nw is odd), every copy loaded and
-// every flag clear. Returns the number of sweeps.
+// One sweep over pieces c0 .. c0 + Q - 1 of the square S4 (rows of Qs 16-byte
+// pieces), rows and pivots 0 .. nw - 1 (row nw zero when nw is odd). Returns
+// whether the calling thread changed something.
 template <typename E>
-__device__ int sweep_square(cooperative_groups::cluster_group& cl, uint4* S4, int32_t Qs, int32_t Q, int32_t nw,
-                            uint32_t (*flags)[kClusterCtas]) {
+__device__ __forceinline__ bool sweep_once(cooperative_groups::cluster_group& cl, uint4* S4, int32_t Qs, int32_t c0,
+                                           int32_t Q, int32_t nw) {
   using AW = RowPair<E>;
   const AW* A = reinterpret_cast<const AW*>(S4);
   const int32_t ra = Qs * 16 / int32_t(sizeof(AW));  // row stride of A
   const int32_t nwe = (nw + 1) & ~1;                 // pivots, in pairs
-  const int t = threadIdx.x;
   const unsigned q = cl.block_rank();
   const int32_t own = int32_t(q) < nw ? (nw - int32_t(q) + kClusterCtas - 1) / kClusterCtas : 0;
   const int32_t items = (own + 1) / 2 * Q;  // (pair of owned rows, piece)
+  bool changed = false;
+  for (int32_t it = threadIdx.x; it < items; it += kClusterThreads) {
+    const int32_t rp = it / Q, c = c0 + it % Q;
+    const int32_t i0 = int32_t(q) + kClusterCtas * (2 * rp), i1 = i0 + kClusterCtas;
+    const bool has1 = i1 < nw;
+    const uint4 x0 = S4[i0 * Qs + c], x1 = has1 ? S4[i1 * Qs + c] : x0;
+    uint4 acc0 = x0, acc1 = x1;
+    const AW* a0p = A + i0 * ra;
+    const AW* a1p = A + (has1 ? i1 : i0) * ra;
+#pragma unroll 4
+    for (int32_t k = 0; k < nwe; k += 2) {
+      const uint4 b0 = S4[k * Qs + c], b1 = S4[(k + 1) * Qs + c];
+      sweep_step(acc0, a0p[k >> 1], b0, b1);
+      sweep_step(acc1, a1p[k >> 1], b0, b1);
+    }
+    if (differs(acc0, x0)) {
+      changed = true;
+      S4[i0 * Qs + c] = acc0;
+#pragma unroll
+      for (int o = 1; o < kClusterCtas; ++o) *cl.map_shared_rank(S4 + i0 * Qs + c, (q + o) % kClusterCtas) = acc0;
+    }
+    if (has1 && differs(acc1, x1)) {
+      changed = true;
+      S4[i1 * Qs + c] = acc1;
+#pragma unroll
+      for (int o = 1; o < kClusterCtas; ++o) *cl.map_shared_rank(S4 + i1 * Qs + c, (q + o) % kClusterCtas) = acc1;
+    }
+  }
+  return changed;
+}
+
+// Sweeps over the first Q pieces until nothing changes, every copy loaded and
+// every flag clear. Returns the number of sweeps.
+template <typename E>
+__device__ int sweep_square(cooperative_groups::cluster_group& cl, uint4* S4, int32_t Qs, int32_t Q, int32_t nw,
+                            uint32_t (*flags)[kClusterCtas]) {
+  const int t = threadIdx.x;
+  const unsigned q = cl.block_rank();
   int sweeps = 0;
   while (sweeps < kMaxSweeps) {
-    bool changed = false;
-    for (int32_t it = t; it < items; it += kClusterThreads) {
-      const int32_t rp = it / Q, c = it % Q;
-      const int32_t i0 = int32_t(q) + kClusterCtas * (2 * rp), i1 = i0 + kClusterCtas;
-      const bool has1 = i1 < nw;
-      const uint4 x0 = S4[i0 * Qs + c], x1 = has1 ? S4[i1 * Qs + c] : x0;
-      uint4 acc0 = x0, acc1 = x1;
-      const AW* a0p = A + i0 * ra;
-      const AW* a1p = A + (has1 ? i1 : i0) * ra;
-#pragma unroll 4
-      for (int32_t k = 0; k < nwe; k += 2) {
-        const uint4 b0 = S4[k * Qs + c], b1 = S4[(k + 1) * Qs + c];
-        sweep_step(acc0, a0p[k >> 1], b0, b1);
-        sweep_step(acc1, a1p[k >> 1], b0, b1);
-      }
-      if (differs(acc0, x0)) {
-        changed = true;
-        S4[i0 * Qs + c] = acc0;
-#pragma unroll
-        for (int o = 1; o < kClusterCtas; ++o)
-          *cl.map_shared_rank(S4 + i0 * Qs + c, (q + o) % kClusterCtas) = acc0;
-      }
-      if (has1 && differs(acc1, x1)) {
-        changed = true;
-        S4[i1 * Qs + c] = acc1;
-#pragma unroll
-        for (int o = 1; o < kClusterCtas; ++o)
-          *cl.map_shared_rank(S4 + i1 * Qs + c, (q + o) % kClusterCtas) = acc1;
-      }
-    }
+    const bool changed = sweep_once<E>(cl, S4, Qs, 0, Q, nw);
     ++sweeps;
     const int any = __syncthreads_or(changed);
     if (any && t < kClusterCtas) *cl.map_shared_rank(&flags[sweeps & 1][q], unsigned(t)) = 1u;
@@ -1047,6 +1055,17 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
 // after the sweeps it writes its rows of p, counts who beats its candidates,
 // hands the counts to the other CTAs and ranks its candidates. Bound by
 // latency: it replaces a chain of eleven launches (m = 64: 10 us).
+//
+// From kFewMin on, where enough candidates have no edge, the square is filled
+// anew with those that have one first (the other rows are zero and are left out,
+// as pivots too), the sweeps run over it alone and one more takes its widths to
+// the other columns: m = 256, int16: 5% with edges 81 -> 27 us, 50% 117 -> 50, 80%
+// 120 -> 100; m = 192, int32: 70 -> 22, 103 -> 45, 106 -> 84. The second filling
+// takes 2 to 4 us. What it saves grows with the entries of the rows left out: at
+// m = 150, int32, 15 rows are about even (56.1 and 58.3 us), 22 save 7 us. Up to
+// 128 candidates, where all of them take no more than 38 us, looking for edges
+// costs more than it saves (m = 64: 15.4 and 15.9 us, all with edges).
+constexpr int32_t kFewMin = 129, kFewSaving = 2400;
 template <typename E>
 __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterThreads, 1)
     closure_small_kernel(const int32_t* __restrict__ d, int32_t m, int64_t bound, int margin, int32_t* __restrict__ p,
@@ -1063,62 +1082,118 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
   const int32_t ls = Qs * kPer16;
   __shared__ uint32_t flags[2][kClusterCtas];
   __shared__ int32_t beaten[kSmallMax];
+  __shared__ uint8_t edges[kSmallMax];               // whether candidate i has an edge
+  __shared__ uint16_t perm[kSmallMax], pos[kSmallMax];  // those with one first: new -> old, old -> new
   const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
   const unsigned q = cl.block_rank();
   const int32_t own = int32_t(q) < m ? (m - int32_t(q) + kClusterCtas - 1) / kClusterCtas : 0;
   if (t < 2 * kClusterCtas) flags[t / kClusterCtas][t % kClusterCtas] = 0u;
+  if (t < kSmallMax) edges[t] = 0;
   if (m & 1)  // the row past the last one, which a pair of pivots reads
     for (int32_t c = t; c < Q; c += kClusterThreads) S4[m * Qs + c] = make_uint4(0u, 0u, 0u, 0u);
   cl.sync();  // every CTA has started before any remote write
   bool bad = false;
-  for (int32_t it = t; it < own * Q; it += kClusterThreads) {
-    const int32_t c = it / own, i = int32_t(q) + kClusterCtas * (it - c * own), j0 = c * kPer16;
-    int32_t x[kPer16], y[kPer16];
+  // the weights of n of this CTA's rows into every square, candidate(x) in its row or column x
+  auto fill = [&](int32_t n, auto candidate) {
+    for (int32_t it = t; it < n * Q; it += kClusterThreads) {
+      const int32_t c = it / n, a = int32_t(q) + kClusterCtas * (it - c * n), i = candidate(a), j0 = c * kPer16;
+      int32_t x[kPer16], y[kPer16];
 #pragma unroll
-    for (int e = 0; e < kPer16; ++e) {
-      x[e] = j0 + e < m ? d[int64_t(i) * m + j0 + e] : 0;
-      y[e] = j0 + e < m ? d[int64_t(j0 + e) * m + i] : 0;
+      for (int e = 0; e < kPer16; ++e) {
+        const int32_t j = j0 + e < m ? candidate(j0 + e) : 0;
+        x[e] = j0 + e < m ? d[int64_t(i) * m + j] : 0;
+        y[e] = j0 + e < m ? d[int64_t(j) * m + i] : 0;
+      }
+      uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int e = 0; e < kPer16; ++e) {
+        bad |= x[e] < 0 || int64_t(x[e]) > bound;
+        const int32_t out = x[e] > y[e] ? x[e] - (margin ? y[e] : 0) : 0;
+        if (sizeof(E) == 2) w[e >> 1] |= (uint32_t(out) & 0xFFFFu) << (16 * (e & 1));
+        else w[e & 3] = uint32_t(out);
+      }
+      const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
+      if (v.x | v.y | v.z | v.w) edges[i] = 1;
+#pragma unroll
+      for (int o = 0; o < kClusterCtas; ++o) *cl.map_shared_rank(S4 + a * Qs + c, unsigned(o)) = v;
     }
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int e = 0; e < kPer16; ++e) {
-      bad |= x[e] < 0 || int64_t(x[e]) > bound;
-      const int32_t out = x[e] > y[e] ? x[e] - (margin ? y[e] : 0) : 0;
-      if (sizeof(E) == 2) w[e >> 1] |= (uint32_t(out) & 0xFFFFu) << (16 * (e & 1));
-      else w[e & 3] = uint32_t(out);
-    }
-    const uint4 v = make_uint4(w[0], w[1], w[2], w[3]);
-#pragma unroll
-    for (int o = 0; o < kClusterCtas; ++o) *cl.map_shared_rank(S4 + i * Qs + c, unsigned(o)) = v;
-  }
+  };
+  fill(own, [](int32_t x) { return x; });
   if (bad) set_status(status, SCHULZE_EDATA);
-  cl.sync();  // every square complete
-  const int sweeps = sweep_square<E>(cl, S4, Qs, Q, m, flags);
-  for (int32_t r = wid; r < own; r += kClusterThreads / 32) {
-    const int32_t i = int32_t(q) + kClusterCtas * r;
-    int32_t c = 0;
-    for (int32_t j = lane; j < m; j += 32) {
-      const int32_t x = j == i ? 0 : int32_t(S[i * ls + j]);
-      p[int64_t(i) * m + j] = x;
-      c += j != i && int32_t(S[j * ls + i]) > x;
+  const bool look = m >= kFewMin;
+  if (look) {  // the own candidates' edges, told to the others
+    __syncthreads();
+    for (int x = t; x < own * kClusterCtas; x += kClusterThreads) {
+      const int32_t i = int32_t(q) + kClusterCtas * (x / kClusterCtas), o = x % kClusterCtas;
+      if (o != int32_t(q)) *cl.map_shared_rank(edges + i, unsigned(o)) = edges[i];
     }
-    c = __reduce_add_sync(0xFFFFFFFFu, c);
-    if (lane < kClusterCtas) *cl.map_shared_rank(beaten + i, unsigned(lane)) = c;
   }
+  cl.sync();  // every square and edge list complete
+  int32_t nw = m;
+  if (look) {
+    nw = __syncthreads_count(t < m && edges[t]);
+    if ((m - nw) * m < kFewSaving) nw = m;
+  }
+  const bool few = nw < m;  // (the same decision in every CTA)
+  int sweeps;
+  if (few) {
+    if (wid == 0) {
+      int32_t seen = 0;  // candidates with edges so far
+      for (int32_t i0 = 0; i0 < m; i0 += 32) {
+        const int32_t i = i0 + lane;
+        const uint32_t b = __ballot_sync(0xFFFFFFFFu, i < m && edges[i]);
+        const int32_t before = seen + __popc(b & ((1u << lane) - 1u));
+        if (i < m) {
+          const int32_t a = edges[i] ? before : nw + i - before;
+          pos[i] = uint16_t(a), perm[a] = uint16_t(i);
+        }
+        seen += __popc(b);
+      }
+    }
+    if (nw & 1)
+      for (int32_t c = t; c < Q; c += kClusterThreads) S4[nw * Qs + c] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();  // (no CTA reads its square before the next cluster barrier)
+    fill(int32_t(q) < nw ? (nw - int32_t(q) + kClusterCtas - 1) / kClusterCtas : 0,
+         [&](int32_t x) { return int32_t(perm[x]); });
+    cl.sync();
+    const int32_t Qw = (nw + kPer16 - 1) / kPer16;
+    sweeps = sweep_square<E>(cl, S4, Qs, Qw, nw, flags);
+    if (Qw < Q) {
+      sweep_once<E>(cl, S4, Qs, Qw, Q - Qw, nw);
+      cl.sync();
+    }
+  } else {
+    sweeps = sweep_square<E>(cl, S4, Qs, Q, m, flags);
+  }
+  auto rows_out = [&](auto width) {  // width(i, j), i != j
+    for (int32_t r = wid; r < own; r += kClusterThreads / 32) {
+      const int32_t i = int32_t(q) + kClusterCtas * r;
+      int32_t c = 0;
+      for (int32_t j = lane; j < m; j += 32) {
+        const int32_t x = j == i ? 0 : width(i, j);
+        p[int64_t(i) * m + j] = x;
+        c += j != i && width(j, i) > x;
+      }
+      c = __reduce_add_sync(0xFFFFFFFFu, c);
+      if (lane < kClusterCtas) *cl.map_shared_rank(beaten + i, unsigned(lane)) = c;
+    }
+  };
+  if (few) rows_out([&](int32_t i, int32_t j) { return edges[i] ? int32_t(S[pos[i] * ls + pos[j]]) : 0; });
+  else rows_out([&](int32_t i, int32_t j) { return int32_t(S[i * ls + j]); });
   cl.sync();  // every count everywhere
   for (int32_t r = wid; r < own; r += kClusterThreads / 32) {
-    const int32_t i = int32_t(q) + kClusterCtas * r, mine = beaten[i];
-    int32_t pos = 0;  // candidates ahead of i by (beaten_by, id)
-    for (int32_t j = lane; j < m; j += 32) pos += beaten[j] < mine || (beaten[j] == mine && j < i);
-    pos = __reduce_add_sync(0xFFFFFFFFu, pos);
+    const int32_t i = int32_t(q) + kClusterCtas * r, count = beaten[i];
+    int32_t ahead = 0;  // candidates ahead of i by (beaten_by, id)
+    for (int32_t j = lane; j < m; j += 32) ahead += beaten[j] < count || (beaten[j] == count && j < i);
+    ahead = __reduce_add_sync(0xFFFFFFFFu, ahead);
     if (lane == 0) {
-      if (bb) bb[i] = mine;
-      if (winners) winners[i] = mine == 0;
-      if (order) order[pos] = i;
+      if (bb) bb[i] = count;
+      if (winners) winners[i] = count == 0;
+      if (order) order[ahead] = i;
     }
   }
   if (t == 0 && q == 0)  // entry updates, in 64 x 64 x 64 tile units
-    atomicAdd(&counters[0], (unsigned long long)sweeps * uint64_t(m) * uint64_t(m) * uint64_t(m) / 262144ull);
+    atomicAdd(&counters[0], (unsigned long long)sweeps * uint64_t(nw) * uint64_t(nw) * uint64_t(nw) / 262144ull);
 }
 
 // Uniform cold columns: u[i] = max(ucol[i], max_x min(W[i][x], ucol[x]))

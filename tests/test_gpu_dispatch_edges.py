@@ -42,6 +42,30 @@ def test_small_closure_both_lanes_margin_and_alignment(m):
     assert S.context().status() == S.OK
 
 
+@pytest.mark.parametrize("m", [1, 2, 3, 31, 64, 65, 128, 129, 130, 191, 192, 255, 256])
+def test_small_closure_with_few_candidates_with_edges(m):
+    """No candidate with an edge, one, a few, two neighbours, the last ones,
+    about half, all but one, and on both sides of the line at which the square
+    is filled anew."""
+    import paper_2505_12976_gb300 as S
+    rs = np.random.Generator(np.random.PCG64(m))
+    full = counts("ties", m, 30000, m) if m > 2 else np.array([[0, 5], [3, 0]], np.int32)[:m, :m]
+    sets = [[], [0], [m - 1], [m - 2, m - 1], rs.permutation(m)[:5], rs.permutation(m)[:m // 4], rs.permutation(m)[:m // 2],
+            np.arange(0, m, 2), np.arange(1, m, 2), rs.permutation(m)[:max(0, m - 1)]]
+    line = -(-2400 // m)  # candidates without an edge
+    sets += [rs.permutation(m)[:max(0, m - line + x)] for x in (0, 1)]
+    for t, keep in enumerate(sets):
+        d = np.zeros_like(full)
+        keep = np.unique(np.clip(np.array(keep, np.int64), 0, m - 1))
+        d[keep] = full[keep] + rs.integers(0, 50, (len(keep), m))
+        np.fill_diagonal(d, 0)
+        for flags in (0, 1, S.F_MARGIN):
+            w = oracle.weights_margin(d) if flags == S.F_MARGIN else oracle.weights(d)
+            want = oracle.closure(w, nthreads=2)
+            eq(host(S.schulze_strongest_paths(cu(d), 30100, flags=flags)), want, f"m={m} set {t} flags={flags}")
+    assert S.context().status() == S.OK
+
+
 @pytest.mark.parametrize("m,n,k", [(1, 4, 1), (2, 5, 1), (8, 30, 8), (65, 50, 64), (192, 40, 192), (193, 60, 20),
                                    (256, 90, 256), (257, 90, 256)])
 @pytest.mark.parametrize("flags", [0, 1, 32])

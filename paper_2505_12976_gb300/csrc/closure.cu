@@ -1241,7 +1241,10 @@ __global__ void __launch_bounds__(512, 1) cold_strip_kernel(E* __restrict__ W, i
                                                             const int32_t* __restrict__ warm,
                                                             unsigned long long* counters,
                                                             const int32_t* __restrict__ hint_valid) {
-  pdl_enter_early();
+  // With a hint cold_product_kernel seldom has work; without one its CTAs are
+  // let in late, when they spread over SMs that the closure has left
+  if (hint_valid) pdl_enter_early();
+  else pdl_enter();
   using Wd = typename std::conditional<sizeof(E) == 2, uint32_t, int32_t>::type;  // one word
   constexpr int kPer = sizeof(Wd) / sizeof(E);                                  // entries per word
   const int32_t nw = *warm;
@@ -1320,14 +1323,18 @@ __global__ void __launch_bounds__(512, 1) cold_strip_kernel(E* __restrict__ W, i
 // may read a W(k, j) that another item is raising at the same time; every
 // value either one sees is the width of a real path and the closed square
 // composes with itself without growing (p(i,x) and p(x,y) give a walk no
-// wider than p(i,y)), so the result is the exact closure either way.
+// wider than p(i,y)), so the result is the exact closure either way. Five CTAs
+// per SM (without the bound 32-bit lanes take registers for three), launched
+// once the closure is done (cold_strip_kernel) where there is no hint: m = 8192
+// with 3000 warm, int32, the whole call 8.32 -> 7.83 ms; with the bound alone 7.80,
+// but m = 2000 with 1000 0.73 -> 0.85 then, as CTAs that came early took the SMs
+// unevenly. (Seven CTAs with 16-bit lanes: 1% less here, and 0.5 us more where
+// they return at once.)
 template <typename E>
-__global__ void __launch_bounds__(kThreads) cold_product_kernel(E* __restrict__ W, int32_t ld, int32_t nb,
-                                                                 int32_t m, const int32_t* __restrict__ warm,
-                                                                 const unsigned long long* __restrict__ prog,
-                                                                 const int32_t* __restrict__ tmax,
-                                                                 unsigned long long* counters,
-                                                                 const int32_t* __restrict__ hint_valid) {
+__global__ void __launch_bounds__(kThreads, 5)
+    cold_product_kernel(E* __restrict__ W, int32_t ld, int32_t nb, int32_t m, const int32_t* __restrict__ warm,
+                        const unsigned long long* __restrict__ prog, const int32_t* __restrict__ tmax,
+                        unsigned long long* counters, const int32_t* __restrict__ hint_valid) {
   pdl_enter_early();
   __shared__ __align__(16) typename Ops<E>::Smem sm;
   if (*warm <= kClusterMaxWarm<E>) return;  // cold_strip_kernel's case

@@ -66,6 +66,7 @@ struct PassArgs {
   const int32_t* asked;     // kMarks: candidates asked about
   const int4* label;        // kMarks: per block its first candidate's ids (x, y), z: all share them
   int32_t *lose, *scc_lose;  // kMarks
+  int32_t* status;          // rows_kernel: kInit sets it, kMarks reads it
 };
 
 // One pass over the pairs of blocks; a thread holds four columns of four rows
@@ -225,6 +226,107 @@ __global__ void __launch_bounds__(256, 4) pair_kernel(PassArgs g) {
   if (s1) serve(B, 1, 0, x2, t1);
 }
 
+// Postprocessing (Alg. 4) without edges: the loser among c, its source and its
+// target, and whether c's incoming edges matter: those of the unknown
+// candidates, and of those with an SCC's label (s = t), which may be an unknown
+// candidate's.
+__device__ __forceinline__ void mark_by_keys(Key f, Key b, int32_t c, int32_t* lose) {
+  const int32_t s = key_id(f), t = key_id(b);
+  if (s < t) {
+    lose[c] = 1;
+  } else if (s > t) {
+    lose[t] = 1;  // an id: t < s
+  } else if (s != kNone) {
+    // smaller low words are wider
+    if (uint32_t(f) < uint32_t(b)) lose[c] = 1;
+    else if (uint32_t(f) > uint32_t(b)) lose[s] = 1;
+  }
+}
+__device__ __forceinline__ bool asks(int32_t status, int32_t s, int32_t t) {
+  return status == kUnknown || (s == t && s != kNone);
+}
+
+// The same passes for few candidates, a warp per candidate on its row of d and
+// of dT (d transposed): a round is one launch that no atomics and no commit
+// follow, and a square of few blocks still gives every SM a warp. Bound by
+// latency and by the host's look at *set after every round (20 to 27 us each).
+// Uniform random d, the whole call, against pairs of blocks: m = 64 740 and 1144
+// us, m = 300 2740 and 4290, m = 700 3550 and 4110, m = 1024 7270 and 7690.
+// *clear is the word that the next round sets when a key changes.
+constexpr int kRowWarps = 4;
+template <int kPass>
+__global__ void __launch_bounds__(32 * kRowWarps) rows_kernel(PassArgs g, const int32_t* __restrict__ dT,
+                                                              int32_t* __restrict__ set, int32_t* __restrict__ clear) {
+  if (kPass == kPropagate && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0;
+  const int lane = threadIdx.x & 31;
+  const int32_t c = blockIdx.x * kRowWarps + (threadIdx.x >> 5), m = g.m;
+  if (c >= m) return;
+  const int32_t *dr = g.d + int64_t(c) * m, *tr = dT + int64_t(c) * m;
+  if (kPass == kInit) {
+    int32_t in = 0, out = 0;
+    for (int32_t u = lane; u < m; u += 32) {
+      const int32_t x = dr[u], o = tr[u];
+      out = max(out, edge(x, o, g.margin)), in = max(in, edge(o, x, g.margin));
+    }
+    in = __reduce_max_sync(0xFFFFFFFFu, in), out = __reduce_max_sync(0xFFFFFFFFu, out);
+    if (lane == 0) g.status[c] = in > out ? kLoser : kUnknown;
+    return;
+  }
+  const Key mf = g.f[c], mb = g.b[c];
+  if (kPass == kPropagate) {
+    Key bf = mf, bb = mb;
+    constexpr int kU = 4;  // loads in flight, also in a last step that not all lanes need
+    for (int32_t u0 = lane; u0 < m; u0 += 32 * kU) {
+      int32_t x[kU], o[kU];
+      Key uf[kU], ub[kU];
+#pragma unroll
+      for (int e = 0; e < kU; ++e) {
+        const int32_t u = u0 + 32 * e;
+        const bool in = u < m;
+        x[e] = in ? dr[u] : 0, o[e] = in ? tr[u] : 0;
+        uf[e] = in ? g.f[u] : 0, ub[e] = in ? g.b[u] : 0;
+      }
+#pragma unroll
+      for (int e = 0; e < kU; ++e) {
+        const int32_t w = g.margin ? abs(o[e] - x[e]) : max(o[e], x[e]);
+        if (o[e] > x[e]) bf = min(bf, along(uf[e], w));  // along (u, c) from u's source
+        if (x[e] > o[e]) bb = min(bb, along(ub[e], w));  // against (c, u) from u's target
+      }
+    }
+#pragma unroll
+    for (int h = 16; h; h >>= 1) {
+      bf = min(bf, __shfl_xor_sync(0xFFFFFFFFu, bf, h));
+      bb = min(bb, __shfl_xor_sync(0xFFFFFFFFu, bb, h));
+    }
+    if (lane == 0) {
+      g.fn[c] = bf, g.bn[c] = bb;
+      if (bf != mf || bb != mb) *set = 1;
+    }
+  } else {
+    const int32_t ms = key_id(mf), mt = key_id(mb);
+    if (lane == 0) mark_by_keys(mf, mb, c, g.lose);
+    if (!asks(g.status[c], ms, mt)) return;
+    bool other = false;  // an incoming edge (u, c) from another SCC
+    for (int32_t u = lane; u < m; u += 32)
+      other |= tr[u] > dr[u] && (key_id(g.f[u]) != ms || key_id(g.b[u]) != mt);
+    if (__any_sync(0xFFFFFFFFu, other) && lane == 0) {
+      if (ms == mt) g.scc_lose[ms == kNone ? m : ms] = 1;
+      else g.lose[c] = 1;
+    }
+  }
+}
+
+// dT = d transposed, through 32 x 32 shared-memory tiles.
+__global__ void __launch_bounds__(256) transpose_kernel(const int32_t* __restrict__ d, int32_t m,
+                                                        int32_t* __restrict__ dT) {
+  __shared__ int32_t tile[32][33];
+  const int32_t j0 = blockIdx.x * 32, i0 = blockIdx.y * 32, x = threadIdx.x & 31;
+  for (int r = threadIdx.x >> 5; r < 32; r += 8) tile[r][x] = i0 + r < m && j0 + x < m ? d[int64_t(i0 + r) * m + j0 + x] : 0;
+  __syncthreads();
+  for (int r = threadIdx.x >> 5; r < 32; r += 8)
+    if (j0 + r < m && i0 + x < m) dT[int64_t(j0 + r) * m + i0 + x] = tile[x][r];
+}
+
 // Initialisation-of-vertices (Alg. 1): c is a loser when its heaviest
 // incoming edge outweighs its heaviest outgoing one.
 __global__ void init_status_kernel(const int32_t* __restrict__ in, const int32_t* __restrict__ out, int32_t m,
@@ -270,10 +372,9 @@ __global__ void __launch_bounds__(kPT) commit_kernel(int32_t m, Key* __restrict_
   }
 }
 
-// Postprocessing (Alg. 4), the marks that need no edges: lose[c] for a loser;
-// and the candidates whose incoming edges matter (the marks pass): the
-// unknown ones, and those with an SCC's label (s = t), which may be an
-// unknown candidate's. A CTA per block of 64.
+// Postprocessing (Alg. 4), the marks that need no edges, the candidates whose
+// incoming edges matter (the marks pass), and what the blocks have in common. A
+// CTA per block of 64.
 __global__ void __launch_bounds__(kPT) label_kernel(const Key* __restrict__ f, const Key* __restrict__ b, int32_t m,
                                                     const int32_t* __restrict__ status, int32_t* __restrict__ lose,
                                                     int32_t* __restrict__ asked, int32_t* __restrict__ flag,
@@ -284,16 +385,8 @@ __global__ void __launch_bounds__(kPT) label_kernel(const Key* __restrict__ f, c
   if (c < m) {
     const int32_t s = key_id(f[c]), t = key_id(b[c]);
     same = s == s0 && t == t0;
-    if (s < t) {
-      lose[c] = 1;
-    } else if (s > t) {
-      lose[t] = 1;  // an id: t < s
-    } else if (s != kNone) {
-      // smaller low words are wider
-      if (uint32_t(f[c]) < uint32_t(b[c])) lose[c] = 1;
-      else if (uint32_t(f[c]) > uint32_t(b[c])) lose[s] = 1;
-    }
-    ask = status[c] == kUnknown || (s == t && s != kNone);
+    mark_by_keys(f[c], b[c], c, lose);
+    ask = asks(status[c], s, t);
     asked[c] = ask;
   }
   const int any = __syncthreads_or(ask), one = __syncthreads_and(same);
@@ -330,9 +423,13 @@ __global__ void winners_out_kernel(const int32_t* __restrict__ status, int32_t m
 
 }  // namespace
 
+// Candidates up to which rows_kernel does the passes (from there on the pairs of
+// blocks, which read d once a round and leave blocks out, are as fast).
+constexpr int32_t kRowsMax = 1024;
+
 size_t propagation_workspace_bytes(int32_t m) {
   const size_t mv = align_up((size_t(m) + 1) * 4, 256);
-  return 4 * align_up(size_t(m) * 8, 256) + 8 * mv + 4096;
+  return 4 * align_up(size_t(m) * 8, 256) + 8 * mv + (m <= kRowsMax ? align_up(size_t(m) * size_t(m) * 4, 256) : 0) + 4096;
 }
 
 int winners_propagation_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, bool margin, int32_t* winners,
@@ -348,30 +445,37 @@ int winners_propagation_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, bo
   int32_t* scc_lose = cv.take<int32_t>(size_t(m) + 1);
   int32_t* asked = cv.take<int32_t>(size_t(m) + 1);
   int32_t* inout = cv.take<int32_t>(2 * size_t(m) + 1);  // heaviest incoming, outgoing edges
-  int32_t* words = cv.take<int32_t>(3);                  // [0] changed, [1] decided, [2] unknown
+  int32_t* words = cv.take<int32_t>(4);                  // [0] changed, [1] decided, [2] unknown, [3] changed (in turn)
   const int32_t nbt = (m + kPT - 1) / kPT;
   int32_t* flag = cv.take<int32_t>(size_t(nbt));
   int4* label = cv.take<int4>(size_t(nbt));
+  const bool rows = m <= kRowsMax && !max_in;
+  int32_t* dT = rows ? cv.take<int32_t>(size_t(m) * size_t(m)) : nullptr;
+  const unsigned row_grid = unsigned((m + kRowWarps - 1) / kRowWarps);
   const unsigned pairs = unsigned(int64_t(nbt) * (nbt + 1) / 2);
   const int g = std::max(1, std::min((m + 255) / 256, 1024));
   PassArgs pa{};
   pa.d = d, pa.m = m, pa.margin = margin ? 1 : 0;
   const bool vec = rows_vec16(d, m);
   pa.in = inout, pa.out = inout + m, pa.flag = flag, pa.f = f, pa.b = b, pa.fn = fn, pa.bn = bn, pa.changed = words;
-  pa.asked = asked, pa.label = label, pa.lose = lose, pa.scc_lose = scc_lose;
+  pa.asked = asked, pa.label = label, pa.lose = lose, pa.scc_lose = scc_lose, pa.status = status;
   {
     Launch L(ctx, stream, "propagation_init", double(m) * double(m) * 4.0);
-    if (!max_in) {
+    if (rows) {
+      const unsigned t = unsigned((m + 31) / 32);
+      transpose_kernel<<<dim3(t, t), 256, 0, stream>>>(d, m, dT);
+      rows_kernel<kInit><<<row_grid, 32 * kRowWarps, 0, stream>>>(pa, dT, nullptr, nullptr);
+    } else if (!max_in) {
       if (cudaMemsetAsync(inout, 0, 2 * size_t(m) * 4, stream) != cudaSuccess) return SCHULZE_ECUDA;
       (vec ? pair_kernel<kInit, true> : pair_kernel<kInit, false>)<<<pairs, 256, 0, stream>>>(pa);
     }
-    init_status_kernel<<<g, 256, 0, stream>>>(max_in ? max_in : pa.in, max_in ? max_out : pa.out, m, status);
+    if (!rows) init_status_kernel<<<g, 256, 0, stream>>>(max_in ? max_in : pa.in, max_in ? max_out : pa.out, m, status);
   }
   if (int rc = check_launch()) return rc;
   int32_t iterations = 0, rounds = 0;
   for (;;) {
     int32_t host[3] = {0, 0, 0};
-    if (cudaMemsetAsync(words, 0, 3 * sizeof(int32_t), stream) != cudaSuccess) return SCHULZE_ECUDA;
+    if (cudaMemsetAsync(words, 0, 4 * sizeof(int32_t), stream) != cudaSuccess) return SCHULZE_ECUDA;
     winners_out_kernel<<<g, 256, 0, stream>>>(status, m, winners, words + 2);
     if (cudaMemcpyAsync(host, words, sizeof(host), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
         cudaStreamSynchronize(stream) != cudaSuccess)
@@ -382,22 +486,33 @@ int winners_propagation_launch(schulze_ctx* ctx, const int32_t* d, int32_t m, bo
     preprocess_kernel<<<nbt, kPT, 0, stream>>>(status, m, f, b, fn, bn, flag, lose, scc_lose);
     // rounds until nothing changes; a chain of m candidates settles in m rounds
     for (int32_t r = 0; r <= m; ++r) {
-      int32_t changed = 0;
-      {
+      int32_t changed = 0, *word = words;
+      if (rows) {
+        Launch L(ctx, stream, "propagation_round", double(m) * double(m) * 8.0);
+        word = words + (r & 1 ? 3 : 0);
+        pa.f = f, pa.b = b, pa.fn = fn, pa.bn = bn;
+        rows_kernel<kPropagate><<<row_grid, 32 * kRowWarps, 0, stream>>>(pa, dT, word, words + (r & 1 ? 0 : 3));
+        std::swap(f, fn), std::swap(b, bn);
+      } else {
         Launch L(ctx, stream, "propagation_round", double(m) * double(m) * 4.0);
         (vec ? pair_kernel<kPropagate, true> : pair_kernel<kPropagate, false>)<<<pairs, 256, 0, stream>>>(pa);
         commit_kernel<<<nbt, kPT, 0, stream>>>(m, f, b, fn, bn, flag, words);
       }
       ++rounds;
-      if (cudaMemcpyAsync(&changed, words, sizeof(int32_t), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+      if (cudaMemcpyAsync(&changed, word, sizeof(int32_t), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
           cudaStreamSynchronize(stream) != cudaSuccess)
         return SCHULZE_ECUDA;
       if (!changed) break;
     }
     {
       Launch L(ctx, stream, "propagation_marks", double(m) * double(m) * 4.0);
-      label_kernel<<<nbt, kPT, 0, stream>>>(f, b, m, status, lose, asked, flag, label);
-      (vec ? pair_kernel<kMarks, true> : pair_kernel<kMarks, false>)<<<pairs, 256, 0, stream>>>(pa);
+      if (rows) {
+        pa.f = f, pa.b = b;
+        rows_kernel<kMarks><<<row_grid, 32 * kRowWarps, 0, stream>>>(pa, dT, nullptr, nullptr);
+      } else {
+        label_kernel<<<nbt, kPT, 0, stream>>>(f, b, m, status, lose, asked, flag, label);
+        (vec ? pair_kernel<kMarks, true> : pair_kernel<kMarks, false>)<<<pairs, 256, 0, stream>>>(pa);
+      }
     }
     apply_kernel<<<g, 256, 0, stream>>>(f, b, m, lose, scc_lose, status, words + 1);
     int32_t decided = 0;

@@ -188,6 +188,14 @@ def test_propagation_block_edges(m, top):
             assert stats == [it, rounds], (m, margin)
 
 
+@pytest.mark.parametrize("m", [257, 500, 1023, 1024, 1025, 1087, 1088, 1089, 1151])
+@pytest.mark.parametrize("top", [2000, 1 << 22])
+def test_propagation_rows_and_blocks(m, top):
+    """The same around the size from which the passes take pairs of blocks
+    instead of rows (m = 1025), at edges of the blocks."""
+    test_propagation_block_edges(m, top)
+
+
 # ------------------------------------------------------------ batch bit planes
 
 @pytest.mark.parametrize("per_tile", [1, 2, 4])

@@ -47,8 +47,8 @@
 // CPU, blocked Floyd-Warshall): 0.9% for Plackett-Luce Zipf(1.1) top-20 lists
 // at m = 8192, 3.7% at m = 2048, 4.6% for top-200 lists at m = 2048, 2.1% for
 // Mallows(0.98) full rankings and 92% for impartial culture at m = 1024. The
-// closure went from 390 to 8.4 ms at m = 16384 (int32, top-20, 0.7% of the
-// updates left) and from 309 to 9.7 ms at m = 18407 (int16, top-200, 4%); it
+// closure went from 390 to 8.4 ms at m = 16384 (int32, top-20, 0.75% of the
+// updates left, measured) and from 309 to 9.8 ms at m = 18407 (int16, top-200, 2.2%); it
 // is now bound by the chain diagonal tile - panel - next diagonal tile of
 // its 256 to 288 rounds (33 us each; 16 us where nothing else runs). Where
 // every update is needed (uniform random d, int32) the tests and bounds cost
@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(1024) relabel_kernel(const int32_t* __restrict
 // there, eight per thread: both passes over the matrix stay coalesced
 // whatever the order (gathering d's columns in strength order took 7.1 ms at
 // m = 16384, int32, a 32-byte sector per entry; weigh_kernel and this form
-// take 0.50 + 0.65 ms). Else (few warm
+// take 0.36 + 0.65 ms). Else (few warm
 // candidates) with x = perm[a] the threads read d[x][perm b] (along row x) and
 // d[perm b][x] (down column x); a candidate y without edges is one no ballot
 // lists, so d[y][x] = 0 and that read is skipped. `chunk` rows (of one tile
@@ -1599,7 +1599,7 @@ int closure_pipeline(schulze_ctx* ctx, int sms, const int32_t* d, int32_t m, int
   {
     // p is written from W (and the uniform cold values); with a side stream
     // it is written there while beaten_by and the ranking come out of W on
-    // stream, with at most four CTAs per SM so that those kernels find room
+    // stream, with at most two CTAs per SM so that those kernels find room
     const bool fork = side && bb_out && ctx && ctx->side_stream;
     cudaStream_t wst = stream;
     raise_smem(ctx, reinterpret_cast<const void*>(widen_kernel<E>));

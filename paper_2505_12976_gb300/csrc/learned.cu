@@ -172,7 +172,7 @@ constexpr int kFPacked = 0, kFNarrow = 1, kFWide = 2;
 // than kCertifyMaxWarm candidates, so the decision does not depend on the
 // order. On the dense profile of m = 18407 a tenth of the CTAs run, 662 ->
 // 134 us for the pass; the propagation then looks for the heaviest edges
-// itself, 315 us.
+// itself, 320 us.
 template <bool kVec, int kMode>
 __global__ void __launch_bounds__(256, kFMinBlocks) features_pass_kernel(const int32_t* __restrict__ d, int32_t m, Acc a,
                                                                          int32_t* __restrict__ seen) {

@@ -1232,7 +1232,12 @@ CompactPlan compact_plan(int64_t n, int32_t m, int32_t k, int sms, uint32_t flag
 bool choose_dense(int64_t n, int32_t m, int32_t k, uint32_t flags) {
   if (flags & SCHULZE_F_TALLY_DENSE) return true;
   if (flags & SCHULZE_F_TALLY_SPARSE) return false;
-  // dense costs ~ m^2 / 2 packed ops per ballot, sparse ~ 4 k^2 / 2
+  // Dense from k = m / 2 on: where packed 16-bit compares (m^2 / 2 operations a
+  // ballot) crossed the sparse form (about 2 k^2). On bit planes the two meet
+  // near k = m / 8 (dense against sparse, m = 1024, n = 20000: k = 102 407 and 285
+  // us, 204 445 and 994, 512 532 and 6000; m = 4096, n = 5000: k = 409 1774 and
+  // 1008, 819 1930 and 4262), so the line leaves time on the table between there
+  // and m / 2. A dense tally reports no candidates with edges (tally_gives_hint).
   return double(k) * double(k) * 4.0 > double(m) * double(m);
 }
 
